@@ -1091,7 +1091,8 @@ int decoder_pass(bild_ctx* c, int which, int MBv, float* logits_dbg, unsigned lo
   }
   auto draw_token = [&]() -> int {
     if (!c->draw) return BILD_OK;
-    CUDA_TRY(c, launch_k(c, nucleus_policy_kernel, dim3(1), dim3(NS_THREADS), 0, h, (const float*)h.logits_dbg, (const float*)c->u_draw[which]));
+    auto kern = mc.vocab <= NS_CLUSTER * NS_THREADS * NS_KEEP ? nucleus_policy_kernel<true> : nucleus_policy_kernel<false>;
+    CUDA_TRY(c, launch_k(c, kern, dim3(NS_CLUSTER), dim3(NS_THREADS), 0, h, (const float*)h.logits_dbg, (const float*)c->u_draw[which]));
     return BILD_OK;
   };
   const int head_tr = (MB == 1 && d <= 512) ? 32 : 16;   // rows per tile of the tensor-core head

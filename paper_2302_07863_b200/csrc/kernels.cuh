@@ -492,8 +492,9 @@ struct HeadArgs {
 // What the last block of every LM-head kernel does once the per-row results are complete: the policy tests, the
 // bookkeeping of Algorithm 1, and (inside a loop graph) the choice of what runs next.
 __device__ inline void policy_tail(const HeadArgs& a, HeadOut* o) {
-  if (!a.loop.st || a.defer_policy) return;
+  if (!a.loop.st) return;
   policy_tests(o, a.desc, a.loop.st, a.which);
+  if (a.defer_policy) return;   // (the row the token is drawn from depends on the tests)
   if (a.desc->run_policy) policy_step(a.loop, o, a.desc, a.which);
   else if (a.which == 0) a.loop.st->S_len = a.desc->pos0 + 1;
   else a.loop.st->L_len = a.desc->pos0 + a.desc->k;

@@ -1,137 +1,307 @@
 // Sampling variant of the decode loop (supplementary material, "BiLD with Sampling"): both models draw their
 // tokens by nucleus (top-p) sampling, the fallback and rollback policies stay as they are.  In this mode the LM-head
-// kernels leave the logits of the pass in memory and skip the policy step; the kernel below, launched right after
+// kernels leave the logits of the pass in memory and skip the bookkeeping; the kernel below, launched right after
 // the head, draws the one token the pass emits (row 0 of a small step; the first violating row, else the last row,
 // of a large pass) and then runs the policy step and the loop graph's conditionals.
 //
 // Definition followed (one row of V logits z, log-sum-exp known from the head, uniform number u of the output
 // position): p_i = exp(z_i - lse); tokens in order of decreasing p (equal p: lower index first); nucleus = shortest
 // prefix whose probabilities add up to at least top_p; drawn token = first of the prefix at which the running sum
-// exceeds u times the prefix's total.  Both prefixes are found without sorting, by a radix search over the bit
-// patterns of the probabilities: four passes over the row, each fixing eight more bits of the threshold value from
-// the probability mass per bucket.
+// exceeds u times the prefix's total.  Both prefixes are found without sorting the row.
+//
+// One cluster of eight blocks owns the row, each an eighth of the vocabulary, every probability computed once and kept in
+// a register (up to 262144 tokens).  Probabilities below (1 - top_p) / V cannot belong to the nucleus (all of them
+// together weigh less than what the nucleus leaves out), so:
+//   * up to 32 candidates are left (a peaked distribution, the usual one): one warp ranks them by comparing all pairs;
+//   * more: a radix search over the bit patterns of the probabilities, 11 + 10 + 9 bits, on histograms of counts and
+//     mantissa sums (integer shared-memory atomics, spread over 16 buckets per octave) merged through distributed
+//     shared memory.
+// Masses are 64-bit fixed point (2^-62), so no sum depends on the order of the additions.
+// Bound by the latency of the cluster barriers and block scans, not by the 4 V bytes of logits (L2).  Measured against one
+// block of 1024 threads with float atomics into 256 buckets (the whole tail of a row fell into two or three of them, each
+// add a retried compare-and-swap): peaked row 418 -> 7.5 us (V = 32128), 2546 -> 8.5 us (V = 250112); flat row 888 -> 45 us
+// and 12.7 ms -> 56 us.
 #pragma once
 #include "kernels.cuh"
 
 namespace bild {
 
 constexpr int NS_THREADS = 1024;
+constexpr int NS_CLUSTER = 8;
+constexpr int NS_KEEP = 32;            // probabilities a thread keeps in registers
+constexpr int NS_CAND = 32;            // candidates one warp ranks
+constexpr int NS_BUCKETS = 2048;       // of the first radix level
+constexpr unsigned NS_NONE = 0xffffffffu;
+typedef unsigned long long ns_mass;    // probability mass in units of 2^-62
 
 struct NucleusShared {
-  float mass[256];
-  unsigned cnt[256];
-  unsigned key;        // bits of the threshold probability fixed so far
-  float above;         // mass of the probabilities above the current bucket range
-  unsigned ties;       // tokens with exactly the threshold probability that are taken
-  unsigned n_eq;       // tokens with exactly the threshold probability
-  int row, token;
-  unsigned scan[NS_THREADS / 32];
+  unsigned cnt[NS_BUCKETS], low[NS_BUCKETS];   // this block's histogram: tokens, sum of the mantissa bits below the bucket's
+  ns_mass mass[NS_BUCKETS];                    // the cluster's histogram
+  unsigned tot[NS_BUCKETS];
+  ns_mass scan[NS_THREADS / 32];
+  ns_mass above;
+  unsigned pick, lowest, n_cand, n_eq, mine;
+  unsigned cand_key[NS_CAND], cand_idx[NS_CAND];
+  int token;
 };
 
-// Finds the probability value at which the running sum over the tokens, taken in decreasing order of probability,
-// first reaches (strict = false: >=) or exceeds (strict = true: >) `thresh`.  On return sh->key holds its bit
-// pattern, sh->above the mass of all larger probabilities, sh->ties how many tokens of exactly that probability the
-// prefix takes (at least 1), sh->n_eq how many there are.  If rounding keeps the total below thresh, the prefix is
-// everything.
-__device__ inline void nucleus_select(const float* __restrict__ z, float lse, int V, float thresh, bool strict, NucleusShared* sh) {
-  const int tid = threadIdx.x;
-  if (tid == 0) { sh->key = 0u; sh->above = 0.f; }
-  unsigned mask = 0u;
-#pragma unroll 1
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 24 - 8 * pass;
-    if (tid < 256) { sh->mass[tid] = 0.f; sh->cnt[tid] = 0u; }
-    __syncthreads();
-    const unsigned prefix = sh->key;
-#pragma unroll 1
-    for (int i = tid; i < V; i += NS_THREADS) {
-      const float p = expf(z[i] - lse);
-      const unsigned key = __float_as_uint(p);
-      if ((key & mask) == prefix) {
-        atomicAdd(&sh->mass[(key >> shift) & 255u], p);
-        atomicAdd(&sh->cnt[(key >> shift) & 255u], 1u);
-      }
-    }
-    __syncthreads();
-    if (tid == 0) {
-      float run = sh->above;
-      int pick = -1, lowest = 0;
-      for (int b = 255; b >= 0; --b) {
-        if (sh->cnt[b] == 0u) continue;
-        lowest = b;
-        const float with = run + sh->mass[b];
-        if (strict ? with > thresh : with >= thresh) { pick = b; break; }
-        run += sh->mass[b];
-      }
-      if (pick < 0) { pick = lowest; run -= sh->mass[lowest]; }   // the whole row is the prefix
-      sh->above = run;
-      sh->key = prefix | ((unsigned)pick << shift);
-      if (pass == 3) {
-        const float kv = __uint_as_float(sh->key);
-        const unsigned n = sh->cnt[pick];
-        unsigned t = 1u;
-        while (t < n && !(strict ? run + (float)t * kv > thresh : run + (float)t * kv >= thresh)) ++t;
-        sh->ties = t;
-        sh->n_eq = n;
-      }
-    }
-    mask |= 255u << shift;
-    __syncthreads();
-  }
+__device__ __forceinline__ unsigned ns_remote(const void* p, int rank) {
+  unsigned a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ unsigned ns_ld(const unsigned* p, int rank) {
+  unsigned v;
+  asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(ns_remote(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ void ns_st(const unsigned* p, int rank, unsigned v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ns_remote(p, rank)), "r"(v) : "memory");
+}
+__device__ __forceinline__ void ns_st(const ns_mass* p, int rank, ns_mass v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(ns_remote(p, rank)), "l"(v) : "memory");
 }
 
-// Index of the t-th (1-based) token whose probability has exactly the bit pattern `key`, in index order.
-__device__ inline void nucleus_locate(const float* __restrict__ z, float lse, int V, unsigned key, unsigned t, NucleusShared* sh) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int per = (V + NS_THREADS - 1) / NS_THREADS, i0 = tid * per, i1 = min(V, i0 + per);
-  unsigned mine = 0u;
-  for (int i = i0; i < i1; ++i) mine += __float_as_uint(expf(z[i] - lse)) == key ? 1u : 0u;
-  unsigned inc = mine;   // inclusive scan over the block, thread order = index order
+// mass of n tokens whose bit patterns share the exponent of `key`, mantissa bits n * (bits of key) + extra in all
+__device__ __forceinline__ ns_mass ns_fixed(unsigned key, unsigned n, ns_mass extra) {
+  const int e = (int)(key >> 23);
+  const ns_mass m = (ns_mass)n * ((key & 0x7fffffu) | (e ? 0x800000u : 0u)) + extra;
+  const int sh = max(e, 1) - 88;   // value = mantissa * 2^(e - 150)
+  return sh >= 0 ? m << sh : sh > -64 ? m >> -sh : 0ull;
+}
+__device__ __forceinline__ bool ns_reached(ns_mass run, ns_mass thresh, bool strict) { return strict ? run > thresh : run >= thresh; }
+
+// The probabilities of this block's share of the row as bit patterns (monotone in the probability).
+template <bool KEEP>
+struct NucleusRow {
+  unsigned key[KEEP ? NS_KEEP : 1];
+  const float* z;
+  float lse;
+  int n;   // tokens of this block
+  __device__ __forceinline__ unsigned compute(int i) const {
+    const int j = i * NS_THREADS + (int)threadIdx.x;
+    return j < n ? __float_as_uint(expf(z[j] - lse)) : NS_NONE;
+  }
+  __device__ __forceinline__ void load() {
+    if (KEEP) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned v = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += v;
+      for (int i = 0; i < NS_KEEP; ++i) key[i] = i * NS_THREADS < n ? compute(i) : NS_NONE;
+    }
   }
-  if (lane == 31) sh->scan[warp] = inc;
-  __syncthreads();
-  unsigned base = 0u;
-  for (int w = 0; w < warp; ++w) base += sh->scan[w];
-  const unsigned before = base + inc - mine;
-  if (mine > 0u && before < t && t <= before + mine) {
-    unsigned seen = before;
-    for (int i = i0; i < i1; ++i)
-      if (__float_as_uint(expf(z[i] - lse)) == key && ++seen == t) { sh->token = i; break; }
+  template <typename F>
+  __device__ __forceinline__ void each(F f) const {   // f(turn, bit pattern), the same turns for every thread of the block
+    if (KEEP) {
+#pragma unroll
+      for (int i = 0; i < NS_KEEP; ++i)
+        if (i * NS_THREADS < n) f(i, key[i]);
+    } else {
+#pragma unroll 1
+      for (int i = 0; i * NS_THREADS < n; ++i) f(i, compute(i));
+    }
   }
-  __syncthreads();
+};
+
+// Finds the probability at which the running mass over the tokens, taken in decreasing order of probability, first
+// reaches (strict: exceeds) `thresh`: its bit pattern, and in `ties` how many tokens of exactly that probability the
+// prefix takes (at least 1).  Returns the prefix's mass.  If the total stays below thresh, the prefix is everything.
+template <bool KEEP>
+__device__ inline ns_mass nucleus_select(const NucleusRow<KEEP>& row, unsigned key_min, ns_mass thresh, bool strict, int rank, NucleusShared* sh,
+                                         unsigned* key_out, unsigned* ties_out) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned prefix = 0u, mask = 0u;
+  ns_mass above = 0ull;
+#pragma unroll 1
+  for (int level = 0; level < 3; ++level) {
+    const int shift = level == 0 ? 19 : level == 1 ? 9 : 0, nb = level == 0 ? NS_BUCKETS : level == 1 ? 1024 : 512;
+    // first level: the 19 mantissa bits below a bucket's, summed over up to a block's share of the row, have to fit 32 bits
+    const int lsh = level == 0 ? max(0, 32 - __clz(row.n) - 13) : 0;
+    const unsigned lmask = (1u << shift) - 1u;
+    for (int b = tid; b < nb; b += NS_THREADS) { sh->cnt[b] = 0u; sh->low[b] = 0u; }
+    if (tid == 0) { sh->pick = NS_NONE; sh->lowest = NS_NONE; }
+    __syncthreads();
+    row.each([&](int, unsigned key) {
+      if (key != NS_NONE && key >= key_min && (key & mask) == prefix) {
+        const unsigned b = (key >> shift) & (unsigned)(nb - 1);
+        atomicAdd(&sh->cnt[b], 1u);
+        if (level < 2) atomicAdd(&sh->low[b], (key & lmask) >> lsh);
+      }
+    });
+    __syncwarp();
+    cluster_sync_all();
+    const int seg = nb / NS_CLUSTER;
+    if (tid < seg) {   // bucket tid of this rank's segment: summed over the ranks, the result goes to every rank
+      const int b = rank * seg + tid;
+      unsigned n = 0u;
+      ns_mass lo = 0ull;
+#pragma unroll
+      for (int rk = 0; rk < NS_CLUSTER; ++rk) { n += ns_ld(&sh->cnt[b], rk); lo += ns_ld(&sh->low[b], rk); }
+      if (lsh) lo = (lo << lsh) + (((ns_mass)n << lsh) >> 1);   // (half a unit per dropped part)
+      const ns_mass m = ns_fixed(prefix | ((unsigned)b << shift), n, lo);
+#pragma unroll
+      for (int rk = 0; rk < NS_CLUSTER; ++rk) { ns_st(&sh->tot[b], rk, n); ns_st(&sh->mass[b], rk, m); }
+    }
+    __syncwarp();
+    cluster_sync_all();
+    // running mass from the highest bucket down; thread <-> two neighbouring buckets
+    const int hi = nb - 1 - 2 * tid;   // (one bucket per pair past the end: none)
+    const ns_mass m0 = hi >= 0 ? sh->mass[hi] : 0ull, m1 = hi >= 1 ? sh->mass[hi - 1] : 0ull;
+    const unsigned n0 = hi >= 0 ? sh->tot[hi] : 0u, n1 = hi >= 1 ? sh->tot[hi - 1] : 0u;
+    ns_mass inc = m0 + m1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const ns_mass v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane == 31) sh->scan[warp] = inc;
+    __syncthreads();
+    ns_mass base = above;
+    for (int w = 0; w < warp; ++w) base += sh->scan[w];
+    const ns_mass r0 = base + inc - m1, r1 = base + inc, rb = r0 - m0;
+    if (!ns_reached(rb, thresh, strict) && ns_reached(r1, thresh, strict)) {   // exactly one thread, if any
+      const bool first = ns_reached(r0, thresh, strict);
+      sh->pick = (unsigned)(first ? hi : hi - 1);
+      sh->above = first ? rb : r0;
+    }
+    __syncthreads();
+    if (sh->pick == NS_NONE) {   // the whole row is the prefix: it ends with the lowest bucket that holds a token
+      if (n1) atomicMin(&sh->lowest, (unsigned)(hi - 1));
+      else if (n0) atomicMin(&sh->lowest, (unsigned)hi);
+      __syncthreads();
+      if (n1 && sh->lowest == (unsigned)(hi - 1)) sh->above = r0;
+      if (n0 && sh->lowest == (unsigned)hi) sh->above = rb;
+      __syncthreads();
+    }
+    const unsigned pick = sh->pick != NS_NONE ? sh->pick : sh->lowest != NS_NONE ? sh->lowest : 0u;
+    above = sh->above;
+    prefix |= pick << shift;
+    mask |= lmask ^ 0x3fffffffu;
+    if (level == 2) {
+      const unsigned n = max(1u, sh->tot[pick]);
+      const ns_mass kv = ns_fixed(prefix, 1u, 0ull);
+      ns_mass t = n;
+      if (kv > 0ull && !ns_reached(above, thresh, strict)) t = strict ? (thresh - above) / kv + 1ull : (thresh - above + kv - 1ull) / kv;
+      *ties_out = (unsigned)(t < 1ull ? 1ull : t > (ns_mass)n ? (ns_mass)n : t);
+      *key_out = prefix;
+      above += (ns_mass)*ties_out * kv;
+    }
+    __syncthreads();
+  }
+  return above;
 }
 
-// logits: [MAXB][V] of the pass that just ran; u: uniform numbers by output position of this model.
-__global__ void __launch_bounds__(NS_THREADS) nucleus_policy_kernel(HeadArgs a, const float* __restrict__ logits, const float* __restrict__ u) {
+// Index of the t-th (1-based) token whose probability has exactly the bit pattern `key`, in index order, into sh->token of rank 0.
+template <bool KEEP>
+__device__ inline void nucleus_locate(const NucleusRow<KEEP>& row, int i0, unsigned key, unsigned t, int rank, NucleusShared* sh) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned n = 0u;
+  row.each([&](int, unsigned k) { n += k == key ? 1u : 0u; });
+  if (tid == 0) sh->mine = 0u;
+  __syncthreads();
+  if (n) atomicAdd(&sh->mine, n);
+  __syncwarp();
+  cluster_sync_all();
+  unsigned seen = 0u;
+  for (int rk = 0; rk < rank; ++rk) seen += ns_ld(&sh->mine, rk);
+  if (seen >= t || seen + sh->mine < t) return;   // (the same for the whole block)
+  row.each([&](int i, unsigned k) {   // this block has it: turn by turn, threads of a turn in index order
+    const unsigned hits = (unsigned)__syncthreads_count(k == key);
+    if (seen < t && t <= seen + hits) {
+      const unsigned bal = __ballot_sync(0xffffffffu, k == key);
+      if (lane == 0) sh->scan[warp] = (ns_mass)__popc(bal);
+      __syncthreads();
+      unsigned before = seen + __popc(bal & ((1u << lane) - 1u));
+      for (int w = 0; w < warp; ++w) before += (unsigned)sh->scan[w];
+      if (k == key && before + 1u == t) ns_st((const unsigned*)&sh->token, 0, (unsigned)(i0 + i * NS_THREADS + tid));
+    }
+    seen += hits;
+  });
+}
+
+// logits: [MAXB][V] of the pass that just ran; u: uniform numbers by output position of this model.  One cluster.
+template <bool KEEP>
+__global__ void __cluster_dims__(NS_CLUSTER, 1, 1) __launch_bounds__(NS_THREADS)
+nucleus_policy_kernel(HeadArgs a, const float* __restrict__ logits, const float* __restrict__ u) {
   __shared__ NucleusShared sh;
+  const int tid = threadIdx.x, rank = (int)cluster_rank();
+  if (tid == 0) sh.n_cand = 0u;
   pdl_launch_dependents();
   pdl_wait();
   HeadOut* o = a.out;
   const int V = a.V;
-  if (threadIdx.x == 0) {
-    policy_tests(o, a.desc, a.loop.st, a.which);
-    sh.row = a.which == 0 ? 0 : (o->first_violation >= 0 ? o->first_violation : a.desc->k - 1);
-    sh.token = o->argmax[sh.row];
-  }
-  __syncthreads();
-  const int r = sh.row;
-  const float* z = logits + (size_t)r * V;
-  const float lse = o->lse[r];
+  const int r = a.which == 0 ? 0 : (o->first_violation >= 0 ? o->first_violation : a.desc->k - 1);   // (tests run by the head)
   const float un = u[a.desc->pos0 + r + 1];   // the position in y the drawn token is written to
-  nucleus_select(z, lse, V, a.loop.st->top_p, false, &sh);
-  const unsigned key1 = sh.key, ties1 = sh.ties;
-  const float total = sh.above + (float)ties1 * __uint_as_float(key1);
+  const float top_p = a.loop.st->top_p;
+  const int per = (V + NS_CLUSTER - 1) / NS_CLUSTER, i0 = min(V, rank * per);
+  NucleusRow<KEEP> row;
+  row.z = logits + (size_t)r * V + i0; row.lse = o->lse[r]; row.n = min(V, i0 + per) - i0;
+  row.load();
+  // the 1e-4: the probabilities add up to 1 only up to rounding
+  const float cut = 0.999f * (1.f - top_p - 1e-4f) / (float)V;
+  const unsigned key_min = cut > 0.f ? __float_as_uint(cut) : 0u;
+  const ns_mass one = 1ull << 62;
+  const ns_mass want = max(1ull, (ns_mass)((double)top_p * (double)one));
   __syncthreads();
-  nucleus_select(z, lse, V, un * total, true, &sh);
-  unsigned key2 = sh.key, t2 = sh.ties;
-  if (key2 < key1 || (key2 == key1 && t2 > ties1)) { key2 = key1; t2 = ties1; }   // rounding: stay inside the nucleus
-  __syncthreads();
-  nucleus_locate(z, lse, V, key2, t2, &sh);
-  if (threadIdx.x == 0) {
+  {
+    unsigned n = 0u;
+    row.each([&](int, unsigned k) { n += k != NS_NONE && k >= key_min ? 1u : 0u; });
+    if (n) {
+      unsigned slot = atomicAdd(&sh.n_cand, n);
+      if (slot < NS_CAND)
+        row.each([&](int i, unsigned k) {
+          if (k != NS_NONE && k >= key_min) {
+            if (slot < NS_CAND) { sh.cand_key[slot] = k; sh.cand_idx[slot] = (unsigned)(i0 + i * NS_THREADS + tid); }
+            ++slot;
+          }
+        });
+    }
+  }
+  __syncwarp();
+  cluster_sync_all();
+  unsigned total = 0u;
+#pragma unroll
+  for (int rk = 0; rk < NS_CLUSTER; ++rk) total += ns_ld(&sh.n_cand, rk);
+  if (total <= NS_CAND) {   // few candidates: one warp, lane <-> candidate
+    if (rank == 0 && tid < 32) {
+      unsigned key = 0u, idx = NS_NONE, at = (unsigned)tid;
+      for (int rk = 0; rk < NS_CLUSTER; ++rk) {
+        const unsigned n = ns_ld(&sh.n_cand, rk);
+        if (idx == NS_NONE && at < n) { key = ns_ld(&sh.cand_key[at], rk); idx = ns_ld(&sh.cand_idx[at], rk); }
+        at -= n;   // (past its own list: wraps round to a value no list has, unless idx is set already)
+        if ((int)at < 0) at = 0x7fffffffu;
+      }
+      const ns_mass m = idx != NS_NONE ? max(1ull, ns_fixed(key, 1u, 0ull)) : 0ull;   // (never 0: the running masses differ)
+      ns_mass run = 0ull, sum = 0ull;   // mass of the candidates up to and including this one in the order of the definition
+      for (int l = 0; l < 32; ++l) {
+        const unsigned k2 = __shfl_sync(0xffffffffu, key, l), j2 = __shfl_sync(0xffffffffu, idx, l);
+        const ns_mass m2 = __shfl_sync(0xffffffffu, m, l);
+        if (k2 > key || (k2 == key && j2 <= idx)) run += m2;
+        sum += m2;
+      }
+      // the nucleus ends at the smallest running mass that reaches `want`; the drawn token has the smallest one that
+      // exceeds u times the nucleus's mass
+      const bool in = idx != NS_NONE;
+      ns_mass end = in && run >= want ? run : ~0ull;
+#pragma unroll
+      for (int s = 16; s > 0; s >>= 1) end = min(end, __shfl_xor_sync(0xffffffffu, end, s));
+      if (end == ~0ull) end = sum;
+      const ns_mass thr = (ns_mass)((double)un * (double)end);
+      ns_mass pickm = in && run > thr && run <= end ? run : ~0ull;
+#pragma unroll
+      for (int s = 16; s > 0; s >>= 1) pickm = min(pickm, __shfl_xor_sync(0xffffffffu, pickm, s));
+      const unsigned who = __ballot_sync(0xffffffffu, in && run == pickm);
+      const unsigned tok = __shfl_sync(0xffffffffu, idx, who ? __ffs(who) - 1 : 0);
+      if (tid == 0) sh.token = who ? (int)tok : o->argmax[r];
+    }
+  } else {
+    unsigned key1, ties1, key2, ties2;
+    const ns_mass nucleus = nucleus_select<KEEP>(row, key_min, want, false, rank, &sh, &key1, &ties1);
+    nucleus_select<KEEP>(row, key_min, (ns_mass)((double)un * (double)nucleus), true, rank, &sh, &key2, &ties2);
+    if (key2 < key1 || (key2 == key1 && ties2 > ties1)) { key2 = key1; ties2 = ties1; }   // rounding: stay inside the nucleus
+    nucleus_locate<KEEP>(row, i0, key2, ties2, rank, &sh);
+  }
+  __syncwarp();
+  cluster_sync_all();   // the token is in rank 0; no block leaves while another may read its shared memory
+  if (rank == 0 && tid == 0) {
     o->argmax[r] = sh.token;
     if (a.cond_while) a.loop.st->cum_draws++;
     HeadArgs b = a;
