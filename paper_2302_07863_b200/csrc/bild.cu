@@ -756,10 +756,14 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   const bild_dec_layer& w = m.dec[l];
   const size_t kvoff = (size_t)l * H * dkv;
   AttnSubArgs a{};
-  a.desc = desc; a.eps = mc.ln_eps; a.d = d; a.I = I; a.H = H; a.dkv = dkv; a.dkv_shift = ilog2(dkv); a.C = C; a.c_shift = ilog2(C);
+  a.desc = desc; a.eps = mc.ln_eps; a.inv_d = 1.f / (float)d; a.d = d; a.I = I; a.H = H; a.dkv = dkv; a.dkv_shift = ilog2(dkv); a.C = C; a.c_shift = ilog2(C);
   a.mb = MB; a.err = &c->st->err;
   a.spin = c->spin_limit; a.skip_copies = c->debug_skip_copies ? 1 : 0;
   a.n_keys_dev = c->enc_len_dev;
+  // When the next kernel's blocks may start their requests.  Behind this kernel's token rows: its 64 KB a block otherwise queue in front
+  // of them (5-row pass 580 -> 552 us).  At once for a single row of more than 512 columns: the kernels are so short then that the
+  // requests would not be back in time (mT5-large 442 -> 416 us, T5-large 356 -> 354 us; 512 columns: 145 -> 135 us the other way).
+  a.early = MB == 1 && d > 512 ? 1 : 0;
   // S1-S3 / L1-L3 (layer 0: with S0 / L0, the rows come from the embedding table)
   if (l == 0 && c->fused_embed) {
     a.emb = (const __nv_bfloat16*)m.w.emb; a.tokens = m.desc->tokens + row0; a.vocab = mc.vocab;
@@ -769,7 +773,7 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   a.kc = m.selfK + kvoff * cap; a.vc = m.selfV + kvoff * cap; a.cap = cap; a.bias = m.dec_bias; a.bias_ld = cap; a.self = 1;
   const AttnSubPlan& pls = m.sub_self[MB == 1 ? 0 : 1];
   a.kc_keys = pls.kc; a.bias_len = pls.bias_len; a.red_keys = pls.red_keys;
-  a.L = attn_sub_layout(d, dkv, 3, C, MB, a.kc_keys, a.bias_len);
+  a.L = attn_sub_layout(d, dkv, 3, C, MB, a.kc_keys, a.bias_len, pls.late);
   CUDA_TRY(c, launch_sub(c, MB == 1 ? attn_sub_kernel<true> : attn_sub_kernel<false>, H * C, C, (size_t)a.L.total, a, !first_plain));
   int rc = after_self();
   if (rc) return rc;
@@ -780,11 +784,11 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   a.kc = m.crossK + kvoff * ecap; a.vc = m.crossV + kvoff * ecap; a.cap = ecap; a.bias = nullptr; a.bias_ld = 0; a.self = 0;
   const AttnSubPlan& plc = m.sub_cross[MB == 1 ? 0 : 1];
   a.kc_keys = plc.kc; a.bias_len = plc.bias_len; a.red_keys = plc.red_keys;
-  a.L = attn_sub_layout(d, dkv, 1, C, MB, a.kc_keys, a.bias_len);
+  a.L = attn_sub_layout(d, dkv, 1, C, MB, a.kc_keys, a.bias_len, plc.late);
   CUDA_TRY(c, launch_sub(c, MB == 1 ? attn_sub_kernel<true> : attn_sub_kernel<false>, H * C, C, (size_t)a.L.total, a));
   // S7-S8 / L7-L8
   FfnSubArgs f{};
-  f.desc = desc; f.eps = mc.ln_eps; f.d = d; f.F = Fd; f.gated = gated ? 1 : 0; f.mb = MB; f.spin = c->spin_limit;
+  f.desc = desc; f.eps = mc.ln_eps; f.inv_d = 1.f / (float)d; f.d = d; f.F = Fd; f.gated = gated ? 1 : 0; f.mb = MB; f.spin = c->spin_limit;
   f.err = &c->st->err; f.x_in = xc; f.x_out = x; f.gain = (const float*)w.ln3;
   f.Wi0 = (const __nv_bfloat16*)w.wi0; f.Wi1 = (const __nv_bfloat16*)w.wi1;
   f.Wfo1 = m.wfo_one + (size_t)l * (Fd / 8) * d; f.Wfo8 = m.wfo_blk + (size_t)l * (Fd / 8) * pack_wfo_dpad(d);
@@ -1888,7 +1892,7 @@ int bild_op_ffn_sublayer(const void* Wi0, const void* Wi1, const void* Wfo, cons
   auto kern = MB == 1 ? ffn_sub_kernel<true> : ffn_sub_kernel<false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) return BILD_ERR_CUDA;
   FfnSubArgs f{};
-  f.desc = o.desc; f.eps = eps; f.d = d; f.F = F; f.gated = gated ? 1 : 0; f.mb = MB; f.spin = SPIN_LIMIT; f.err = o.err;
+  f.desc = o.desc; f.eps = eps; f.inv_d = 1.f / (float)d; f.d = d; f.F = F; f.gated = gated ? 1 : 0; f.mb = MB; f.spin = SPIN_LIMIT; f.err = o.err;
   f.x_in = x_in; f.x_out = x_out; f.gain = gain; f.Wi0 = (const __nv_bfloat16*)Wi0; f.Wi1 = (const __nv_bfloat16*)Wi1; f.Wfo1 = wfo_one; f.Wfo8 = wfo_blk;
   f.nparts = np; f.L = ffn_sub_layout(d, F, gated, sms * np, sms, MB);
   for (int p = 0; p < np; ++p) {
@@ -1930,12 +1934,12 @@ int bild_op_attn_sublayer(int self, const void* Wp, const void* Wo, const float*
   auto kern = MB == 1 ? attn_sub_kernel<true> : attn_sub_kernel<false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) return BILD_ERR_CUDA;
   AttnSubArgs a{};
-  a.desc = o.desc; a.eps = eps; a.d = d; a.I = I; a.H = H; a.dkv = dkv; a.dkv_shift = ilog2(dkv); a.C = C; a.c_shift = ilog2(C);
+  a.desc = o.desc; a.eps = eps; a.inv_d = 1.f / (float)d; a.d = d; a.I = I; a.H = H; a.dkv = dkv; a.dkv_shift = ilog2(dkv); a.C = C; a.c_shift = ilog2(C);
   a.kc_keys = kc_keys; a.bias_len = bias_len; a.red_keys = pl.red_keys; a.mb = MB; a.err = o.err; a.spin = SPIN_LIMIT; a.skip_copies = 0;
   a.n_keys_dev = o.nkeys; a.x_in = x_in; a.x_out = x_out; a.x_zero = o.zero; a.gain = gain;
   a.Wp = (const __nv_bfloat16*)Wp; a.Wo = (const __nv_bfloat16*)Wo; a.kc = kc; a.vc = vc; a.cap = cap;
   a.bias = bias_by_dist; a.bias_ld = cap; a.self = self ? 1 : 0;
-  a.L = attn_sub_layout(d, dkv, P, C, MB, kc_keys, bias_len);
+  a.L = attn_sub_layout(d, dkv, P, C, MB, kc_keys, bias_len, pl.late);
   if (launch_sub(&tmp, kern, H * C, C, (size_t)a.L.total, a) != cudaSuccess) return BILD_ERR_CUDA;
   return op_finish(s, o);
 }

@@ -4,15 +4,14 @@
 //     for self-attention, S4-S6 / L4-L6 for cross-attention).  A cluster of C blocks owns one head:
 //     rank r multiplies its share of the head's q|k|v rows (weights fetched by bulk copies BEFORE
 //     the dependency wait of the programmatic launch), the cluster exchanges the k x 3 x d_kv results
-//     through distributed shared memory, rank r then attends over its share of the keys, the
+//     through distributed shared memory (asynchronous stores that an mbarrier counts), rank r then attends over its share of the keys, the
 //     per-rank (max, sum, weighted values) records are exchanged the same way, and every rank
 //     multiplies the merged head output with its share of the rows of W_o's column slice; while a head has few keys
 //     (they fit one staged chunk) every rank attends over all of them instead and the second exchange falls away;
 //     the first kernel of a pass takes its rows from the embedding table (S0 / L0);
 //   * ffn_sub_kernel: x_out = x_in + W_fo * act(W_i * rms_norm(x_in))   (S7-S8 / L7-L8).  Block b owns a
-//     slice of d_ff (a multiple of 8 rows): the rows of W_i (and of the gate matrix) in shared memory and the
-//     matching columns of W_fo in registers (from a copy laid out in load order), so the hidden activations never
-//     leave the block.
+//     slice of d_ff (a multiple of 8 rows): the rows of W_i (and of the gate matrix) and the matching columns of W_fo
+//     (from a copy laid out in load order), so the hidden activations never leave the block.
 // Both kernels produce partial sums over heads / slices of d_ff of the d_model outputs.  They are added
 // into x_out with vector reductions at the L2 (red.global.add); x_out was zeroed by the kernel before the
 // previous one, one designated block adds x_in (the residual term), and every kernel zeroes the buffer
@@ -24,18 +23,16 @@
 namespace bild {
 
 constexpr int SUB_THREADS = 256;
-constexpr int SUB_PSUM = SL_PSUM;   // bytes of partial sums of sl_items / sl_mma
 constexpr int SUB_RECPAD = 4;       // record of a rank and row = [max, sum, -, -, values[d_kv]]
-constexpr int SUB_MAX_ROWS = 4 * SL_QUADS;   // weight rows of one block and phase (limit of sl_items / sl_mma)
+constexpr int SUB_MAX_ROWS = 48;             // weight rows of one block and phase: three 16-row tiles
 constexpr int SUB_FO_REGS = 32;              // most rows of d_ff a block takes: its columns of W_fo fill 64 registers of a thread
 constexpr int SUB_HALF_SM = 113 * 1024;      // shared memory of a block that leaves room for a second one on the SM
 constexpr int SUB_MB = 8;                    // token rows of the block variant (one 8-token tile of the tensor-core instruction)
 
 struct SubShared {
-  unsigned long long wbar;
-  float inv[MAXB];
-  float ssq[8][MAXB];
-  float rmax[MAXB], rsum[MAXB], rscale[MAXB];
+  unsigned long long wbar;      // weight copies
+  unsigned long long xbar[2];   // exchanges within the cluster
+  float ssq[8][SUB_MB];         // the warps' sums of squares of the token rows
   int failed;
 };
 
@@ -78,7 +75,6 @@ __device__ __forceinline__ void sub_wait(SubShared* sh, int* err, unsigned long 
   atomicExch(err, (int)BILD_ERR_TIMEOUT);
 }
 
-__device__ __forceinline__ void sub_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 // (nothing to publish: does not wait for the loads in flight)
 __device__ __forceinline__ void sub_cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void sub_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -86,159 +82,232 @@ __device__ __forceinline__ void sub_cp16(void* dst_smem, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void sub_cp_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// dot product (weight row `row`, token row m) from the partial sums of sl_items<1> (ONE) or sl_mma<1>, added in warp order
-template <bool ONE>
-__device__ __forceinline__ float sub_total(const float* psum, int row, int m, int nrows, int K) {
-  float t = 0.f;
-  if (ONE) {
-    const int nkb = (K + 255) >> 8, qd = row >> 2, first = qd * nkb;
-    const float* p = psum + (size_t)(qd * 8) * 32 + (row & 3);
-#pragma unroll
-    for (int wv = 0; wv < 8; ++wv)
-      if (((wv - first) & 7) < nkb) t += p[wv * 32];   // warp wv took part in this quad
-  } else {   // fragment layout of the instruction: row = group (+ 8), token = 2 * (lane & 3) (+ 1); one tile of 8 tokens
-    const int MT = (nrows + 15) >> 4, ks_sh = MT == 1 ? 3 : MT == 2 ? 2 : 1;
-    const int mt = row >> 4, rr = row & 15;
-    const float* p = psum + ((size_t)(mt << ks_sh) * 32 + (rr & 7) * 4 + (m >> 1)) * 4 + (rr >> 3) * 2 + (m & 1);
-    float v[8];
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) v[ks] = ks < (1 << ks_sh) ? p[(size_t)ks * 128] : 0.f;   // loads side by side
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) t += v[ks];
-  }
-  return t;
+__device__ __forceinline__ bool sub_try_cluster(uint32_t bar, uint32_t parity) {   // (what the cluster's other blocks wrote is visible after it)
+  uint32_t ok;
+  asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+// Wait for the values the cluster's blocks store into this one (sub_push).  Every block sends its part after bounded waits of
+// its own, so the limit here is only a last bound, above theirs.
+__device__ __forceinline__ void sub_wait_exchange(SubShared* sh, int* err, unsigned long long* bar, unsigned spin) {
+  const uint32_t b = smem_u32(bar);
+  const unsigned lim = (spin > SPIN_LIMIT ? spin : SPIN_LIMIT) * 4u;
+  for (unsigned it = 0; it < lim; ++it)
+    if (sub_try_cluster(b, 0)) return;
+  sh->failed = 1;
+  atomicExch(err, (int)BILD_ERR_TIMEOUT);
+}
+// Stores into the shared memory of block `rank` of the cluster that count down the bytes its mbarrier `bar` expects: the
+// receiver waits for the bytes, nobody for a cluster-wide barrier with its release of everything written before (which cost
+// 883 cycles per exchange against 510 of these stores, eight blocks, 192 values each to everyone).
+__device__ __forceinline__ uint32_t sub_mapa(uint32_t a, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void sub_push(const float* dst, const unsigned long long* bar, uint32_t rank, float v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+               ::"r"(sub_mapa(smem_u32(dst), rank)), "r"(__float_as_uint(v)), "r"(sub_mapa(smem_u32(bar), rank)) : "memory");
+}
+__device__ __forceinline__ void sub_push4(const float* dst, const unsigned long long* bar, uint32_t rank, float4 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(sub_mapa(smem_u32(dst), rank)), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
+               "r"(__float_as_uint(v.w)), "r"(sub_mapa(smem_u32(bar), rank)) : "memory");
 }
 
-// Token rows, after the dependency wait (d <= 1024: one 128-bit load per thread and row).  The loads are issued first
-// thing after the wait, for the rows of the pass (the row count is read before the wait); sub_rows_finish then writes
-// x * gain into Xs and 1 / rms into
-// sh->inv (returned for the single row of ONE).  The raw values of the columns [seed0, seed1) (multiples of 4) also go
-// to sSeed[m][column - seed0]: the residual term the block adds.
-// Block variant: the normalised token rows wait in shared memory as bf16 heads [SUB_MB][d / 2 + 4] (two values a word)
-// followed by their bf16 remainders in the same layout: d + 8 words a row in all, as for the fp32 rows of the single-row
-// variant.  The row stride of d / 2 + 4 words is 4 times an odd number for d a multiple of 32: the eight rows a warp
-// reads side by side fall into different banks.
-__host__ __device__ inline int sub_split_stride(int d) { return (d >> 1) + 4; }
-
-// Products of up to 48 weight rows (shared memory, row stride rowst bytes) with the token rows on mma.sync m16n8k16, one tile
-// of 8 token rows: warp w works on row tile w / KS and on the w % KS-th part of K (KS = 8, 4 or 2 for 1, 2 or 3 row tiles),
-// as sl_mma<1>, with the right operand read ready-made; partial sums in the same place and layout (sub_total<false>).
-__device__ __forceinline__ void sub_mma_split(const unsigned char* sW, int rowst, int nrows, int K, const float* Xs, int mg, float* psum,
-                                              int warp, int lane) {
-  const int MT = (nrows + 15) >> 4, ks_sh = MT == 1 ? 3 : MT == 2 ? 2 : 1, KS = 1 << ks_sh;
-  if (warp >= MT * KS) return;
-  const int mt = warp >> ks_sh, ks = warp & (KS - 1);
-  const int steps = K >> 4, per = (steps + KS - 1) >> ks_sh;   // K is a multiple of 16 here
-  const int s0 = ks * per, s1 = min(steps, s0 + per);
-  const int g = lane >> 2, t = lane & 3, hw = sub_split_stride(K);
-  const unsigned char* pa0 = sW + (size_t)min(mt * 16 + g, nrows - 1) * rowst + t * 4;
-  const unsigned char* pa1 = sW + (size_t)min(mt * 16 + g + 8, nrows - 1) * rowst + t * 4;
-  const uint32_t* xh = reinterpret_cast<const uint32_t*>(Xs) + (size_t)min(g, mg - 1) * hw + t;
-  const uint32_t* xl = xh + (size_t)SUB_MB * hw;
-  float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};   // heads and remainders: two independent chains
-#pragma unroll 4
-  for (int st = s0; st < s1; ++st) {
-    const int k0 = st << 4;
-    const uint32_t a0 = *reinterpret_cast<const uint32_t*>(pa0 + k0 * 2), a1 = *reinterpret_cast<const uint32_t*>(pa1 + k0 * 2);
-    const uint32_t a2 = *reinterpret_cast<const uint32_t*>(pa0 + k0 * 2 + 16), a3 = *reinterpret_cast<const uint32_t*>(pa1 + k0 * 2 + 16);
-    const uint32_t h0 = xh[k0 >> 1], h1 = xh[(k0 >> 1) + 4], l0 = xl[k0 >> 1], l1 = xl[(k0 >> 1) + 4];
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(h0), "r"(h1));
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(e[0]), "+f"(e[1]), "+f"(e[2]), "+f"(e[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(l0), "r"(l1));
-  }
-  *reinterpret_cast<float4*>(psum + ((size_t)warp * 32 + lane) * 4) = make_float4(c[0] + e[0], c[1] + e[1], c[2] + e[2], c[3] + e[3]);
+__device__ __forceinline__ void sub_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+__device__ __forceinline__ void sub_mma8(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
+  asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(b0));
+}
+// two fp32 values as a pair of bf16 heads and a pair of bf16 remainders
+__device__ __forceinline__ void sub_split(float x, float y, uint32_t& h, uint32_t& l) {
+  h = sl_pack_bf16(x, y);
+  l = sl_pack_bf16(x - __uint_as_float(h << 16), y - __uint_as_float(h & 0xffff0000u));
+}
+// ... and as three (24 mantissa bits: the fp32 values themselves)
+__device__ __forceinline__ void sub_split3(float x, float y, uint32_t& h, uint32_t& m, uint32_t& l) {
+  h = sl_pack_bf16(x, y);
+  const float rx = x - __uint_as_float(h << 16), ry = y - __uint_as_float(h & 0xffff0000u);
+  m = sl_pack_bf16(rx, ry);
+  l = sl_pack_bf16(rx - __uint_as_float(m << 16), ry - __uint_as_float(m & 0xffff0000u));
+}
+
+// ------------------------------------------------------------------------------------------------
+// Products of a block's weight rows with the token rows
+// ------------------------------------------------------------------------------------------------
+// Warp w owns the columns [w CW, (w + 1) CW) of every row (CW = 32 x sub_chunks(d), 128 for d = 1024): it fetches that slice of
+// the token rows from the L2, multiplies it with the norm gain, splits it into bf16 parts in its own piece of shared memory
+// and multiplies it with its slice of the weight rows on mma.sync m16n8k16 -- no block barrier between the token rows and the
+// products; the one barrier behind the products covers the eight warps' partial sums and their sums of squares (1 / rms is a
+// factor of the sums).  Within a chunk of 32 columns the instruction's column positions are dealt so that a lane's 16-byte load
+// holds the operands of two instructions (position 2 t, 2 t + 1 | 2 t + 8, 2 t + 9 of instruction i <-> columns
+// 8 t + 4 i + 0, 1 | 2, 3), weights and token rows alike.
+// A single token row is three columns of the right operand: its bf16 head, remainder and second remainder, so the products are
+// those of the fp32 row at one instruction per 16 x 16 weights (multiply-adds with a warp reduction took twice the time of
+// rows + norm + products together: 2.2 -> 1.1 us per attention kernel of the large model).
+// A block of token rows is multiplied twice, heads and remainders, into two accumulator chains.
+__host__ __device__ inline int sub_chunks(int d) { return ((d + 31) / 32 + 7) / 8; }                 // 32-column chunks per warp: 1..4
+__host__ __device__ inline int sub_wst(int d) { return (d * 2 + 127) / 128 * 128 + 64; }            // bytes from weight row to weight row: 64 mod 128
+__host__ __device__ inline int sub_xst(int d) { return (d / 2 + 31) / 32 * 32 + 16; }               // words from token row to token row: 16 mod 32
+__host__ __device__ inline int sub_pst(int rows) { return (rows + 15) / 16 * 16 + 4; }              // floats of partial sums per token: 2 p = 8 mod 32
+__host__ __device__ inline int sub_xs_bytes(int d, int mb) { return (mb == 1 ? 3 : 2 * SUB_MB) * sub_xst(d) * 4; }
+__host__ __device__ inline int sub_psum_bytes(int rows, int mb) { return 8 * (mb == 1 ? 1 : SUB_MB) * sub_pst(rows) * 4; }
 
 template <bool ONE>
 struct SubRows { float4 v[ONE ? 1 : SUB_MB]; };
 
+// this lane's four columns of the token rows (after the dependency wait)
 template <bool ONE>
-__device__ __forceinline__ void sub_rows_issue(const float* __restrict__ x_in, int rows, int d, int tid, SubRows<ONE>& rw) {
-  if (tid * 4 < d) {   // rows: the rows of the pass
+__device__ __forceinline__ void sub_rows_issue(const float* __restrict__ x_in, int rows, int d, int col, bool on, SubRows<ONE>& rw) {
 #pragma unroll
-    for (int i = 0; i < (ONE ? 1 : SUB_MB); ++i)
-      if (i < rows) rw.v[i] = __ldcg(reinterpret_cast<const float4*>(x_in + (size_t)i * d) + tid);
-  }
+  for (int i = 0; i < (ONE ? 1 : SUB_MB); ++i)
+    if (on && i < rows) rw.v[i] = __ldcg(reinterpret_cast<const float4*>(x_in + (size_t)i * d + col));
 }
 
 // The first sub-layer of a pass takes its rows from the embedding table (S0 / L0): row i = E[token_i], bf16.
 template <bool ONE>
 __device__ __forceinline__ void sub_rows_embed(const __nv_bfloat16* __restrict__ E, const int* __restrict__ tokens, int vocab, int rows,
-                                               int d, int tid, SubRows<ONE>& rw) {
-  if (tid * 4 < d) {
+                                               int d, int col, bool on, SubRows<ONE>& rw) {
 #pragma unroll
-    for (int i = 0; i < (ONE ? 1 : SUB_MB); ++i)
-      if (i < rows) {
-        int t = tokens[i];
-        t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
-        const uint2 w = __ldg(reinterpret_cast<const uint2*>(E + (size_t)t * d) + tid);
-        rw.v[i] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
-                              __uint_as_float(w.y & 0xffff0000u));
-      }
-  }
+  for (int i = 0; i < (ONE ? 1 : SUB_MB); ++i)
+    if (on && i < rows) {
+      int t = tokens[i];
+      t = t < 0 ? 0 : (t >= vocab ? vocab - 1 : t);
+      const uint2 w = __ldg(reinterpret_cast<const uint2*>(E + (size_t)t * d + col));
+      rw.v[i] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                            __uint_as_float(w.y & 0xffff0000u));
+    }
 }
 
+// Splits x * gain into the warp's slice of Xs and leaves the warp's sums of squares in sh->ssq.  Xs: [part][row] rows of
+// sub_xst(d) words; `stores`: this lane's columns lie in the warp's slice, `on`: and inside the rows.  The raw values of the
+// columns [seed0, seed1) go to sSeed[m][column - seed0]: the residual term the block adds.
 template <bool ONE>
-__device__ __forceinline__ float sub_rows_finish(const SubRows<ONE>& rw, int k, int d, float4 g, float eps, float* Xs, int xst,
-                                                 SubShared* sh, float* sSeed, int seed0, int seed1, int tid, int lane, int warp) {
-  const int d4 = d >> 2, c = tid * 4;
-  const bool on = tid < d4, sd = c >= seed0 && c < seed1;
-  if (ONE) {
-    float ss = 0.f;
-    if (on) {
-      float4 w = rw.v[0];
-      ss = w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
-      if (sd) *reinterpret_cast<float4*>(sSeed + (c - seed0)) = w;
+__device__ __forceinline__ void sub_rows_split(const SubRows<ONE>& rw, int k, int col, bool stores, bool on, float4 g, uint32_t* Xs, int xst,
+                                               SubShared* sh, float* sSeed, int seed0, int seed1, int lane, int warp) {
+  const bool sd = on && col >= seed0 && col < seed1;
+  float q[ONE ? 1 : SUB_MB];
+#pragma unroll
+  for (int i = 0; i < (ONE ? 1 : SUB_MB); ++i) {
+    q[i] = 0.f;
+    if (stores && i < k) {
+      float4 w = on ? rw.v[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      q[i] = w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
+      if (sd) *reinterpret_cast<float4*>(sSeed + (size_t)i * (seed1 - seed0) + (col - seed0)) = w;
       w.x *= g.x; w.y *= g.y; w.z *= g.z; w.w *= g.w;
-      *reinterpret_cast<float4*>(Xs + c) = w;
+      uint32_t h0, h1, l0, l1, m0, m1;
+      if (ONE) {
+        sub_split3(w.x, w.y, h0, m0, l0); sub_split3(w.z, w.w, h1, m1, l1);
+        *reinterpret_cast<uint2*>(Xs + xst + (col >> 1)) = make_uint2(m0, m1);
+        *reinterpret_cast<uint2*>(Xs + 2 * xst + (col >> 1)) = make_uint2(l0, l1);
+      } else {
+        sub_split(w.x, w.y, h0, l0); sub_split(w.z, w.w, h1, l1);
+        *reinterpret_cast<uint2*>(Xs + (size_t)(SUB_MB + i) * xst + (col >> 1)) = make_uint2(l0, l1);
+      }
+      *reinterpret_cast<uint2*>(Xs + (size_t)i * xst + (col >> 1)) = make_uint2(h0, h1);
     }
-    ss = warp_sum(ss);
-    if (lane == 0) sh->ssq[warp][0] = ss;
-    __syncthreads();
-    ss = 0.f;
-#pragma unroll
-    for (int wv = 0; wv < 8; ++wv) ss += sh->ssq[wv][0];
-    return rsqrtf(ss / (float)d + eps);
+  }
+  if (ONE) {
+    const float s = warp_sum(q[0]);
+    if (lane == 0) sh->ssq[warp][0] = s;
   } else {
-    float q[SUB_MB];
+    float qq[SUB_MB];
 #pragma unroll
-    for (int i = 0; i < SUB_MB; ++i) {
-      q[i] = 0.f;
-      if (on && i < k) {
-        float4 w = rw.v[i];
-        q[i] = w.x * w.x + w.y * w.y + w.z * w.z + w.w * w.w;
-        if (sd) *reinterpret_cast<float4*>(sSeed + (size_t)i * (seed1 - seed0) + (c - seed0)) = w;
-        w.x *= g.x; w.y *= g.y; w.z *= g.z; w.w *= g.w;
-        // stored as bf16 heads and bf16 remainders, the form the tensor-core products read (sub_mma_split)
-        const uint32_t h0 = sl_pack_bf16(w.x, w.y), h1 = sl_pack_bf16(w.z, w.w);
-        const uint32_t l0 = sl_pack_bf16(w.x - __uint_as_float(h0 << 16), w.y - __uint_as_float(h0 & 0xffff0000u));
-        const uint32_t l1 = sl_pack_bf16(w.z - __uint_as_float(h1 << 16), w.w - __uint_as_float(h1 & 0xffff0000u));
-        uint32_t* xh = reinterpret_cast<uint32_t*>(Xs);
-        const int hw = sub_split_stride(d);
-        *reinterpret_cast<uint2*>(xh + (size_t)i * hw + 2 * tid) = make_uint2(h0, h1);
-        *reinterpret_cast<uint2*>(xh + (size_t)(SUB_MB + i) * hw + 2 * tid) = make_uint2(l0, l1);
+    for (int i = 0; i < SUB_MB; ++i) qq[i] = q[ONE ? 0 : i];
+    const float r8 = treduce<SUB_MB>(qq, lane);   // lanes 4 i hold the warp's sum of row i
+    if ((lane & 3) == 0) sh->ssq[warp][lane >> 2] = r8;
+  }
+  __syncwarp();
+}
+// 1 / x to the last bit but one: the hardware's approximation and a Newton step (a full division is a chain several times as long)
+__device__ __forceinline__ float sub_rcp(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r * (2.f - x * r);
+}
+// 1 / rms of token row m from the warps' sums of squares (after the barrier behind the products)
+__device__ __forceinline__ float sub_inv(const SubShared* sh, int m, float inv_d, float eps) {
+  float s[8];
+#pragma unroll
+  for (int w = 0; w < 8; ++w) s[w] = sh->ssq[w][m];
+  return rsqrtf((((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]))) * inv_d + eps);
+}
+
+// the left operands of this warp's slice of the 16-row tile `mt` (chunks past the end of the rows: zero)
+__device__ __forceinline__ void sub_frags(const unsigned char* sW, int wst, int nrows, int d, int mt, int col0, int nch, int lane, uint4 (&f)[4][2]) {
+  const int g = lane >> 2, t = lane & 3;
+  const unsigned char* p0 = sW + (size_t)min(mt * 16 + g, nrows - 1) * wst + (col0 + 8 * t) * 2;
+  const unsigned char* p1 = sW + (size_t)min(mt * 16 + g + 8, nrows - 1) * wst + (col0 + 8 * t) * 2;
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch) {
+    const bool in = ch < nch && col0 + ch * 32 + 8 * t < d;
+    f[ch][0] = in ? *reinterpret_cast<const uint4*>(p0 + ch * 64) : make_uint4(0u, 0u, 0u, 0u);
+    f[ch][1] = in ? *reinterpret_cast<const uint4*>(p1 + ch * 64) : make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+// the right operands: the warp's slice of the token rows
+template <bool ONE> struct SubB { uint4 h[4], l[ONE ? 1 : 4]; };
+template <bool ONE>
+__device__ __forceinline__ void sub_bfrags(const uint32_t* Xs, int xst, int k, int col0, int nch, int lane, SubB<ONE>& b) {
+  const int g = lane >> 2, t = lane & 3;
+  const uint32_t* p = Xs + (size_t)min(g, (ONE ? 3 : k) - 1) * xst + (col0 >> 1) + 4 * t;
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch)
+    if (ch < nch) {
+      b.h[ch] = *reinterpret_cast<const uint4*>(p + ch * 16);
+      if (!ONE) b.l[ONE ? 0 : ch] = *reinterpret_cast<const uint4*>(p + (size_t)SUB_MB * xst + ch * 16);
+    }
+}
+// one 16-row tile; the warp's partial sums go to psum [warp][token][sub_pst(rows)]
+template <bool ONE>
+__device__ __forceinline__ void sub_tile(const uint4 (&f)[4][2], const SubB<ONE>& b, int nch, int nrows, int mt, float* psum, int warp, int lane) {
+  const int g = lane >> 2, t = lane & 3, pst = sub_pst(nrows), row = mt * 16 + g;
+  float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int ch = 0; ch < 4; ++ch)
+    if (ch < nch) {
+      const uint4 a0 = f[ch][0], a1 = f[ch][1];
+      sub_mma(c, a0.x, a1.x, a0.y, a1.y, b.h[ch].x, b.h[ch].y);
+      if (ONE) {
+        sub_mma(e, a0.z, a1.z, a0.w, a1.w, b.h[ch].z, b.h[ch].w);
+      } else {
+        sub_mma(e, a0.x, a1.x, a0.y, a1.y, b.l[ONE ? 0 : ch].x, b.l[ONE ? 0 : ch].y);
+        sub_mma(c, a0.z, a1.z, a0.w, a1.w, b.h[ch].z, b.h[ch].w);
+        sub_mma(e, a0.z, a1.z, a0.w, a1.w, b.l[ONE ? 0 : ch].z, b.l[ONE ? 0 : ch].w);
       }
     }
-    const float r8 = treduce<8>(q, lane);   // lanes 4 i hold the warp's sum of row i
-    if ((lane & 3) == 0) sh->ssq[warp][lane >> 2] = r8;
-    __syncthreads();
-    if (tid < k) {
-      float ss = 0.f;
 #pragma unroll
-      for (int wv = 0; wv < 8; ++wv) ss += sh->ssq[wv][tid];
-      sh->inv[tid] = rsqrtf(ss / (float)d + eps);
+  for (int i = 0; i < 4; ++i) c[i] += e[i];
+  if (ONE) {   // accumulator columns 0, 1 (lane t = 0) and 2 (lane t = 1): the three parts of the token row
+    const float z0 = __shfl_down_sync(0xffffffffu, c[0], 1), z2 = __shfl_down_sync(0xffffffffu, c[2], 1);
+    if (t == 0) {
+      psum[(size_t)warp * pst + row] = c[0] + c[1] + z0;
+      psum[(size_t)warp * pst + row + 8] = c[2] + c[3] + z2;
     }
-    __syncthreads();
-    return 0.f;
+  } else {
+    float* p = psum + (size_t)(warp * SUB_MB + 2 * t) * pst + row;
+    p[0] = c[0]; p[pst] = c[1]; p[8] = c[2]; p[pst + 8] = c[3];
   }
+}
+// dot product (weight row, token row) over all warps, in a fixed order
+template <bool ONE>
+__device__ __forceinline__ float sub_total(const float* psum, int row, int m, int pst) {
+  const float* p = psum + (size_t)m * pst + row;
+  float v[8];
+#pragma unroll
+  for (int w = 0; w < 8; ++w) v[w] = p[w * (ONE ? 1 : SUB_MB) * pst];   // (a warp without columns left zeros)
+  return ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
 }
 
 // ------------------------------------------------------------------------------------------------
 // Attention sub-layer
 // ------------------------------------------------------------------------------------------------
-struct AttnSubLayout { int wq, xs, kv, kv_late, qkv, psum, probs, bias, seed, sa, red, recloc, loc, out, sh, total; };
+struct AttnSubLayout { int wq, kv, kv_late, xs, rec, rrec, qkv, psum, sa, out, bias, seed, sh, total; };
 
 struct AttnSubArgs {
   const CallDesc* desc;
@@ -249,7 +318,7 @@ struct AttnSubArgs {
   float* x_out;         // [MAXB][d] zero on entry; receives x_in + the sub-layer's output
   float* x_zero;        // [MAXB][d] cleared for the kernel after this one
   const float* gain;
-  float eps;
+  float eps, inv_d;          // inv_d: 1 / d
   const __nv_bfloat16* Wp;   // self: [3 I][d] (q rows, then k, then v); cross: [I][d]
   const __nv_bfloat16* Wo;   // [d][I]
   float* kc;                 // [H][cap][dkv] keys of this layer (self: rows pos0.. are appended; cross: read only)
@@ -266,6 +335,7 @@ struct AttnSubArgs {
   int mb;                    // token rows the shared memory is sized for
   unsigned spin;             // polls of the weight barrier before the kernel gives up
   int skip_copies;           // test of the time-out path: the weight copies are announced but not issued
+  int early;                 // 1: the next kernel may start at once, 0: once this kernel has its token rows
   int* err;
   AttnSubLayout L;
 };
@@ -273,31 +343,24 @@ struct AttnSubArgs {
 // Shared memory is kept under half an SM's (113 KB) where possible, so that the next kernel's blocks can sit beside
 // this kernel's and run their prologue and weight fetch in its shadow (and so that 16 clusters of 8 are resident at
 // once: above that size an SM takes one block, and a B200 then holds only 15 such clusters).
-inline AttnSubLayout attn_sub_layout(int d, int dkv, int P, int C, int mb, int kc, int bias_len) {
+// late: the keys / values are staged where the projection's weight rows were, once those wait in registers.
+inline AttnSubLayout attn_sub_layout(int d, int dkv, int P, int C, int mb, int kc, int bias_len, int late) {
   AttnSubLayout L;
-  const int npr = (P * dkv + C - 1) / C, no = (d + C - 1) / C;
-  const int wq_b = sub_up16(npr * (d * 2 + SL_WPAD)), kv_b = sub_up16(kc * (sub_kv_stride(dkv) + dkv + 4) * 4);
+  const int npr = (P * dkv + C - 1) / C, no = (d + C - 1) / C, rec = dkv + SUB_RECPAD;
+  const int wq_b = sub_up16(npr * sub_wst(d)), kv_b = sub_up16(kc * (sub_kv_stride(dkv) + dkv + 4) * 4);
   int off = 0;
-  // block variant, self-attention: the keys / values of the rank are staged where the projection rows were, once the
-  // products are done (they depend on the cache position anyway); otherwise they have an area of their own and the
-  // encoder keys are requested in the prologue
-  L.kv_late = (mb > 1 && P == 3 && kv_b <= wq_b) ? 1 : 0;
-  L.wq = off; off += wq_b;
-  const int xs_b = mb * (d + SL_XPAD) * 4, rec_b = C * mb * (dkv + SUB_RECPAD) * 4;
-  L.xs = off; off += sub_up16(xs_b > rec_b ? xs_b : rec_b);   // the records of the merge reuse the token rows
-  if (L.kv_late) L.kv = L.wq;
-  else { L.kv = off; off += kv_b; }
-  L.qkv = off; off += sub_up16(mb * P * dkv * 4);
-  // partial sums of the products; afterwards the merged head output and this rank's record
-  const int ps_b = mb == 1 ? ((npr + 3) / 4) * 8 * 32 * 4 : 8 * 128 * 4, after_b = sub_up16(mb * dkv * 4) + sub_up16(mb * (dkv + SUB_RECPAD) * 4);
-  L.psum = off; L.sa = off; L.recloc = off + sub_up16(mb * dkv * 4);
-  off += sub_up16(ps_b > after_b ? ps_b : after_b);
-  L.probs = off; off += sub_up16(mb * (kc + 4) * 4);
+  L.kv_late = late;
+  L.wq = off; off += late ? std::max(wq_b, kv_b) : wq_b;
+  L.kv = late ? L.wq : off; off += late ? 0 : kv_b;
+  // token rows; afterwards the warps' records and the ranks' records
+  L.xs = off; L.rec = off; L.rrec = off + sub_up16(8 * mb * rec * 4);
+  off += std::max(sub_up16(sub_xs_bytes(d, mb)), sub_up16(8 * mb * rec * 4) + sub_up16(C * mb * rec * 4));
+  L.qkv = off; off += sub_up16(mb * (P * dkv + 16) * 4);
+  // partial sums of the products; afterwards the merged head output and the output tile (block variant)
+  L.psum = off; L.sa = off; L.out = off + sub_up16(mb * (dkv + 4) * 4);
+  off += std::max(sub_up16(sub_psum_bytes(npr, mb)), mb == 1 ? 0 : sub_up16(mb * (dkv + 4) * 4) + sub_up16(SUB_MB * (no + 4) * 4));
   L.bias = off; off += sub_up16(bias_len * 4);
   L.seed = off; off += sub_up16(mb * no * 4);
-  L.red = off; off += sub_up16(SUB_THREADS * 16 + 64 * 4);   // single row: [key part][d_kv] weighted values, then the parts' sums
-  L.loc = off; off += sub_up16(mb * npr * 4);
-  L.out = off; off += mb == 1 ? 0 : sub_up16(SUB_MB * (no + 4) * 4);
   L.sh = off; off += sub_up16((int)sizeof(SubShared));
   L.total = off;
   return L;
@@ -307,71 +370,237 @@ inline AttnSubLayout attn_sub_layout(int d, int dkv, int P, int C, int mb, int k
 // `all_keys` > 0 asks for a chunk that holds up to that many keys so that short caches need no second exchange; the
 // chunk shrinks until the layout for passes of `mb` rows (1: the single-row kernel, SUB_MB: the block kernel; each has a plan
 // of its own) stays under `prefer` bytes (half an SM), else under `limit`.
-struct AttnSubPlan { int kc, bias_len, red_keys; bool ok; };
+struct AttnSubPlan { int kc, bias_len, red_keys, late; bool ok; };
 inline AttnSubPlan attn_sub_plan(int d, int dkv, int P, int C, int keys_cap, int all_keys, int prefer, int limit, int mb) {
   AttnSubPlan pl;
   const int per_rank = (keys_cap + C - 1) / C;
-  const int need = std::min(64, sub_up16(per_rank)), want = std::min(128, sub_up16(std::min(all_keys, keys_cap)));
+  const int need = std::min(64, sub_up16(per_rank)), want = std::min(128, sub_up16(std::max(per_rank, std::min(all_keys, keys_cap))));
   auto blen = [&](int kc) { return P == 3 ? (std::max(per_rank, kc) + MAXB + 8 + 3) / 4 * 4 : 4; };
   auto fits = [&](int kc, int lim) {
-    return attn_sub_layout(d, dkv, P, C, mb, kc, blen(kc)).total <= lim;
+    for (pl.late = 0; pl.late < (P == 3 && (P * dkv + C - 1) / C <= 32 ? 2 : 1); ++pl.late)   // (cross-attention: its keys are requested first
+      // thing, into an area of their own; more than 32 weight rows do not all wait in registers)
+      if (attn_sub_layout(d, dkv, P, C, mb, kc, blen(kc), pl.late).total <= lim) return true;
+    pl.late = 0;
+    return false;
   };
   int kc = std::max(need, want);
   while (kc > need && !fits(kc, prefer)) kc -= 16;
   while (kc > 16 && !fits(kc, limit)) kc -= 16;
   pl.kc = kc; pl.bias_len = blen(kc); pl.ok = fits(kc, limit);
+  if (fits(kc, prefer)) pl.ok = true;
+  else fits(kc, limit);
   pl.red_keys = all_keys > 0 ? kc : 0;
   return pl;
 }
 
-// ONE: a single token row (the small model's step, the large model's single-row pass): SIMT products, no loops over rows.
+// (max, sum, values) records of one token row added up, channels [4 u, 4 u + 4), and their sum; u < 0: the merged (max, sum, -, -)
+template <bool EIGHT>   // n is 8
+__device__ __forceinline__ float4 sub_merge_t(const float* rec, int stride, int n, int u, float& sum) {
+  float m[8], l[8];
+  const int uo = u < 0 ? 0 : SUB_RECPAD + 4 * u;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {   // (loads side by side; past the last record: the last one again, with weight 0)
+    const float2 ml = *reinterpret_cast<const float2*>(rec + (EIGHT ? i : min(i, n - 1)) * stride);
+    m[i] = ml.x; l[i] = EIGHT || i < n ? ml.y : 0.f;
+  }
+  const float gm = fmaxf(fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])), fmaxf(fmaxf(m[4], m[5]), fmaxf(m[6], m[7])));
+  float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  sum = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float4 v = *reinterpret_cast<const float4*>(rec + (EIGHT ? i : min(i, n - 1)) * stride + uo);
+    const float w = l[i] > 0.f ? __expf(m[i] - gm) : 0.f;
+    sum += w * l[i];
+    o.x += w * v.x; o.y += w * v.y; o.z += w * v.z; o.w += w * v.w;
+  }
+  return u < 0 ? make_float4(gm, sum, 0.f, 0.f) : o;
+}
+__device__ __forceinline__ float4 sub_merge(const float* rec, int stride, int n, int u, float& sum) {
+  return n == 8 ? sub_merge_t<true>(rec, stride, 8, u, sum) : sub_merge_t<false>(rec, stride, n, u, sum);
+}
+
+// One token row: this warp's keys of the chunk, eight at a time, two eights side by side.  Lane (key, channel quarter) scores,
+// lane <-> two channels (one, with d_kv = 32 or 16) of the weighted values; everything stays in the warp.
+struct SubAtt1 { float run, sum; float2 acc; };
+template <typename KP, typename VP>
+__device__ __forceinline__ void sub_attend_one(const float4 (&q)[4], int dq4, int dkv, int nk, KP kp, VP vp, const float* sBias, int bias0, bool biased,
+                                               SubAtt1& st, int warp, int lane) {
+  const int key = lane >> 2, qt = lane & 3, cw = dkv >= 64 ? 2 : 1, ch = min(lane * cw, dkv - cw);
+#pragma unroll 1
+  for (int t0 = warp * 8; t0 < nk; t0 += 128) {
+    const bool two = t0 + 64 < nk;
+    float s[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int j = t0 + 64 * h + key;
+      s[h] = -INFINITY;
+      if (h == 0 || two) {
+        const float* p = kp(min(j, nk - 1));
+        float a = 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (u < dq4) {
+            const float4 k4 = *reinterpret_cast<const float4*>(p + (u * 4 + qt) * 4);
+            a += q[u].x * k4.x + q[u].y * k4.y + q[u].z * k4.z + q[u].w * k4.w;
+          }
+        a += __shfl_xor_sync(0xffffffffu, a, 1);
+        a += __shfl_xor_sync(0xffffffffu, a, 2);
+        if (j < nk) s[h] = biased ? a + sBias[bias0 - j] : a;
+      }
+    }
+    float mx = fmaxf(s[0], s[1]);
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    const float nw = fmaxf(st.run, mx), sc = st.run == -INFINITY ? 0.f : __expf(st.run - nw);
+    const float p0 = __expf(s[0] - nw), p1 = __expf(s[1] - nw);   // (a key that is not there: 0)
+    st.run = nw;
+    st.sum = st.sum * sc + p0 + p1;          // per lane: the keys of its quad
+    st.acc.x *= sc; st.acc.y *= sc;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (h == 0 || two) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float w = __shfl_sync(0xffffffffu, h ? p1 : p0, i * 4);
+          const float* v = vp(min(t0 + 64 * h + i, nk - 1)) + ch;
+          if (cw == 2) {
+            const float2 v2 = *reinterpret_cast<const float2*>(v);
+            st.acc.x += w * v2.x; st.acc.y += w * v2.y;
+          } else {
+            st.acc.x += w * v[0];
+          }
+        }
+      }
+  }
+}
+
+// Up to 8 token rows: this warp's keys of the chunk, eight at a time, on mma.sync: scores (token rows x keys, 16 channels per
+// m16n8k16) leave a lane (token g; keys 2 t, 2 t + 1) with just the left operand of the weighted values (token rows x channels,
+// eight keys per m16n8k8), so soft-max and both products stay in the warp, without a barrier.  Queries, keys, probabilities and
+// values each as a bf16 head and remainder, three of the four products kept.  Channels are dealt to the instruction's positions so that
+// keys and values arrive with 16-byte loads: score step i, positions (2 t, 2 t + 1 | 2 t + 8, 2 t + 9) <-> channels
+// 16 i + 4 t + 0, 1 | 2, 3; value column g of tile n <-> channel 32 (n / 4) + 4 g + n % 4 (d_kv = 16: 2 g + n).
+struct SubAtt8 { float run, sum; float o[8][4]; };
+struct SubQ8 { uint32_t h[4][2], l[4][2]; };
+template <typename KP, typename VP>
+__device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk, KP kp, VP vp, const float* sBias, int bias0, bool biased, int limit,
+                                                 SubAtt8& st, int warp, int lane) {
+  // bias0 - j: index of the bias of key j for this lane's token; limit: the last key this lane's token sees
+  const int g = lane >> 2, t = lane & 3;
+#pragma unroll 1
+  for (int t0 = warp * 8; t0 < nk; t0 += 64) {
+    float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f}, f[4] = {0.f, 0.f, 0.f, 0.f};
+    const float* k0 = kp(min(t0 + g, nk - 1)) + 4 * t;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i * 16 < dkv) {
+        const float4 k4 = *reinterpret_cast<const float4*>(k0 + i * 16);
+        uint32_t h0, h1, l0, l1;
+        sub_split(k4.x, k4.y, h0, l0); sub_split(k4.z, k4.w, h1, l1);
+        sub_mma(c, q.h[i][0], 0u, q.h[i][1], 0u, h0, h1);
+        sub_mma(e, q.l[i][0], 0u, q.l[i][1], 0u, h0, h1);
+        sub_mma(f, q.h[i][0], 0u, q.h[i][1], 0u, l0, l1);
+      }
+    float s0 = c[0] + (e[0] + f[0]), s1 = c[1] + (e[1] + f[1]);
+    const int ja = t0 + 2 * t, jb = ja + 1;
+    if (biased) {
+      s0 += sBias[max(0, bias0 - ja)]; s1 += sBias[max(0, bias0 - jb)];
+    }
+    if (ja > limit) s0 = -INFINITY;
+    if (jb > limit) s1 = -INFINITY;
+    float mx = fmaxf(s0, s1);
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+    const float nw = fmaxf(st.run, mx);
+    const float sc = st.run == -INFINITY ? 0.f : __expf(st.run - nw);
+    const float p0 = s0 == -INFINITY ? 0.f : __expf(s0 - nw), p1 = s1 == -INFINITY ? 0.f : __expf(s1 - nw);
+    st.run = nw;
+    st.sum = st.sum * sc + p0 + p1;   // per lane: its two keys
+    uint32_t ph, pl;
+    sub_split(p0, p1, ph, pl);
+    const float* va = vp(min(ja, nk - 1));
+    const float* vb = vp(min(jb, nk - 1));
+#pragma unroll
+    for (int n4 = 0; n4 < 2; ++n4)
+      if (n4 * 32 < dkv) {
+        float4 x, y;
+        if (dkv >= 32) {
+          x = *reinterpret_cast<const float4*>(va + n4 * 32 + 4 * g); y = *reinterpret_cast<const float4*>(vb + n4 * 32 + 4 * g);
+        } else {
+          const float2 x2 = *reinterpret_cast<const float2*>(va + 2 * g), y2 = *reinterpret_cast<const float2*>(vb + 2 * g);
+          x = make_float4(x2.x, x2.y, 0.f, 0.f); y = make_float4(y2.x, y2.y, 0.f, 0.f);
+        }
+        const float xs[4] = {x.x, x.y, x.z, x.w}, ys[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+          float (&o)[4] = st.o[n4 * 4 + n];
+          o[0] *= sc; o[1] *= sc;
+          uint32_t vh, vl;
+          sub_split(xs[n], ys[n], vh, vl);
+          sub_mma8(o, ph, 0u, vh);
+          sub_mma8(o, pl, 0u, vh);
+          sub_mma8(o, ph, 0u, vl);
+        }
+      }
+  }
+}
+
+// ONE: a single token row (the small model's step, the large model's single-row pass); else 2 to 8 rows.
+// Bound by the latency of its dependent chain (3-10 % of the memory's rate, 3-10 % of the tensor pipe): token rows from the L2,
+// products, exchange of q | k | v within the head's cluster, attention, [exchange of the ranks' records], output products, reductions
+// at the L2.  What is off the chain is done before the dependency wait: the weight rows wait as operands in registers, W_o's too,
+// the cached keys and values in shared memory.  Between barriers each warp works alone: three (four) block barriers and one
+// (two) waits for the cluster per kernel.
+// Measured, T5-large shapes, pass of 24 layers, cache 32, 512 encoder keys, before -> after this form of the kernels (both
+// sub-layer kernels; before: token rows and norm for the whole block, then products from shared memory, cluster barriers, scores,
+// soft-max and values with a block barrier each): 1 row 473 -> 355 us, 5 rows 632 -> 550 us, 8 rows 691 -> 597 us, 16 rows
+// 1080 -> 831 us; T5-small 100 -> 83 us.
 template <bool ONE>
-__global__ void __launch_bounds__(SUB_THREADS) attn_sub_kernel(const AttnSubArgs a) {
+__global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubArgs a) {
   extern __shared__ __align__(1024) unsigned char sub_smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int C = a.C, d = a.d, dkv = a.dkv, P = a.self ? 3 : 1, R = P * dkv;
   const int h = blockIdx.x >> a.c_shift, r = (int)cluster_rank();
   const int pr0 = (r * R) >> a.c_shift, npr = (((r + 1) * R) >> a.c_shift) - pr0;   // rows of the head's q|k|v projection
   const int no = d >> a.c_shift, o0 = r * no;                                         // output rows of W_o
-  const int rowbytes = d * 2 + SL_WPAD, xst = d + SL_XPAD, kvst = sub_kv_stride(dkv);
-  const int vst = dkv + 4;   // row stride of the staged values: rows 2 t and channels g of a tensor-core tile hit 32 banks
+  const int wst = sub_wst(d), xst = sub_xst(d), kvst = sub_kv_stride(dkv), qst = R + 16, recst = dkv + SUB_RECPAD;
+  const int vst = dkv + 4;   // row stride of the staged values: the rows 2 t and channels 4 g of a tile hit 32 banks
   unsigned char* sWq = sub_smem + a.L.wq;
-  float* Xs = reinterpret_cast<float*>(sub_smem + a.L.xs);
-  float* rec = Xs;
+  uint32_t* Xs = reinterpret_cast<uint32_t*>(sub_smem + a.L.xs);
+  float* sRec = reinterpret_cast<float*>(sub_smem + a.L.rec);     // [8 warps][mb][recst]
+  float* sRrec = reinterpret_cast<float*>(sub_smem + a.L.rrec);   // [C ranks][mb][recst]
   float* sK = reinterpret_cast<float*>(sub_smem + a.L.kv);
   float* sV = sK + (size_t)a.kc_keys * kvst;
-  float* sQKV = reinterpret_cast<float*>(sub_smem + a.L.qkv);
+  float* sQKV = reinterpret_cast<float*>(sub_smem + a.L.qkv);     // [mb][qst]
   float* psum = reinterpret_cast<float*>(sub_smem + a.L.psum);
-  float* sP = reinterpret_cast<float*>(sub_smem + a.L.probs);
   float* sBias = reinterpret_cast<float*>(sub_smem + a.L.bias);
   float* sSeed = reinterpret_cast<float*>(sub_smem + a.L.seed);
-  float* sA = reinterpret_cast<float*>(sub_smem + a.L.sa);
-  float* sRed = reinterpret_cast<float*>(sub_smem + a.L.red);
-  float* recLoc = reinterpret_cast<float*>(sub_smem + a.L.recloc);
-  float* sLoc = reinterpret_cast<float*>(sub_smem + a.L.loc);
+  float* sA = reinterpret_cast<float*>(sub_smem + a.L.sa);        // [mb][dkv + 4]
   SubShared* sh = reinterpret_cast<SubShared*>(sub_smem + a.L.sh);
-  const int pst = a.kc_keys + 4, recst = dkv + SUB_RECPAD;
+  const int cpw = sub_chunks(d), col0 = warp * 32 * cpw, nch = max(0, min(cpw, (d - col0 + 31) >> 5));
+  const int col = col0 + lane * 4;
+  const bool stores = lane * 4 < 32 * nch, on = stores && col < d;   // this lane's four columns of the token rows
   SUB_STAMP_BEGIN();
 
   if (tid == 0) {
     mbar_init(smem_u32(&sh->wbar), 1);
+    mbar_init(smem_u32(&sh->xbar[0]), 1);
+    mbar_init(smem_u32(&sh->xbar[1]), 1);
     sh->failed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     mbar_expect(smem_u32(&sh->wbar), (uint32_t)(npr * d * 2));
   }
   __syncthreads();
-  SUB_STAMP();            // P0: barrier initialised
-  pdl_launch_dependents();
+  if (a.early) pdl_launch_dependents();
   // weights depend on nothing: requested before the dependency wait.  Row i is copied by lane i / 8 of warp i % 8:
   // the copies a warp issues go out one after the other (about 25 ns each), the warps issue side by side
   {
     const int i = ((tid & 31) << 3) | (tid >> 5);
     if (i < npr && !a.skip_copies) {
       const int j = pr0 + i, part = j >> a.dkv_shift, ch = j & (dkv - 1);
-      bulk_g2s(smem_u32(sWq + (size_t)i * rowbytes), a.Wp + ((size_t)part * a.I + h * dkv + ch) * d, (uint32_t)(d * 2), smem_u32(&sh->wbar));
+      bulk_g2s(smem_u32(sWq + (size_t)i * wst), a.Wp + ((size_t)part * a.I + h * dkv + ch) * d, (uint32_t)(d * 2), smem_u32(&sh->wbar));
     }
   }
-  SUB_STAMP();            // P1: copies issued
   // output projection: warp w owns rows 16 w .. 16 w + 15 of this rank's share of W_o's column slice.  Thread (g, t) of the
   // warp keeps, of rows g and g + 8, the channels [t d_kv / 4, (t + 1) d_kv / 4), two per register: as it stands the left
   // operand of mma.sync m16n8k16 with the channels of a 16-channel step dealt out four to a thread
@@ -393,7 +622,7 @@ __global__ void __launch_bounds__(SUB_THREADS) attn_sub_kernel(const AttnSubArgs
     }
   }
   float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (tid * 4 < d) g4 = __ldg(reinterpret_cast<const float4*>(a.gain) + tid);
+  if (on) g4 = __ldg(reinterpret_cast<const float4*>(a.gain + col));
   const float* Kh = a.kc + (size_t)h * a.cap * dkv;
   const float* Vh = a.vc + (size_t)h * a.cap * dkv;
   // stages keys / values [c0, c1) of the cache into sK / sV rows 0.. (asynchronous 16-byte copies)
@@ -416,7 +645,7 @@ __global__ void __launch_bounds__(SUB_THREADS) attn_sub_kernel(const AttnSubArgs
     j0 = red ? 0 : (r * n_keys) >> a.c_shift; j1 = red ? n_keys : ((r + 1) * n_keys) >> a.c_shift;
     stage_cached(j0, min(j1, j0 + a.kc_keys));
     // a share of more than one chunk: the later chunks are asked into the L2 now (they are staged when the first is used up)
-    const int later = (j1 - j0 - a.kc_keys) * (dkv >> 5);   // 128-byte lines of keys (as many again of values)
+    const int later = (j1 - j0 - a.kc_keys) * dkv / 32;   // 128-byte lines of keys (as many again of values)
 #pragma unroll 1
     for (int i = tid; i < later; i += SUB_THREADS) {
       const size_t o = (size_t)(j0 + a.kc_keys) * dkv + (size_t)i * 32;
@@ -436,369 +665,264 @@ __global__ void __launch_bounds__(SUB_THREADS) attn_sub_kernel(const AttnSubArgs
     j0 = red ? 0 : (r * n_keys) >> a.c_shift; j1 = red ? n_keys : ((r + 1) * n_keys) >> a.c_shift;
     if (!a.L.kv_late) stage_cached(j0, min(min(j1, pos0), j0 + a.kc_keys));
   }
+  if (tid == 0) {   // what the exchanges bring: the head's q | k | v of every row, one record per rank and row
+    mbar_expect(smem_u32(&sh->xbar[0]), (uint32_t)(R * k * 4));
+    if (!red) mbar_expect(smem_u32(&sh->xbar[1]), (uint32_t)(C * k * recst * 4));
+  }
   // relative-position bias of the distances this rank meets
   const int dist_lo = max(0, pos0 - (j1 - 1));
   const int bias_cnt = a.self ? min(pos0 + k - j0 - dist_lo, a.bias_len) : 0;
 #pragma unroll 1
   for (int i = tid; i < bias_cnt; i += SUB_THREADS) sBias[i] = __ldg(a.bias + (size_t)h * a.bias_ld + dist_lo + i);
   SubRows<ONE> rw;
-  if (a.emb) sub_rows_embed<ONE>(a.emb, a.tokens, a.vocab, k, d, tid, rw);   // (tokens: part of the descriptor; the table: weights)
-  SUB_STAMP();            // P2: loads issued, keys requested
+  if (a.emb) sub_rows_embed<ONE>(a.emb, a.tokens, a.vocab, k, d, col, on, rw);   // (tokens: part of the descriptor; the table: weights)
+  __syncwarp();
   sub_cluster_arrive_relaxed();   // (0) this block is up: its shared memory may be written by the cluster
-  SUB_STAMP();            // 0: prologue
+  SUB_STAMP();            // 0: requests
+  // the weight rows become operands (two 16-row tiles in registers), then the keys may take their place
+  const int mt = (npr + 15) >> 4;
+  uint4 fr[2][4][2];
+  sub_wait(sh, a.err, &sh->wbar, 0, a.spin);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (i < mt) sub_frags(sWq, wst, npr, d, i, col0, nch, lane, fr[i]);
+  if (a.L.kv_late) {
+    __syncthreads();
+    stage_cached(j0, min(min(j1, pos0), j0 + a.kc_keys));
+  }
+  SUB_STAMP();            // 1: weights in registers
   pdl_wait();
-  SUB_STAMP();            // 1: dependency wait
-  if (!a.emb) sub_rows_issue<ONE>(a.x_in, k, d, tid, rw);
+  SUB_STAMP();            // 2: dependency wait
+  if (!a.emb) sub_rows_issue<ONE>(a.x_in, k, d, col, on, rw);
   {   // clear the buffer the next kernel accumulates into
     const int n4 = k * (d >> 2);
 #pragma unroll 1
     for (int i = blockIdx.x * SUB_THREADS + tid; i < n4; i += gridDim.x * SUB_THREADS)
       reinterpret_cast<float4*>(a.x_zero)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  const float inv1 = sub_rows_finish<ONE>(rw, k, d, g4, a.eps, Xs, xst, sh, sSeed, h == 0 ? o0 : 0, h == 0 ? o0 + no : 0, tid, lane, warp);
-  SUB_STAMP();            // 2: token rows + norm
-  sub_wait(sh, a.err, &sh->wbar, 0, a.spin);
-  SUB_STAMP();            // 3: wait for the weights
+  sub_rows_split<ONE>(rw, k, col, stores, on, g4, Xs, xst, sh, sSeed, h == 0 ? o0 : 0, h == 0 ? o0 + no : 0, lane, warp);
+  if (!a.early) pdl_launch_dependents();
+  SUB_STAMP();            // 3: token rows
+  const int pst = sub_pst(npr);
   // ---- phase A: this rank's q|k|v rows for all token rows -----------------------------------
-  if (ONE) sl_items<1>(sWq, rowbytes, npr, d, Xs, xst, psum, warp, lane);
-  else sub_mma_split(sWq, rowbytes, npr, d, Xs, k, psum, warp, lane);
+  {
+    SubB<ONE> b;
+    sub_bfrags<ONE>(Xs, xst, k, col0, nch, lane, b);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i < mt) sub_tile<ONE>(fr[i], b, nch, npr, i, psum, warp, lane);
+    if (mt > 2) {   // (heads over fewer than eight blocks; never with kv_late)
+      sub_frags(sWq, wst, npr, d, 2, col0, nch, lane, fr[0]);
+      sub_tile<ONE>(fr[0], b, nch, npr, 2, psum, warp, lane);
+    }
+  }
+  sub_cp_wait();          // (first chunk of keys / values)
   __syncthreads();
-  if (a.L.kv_late) stage_cached(j0, min(min(j1, pos0), j0 + a.kc_keys));   // the projection rows are done with: their place takes the keys
   SUB_STAMP();            // 4: q|k|v products
   sub_cluster_wait();     // (0) every block of the cluster is up
-  if (ONE || (npr & 3) || (pr0 & 3)) {   // one (value, destination rank) pair per thread and turn
+  if (!ONE && ((npr | pr0) & 3) == 0 && npr <= 32) {   // warp <-> token row: values in lanes, then four at a time to every rank
+    const int m = warp, n4 = npr >> 2, tot = n4 << a.c_shift;
+    if (m < k) {
+      float v = 0.f;
+      if (lane < npr) {
+        v = sub_total<ONE>(psum, lane, m, pst) * sub_inv(sh, m, a.inv_d, a.eps);
+        const int j = pr0 + lane;
+        if (a.self && j >= dkv && pos0 + m < a.cap)
+          (j < 2 * dkv ? a.kc : a.vc)[((size_t)h * a.cap + pos0 + m) * dkv + (j & (dkv - 1))] = v;
+      }
+#pragma unroll 1
+      for (int i0 = 0; i0 < tot; i0 += 32) {
+        const int i = i0 + lane, q = i >> a.c_shift, rk = i & (C - 1);
+        float4 o;
+        o.x = __shfl_sync(0xffffffffu, v, (4 * q) & 31); o.y = __shfl_sync(0xffffffffu, v, (4 * q + 1) & 31);
+        o.z = __shfl_sync(0xffffffffu, v, (4 * q + 2) & 31); o.w = __shfl_sync(0xffffffffu, v, (4 * q + 3) & 31);
+        if (i < tot) sub_push4(sQKV + (size_t)m * qst + pr0 + 4 * q, &sh->xbar[0], (uint32_t)rk, o);
+      }
+    }
+  } else {   // one (value, destination rank) pair per thread and turn
     const int tot = (npr * k) << a.c_shift;
 #pragma unroll 1
     for (int idx = tid; idx < tot; idx += SUB_THREADS) {
       const int rk = idx & (C - 1), rest = idx >> a.c_shift, m = ONE ? 0 : rest / npr, i = rest - m * npr;
-      const float v = sub_total<ONE>(psum, i, m, npr, d) * (ONE ? inv1 : sh->inv[m]);
+      const float v = sub_total<ONE>(psum, i, m, pst) * sub_inv(sh, m, a.inv_d, a.eps);
       const int j = pr0 + i;
-      st_cluster_f1(smem_u32(sQKV + (size_t)m * R + j), (uint32_t)rk, v);
+      sub_push(sQKV + (size_t)m * qst + j, &sh->xbar[0], (uint32_t)rk, v);
       if (a.self && rk == r && j >= dkv && pos0 + m < a.cap)
         (j < 2 * dkv ? a.kc : a.vc)[((size_t)h * a.cap + pos0 + m) * dkv + (j & (dkv - 1))] = v;
     }
-  } else {   // values first, then one 16-byte store per thread and turn
-#pragma unroll 1
-    for (int idx = tid; idx < npr * k; idx += SUB_THREADS) {
-      const int m = idx / npr, i = idx - m * npr;
-      const float v = sub_total<ONE>(psum, i, m, npr, d) * sh->inv[m];
-      const int j = pr0 + i;
-      sLoc[idx] = v;
-      if (a.self && j >= dkv && pos0 + m < a.cap)
-        (j < 2 * dkv ? a.kc : a.vc)[((size_t)h * a.cap + pos0 + m) * dkv + (j & (dkv - 1))] = v;
-    }
-    __syncthreads();
-    const int n4 = npr >> 2, tot = (n4 * k) << a.c_shift;
-#pragma unroll 1
-    for (int idx = tid; idx < tot; idx += SUB_THREADS) {
-      const int rk = idx & (C - 1), rest = idx >> a.c_shift, m = rest / n4, q = rest - m * n4;
-      st_cluster_f4(smem_u32(sQKV + (size_t)m * R + pr0 + q * 4), (uint32_t)rk, *reinterpret_cast<const float4*>(sLoc + (size_t)m * npr + q * 4));
-    }
   }
   SUB_STAMP();            // 5: exchange stores
-  sub_cluster_arrive();   // (1) q, new keys and new values of the head are complete in every block
-  sub_cluster_wait();
-  SUB_STAMP();            // 6: cluster barrier 1
-  // ---- phase B: attention of the k rows over the keys [j0, j1) ---------------------------------
-  // single row, value phase: thread = (group of four channels, key part)
-  const int cg4 = tid & ((dkv >> 2) - 1), part4 = tid >> (a.dkv_shift - 2), nparts4 = SUB_THREADS >> (a.dkv_shift - 2);
-  float4 acc4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int dq4 = dkv >> 4;   // 16-byte units per channel quarter (d_kv <= 64)
-  constexpr int RPP = ONE ? 1 : 2;   // rows per thread in the value phase (up to 8 rows over at least 4 parts)
-  float acc[RPP], run1 = -INFINITY, lsum1 = 0.f;
+  sub_wait_exchange(sh, a.err, &sh->xbar[0], a.spin);   // q, new keys and new values of the head are complete
+  SUB_STAMP();            // 6: exchange 1
+  // ---- phase B: attention of the k rows over the keys [j0, j1), every warp on keys of its own -----------------
+  constexpr int MBC = ONE ? 1 : SUB_MB;
+  const int og_k = min(og, k - 1);
+  SubAtt1 s1;
+  SubAtt8 s8;
+  float4 q1[4];
+  SubQ8 q8;
+  if (ONE) {
+    s1.run = -INFINITY; s1.sum = 0.f; s1.acc = make_float2(0.f, 0.f);
 #pragma unroll
-  for (int i = 0; i < RPP; ++i) acc[i] = 0.f;
-  if (!ONE && tid < MAXB) { sh->rmax[tid] = -INFINITY; sh->rsum[tid] = 0.f; sh->rscale[tid] = 1.f; }
+    for (int u = 0; u < 4; ++u)
+      if (u * 16 < dkv) q1[u] = *reinterpret_cast<const float4*>(sQKV + (u * 4 + ot) * 4);
+  } else {
+    s8.run = -INFINITY; s8.sum = 0.f;
+#pragma unroll
+    for (int n = 0; n < 8; ++n) { s8.o[n][0] = 0.f; s8.o[n][1] = 0.f; s8.o[n][2] = 0.f; s8.o[n][3] = 0.f; }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i * 16 < dkv) {
+        float4 q4 = *reinterpret_cast<const float4*>(sQKV + (size_t)og_k * qst + i * 16 + 4 * ot);
+        if (og >= k) q4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        sub_split(q4.x, q4.y, q8.h[i][0], q8.l[i][0]);
+        sub_split(q4.z, q4.w, q8.h[i][1], q8.l[i][1]);
+      }
+  }
 #pragma unroll 1
   for (int c0 = j0; c0 < j1; c0 += a.kc_keys) {
     const int c1 = min(j1, c0 + a.kc_keys), nk = c1 - c0;
     if (c0 > j0) {   // later chunks: staged now (the first one is on its way since the prologue)
       __syncthreads();
       stage_cached(c0, a.self ? min(c1, pos0) : c1);
-    }
-    if (a.self) {   // keys of this pass come from the exchange buffer
-      const int n0 = max(c0, pos0), cnt = (c1 - n0) << a.dkv_shift;
-#pragma unroll 1
-      for (int i = tid; i < cnt; i += SUB_THREADS) {
-        const int jj = i >> a.dkv_shift, cc = i & (dkv - 1), mm = n0 + jj - pos0;
-        sK[(size_t)(n0 + jj - c0) * kvst + cc] = sQKV[(size_t)mm * R + dkv + cc];
-        sV[(size_t)(n0 + jj - c0) * vst + cc] = sQKV[(size_t)mm * R + 2 * dkv + cc];
-      }
-    }
-    sub_cp_wait();
-    __syncthreads();
-    SUB_STAMP();          // B1: keys / values staged
-    if (ONE) {   // scores: four threads per key, one channel quarter each (16-byte units interleaved over the quarters);
-                 // two keys (64 apart) per thread and turn so that their loads are in flight together
-      const int qt = tid & 3;
-      const float* qp = sQKV;
-#pragma unroll 1
-      for (int j0b = 0; j0b < nk; j0b += SUB_THREADS / 2) {   // (the same trip count for every thread: the quads shuffle)
-        const int jb = j0b + (tid >> 2), jc = jb + SUB_THREADS / 4;
-        const bool va = jb < nk, vb = jc < nk;
-        const float* pa = sK + (size_t)(va ? jb : 0) * kvst;
-        const float* pb = sK + (size_t)(vb ? jc : 0) * kvst;
-        float sa = 0.f, sb = 0.f;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (u < dq4) {
-            const float4 q4 = *reinterpret_cast<const float4*>(qp + (u * 4 + qt) * 4);
-            const float4 ka = *reinterpret_cast<const float4*>(pa + (u * 4 + qt) * 4);
-            const float4 kb = *reinterpret_cast<const float4*>(pb + (u * 4 + qt) * 4);
-            sa += q4.x * ka.x + q4.y * ka.y + q4.z * ka.z + q4.w * ka.w;
-            sb += q4.x * kb.x + q4.y * kb.y + q4.z * kb.z + q4.w * kb.w;
-          }
-        sa += __shfl_xor_sync(0xffffffffu, sa, 1); sb += __shfl_xor_sync(0xffffffffu, sb, 1);
-        sa += __shfl_xor_sync(0xffffffffu, sa, 2); sb += __shfl_xor_sync(0xffffffffu, sb, 2);
-        if (qt == 0) {
-          if (a.self) {   // (a single row sees every key up to its own position: all of them)
-            if (va) sa += sBias[min(pos0 - (c0 + jb) - dist_lo, a.bias_len - 1)];
-            if (vb) sb += sBias[min(pos0 - (c0 + jc) - dist_lo, a.bias_len - 1)];
-          }
-          if (va) sP[jb] = sa;
-          if (vb) sP[jc] = sb;
-        }
-      }
-    } else {
-      // scores on mma.sync m16n8k16: 16 keys of the chunk are the rows of the left operand, the token rows the columns of
-      // the right one, 16 channels per step; keys and queries each as a bf16 head and a bf16 remainder, three products kept.
-      // Warp w takes the key tiles w, w + 8, ...
-      const int g = lane >> 2, t = lane & 3;
-#pragma unroll 1
-      for (int t0 = warp * 16; t0 < nk; t0 += 16 * (SUB_THREADS / 32)) {
-        float c0a = 0.f, c1a = 0.f, c2a = 0.f, c3a = 0.f, c0b = 0.f, c1b = 0.f, c2b = 0.f, c3b = 0.f, c0c = 0.f, c1c = 0.f, c2c = 0.f, c3c = 0.f;
-        const float* ka = sK + (size_t)min(t0 + g, nk - 1) * kvst + 2 * t;
-        const float* kb = sK + (size_t)min(t0 + g + 8, nk - 1) * kvst + 2 * t;
-        const float* qp = sQKV + (size_t)min(g, k - 1) * R + 2 * t;
-#pragma unroll
-        for (int st = 0; st < 4; ++st)
-          if (st * 16 < dkv) {
-            const float2 a0 = *reinterpret_cast<const float2*>(ka + st * 16), a1 = *reinterpret_cast<const float2*>(kb + st * 16);
-            const float2 a2 = *reinterpret_cast<const float2*>(ka + st * 16 + 8), a3 = *reinterpret_cast<const float2*>(kb + st * 16 + 8);
-            float2 b0 = *reinterpret_cast<const float2*>(qp + st * 16), b1 = *reinterpret_cast<const float2*>(qp + st * 16 + 8);
-            if (g >= k) { b0 = make_float2(0.f, 0.f); b1 = b0; }
-            const uint32_t ah0 = sl_pack_bf16(a0.x, a0.y), ah1 = sl_pack_bf16(a1.x, a1.y), ah2 = sl_pack_bf16(a2.x, a2.y), ah3 = sl_pack_bf16(a3.x, a3.y);
-            const uint32_t al0 = sl_pack_bf16(a0.x - __uint_as_float(ah0 << 16), a0.y - __uint_as_float(ah0 & 0xffff0000u));
-            const uint32_t al1 = sl_pack_bf16(a1.x - __uint_as_float(ah1 << 16), a1.y - __uint_as_float(ah1 & 0xffff0000u));
-            const uint32_t al2 = sl_pack_bf16(a2.x - __uint_as_float(ah2 << 16), a2.y - __uint_as_float(ah2 & 0xffff0000u));
-            const uint32_t al3 = sl_pack_bf16(a3.x - __uint_as_float(ah3 << 16), a3.y - __uint_as_float(ah3 & 0xffff0000u));
-            const uint32_t bh0 = sl_pack_bf16(b0.x, b0.y), bh1 = sl_pack_bf16(b1.x, b1.y);
-            const uint32_t bl0 = sl_pack_bf16(b0.x - __uint_as_float(bh0 << 16), b0.y - __uint_as_float(bh0 & 0xffff0000u));
-            const uint32_t bl1 = sl_pack_bf16(b1.x - __uint_as_float(bh1 << 16), b1.y - __uint_as_float(bh1 & 0xffff0000u));
-#define SUB_MMA_S(C0, C1, C2, C3, A0, A1, A2, A3, B0, B1)                                                                        \
-            asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};" \
-                         : "+f"(C0), "+f"(C1), "+f"(C2), "+f"(C3) : "r"(A0), "r"(A1), "r"(A2), "r"(A3), "r"(B0), "r"(B1))
-            SUB_MMA_S(c0a, c1a, c2a, c3a, ah0, ah1, ah2, ah3, bh0, bh1);
-            SUB_MMA_S(c0b, c1b, c2b, c3b, al0, al1, al2, al3, bh0, bh1);
-            SUB_MMA_S(c0c, c1c, c2c, c3c, ah0, ah1, ah2, ah3, bl0, bl1);
-#undef SUB_MMA_S
-          }
-        // accumulators: keys t0 + g and t0 + g + 8, token rows 2 t and 2 t + 1
-        const float cv[4] = {c0a + (c0b + c0c), c1a + (c1b + c1c), c2a + (c2b + c2c), c3a + (c3b + c3c)};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int jj = t0 + g + 8 * (i >> 1), m = 2 * t + (i & 1);
-          if (jj < nk && m < k) {
-            float sc = cv[i];
-            if (a.self) {
-              const int dist = pos0 + m - (c0 + jj);   // causal inside the block: row m sees keys up to its own position
-              sc = dist >= 0 ? sc + sBias[min(dist - dist_lo, a.bias_len - 1)] : -INFINITY;
-            }
-            sP[(size_t)m * pst + jj] = sc;
-          }
-        }
-      }
-    }
-    __syncthreads();
-    SUB_STAMP();          // B2: scores
-    if (ONE) {
-      // every warp finds the chunk's maximum; thread (group of four channels, key part) then exponentiates and weighs its keys
-      float mx = -INFINITY;
-#pragma unroll 4
-      for (int jj = lane; jj < nk; jj += 32) mx = fmaxf(mx, sP[jj]);   // (unrolled: the loads of a thread side by side)
-      mx = warp_max(mx);
-      const float nw = fmaxf(run1, mx), sc = run1 == -INFINITY ? 0.f : __expf(run1 - nw);
-      float4 t4 = make_float4(acc4.x * sc, acc4.y * sc, acc4.z * sc, acc4.w * sc);
-      float l = lsum1 * sc;
-#pragma unroll 4
-      for (int jj = part4; jj < nk; jj += nparts4) {
-        const float p = __expf(sP[jj] - nw);
-        const float4 v = *reinterpret_cast<const float4*>(sV + (size_t)jj * vst + cg4 * 4);
-        l += p;
-        t4.x += p * v.x; t4.y += p * v.y; t4.z += p * v.z; t4.w += p * v.w;
-      }
-      acc4 = t4; lsum1 = l; run1 = nw;
-    } else {
-      // running soft-max, one warp per row
-#pragma unroll 1
-      for (int m = warp; m < k; m += SUB_THREADS / 32) {
-        float mx = -INFINITY;
-        for (int jj = lane; jj < nk; jj += 32) mx = fmaxf(mx, sP[(size_t)m * pst + jj]);
-        mx = warp_max(mx);
-        const float old = sh->rmax[m], nw = fmaxf(old, mx);
-        float sum = 0.f;
-        for (int jj = lane; jj < ((nk + 15) & ~15); jj += 32) {   // (zeros up to the end of the last 16-key step)
-          const float p = (jj >= nk || nw == -INFINITY) ? 0.f : __expf(sP[(size_t)m * pst + jj] - nw);
-          sP[(size_t)m * pst + jj] = p;
-          sum += p;
-        }
-        sum = warp_sum(sum);
-        if (lane == 0) {
-          const float sc = nw == -INFINITY ? 1.f : __expf(old - nw);
-          sh->rscale[m] = sc;
-          sh->rsum[m] = sh->rsum[m] * sc + sum;
-          sh->rmax[m] = nw;
-        }
-      }
+      sub_cp_wait();
       __syncthreads();
-      SUB_STAMP();        // B3: soft-max (block variant)
-      // weighted values on mma.sync m16n8k16: out[row][channel] = sum_j p[row][j] v[j][channel]; the token rows are the
-      // rows of the left operand (8..15 zero), warp w owns the channels 8 w .. 8 w + 7, 16 keys per step; probabilities
-      // and values each as a bf16 head and a bf16 remainder, three products kept
-      if (warp * 8 < dkv) {
-        const int g = lane >> 2, t = lane & 3, n0 = warp * 8;
-        const float rs = g < k ? sh->rscale[g] : 1.f;
-        acc[0] *= rs; acc[1] *= rs;
-        float c2 = 0.f, c3 = 0.f, d0 = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;   // (d: the products with the remainders, a chain of their own)
-        const uint32_t zero = 0u;
-#pragma unroll 2
-        for (int k0 = 0; k0 < nk; k0 += 16) {
-          float2 p0 = make_float2(0.f, 0.f), p1 = p0;
-          if (g < k) {
-            p0 = *reinterpret_cast<const float2*>(sP + (size_t)g * pst + k0 + 2 * t);
-            p1 = *reinterpret_cast<const float2*>(sP + (size_t)g * pst + k0 + 2 * t + 8);
+    }
+    // keys of this pass come from the exchange buffer
+    const int own0 = a.self ? pos0 - c0 : nk;
+    auto kp = [&](int j) { return j >= own0 ? sQKV + (size_t)(j - own0) * qst + dkv : sK + (size_t)j * kvst; };
+    auto vp = [&](int j) { return j >= own0 ? sQKV + (size_t)(j - own0) * qst + 2 * dkv : sV + (size_t)j * vst; };
+    if (ONE) sub_attend_one(q1, dkv >> 4, dkv, nk, kp, vp, sBias, pos0 - c0 - dist_lo, a.self != 0, s1, warp, lane);
+    else sub_attend_block(q8, dkv, nk, kp, vp, sBias, pos0 + og - c0 - dist_lo, a.self != 0, a.self ? min(nk - 1, pos0 + og_k - c0) : nk - 1, s8, warp, lane);
+  }
+  // the warp's record of every row: max, sum, weighted values
+  if (ONE) {
+    float l = s1.sum;
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    float* rp = sRec + (size_t)warp * recst;
+    if (lane == 0) *reinterpret_cast<float4*>(rp) = make_float4(s1.run, l, 0.f, 0.f);
+    if (dkv >= 64) *reinterpret_cast<float2*>(rp + SUB_RECPAD + 2 * lane) = s1.acc;
+    else if (lane < dkv) rp[SUB_RECPAD + lane] = s1.acc.x;
+  } else {
+    float l = s8.sum;
+    l += __shfl_xor_sync(0xffffffffu, l, 1);
+    l += __shfl_xor_sync(0xffffffffu, l, 2);
+    if (og < k) {
+      float* rp = sRec + (size_t)(warp * MBC + og) * recst;
+      if (ot == 0) *reinterpret_cast<float4*>(rp) = make_float4(s8.run, l, 0.f, 0.f);
+      rp += SUB_RECPAD;
+      if (dkv == 16) {
+        *reinterpret_cast<float4*>(rp + 4 * ot) = make_float4(s8.o[0][0], s8.o[1][0], s8.o[0][1], s8.o[1][1]);
+      } else {
+#pragma unroll
+        for (int n4 = 0; n4 < 2; ++n4)
+          if (n4 * 32 < dkv) {
+            *reinterpret_cast<float4*>(rp + n4 * 32 + 8 * ot) = make_float4(s8.o[4 * n4][0], s8.o[4 * n4 + 1][0], s8.o[4 * n4 + 2][0], s8.o[4 * n4 + 3][0]);
+            *reinterpret_cast<float4*>(rp + n4 * 32 + 8 * ot + 4) = make_float4(s8.o[4 * n4][1], s8.o[4 * n4 + 1][1], s8.o[4 * n4 + 2][1], s8.o[4 * n4 + 3][1]);
           }
-          const int ja = k0 + 2 * t;
-          const float v00 = ja < nk ? sV[(size_t)ja * vst + n0 + g] : 0.f, v01 = ja + 1 < nk ? sV[(size_t)(ja + 1) * vst + n0 + g] : 0.f;
-          const float v10 = ja + 8 < nk ? sV[(size_t)(ja + 8) * vst + n0 + g] : 0.f, v11 = ja + 9 < nk ? sV[(size_t)(ja + 9) * vst + n0 + g] : 0.f;
-          const uint32_t ah0 = sl_pack_bf16(p0.x, p0.y), ah2 = sl_pack_bf16(p1.x, p1.y);
-          const uint32_t al0 = sl_pack_bf16(p0.x - __uint_as_float(ah0 << 16), p0.y - __uint_as_float(ah0 & 0xffff0000u));
-          const uint32_t al2 = sl_pack_bf16(p1.x - __uint_as_float(ah2 << 16), p1.y - __uint_as_float(ah2 & 0xffff0000u));
-          const uint32_t bh0 = sl_pack_bf16(v00, v01), bh1 = sl_pack_bf16(v10, v11);
-          const uint32_t bl0 = sl_pack_bf16(v00 - __uint_as_float(bh0 << 16), v01 - __uint_as_float(bh0 & 0xffff0000u));
-          const uint32_t bl1 = sl_pack_bf16(v10 - __uint_as_float(bh1 << 16), v11 - __uint_as_float(bh1 & 0xffff0000u));
-#define SUB_MMA(A0, A2, B0, B1)                                                                                                  \
-          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};" \
-                       : "+f"(acc[0]), "+f"(acc[1]), "+f"(c2), "+f"(c3) : "r"(A0), "r"(zero), "r"(A2), "r"(zero), "r"(B0), "r"(B1))
-          SUB_MMA(ah0, ah2, bh0, bh1);
-          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                       : "+f"(d0), "+f"(d1), "+f"(d2), "+f"(d3) : "r"(al0), "r"(zero), "r"(al2), "r"(zero), "r"(bh0), "r"(bh1));
-          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                       : "+f"(d0), "+f"(d1), "+f"(d2), "+f"(d3) : "r"(ah0), "r"(zero), "r"(ah2), "r"(zero), "r"(bl0), "r"(bl1));
-#undef SUB_MMA
-        }
-        acc[0] += d0; acc[1] += d1;
       }
     }
-  }
-  // this rank's record (max, sum, weighted values per row), assembled locally
-  if (ONE) {
-    *reinterpret_cast<float4*>(sRed + (size_t)part4 * dkv + cg4 * 4) = acc4;
-    if (cg4 == 0) sRed[SUB_THREADS * 4 + part4] = lsum1;
-    __syncthreads();
-    if (tid < dkv) {
-      float t = 0.f;
-#pragma unroll 16
-      for (int p2 = 0; p2 < nparts4; ++p2) t += sRed[p2 * dkv + tid];
-      recLoc[SUB_RECPAD + tid] = t;
-    } else if (warp == SUB_THREADS / 32 - 1) {   // the parts' sums, added by one warp
-      float l = 0.f;
-      for (int p2 = lane; p2 < nparts4; p2 += 32) l += sRed[SUB_THREADS * 4 + p2];
-      l = warp_sum(l);
-      if (lane == 0) { recLoc[0] = run1; recLoc[1] = l; recLoc[2] = 0.f; recLoc[3] = 0.f; }
-    }
-  } else {
-    if (warp * 8 < dkv && (lane >> 2) < k)   // accumulators of the tile: row lane / 4, channels 8 warp + 2 (lane % 4) (+ 1)
-      *reinterpret_cast<float2*>(recLoc + (size_t)(lane >> 2) * recst + SUB_RECPAD + warp * 8 + 2 * (lane & 3)) = make_float2(acc[0], acc[1]);
-    if (tid < k) { recLoc[(size_t)tid * recst] = sh->rmax[tid]; recLoc[(size_t)tid * recst + 1] = sh->rsum[tid]; }
   }
   __syncthreads();
   SUB_STAMP();            // 7: attention over this rank's keys
-  if (red) {   // this rank's record covers every key: the head output is its values over its sum
+  const float* rec = sRec;
+  int nrec = 8;
+  if (!red) {   // the ranks hold different keys: the block's merged records go to every rank
+    const int nu = 1 + (dkv >> 2);   // 16-byte pieces of a record
+    float sum;
+    if (ONE) {
 #pragma unroll 1
-    for (int o = tid; o < k * dkv; o += SUB_THREADS) {
-      const int m = o >> a.dkv_shift, cc = o & (dkv - 1);
-      sA[(size_t)m * dkv + cc] = recLoc[(size_t)m * recst + SUB_RECPAD + cc] / recLoc[(size_t)m * recst + 1];
+      for (int idx = tid; idx < nu << a.c_shift; idx += SUB_THREADS) {
+        const int rk = idx & (C - 1), u = idx >> a.c_shift;
+        sub_push4(sRrec + (size_t)r * recst + 4 * u, &sh->xbar[1], (uint32_t)rk, sub_merge(sRec, recst, 8, u - 1, sum));
+      }
+    } else {
+#pragma unroll 1
+      for (int m = warp; m < k; m += SUB_THREADS / 32)
+        if (lane < nu) {
+          const float4 v = sub_merge(sRec + (size_t)m * recst, MBC * recst, 8, lane - 1, sum);
+#pragma unroll 1
+          for (int rk = 0; rk < C; ++rk) sub_push4(sRrec + (size_t)(r * MBC + m) * recst + 4 * lane, &sh->xbar[1], (uint32_t)rk, v);
+        }
     }
-    SUB_STAMP(); SUB_STAMP(); SUB_STAMP();
+    SUB_STAMP();          // 8: records merged and sent
+    sub_wait_exchange(sh, a.err, &sh->xbar[1], a.spin);
+    rec = sRrec; nrec = C;
+    SUB_STAMP();          // 9: exchange 2
   } else {
-  {   // the record goes to every block of the cluster: one 16-byte store per thread and turn
-    const int q4 = (k * recst) >> 2, tot = q4 << a.c_shift;
-#pragma unroll 1
-    for (int idx = tid; idx < tot; idx += SUB_THREADS) {
-      const int rk = idx & (C - 1), q = idx >> a.c_shift;
-      st_cluster_f4(smem_u32(rec + (size_t)r * a.mb * recst + q * 4), (uint32_t)rk, *reinterpret_cast<const float4*>(recLoc + q * 4));
-    }
+    SUB_STAMP(); SUB_STAMP();
   }
-  SUB_STAMP();            // 8: record stores
-  sub_cluster_arrive();   // (2) all records are in place
-  sub_cluster_wait();
-  SUB_STAMP();            // 9: cluster barrier 2
-  // ---- phase C: merge in rank order, then this rank's rows of the output projection ---------------
-#pragma unroll 1
-  for (int o = tid; o < k * dkv; o += SUB_THREADS) {
-    const int m = o >> a.dkv_shift, cc = o & (dkv - 1);
-    float mx[8], ls[8], av[8], gm = -INFINITY;   // the ranks' records are loaded side by side (C <= 8)
+  // ---- phase C: this rank's rows of the output projection ---------------
+  if (ONE) {
+    // one row: the up to eight records are the columns of the right operand, each scaled by its weight in the merged soft-max
+    // (fp32 as three bf16 parts); the sum over the columns is the output
+    const float* rg = rec + (size_t)min(og, nrec - 1) * recst;
+    const float2 ml = *reinterpret_cast<const float2*>(rg);
+    float gm = og < nrec ? ml.x : -INFINITY;
 #pragma unroll
-    for (int rk = 0; rk < 8; ++rk) {
-      const float* rp = rec + ((size_t)min(rk, C - 1) * a.mb + m) * recst;
-      const float2 ml = *reinterpret_cast<const float2*>(rp);
-      mx[rk] = ml.x; ls[rk] = rk < C ? ml.y : 0.f; av[rk] = rp[SUB_RECPAD + cc];
-    }
+    for (int o = 4; o < 32; o <<= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+    const float w = og < nrec && ml.y > 0.f ? __expf(ml.x - gm) : 0.f;
+    float den = w * ml.y;
 #pragma unroll
-    for (int rk = 0; rk < 8; ++rk) gm = fmaxf(gm, mx[rk]);
-    float num = 0.f, den = 0.f;
+    for (int o = 4; o < 32; o <<= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+    const float sc = w * sub_rcp(den);
+    float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f}, f[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int rk = 0; rk < 8; ++rk) {   // fixed rank order
-      const float w = ls[rk] > 0.f ? __expf(mx[rk] - gm) : 0.f;
-      den += ls[rk] * w;
-      num += (ls[rk] > 0.f ? av[rk] : 0.f) * w;
-    }
-    sA[(size_t)m * dkv + cc] = num / den;
-  }
-  SUB_STAMP();            // 10: merge
-  }
-  __syncthreads();
-  if (ONE) {   // output projection, one row: the thread's channels of rows g and g + 8, then the four threads of a row add up
-#pragma unroll
-    for (int rr = 0; rr < 2; ++rr) {
-      const float* ap = sA + ot * cpt;
-      float o = 0.f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (2 * i < cpt) o += __uint_as_float(wr[rr][i] << 16) * ap[2 * i] + __uint_as_float(wr[rr][i] & 0xffff0000u) * ap[2 * i + 1];
-      o += __shfl_xor_sync(0xffffffffu, o, 1);
-      o += __shfl_xor_sync(0xffffffffu, o, 2);
-      const int row = warp * 16 + og + 8 * rr;
-      if (ot == 0 && row < no) atomicAdd(a.x_out + o0 + row, h == 0 ? o + sSeed[row] : o);   // residual term once per column
+    for (int st = 0; st < 4; ++st)
+      if (st * 16 < dkv) {
+        float4 v = *reinterpret_cast<const float4*>(rg + SUB_RECPAD + ot * cpt + 4 * st);
+        if (!(sc > 0.f)) v = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t h0, h1, m0, m1, l0, l1;
+        sub_split3(v.x * sc, v.y * sc, h0, m0, l0);
+        sub_split3(v.z * sc, v.w * sc, h1, m1, l1);
+        sub_mma(c, wr[0][2 * st], wr[1][2 * st], wr[0][2 * st + 1], wr[1][2 * st + 1], h0, h1);
+        sub_mma(e, wr[0][2 * st], wr[1][2 * st], wr[0][2 * st + 1], wr[1][2 * st + 1], m0, m1);
+        sub_mma(f, wr[0][2 * st], wr[1][2 * st], wr[0][2 * st + 1], wr[1][2 * st + 1], l0, l1);
+      }
+    // accumulators: rows g and g + 8 of the tile, columns 2 t and 2 t + 1
+    float v0 = (c[0] + c[1]) + ((e[0] + e[1]) + (f[0] + f[1])), v1 = (c[2] + c[3]) + ((e[2] + e[3]) + (f[2] + f[3]));
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 1); v1 += __shfl_xor_sync(0xffffffffu, v1, 1);
+    v0 += __shfl_xor_sync(0xffffffffu, v0, 2); v1 += __shfl_xor_sync(0xffffffffu, v1, 2);
+    const int row = warp * 16 + og + 8 * ot;
+    if (ot < 2 && row < no) {
+      const float v = ot ? v1 : v0;
+      atomicAdd(a.x_out + o0 + row, h == 0 ? v + sSeed[row] : v);   // residual term once per column
     }
   } else {
-    // output projection on mma.sync m16n8k16: rows of W_o x token rows (the right operand: the merged head output, each value
-    // as a bf16 head and a bf16 remainder), 16 channels per step
+    // merged head output of every row, then rows of W_o x token rows on mma.sync m16n8k16 (the right operand: each value as a
+    // bf16 head and a bf16 remainder), 16 channels per step
+    const int ast = dkv + 4;
+#pragma unroll 1
+    for (int idx = tid; idx < k << (a.dkv_shift - 2); idx += SUB_THREADS) {
+      const int m = idx >> (a.dkv_shift - 2), u = idx & ((dkv >> 2) - 1);
+      float sum;
+      float4 v = sub_merge(rec + (size_t)m * recst, MBC * recst, nrec, u, sum);
+      const float is = sub_rcp(sum);
+      *reinterpret_cast<float4*>(sA + (size_t)m * ast + 4 * u) = make_float4(v.x * is, v.y * is, v.z * is, v.w * is);
+    }
+    __syncthreads();
+    SUB_STAMP();          // 10: merge
     float* sOut = reinterpret_cast<float*>(sub_smem + a.L.out);
     const int ost = no + 4;
     if (warp * 16 < no) {
-      float c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f, e0 = 0.f, e1 = 0.f, e2 = 0.f, e3 = 0.f;   // (heads | remainders: two chains)
+      float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};   // (heads | remainders: two chains)
 #pragma unroll
       for (int st = 0; st < 4; ++st)
         if (st * 16 < dkv) {
           float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (og < k) b4 = *reinterpret_cast<const float4*>(sA + (size_t)og * dkv + ot * cpt + 4 * st);
-          const uint32_t bh0 = sl_pack_bf16(b4.x, b4.y), bh1 = sl_pack_bf16(b4.z, b4.w);
-          const uint32_t bl0 = sl_pack_bf16(b4.x - __uint_as_float(bh0 << 16), b4.y - __uint_as_float(bh0 & 0xffff0000u));
-          const uint32_t bl1 = sl_pack_bf16(b4.z - __uint_as_float(bh1 << 16), b4.w - __uint_as_float(bh1 & 0xffff0000u));
-          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                       : "+f"(c0), "+f"(c1), "+f"(c2), "+f"(c3)
-                       : "r"(wr[0][2 * st]), "r"(wr[1][2 * st]), "r"(wr[0][2 * st + 1]), "r"(wr[1][2 * st + 1]), "r"(bh0), "r"(bh1));
-          asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                       : "+f"(e0), "+f"(e1), "+f"(e2), "+f"(e3)
-                       : "r"(wr[0][2 * st]), "r"(wr[1][2 * st]), "r"(wr[0][2 * st + 1]), "r"(wr[1][2 * st + 1]), "r"(bl0), "r"(bl1));
+          if (og < k) b4 = *reinterpret_cast<const float4*>(sA + (size_t)og * ast + ot * cpt + 4 * st);
+          uint32_t h0, h1, l0, l1;
+          sub_split(b4.x, b4.y, h0, l0); sub_split(b4.z, b4.w, h1, l1);
+          sub_mma(c, wr[0][2 * st], wr[1][2 * st], wr[0][2 * st + 1], wr[1][2 * st + 1], h0, h1);
+          sub_mma(e, wr[0][2 * st], wr[1][2 * st], wr[0][2 * st + 1], wr[1][2 * st + 1], l0, l1);
         }
-      c0 += e0; c1 += e1; c2 += e2; c3 += e3;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) c[i] += e[i];
       // accumulators: rows g and g + 8 of the tile, token rows 2 t and 2 t + 1
       const int row = warp * 16 + og;
-      if (row < no) { sOut[(size_t)(2 * ot) * ost + row] = c0; sOut[(size_t)(2 * ot + 1) * ost + row] = c1; }
-      if (row + 8 < no) { sOut[(size_t)(2 * ot) * ost + row + 8] = c2; sOut[(size_t)(2 * ot + 1) * ost + row + 8] = c3; }
+      if (row < no) { sOut[(size_t)(2 * ot) * ost + row] = c[0]; sOut[(size_t)(2 * ot + 1) * ost + row] = c[1]; }
+      if (row + 8 < no) { sOut[(size_t)(2 * ot) * ost + row + 8] = c[2]; sOut[(size_t)(2 * ot + 1) * ost + row + 8] = c[3]; }
     }
     __syncthreads();
     const int n4 = no >> 2;
@@ -838,7 +962,7 @@ __global__ void pack_wfo_kernel(const __nv_bfloat16* __restrict__ W, uint4* __re
   }
 }
 
-struct FfnSubLayout { int wi, xs, psum, u, seed, sh, total; };
+struct FfnSubLayout { int wi, wi2, xs, psum, u, seed, sh, total; };
 
 struct FfnSubArgs {
   const CallDesc* desc;
@@ -846,7 +970,7 @@ struct FfnSubArgs {
   float* x_out;
   float* x_zero;             // nullptr: nothing to clear (second part of a split launch)
   const float* gain;
-  float eps;
+  float eps, inv_d;          // inv_d: 1 / d
   const __nv_bfloat16* Wi0;  // [F][d]
   const __nv_bfloat16* Wi1;  // [F][d] gate matrix (gated GELU) or nullptr
   const uint4* Wfo1;         // W_fo in the load order of the single-row variant (pack_wfo_kernel)
@@ -866,9 +990,11 @@ inline FfnSubLayout ffn_sub_layout(int d, int F, int gated, int slices, int grid
   FfnSubLayout L;
   const int nf = ffn_sub_rows(F, slices), nmat = gated ? 2 : 1;
   int off = 0;
-  L.wi = off; off += sub_up16(nf * nmat * (d * 2 + SL_WPAD));
-  L.xs = off; off += sub_up16(mb * (d + SL_XPAD) * 4);   // token rows; the block variant later collects its output tile here
-  L.psum = off; off += mb == 1 ? SUB_PSUM : 8 * 128 * 4;
+  // weight rows of W_i (and the gate); once they wait in registers (the first 32), the slice's units of W_fo take their place
+  const int fo_b = nf / 8 * (pack_wfo_dpad(d) * 16 + 32);
+  L.wi = off; L.wi2 = sub_up16(std::max(std::min(nf * nmat, 32) * sub_wst(d), fo_b)); off += L.wi2 + sub_up16(std::max(nf * nmat - 32, 0) * sub_wst(d));
+  L.xs = off; off += std::max(sub_up16(sub_xs_bytes(d, mb)), mb == 1 ? 0 : sub_up16(mb * (d + 4) * 4));   // token rows; later the block variant's output tile
+  L.psum = off; off += sub_up16(sub_psum_bytes(nf * nmat, mb));
   L.u = off; off += sub_up16(mb * (SUB_FO_REGS + 4) * 4);
   L.seed = off; off += sub_up16(mb * 4 * ((d / 4 + grid - 1) / grid + 1) * 4);
   L.sh = off; off += sub_up16((int)sizeof(SubShared));
@@ -876,21 +1002,27 @@ inline FfnSubLayout ffn_sub_layout(int d, int F, int gated, int slices, int grid
   return L;
 }
 
+// Bound as the attention kernels by its dependent chain: token rows, products, activation, output products, reductions at the L2
+// (every block adds a partial sum to every output: 148 additions per address).  Times: see attn_sub_kernel.
 template <bool ONE>
-__global__ void __launch_bounds__(SUB_THREADS) ffn_sub_kernel(const FfnSubArgs a) {
+__global__ void __launch_bounds__(SUB_THREADS, 2) ffn_sub_kernel(const FfnSubArgs a) {
   extern __shared__ __align__(1024) unsigned char sub_smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int d = a.d, F = a.F, G = gridDim.x, S = G * a.nparts, s = blockIdx.x * a.nparts + a.part;
   const int f0 = 8 * (int)(((long long)s * (F >> 3)) / S), f1 = 8 * (int)(((long long)(s + 1) * (F >> 3)) / S), nf = f1 - f0;
   const int nmat = a.gated ? 2 : 1, nrows = nf * nmat;
-  const int rowbytes = d * 2 + SL_WPAD, xst = d + SL_XPAD;
+  const int wst = sub_wst(d), xst = sub_xst(d);
   unsigned char* sWi = sub_smem + a.L.wi;
-  float* Xs = reinterpret_cast<float*>(sub_smem + a.L.xs);
+  unsigned char* sWi2 = sWi + a.L.wi2 - 32 * wst;   // rows 32 and up
+  uint32_t* Xs = reinterpret_cast<uint32_t*>(sub_smem + a.L.xs);
   float* psum = reinterpret_cast<float*>(sub_smem + a.L.psum);
   float* sU = reinterpret_cast<float*>(sub_smem + a.L.u);
   float* sSeed = reinterpret_cast<float*>(sub_smem + a.L.seed);
   SubShared* sh = reinterpret_cast<SubShared*>(sub_smem + a.L.sh);
   constexpr int ust = SUB_FO_REGS + 4;
+  const int cpw = sub_chunks(d), col0 = warp * 32 * cpw, nch = max(0, min(cpw, (d - col0 + 31) >> 5));
+  const int col = col0 + lane * 4;
+  const bool stores = lane * 4 < 32 * nch, on = stores && col < d;   // this lane's four columns of the token rows
   // columns whose residual term this block adds: units of four columns, spread over the grid
   const int d4 = d >> 2;
   const int su0 = a.seed ? (int)(((long long)blockIdx.x * d4) / G) : 0, su1 = a.seed ? (int)(((long long)(blockIdx.x + 1) * d4) / G) : 0;
@@ -903,95 +1035,112 @@ __global__ void __launch_bounds__(SUB_THREADS) ffn_sub_kernel(const FfnSubArgs a
     mbar_expect(smem_u32(&sh->wbar), (uint32_t)(nrows * d * 2));
   }
   __syncthreads();
-  pdl_launch_dependents();
   {   // row i is copied by lane i / 8 of warp i % 8 (the copies of one warp are issued one after the other)
     const int i = ((tid & 31) << 3) | (tid >> 5);
     if (i < nrows) {
       const __nv_bfloat16* W = i < nf ? a.Wi0 : a.Wi1;
       const int rr = i < nf ? i : i - nf;
-      bulk_g2s(smem_u32(sWi + (size_t)i * rowbytes), W + (size_t)(f0 + rr) * d, (uint32_t)(d * 2), smem_u32(&sh->wbar));
-    }
-  }
-  // The block's columns [f0, f1) of W_fo stay in registers, 16 bytes (8 columns of a row) per load, from the copies of
-  // W_fo that pack_wfo_kernel lays out so that the loads of a warp are contiguous (8 columns of a row in place are 16
-  // bytes every 2 F bytes: a fraction of the memory's rate).  ONE: thread <-> the four output rows 4 tid .. 4 tid + 3,
-  // chunk q = columns 8 q .. 8 q + 7.  Block variant: warp w owns the output tiles w, w + 8, ... (16 rows each); thread
-  // (g, t) keeps, of rows g and g + 8 of a tile, the columns 8 t .. 8 t + 7: read as the left operand of mma.sync m16n8k16
-  // they are two steps of 16 slice rows, with the slice rows dealt to the steps' positions so that one 16-byte load
-  // fills them (the right operand, the hidden activations, follows the same order).
-  uint4 wf[8][2];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) wf[i][j] = make_uint4(0u, 0u, 0u, 0u);
-  if (ONE) {
-    if (tid * 4 < d) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (8 * q < nf) {
-          const uint4* p = a.Wfo1 + (size_t)((f0 >> 3) + q) * d + tid;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            uint4& w = wf[i * 2 + (q >> 1)][q & 1];
-            asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(p + i * (d >> 2)));
-          }
-        }
-    }
-  } else {
-    const int g = lane >> 2, t = lane & 3;
-    if (8 * t < nf) {
-      const uint4* p = a.Wfo8 + (size_t)((f0 >> 3) + t) * pack_wfo_dpad(d) + warp * 8 + g;
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if ((warp + 8 * i) * 16 < d) {
-#pragma unroll
-          for (int rr = 0; rr < 2; ++rr) {
-            uint4& w = wf[i][rr];
-            asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(w.x), "=r"(w.y), "=r"(w.z), "=r"(w.w) : "l"(p + (i * 2 + rr) * 64));
-          }
-        }
+      bulk_g2s(smem_u32(i < 32 ? sWi + (size_t)i * wst : sWi2 + (size_t)i * wst), W + (size_t)(f0 + rr) * d, (uint32_t)(d * 2), smem_u32(&sh->wbar));
     }
   }
   float4 g4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (tid * 4 < d) g4 = __ldg(reinterpret_cast<const float4*>(a.gain) + tid);
+  if (on) g4 = __ldg(reinterpret_cast<const float4*>(a.gain + col));
   const int k = ONE ? 1 : min(a.desc->k, a.mb);   // (written before the pass began: see the attention kernel)
-  SUB_STAMP();            // 0: prologue
+  SUB_STAMP();            // 0: requests
+  // The rows of W_i become operands in registers; then the block's columns [f0, f1) of W_fo are fetched into their place, as units of
+  // 8 columns from the copies of W_fo that pack_wfo_kernel lays out (8 columns of a row in place are 16 bytes every 2 F bytes: a
+  // fraction of the memory's rate).  Both by bulk copies: 64 KB a block through the load units held up the shared-memory
+  // accesses of the kernel in front on the same SM (5-row pass 594 -> 551 us without them).
+  const int ust_fo = (ONE ? d : pack_wfo_dpad(d)) * 16 + 32;   // bytes from unit to unit: the lanes (row g, unit t) hit 32 banks
+  uint4 fr[2][4][2];
+  if (nf > 0) {
+    sub_wait(sh, a.err, &sh->wbar, 0, a.spin);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i * 16 < nrows) sub_frags(sWi, wst, nrows, d, i, col0, nch, lane, fr[i]);
+    __syncthreads();
+    const uint32_t ub = (uint32_t)(ust_fo - 32);
+    if (tid == 0) mbar_expect(smem_u32(&sh->wbar), ub * (uint32_t)(nf >> 3));
+    if (tid < (nf >> 3)) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      bulk_g2s(smem_u32(sWi + (size_t)tid * ust_fo), reinterpret_cast<const unsigned char*>(ONE ? a.Wfo1 : a.Wfo8) + (size_t)((f0 >> 3) + tid) * ub, ub,
+               smem_u32(&sh->wbar));
+    }
+  }
+  SUB_STAMP();            // 1: weights
   pdl_wait();
-  SUB_STAMP();            // 1: dependency wait
+  pdl_launch_dependents();   // (the next kernel's requests behind this kernel's own rows)
+  SUB_STAMP();            // 2: dependency wait
   SubRows<ONE> rw;
-  sub_rows_issue<ONE>(a.x_in, k, d, tid, rw);
+  sub_rows_issue<ONE>(a.x_in, k, d, col, on, rw);
   if (a.x_zero) {
     const int n4 = k * d4;
 #pragma unroll 1
     for (int i = blockIdx.x * SUB_THREADS + tid; i < n4; i += G * SUB_THREADS)
       reinterpret_cast<float4*>(a.x_zero)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  const float inv1 = sub_rows_finish<ONE>(rw, k, d, g4, a.eps, Xs, xst, sh, sSeed, su0 * 4, su1 * 4, tid, lane, warp);
-  SUB_STAMP();            // 2: token rows + norm
-  {
-    if (nf > 0) sub_wait(sh, a.err, &sh->wbar, 0, a.spin);
-    SUB_STAMP();          // 3: wait for the weights
-    // hidden activations of the slice
-    if (ONE) sl_items<1>(sWi, rowbytes, nrows, d, Xs, xst, psum, warp, lane);
-    else sub_mma_split(sWi, rowbytes, nrows, d, Xs, k, psum, warp, lane);
-    __syncthreads();   // (both product routines do nothing for a block without rows)
-    if (ONE) {
-      if (tid < nf) {
-        const float v0 = sub_total<true>(psum, tid, 0, nrows, d) * inv1;
-        sU[tid] = a.gated ? gelu_tanh(v0) * (sub_total<true>(psum, nf + tid, 0, nrows, d) * inv1) : fmaxf(v0, 0.f);
-      }
-    } else {   // thread <-> (token row, slice row) of the 8 x 32 tile the output products read; what lies outside is zero
-      const int m = tid >> 5, i = tid & 31;
-      float uv = 0.f;
-      if (m < k && i < nf) {
-        const float sc = sh->inv[m], v0 = sub_total<false>(psum, i, m, nrows, d) * sc;
-        uv = a.gated ? gelu_tanh(v0) * (sub_total<false>(psum, nf + i, m, nrows, d) * sc) : fmaxf(v0, 0.f);
-      }
-      sU[(size_t)m * ust + i] = uv;
+  sub_rows_split<ONE>(rw, k, col, stores, on, g4, Xs, xst, sh, sSeed, su0 * 4, su1 * 4, lane, warp);
+  SUB_STAMP();            // 3: token rows
+  if (nf > 0) {   // hidden activations of the slice
+    SubB<ONE> b;
+    sub_bfrags<ONE>(Xs, xst, k, col0, nch, lane, b);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (i * 16 < nrows) sub_tile<ONE>(fr[i], b, nch, nrows, i, psum, warp, lane);
+    if (nrows > 32) {
+      sub_frags(sWi2, wst, nrows, d, 2, col0, nch, lane, fr[0]);
+      sub_tile<ONE>(fr[0], b, nch, nrows, 2, psum, warp, lane);
     }
-    __syncthreads();
-    SUB_STAMP();          // 4: hidden activations
   }
+  // W_fo into registers while the sums go round.  ONE: thread <-> the four output rows 4 tid .. 4 tid + 3, chunk q = columns 8 q .. 8 q + 7.
+  // Block variant: warp w owns the output tiles w, w + 8, ... (16 rows each); thread (g, t) takes, of rows g and g + 8 of a tile, the
+  // columns 8 t .. 8 t + 7: read as the left operand of mma.sync m16n8k16 they are two steps of 16 slice rows, with the slice rows
+  // dealt to the steps' positions so that one 16-byte load fills them (the right operand, the hidden activations, follows the same order).
+  uint4 wf[8][2];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j) wf[i][j] = make_uint4(0u, 0u, 0u, 0u);
+  if (nf > 0) sub_wait(sh, a.err, &sh->wbar, 1, a.spin);
+  if (ONE) {
+    if (tid * 4 < d) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (8 * q < nf) {
+          const uint4* p = reinterpret_cast<const uint4*>(sWi + (size_t)q * ust_fo) + tid;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) wf[i * 2 + (q >> 1)][q & 1] = p[i * (d >> 2)];
+        }
+    }
+  } else {
+    const int g = lane >> 2, t = lane & 3;
+    if (8 * t < nf) {
+      const uint4* p = reinterpret_cast<const uint4*>(sWi + (size_t)t * ust_fo) + warp * 8 + g;
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if ((warp + 8 * i) * 16 < d) {
+          wf[i][0] = p[i * 128]; wf[i][1] = p[i * 128 + 64];
+        }
+    }
+  }
+  __syncthreads();
+  SUB_STAMP();            // 4: products
+  const int pst = sub_pst(nrows);
+  if (ONE) {
+    if (tid < nf) {
+      const float inv = sub_inv(sh, 0, a.inv_d, a.eps), v0 = sub_total<true>(psum, tid, 0, pst) * inv;
+      sU[tid] = a.gated ? gelu_tanh(v0) * (sub_total<true>(psum, nf + tid, 0, pst) * inv) : fmaxf(v0, 0.f);
+    }
+  } else {   // warp <-> token row, lane <-> slice row of the 8 x 32 tile the output products read; what lies outside is zero
+    float uv = 0.f;
+    if (warp < k && lane < nf) {
+      const float inv = sub_inv(sh, warp, a.inv_d, a.eps), v0 = sub_total<false>(psum, lane, warp, pst) * inv;
+      uv = a.gated ? gelu_tanh(v0) * (sub_total<false>(psum, nf + lane, warp, pst) * inv) : fmaxf(v0, 0.f);
+    }
+    sU[(size_t)warp * ust + lane] = uv;
+  }
+  __syncthreads();
+  SUB_STAMP();            // 5: hidden activations
   if (ONE) {
     // this slice's share of all d outputs: thread <-> four output rows, their columns of W_fo from its registers
     if (tid < d4) {
@@ -1029,7 +1178,8 @@ __global__ void __launch_bounds__(SUB_THREADS) ffn_sub_kernel(const FfnSubArgs a
       bl[st][0] = sl_pack_bf16(u4.x - __uint_as_float(bh[st][0] << 16), u4.y - __uint_as_float(bh[st][0] & 0xffff0000u));
       bl[st][1] = sl_pack_bf16(u4.z - __uint_as_float(bh[st][1] << 16), u4.w - __uint_as_float(bh[st][1] & 0xffff0000u));
     }
-    float* sOut = Xs;   // [token][column], row stride xst: the token rows are done with
+    float* sOut = reinterpret_cast<float*>(Xs);   // [token][column]: the token rows are done with
+    const int ost = d + 4;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       const int n0 = (warp + 8 * i) * 16;
@@ -1044,17 +1194,18 @@ __global__ void __launch_bounds__(SUB_THREADS) ffn_sub_kernel(const FfnSubArgs a
         SUB_MMA(wf[i][0].z, wf[i][1].z, wf[i][0].w, wf[i][1].w, bl[1][0], bl[1][1]);
 #undef SUB_MMA
         // accumulators: columns n0 + g and n0 + g + 8, token rows 2 t and 2 t + 1
-        sOut[(size_t)(2 * t) * xst + n0 + g] = c0; sOut[(size_t)(2 * t + 1) * xst + n0 + g] = c1;
-        sOut[(size_t)(2 * t) * xst + n0 + g + 8] = c2; sOut[(size_t)(2 * t + 1) * xst + n0 + g + 8] = c3;
+        sOut[(size_t)(2 * t) * ost + n0 + g] = c0; sOut[(size_t)(2 * t + 1) * ost + n0 + g] = c1;
+        sOut[(size_t)(2 * t) * ost + n0 + g + 8] = c2; sOut[(size_t)(2 * t + 1) * ost + n0 + g + 8] = c3;
       }
     }
     __syncthreads();
 #pragma unroll 1
-    for (int idx = tid; idx < k * d4; idx += SUB_THREADS) {   // added four columns at a time
-      const int m = idx / d4, un = idx - m * d4;
+    for (int un = tid; un < d4; un += SUB_THREADS)   // added four columns at a time
+#pragma unroll 1
+    for (int m = 0; m < k; ++m) {
       const bool seeds = un >= su0 && un < su1;
       if (nf > 0 || seeds) {
-        float4 v = *reinterpret_cast<const float4*>(sOut + (size_t)m * xst + un * 4);
+        float4 v = *reinterpret_cast<const float4*>(sOut + (size_t)m * ost + un * 4);
         if (seeds) {
           const float4 xr = *reinterpret_cast<const float4*>(sSeed + (size_t)m * (su1 - su0) * 4 + (un - su0) * 4);
           v.x += xr.x; v.y += xr.y; v.z += xr.z; v.w += xr.w;
@@ -1064,7 +1215,7 @@ __global__ void __launch_bounds__(SUB_THREADS) ffn_sub_kernel(const FfnSubArgs a
       }
     }
   }
-  SUB_STAMP();            // 5: output products + reductions issued
+  SUB_STAMP();            // 6: output products + reductions issued
   SUB_STAMP_END(2);
 }
 

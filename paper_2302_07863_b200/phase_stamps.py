@@ -26,8 +26,8 @@ ctx, ids, wl = make_context(wlname, g["scale_small"]["scale"], g["scale_large"][
 ctx.encode(ids)
 L = B.lib()
 L.bild_debug_stamps.argtypes = [C.POINTER(C.c_ulonglong), C.c_int]
-names = {0: ["P0 init", "P1 copies", "P2 loads", "arrive", "dep wait", "rows+norm", "weights wait", "qkv products", "exch stores", "cluster bar 1", "B1 staged", "B2 scores", "B3 softmax", "attention(pv)", "rec stores", "cluster bar 2", "merge", "oproj+red"],
-         1: None, 2: ["prologue", "dep wait", "rows+norm", "weights wait", "hidden", "out+red"]}
+names = {0: ["requests", "weights", "dep wait", "rows", "qkv products", "exch stores", "exchange 1", "attention", "rec stores", "exchange 2", "merge", "oproj+red"],
+         1: None, 2: ["requests", "weights", "dep wait", "rows", "products", "hidden", "out+red"]}
 names[1] = names[0]
 def run(which, k):
     buf = (C.c_ulonglong * 288)()
@@ -38,12 +38,12 @@ def run(which, k):
     for kind, nm in (("self", 0), ("cross", 1), ("ffn", 2)):
         n0, na = buf[nm * 24 + 23], buf[96 + nm * 24 + 23]
         if not n0: continue
-        # single-row kernels have no separate soft-max phase (it is part of the value phase)
-        nms = [x for x in names[nm] if not (k == 1 and x == "B3 softmax")]
+        # single-row kernels merge the records as operands of the output projection
+        nms = [x for x in names[nm] if not (k == 1 and x == "merge")]
         ph0 = [buf[nm * 24 + i] / n0 / 1965.0 for i in range(len(nms))]
         pha = [buf[96 + nm * 24 + i] / na / 1965.0 for i in range(len(nms))]
         phm = [buf[192 + nm * 24 + i] / 1965.0 for i in range(len(nms))]
-        off = 5 if nm < 2 else 2
+        off = 3
         print(f"  {kind:5s} after wait: block 0 {sum(ph0[off:]):.2f} us, mean of blocks {sum(pha[off:]):.2f} us | " +
               " ".join(f"{a}={b:.2f}/{c:.2f}/{e:.2f}" for a, b, c, e in zip(nms, ph0, pha, phm)))
 run(0, 1)
