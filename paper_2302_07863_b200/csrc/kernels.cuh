@@ -487,6 +487,10 @@ struct HeadArgs {
   int sw_bodies;
   int pass_kind;                 // which pass counter the kernel bumps inside a loop graph: 0 small, 1 block, 2 single row, 3 up to 8 rows
   int defer_policy;              // sampling: the head leaves policy and loop control to the kernel that draws the token
+  // single-step calls: pinned HOST memory the results are written to (five to fifty words over the bus, on their way while the
+  // kernel ends, instead of two copies behind it); nullptr otherwise
+  HeadOut* host_head;
+  DevState* host_state;
 };
 
 // What the last block of every LM-head kernel does once the per-row results are complete: the policy tests, the
@@ -498,6 +502,15 @@ __device__ inline void policy_tail(const HeadArgs& a, HeadOut* o) {
   if (a.desc->run_policy) policy_step(a.loop, o, a.desc, a.which);
   else if (a.which == 0) a.loop.st->S_len = a.desc->pos0 + 1;
   else a.loop.st->L_len = a.desc->pos0 + a.desc->k;
+  if (a.host_head) {
+    volatile HeadOut* w = a.host_head;
+    const int k = a.which == 0 ? 1 : a.desc->k;
+    for (int i = 0; i < k; ++i) { w->argmax[i] = o->argmax[i]; w->lse[i] = o->lse[i]; w->d[i] = o->d[i]; }
+    w->zmax[0] = o->zmax[0]; w->pmax = o->pmax; w->fallback = o->fallback;
+    w->first_violation = o->first_violation; w->next_token = o->next_token;
+    volatile DevState* v = a.host_state;
+    v->S_len = a.loop.st->S_len; v->L_len = a.loop.st->L_len; v->err = *(volatile int*)&a.loop.st->err;
+  }
   if (a.cond_while) {
     a.loop.st->cum_passes[a.pass_kind]++;
     cudaGraphSetConditional(a.cond_while, a.loop.st->done ? 0u : 1u);
@@ -656,7 +669,9 @@ __global__ void __launch_bounds__(HEAD_THREADS) lm_head_kernel(HeadArgs a) {
 // ---------------------------------------------------------------------------------
 struct TokList { int t[MAXB]; };
 
-__global__ void set_desc_kernel(CallDesc* d, const DevState* st, int which, int k, TokList toks) {
+// The next single-step call of model `which`: k tokens at the end of its cache, and the threshold its test uses.
+__global__ void set_call_kernel(CallDesc* d, DevState* st, int which, int k, float alpha, TokList toks) {
+  if (which == 0) st->alpha_fb = alpha; else st->alpha_rb = alpha;
   d->k = k;
   d->pos0 = which == 0 ? st->S_len : st->L_len;
   d->run_policy = 0;
@@ -682,11 +697,6 @@ __global__ void split_desc_kernel(const CallDesc* d, CallDesc* lo, CallDesc* hi)
   const int k = d->k, klo = k < SUB_CHUNK ? k : SUB_CHUNK;
   lo->k = klo; lo->pos0 = d->pos0; lo->run_policy = 0;
   hi->k = k - klo; hi->pos0 = d->pos0 + klo; hi->run_policy = 0;
-}
-
-__global__ void set_alpha_kernel(DevState* st, float alpha_fb, float alpha_rb) {
-  st->alpha_fb = alpha_fb;
-  st->alpha_rb = alpha_rb;
 }
 
 __global__ void rewind_kernel(DevState* st, int which, int new_len) {
