@@ -17,6 +17,7 @@
 #include "enc_gemm.cuh"
 #include "enc_attention.cuh"
 #include "sublayer.cuh"
+#include "cluster_pass.cuh"
 #include "sampling.cuh"
 
 using namespace bild;
@@ -125,6 +126,10 @@ struct Model {
   CallDesc* desc_hi = nullptr;
   AttnSubPlan sub_self[2]{}, sub_cross[2]{};   // chunk sizes of the attention sub-layers: [0] single-row kernel, [1] block kernel
   int sub_parts = 1;                 // launches the feed-forward sub-layer is split into
+  bild_dec_layer* layers_dev = nullptr;   // DEVICE copy of `dec`
+  bool cpass = false;                // small model: all layers of a pass in one cluster kernel
+  float *cp_wo = nullptr, *cp_wfo = nullptr;   // its copies of W_o and W_fo (cp_pack_kernel)
+  int cp_keys = 0;                   // cached keys per head that kernel stages
 };
 
 }  // namespace
@@ -257,11 +262,19 @@ int check_config(const bild_config* cfg, std::string& why) {
   return BILD_OK;
 }
 
-int head_grid_for(int V) { return std::max(1, std::min(HEAD_GRID_MAX, (V + 63) / 64)); }
+int head_grid_for(int V) { return std::max(1, std::min(HEAD_GRID_MAX, (V + 15) / 16)); }   // (16 rows: one round of a block's warps)
 // partial records either head kernel may write (block head: grid x MAXB; single-row head: up to V / 8 blocks)
 size_t head_partial_count(int V) {
   // block head: grid x MAXB; single-row head: up to V / 8 blocks; one-block-per-SM head: SMs x MAXB
   return std::max(std::max((size_t)head_grid_for(V) * MAXB, (size_t)(V + 7) / 8 + 8), (size_t)MAX_GRID_SM * MAXB);
+}
+
+// Models whose passes may run in one cluster kernel (cluster_pass.cuh): fp32, rows of at most 256 columns and layers of at most 2 MB.
+// Beyond that eight SMs take longer to read a layer than one kernel per operation to go through it.
+bool cpass_size_ok(const bild_model_cfg& mc, int dtype) {
+  const size_t I = (size_t)mc.n_heads * mc.d_kv;
+  return dtype == BILD_FP32 && mc.d_model <= 256 &&
+         4 * mc.d_model * (6 * I + (mc.ffn_kind == BILD_FFN_GATED_GELU ? 3 : 2) * (size_t)mc.d_ff) <= (size_t)2 << 20;
 }
 
 // Lays out everything the context keeps on the device.
@@ -304,6 +317,11 @@ void plan(bild_ctx* c, Bump& b) {
     m.desc_lo = b.take<CallDesc>(1);
     m.desc_hi = b.take<CallDesc>(1);
     m.logits = b.take<float>((size_t)MAXB * mc.vocab);
+    m.layers_dev = b.take<bild_dec_layer>(mc.n_layers);
+    if (cpass_size_ok(mc, cfg.dtype)) {
+      m.cp_wo = b.take<float>((size_t)mc.n_layers * 2 * mc.d_model * m.inner);
+      m.cp_wfo = b.take<float>((size_t)mc.n_layers * mc.d_model * mc.d_ff);
+    }
     m.xb = b.take<float>((size_t)MAXB * mc.d_model);
     m.xc = b.take<float>((size_t)MAXB * mc.d_model);
     {   // W_fo of every decoder layer in the load order of the fused feed-forward kernels (two orders: one row, blocks)
@@ -721,6 +739,63 @@ int setup_fused(bild_ctx* c, Model& m) {
   return BILD_OK;
 }
 
+// Decides whether the decoder passes of model `m` run in one cluster kernel, and lays out its copies of W_o and W_fo.
+int setup_cpass(bild_ctx* c, Model& m) {
+  m.cpass = false;
+  const bild_model_cfg& mc = m.c;
+  const bool gated = mc.ffn_kind == BILD_FFN_GATED_GELU;
+  if (c->fused_on < 3 || c->debug_skip_copies || !cpass_size_ok(mc, c->cfg.dtype)) return BILD_OK;
+  int smem_max = 0, dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return BILD_OK;
+  }
+  for (m.cp_keys = 128; m.cp_keys >= 16; m.cp_keys >>= 1)
+    if (cp_layout(mc.d_model, mc.d_kv, cp_slice_max(mc.d_ff), gated, 4, SUB_MB, mc.n_layers, m.cp_keys).total <= smem_max) break;
+  if (m.cp_keys < 16) return BILD_OK;
+  auto aligned = [](const void* p) { return ((uintptr_t)p & 15) == 0; };
+  for (const bild_dec_layer& w : m.dec)
+    if (!aligned(w.wqkv) || !aligned(w.wo) || !aligned(w.wcq) || !aligned(w.wco) || !aligned(w.wi0) || !aligned(w.wfo) || (gated && !aligned(w.wi1)) ||
+        !aligned(w.ln1) || !aligned(w.ln2) || !aligned(w.ln3))
+      return BILD_OK;
+  const void* kerns[2] = {(const void*)cluster_pass_kernel<1>, (const void*)cluster_pass_kernel<8>};
+  for (const void* k : kerns)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) { cudaGetLastError(); return BILD_OK; }
+  CUDA_TRY(c, cudaMemcpyAsync(m.layers_dev, m.dec.data(), m.dec.size() * sizeof(bild_dec_layer), cudaMemcpyHostToDevice, c->stream));
+  cp_pack_kernel<<<mc.n_layers, 512, 0, c->stream>>>(m.layers_dev, mc.d_model, m.inner, mc.d_kv, mc.d_ff, m.cp_wo, m.cp_wfo);
+  (*c->cnt)++;
+  CUDA_TRY(c, cudaGetLastError());
+  m.cpass = true;
+  return BILD_OK;
+}
+
+// A pass of the rows described by `desc` (row0: the first one's place in the call).
+cudaError_t launch_cpass_rows(bild_ctx* c, Model& m, int mb, const CallDesc* desc, int row0) {
+  const bild_model_cfg& mc = m.c;
+  CPassArgs a{};
+  a.desc = desc; a.tokens = m.desc->tokens + row0; a.layers = m.layers_dev; a.wo_pack = m.cp_wo; a.wfo_pack = m.cp_wfo; a.n_layers = mc.n_layers; a.d = mc.d_model; a.I = m.inner;
+  a.H = mc.n_heads; a.dkv = mc.d_kv; a.dkv_shift = ilog2(mc.d_kv); a.F = mc.d_ff; a.gated = mc.ffn_kind == BILD_FFN_GATED_GELU ? 1 : 0;
+  a.vocab = mc.vocab; a.eps = mc.ln_eps; a.inv_d = 1.f / (float)mc.d_model; a.emb = m.w.emb;
+  a.selfK = m.selfK; a.selfV = m.selfV; a.crossK = m.crossK; a.crossV = m.crossV; a.cap = c->cfg.max_dec_len; a.ecap = c->cfg.max_enc_len;
+  a.bias = m.dec_bias; a.n_keys_dev = c->enc_len_dev; a.x_out = m.x + (size_t)row0 * mc.d_model; a.mb = mb; a.kv_keys = m.cp_keys;
+  a.spin = c->spin_limit; a.err = &c->st->err;
+  const size_t smem = cp_layout(mc.d_model, mc.d_kv, cp_slice_max(mc.d_ff), a.gated, 4, mb, mc.n_layers, m.cp_keys).total;
+  auto kern = mb == 1 ? cluster_pass_kernel<1> : cluster_pass_kernel<8>;
+  return launch_k(c, kern, dim3(CP_C), dim3(CP_THREADS), smem, a);
+}
+cudaError_t launch_cpass(bild_ctx* c, Model& m, int MBv) {
+  if (MBv <= SUB_MB) return launch_cpass_rows(c, m, MBv, m.desc, 0);
+  // 9 to 16 rows: two chunks, the second (plain launch: it stages keys of the first before any wait) behind the first
+  split_desc_kernel<<<1, 1, 0, c->stream>>>(m.desc, m.desc_lo, m.desc_hi);
+  (*c->cnt)++;
+  const bool pdl = c->use_pdl;
+  c->use_pdl = false;
+  cudaError_t e = launch_cpass_rows(c, m, SUB_MB, m.desc_lo, 0);
+  if (e == cudaSuccess) e = launch_cpass_rows(c, m, SUB_MB, m.desc_hi, SUB_CHUNK);
+  c->use_pdl = pdl;
+  return e;
+}
+
 template <typename Arg>
 cudaError_t launch_sub(bild_ctx* c, void (*kern)(Arg), int grid, int cluster, size_t smem, const Arg& a, bool pdl_ok = true) {
   cudaLaunchConfig_t cfg = {};
@@ -1021,11 +1096,13 @@ int decoder_pass(bild_ctx* c, int which, int MBv, float* logits_dbg, unsigned lo
   const int d = mc.d_model, I = m.inner, F = mc.d_ff, H = mc.n_heads, dkv = mc.d_kv;
   const int cap = c->cfg.max_dec_len, ecap = c->cfg.max_enc_len, dt = c->cfg.dtype;
   // blocks of 9 to 16 rows: two chunks of the 8-row kernels side by side (the caller guarantees more than 8 rows)
-  const bool chunked = m.fused && which == 1 && MBv == MAXB && c->fused_on >= 3;
-  const bool fused = chunked || (m.fused && (MBv == 1 || (MBv == SUB_MB && c->fused_on >= 2)));
+  const bool small = m.cpass;   // all layers in one kernel
+  const bool chunked = !small && m.fused && which == 1 && MBv == MAXB && c->fused_on >= 3;
+  const bool fused = chunked || (!small && m.fused && (MBv == 1 || (MBv == SUB_MB && c->fused_on >= 2)));
   // (fused sub-layer kernels: the first one gathers the embedding rows itself; the buffer it adds into is clear, every
   // pass leaves it so and a generation starts with it cleared)
-  if (!(fused && c->fused_embed))
+  if (small) CUDA_TRY(c, launch_cpass(c, m, MBv));
+  else if (!(fused && c->fused_embed))
     CUDA_TRY(c, launch_embed(c, m.w.emb, m.desc->tokens, &m.desc->k, 0, MB, d, mc.vocab, m.x, fused ? m.xb : nullptr));
   if (fused) {
     int rc = chunked ? fused_layers_two_chunks(c, m) : fused_layers(c, m, MBv);
@@ -1039,7 +1116,7 @@ int decoder_pass(bild_ctx* c, int which, int MBv, float* logits_dbg, unsigned lo
   int ns_self = 1;
   while (ns_self < 8 && (cap + ns_self - 1) / ns_self > 256) ns_self *= 2;
   const int ns_cross = pick_nsplit(H, ecap);
-  for (int l = 0; l < (fused ? 0 : mc.n_layers); ++l) {
+  for (int l = 0; l < (fused || small ? 0 : mc.n_layers); ++l) {
     const bild_dec_layer& w = m.dec[l];
     const size_t kvoff = (size_t)l * H * dkv;
     LinArgs a{};
@@ -1322,7 +1399,7 @@ int build_graphs_once(bild_ctx* c, int base) {
     CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hi, graph[0], 0, cudaGraphCondAssignDefault));
     CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hi1, graph[0], 0, cudaGraphCondAssignDefault));
     // passes of 2 to 8 rows have a branch of their own where they run on the fused sub-layer kernels
-    const bool body8 = c->m[1].fused && c->fused_on >= 2;
+    const bool body8 = c->m[1].cpass || (c->m[1].fused && c->fused_on >= 2);
     if (body8) CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hi8, graph[0], 0, cudaGraphCondAssignDefault));
     cudaGraph_t body = nullptr, ifbody = nullptr, if1body = nullptr, if8body = nullptr;
     int rc = add_cond(c, graph[0], nullptr, 0, hw, cudaGraphCondTypeWhile, &body);
@@ -1590,6 +1667,7 @@ int bild_create_tuned(const bild_config* cfg, const bild_weights* small_w, const
   if (cudaMemsetAsync(workspace, 0, c->ws_bytes, c->stream) != cudaSuccess) { bild_destroy(c); return BILD_ERR_CUDA; }
   for (int i = 0; i < 2; ++i) {
     rc = setup_fused(c, c->m[i]);
+    if (rc == BILD_OK) rc = setup_cpass(c, c->m[i]);
     if (rc) { bild_destroy(c); return rc; }
   }
   rc = build_bias_tables(c);

@@ -594,13 +594,20 @@ __global__ void __launch_bounds__(HEAD_THREADS) lm_head_kernel(HeadArgs a) {
       }
     }
     float z = 0.f;
+    if constexpr (RW * MB == 32) {   // one transposed reduction: lane r MB + m ends with the sum of its (row, token row)
+      float v[32];
 #pragma unroll
-    for (int r = 0; r < RW; ++r)
+      for (int i = 0; i < 32; ++i) v[i] = acc[i / MB][i % MB];
+      z = treduce<32>(v, lane);
+    } else {
 #pragma unroll
-      for (int m = 0; m < MB; ++m) {
-        const float s = warp_sum(acc[r][m]);
-        if (lane == r * MB + m) z = s;
-      }
+      for (int r = 0; r < RW; ++r)
+#pragma unroll
+        for (int m = 0; m < MB; ++m) {
+          const float s = warp_sum(acc[r][m]);
+          if (lane == r * MB + m) z = s;
+        }
+    }
     const int n = n0 + my_r;
     if (lane < RW * MB && my_m < mrows && n < ne) {
       z *= a.scale;

@@ -51,3 +51,35 @@ def test_drawn_token_over_vocabulary_sizes(torch_cuda, vocab, scale, equal):
             assert c[at] <= uu[1] * c[n] + 1e-5 and c[at + 1] >= uu[1] * c[n] - 1e-5, (top_p, u, margin)
     assert checked >= 2
     ctx.close()
+
+
+@pytest.mark.parametrize("name,n_layers,d,H,dkv,F,ffn", [("a", 3, 64, 3, 16, 136, "gated_gelu"), ("b", 2, 128, 10, 16, 40, "relu"),
+                                                         ("c", 2, 256, 2, 64, 64, "gated_gelu"), ("d", 1, 72, 1, 128, 520, "relu")])
+def test_small_fp32_passes_match_oracle(torch_cuda, name, n_layers, d, H, dkv, F, ffn):
+    """Passes of small fp32 models in one cluster kernel: fewer and more heads than blocks, slices of unequal size and empty ones,
+    1 to 16 rows, caches around the count of staged keys."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200.binding import FP32, Config, Context, model_cfg, upload_model
+    torch = torch_cuda
+    s = dataclasses.replace(MODEL_SHAPES["tiny_s"], name=name, n_layers=n_layers, d_model=d, n_heads=H, d_kv=dkv, d_ff=F, ffn=ffn, vocab=97)
+    w = gen_model(s, 5, "fp32")
+    dev = upload_model(w, "cuda:0")
+    ctx = Context(Config(model_cfg(s, 3.0), model_cfg(s, 3.0), FP32, 150, 150, 15, 0, -1, 0), s, dev, s, dev)
+    rng = np.random.default_rng(d)
+    ids = rng.integers(2, 97, size=140).astype(np.int32)
+    ctx.encode(ids)
+    m = Model(s, w, 3.0)
+    st, st1 = m.start(ids, 150), m.start(ids, 150)
+    buf = torch.empty((16, 97), dtype=torch.float32, device="cuda")
+    toks = [int(t) for t in rng.integers(2, 97, size=150)]
+    at = 0
+    for k in (1, 2, 3, 5, 8, 9, 16, 16, 16, 16, 16, 16, 4, 1, 7, 13):   # the cache grows past 128 rows
+        ctx.large_verify(toks[at:at + k], 10.0, buf)
+        z = m.forward_block(st, toks[at:at + k])
+        assert np.max(np.abs(buf[:k].cpu().numpy() - z)) <= 1e-4 * max(1.0, np.max(np.abs(z))), (k, at)
+        at += k
+    for t in toks[:5]:
+        ctx.small_step(t, 0.5, buf)
+        z = m.forward_one(st1, t)
+        assert np.max(np.abs(buf[0].cpu().numpy() - z)) <= 1e-4 * max(1.0, np.max(np.abs(z)))
+    ctx.close()
