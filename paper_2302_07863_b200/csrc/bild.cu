@@ -16,6 +16,7 @@
 #include "umma_linear.cuh"
 #include "enc_gemm.cuh"
 #include "enc_attention.cuh"
+#include "enc_flash.cuh"
 #include "sublayer.cuh"
 #include "cluster_pass.cuh"
 #include "sampling.cuh"
@@ -112,6 +113,8 @@ struct Model {
   std::vector<CUtensorMap> tmaps;
   bool umma = false;
   // encoder GEMM: descriptors of the bf16 head / remainder matrices of the layer input, by row length (d, inner, d_ff)
+  CUtensorMap tmAtt[6];       // encoder attention: queries, keys (heads, remainders each), transposed values
+  bool enc_flash = false;     // encoder attention on tcgen05
   CUtensorMap tmH[2][3][2];   // [buffer pair][row length d / inner / d_ff][head, remainder]
   bool enc_gemm = false;
   int index = 0;   // 0 small, 1 large
@@ -151,6 +154,7 @@ struct bild_ctx {
   // encoder temporaries, one set per model (the two encoders run side by side on two streams)
   struct EncBuf {
     float *ex = nullptr, *eq = nullptr, *ek = nullptr, *ev = nullptr, *eatt = nullptr, *eu = nullptr;
+    EgQkv qkv{};   // projected queries, keys, values of the layer at hand as enc_flash_kernel reads them
     __nv_bfloat16 *exh[2] = {nullptr, nullptr}, *exl[2] = {nullptr, nullptr};   // two pairs (bf16 head, remainder) of layer inputs
   } eb[2];
   cudaStream_t enc_stream = nullptr;   // the small model's encoder runs here, the large model's on the caller's stream
@@ -342,6 +346,12 @@ void plan(bild_ctx* c, Bump& b) {
     e.ev = b.take<float>((size_t)ecap * I);
     e.eatt = b.take<float>(ecap16 * I);
     e.eu = b.take<float>(ecap16 * F);
+    if (cfg.dtype == BILD_BF16 && mc.d_kv == EA_D) {
+      e.qkv.qh = b.take<__nv_bfloat16>(ecap128 * I); e.qkv.ql = b.take<__nv_bfloat16>(ecap128 * I);
+      e.qkv.kh = b.take<__nv_bfloat16>(ecap128 * I); e.qkv.kl = b.take<__nv_bfloat16>(ecap128 * I);
+      e.qkv.vh = b.take<__nv_bfloat16>(ecap128 * I); e.qkv.vl = b.take<__nv_bfloat16>(ecap128 * I);
+      e.qkv.ldv = (int)ecap128;
+    }
     for (int pr = 0; pr < 2; ++pr) {
       e.exh[pr] = b.take<__nv_bfloat16>(ecap128 * std::max(std::max(d, I), F));
       e.exl[pr] = b.take<__nv_bfloat16>(ecap128 * std::max(std::max(d, I), F));
@@ -609,11 +619,11 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// Descriptor of a row-major bf16 matrix [N][K] for boxes of 128 rows x 64 columns, 128-byte swizzle.
-bool make_tmap(EncodeTiledFn enc, const void* W, int N, int K, CUtensorMap* out) {
+// Descriptor of a row-major bf16 matrix [N][K] for boxes of box_rows x 64 columns, 128-byte swizzle.
+bool make_tmap(EncodeTiledFn enc, const void* W, int N, int K, CUtensorMap* out, int box_rows = UM_TILE_M) {
   cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)N};
   cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-  cuuint32_t box[2] = {UM_KB, UM_TILE_M};
+  cuuint32_t box[2] = {UM_KB, (cuuint32_t)box_rows};
   cuuint32_t es[2] = {1, 1};
   return enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(W), dims, strides, box, es,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -680,6 +690,19 @@ void setup_umma(bild_ctx* c, Model& m) {
     return;
   }
   m.enc_gemm = true;
+  // encoder attention on tcgen05 (the mma.sync kernel remains behind bild_tuning.enc_attn_groups = 1, 2)
+  m.enc_flash = false;
+  const EgQkv& pj = c->eb[m.index].qkv;
+  if (!pj.qh || !c->enc_attn_mma || c->enc_attn_groups < EA_MAX_GROUPS || ef_smem_bytes(c->cfg.max_enc_len) > (size_t)maxsm) return;
+  const void* mats[6] = {pj.qh, pj.ql, pj.kh, pj.kl, pj.vh, pj.vl};
+  for (int i = 0; i < 6; ++i)
+    if (!make_tmap(enc, mats[i], i < 4 ? ecap128 : m.inner, i < 4 ? m.inner : ecap128, &m.tmAtt[i], i < 2 ? EF_ROWS : EF_KEYS)) return;
+  if (cudaFuncSetAttribute(enc_flash_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ef_smem_bytes(c->cfg.max_enc_len)) != cudaSuccess ||
+      cudaFuncSetAttribute(enc_flash_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ef_smem_bytes(c->cfg.max_enc_len)) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  m.enc_flash = true;
 }
 
 // ---- fused sub-layer kernels ------------------------------------------------------------------
@@ -1039,6 +1062,8 @@ cudaError_t launch_dec_linear(bild_ctx* c, Model& m, int MB, const LinArgs& a, i
 // The input pair is buffer `pair`; `split` false: it already holds the input (written by the kernel in front or by
 // an earlier call); `out_pair` >= 0: a ReLU / gated epilogue writes its output as the pair `out_pair` instead of fp32.
 cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, int which_map, bool split, int pair, int out_pair) {
+  // the projection in front of the tcgen05 attention leaves bf16 heads and remainders
+  const EgQkv qkv = which_map == TM_EQKV && m.enc_flash ? c->eb[m.index].qkv : EgQkv{};
   const int E = a.M, tiles_tok = (E + EG_TOK - 1) / EG_TOK;
   const int ki = a.K == m.c.d_model ? 0 : a.K == m.inner ? 1 : 2;
   if (split) {
@@ -1058,10 +1083,32 @@ cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, 
     grid.z = z;
   }
   if (gated)
-    return launch_k(c, enc_gemm_kernel<true>, grid, dim3(EG_THREADS), eg_smem_bytes<true>(), a, &c->st->err, oh, ol, t[which_map],
+    return launch_k(c, enc_gemm_kernel<true>, grid, dim3(EG_THREADS), eg_smem_bytes<true>(), a, &c->st->err, oh, ol, qkv, t[which_map],
                     t[which_map == TM_EWI0 ? TM_EWI1 : which_map], m.tmH[pair][ki][0], m.tmH[pair][ki][1]);
-  return launch_k(c, enc_gemm_kernel<false>, grid, dim3(EG_THREADS), eg_smem_bytes<false>(), a, &c->st->err, oh, ol, t[which_map],
+  return launch_k(c, enc_gemm_kernel<false>, grid, dim3(EG_THREADS), eg_smem_bytes<false>(), a, &c->st->err, oh, ol, qkv, t[which_map],
                   t[which_map], m.tmH[pair][ki][0], m.tmH[pair][ki][1]);
+}
+
+// Encoder attention on tcgen05; two blocks share a query tile's keys while the grid leaves half of the SMs idle (and there are two tiles).
+cudaError_t launch_enc_flash(bild_ctx* c, Model& m, const EncFlashArgs& f) {
+  const int rows = (f.M + EF_ROWS - 1) / EF_ROWS, cs = f.M > 2 * EF_KEYS && 2 * f.H * rows <= c->sms ? 2 : 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(f.H * cs, rows); cfg.blockDim = dim3(EF_THREADS); cfg.dynamicSmemBytes = ef_smem_bytes(f.M); cfg.stream = c->stream;
+  cudaLaunchAttribute at[2];
+  int na = 0;
+  if (c->use_pdl) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+  }
+  if (cs > 1) {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = cs; at[na].val.clusterDim.y = 1; at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  cfg.attrs = at; cfg.numAttrs = na;
+  (*c->cnt)++;
+  return cudaLaunchKernelEx(&cfg, cs > 1 ? enc_flash_kernel<2> : enc_flash_kernel<1>, f, m.tmAtt[0], m.tmAtt[1], m.tmAtt[2], m.tmAtt[3], m.tmAtt[4], m.tmAtt[5]);
 }
 
 // Linear layer of the encoder over rb blocks of MAXB rows.
@@ -1223,12 +1270,19 @@ int encoder_pass(bild_ctx* c, int which) {
     // norm(x) -> pair 0 -> QKV; attention -> pair 1 -> O; norm(x) -> pair 0 -> FFN-up -> pair 1 -> FFN-down
     const bool fuse = m.enc_gemm && c->enc_attn_mma && dkv == EA_D;
     CUDA_TRY(c, launch_enc_linear(c, m, a, rb, l, TM_EQKV, true, 0));
+    if (m.enc_flash) {
+      EncFlashArgs f{};
+      f.bias = m.enc_bias; f.bias_ld = 2 * ecap - 1; f.bias_off = ecap - 1; f.n_keys_dev = c->enc_len_dev; f.M = E; f.H = H;
+      f.oh = B.exh[1]; f.ol = B.exl[1]; f.err = &c->st->err;
+      CUDA_TRY(c, launch_enc_flash(c, m, f));
+    } else {
     BAttnArgs t{};
     t.q = B.eq; t.ldq = I; t.kc = B.ek; t.vc = B.ev; t.cap = ecap; t.out = B.eatt; t.ldo = I;
     t.bias = m.enc_bias; t.bias_ld = 2 * ecap - 1; t.bias_off = ecap - 1; t.mode = 2; t.dkv = dkv; t.H = H;
     t.n_keys_dev = c->enc_len_dev; t.M = E; t.part = m.att_part; t.counters = m.att_cnt; t.nsplit = 1;
     t.err = &c->st->err;
     CUDA_TRY(c, launch_battn(c, MAXB, t, rb, ecap, fuse ? B.exh[1] : nullptr, fuse ? B.exl[1] : nullptr));
+    }
     LinArgs o{};
     o.M = E; o.W0 = w.wo; o.X = B.eatt; o.ldx = I; o.N = d; o.K = I; o.epi = EPI_RESID; o.Y = B.ex; o.ldy = d;
     CUDA_TRY(c, launch_enc_linear(c, m, o, rb, l, TM_EO, !fuse, 1));
