@@ -129,6 +129,7 @@ struct Model {
   CallDesc* desc_hi = nullptr;
   AttnSubPlan sub_self[2]{}, sub_cross[2]{};   // chunk sizes of the attention sub-layers: [0] single-row kernel, [1] block kernel
   int sub_parts = 1;                 // launches the feed-forward sub-layer is split into
+  int sub_grid[2] = {0, 0};          // blocks of a feed-forward launch: [0] single-row kernel, [1] block kernel
   bild_dec_layer* layers_dev = nullptr;   // DEVICE copy of `dec`
   bool cpass = false;                // small model: all layers of a pass in one cluster kernel
   float *cp_wo = nullptr, *cp_wfo = nullptr;   // its copies of W_o and W_fo (cp_pack_kernel)
@@ -756,6 +757,16 @@ int setup_fused(bild_ctx* c, Model& m) {
     (*c->cnt)++;
   }
   CUDA_TRY(c, cudaGetLastError());
+  // One block per SM; more where that brings the block variant's shared memory under half an SM's, so that its blocks sit beside the
+  // attention kernel's in front and their weights arrive in its shadow (gated slices of 24 rows: 148 KB, of 16 rows: 112 KB; mT5-large,
+  // 5 rows: a pass of two 642 -> 600 us, of five 642 -> 637, of sixteen 1033 -> 912)
+  m.sub_grid[0] = m.sub_grid[1] = c->sms;
+  if (parts == 1 && ffn_sub_layout(d, F, gated, c->sms, c->sms, SUB_MB).total > SUB_HALF_SM)
+    for (int rows = ffn_sub_rows(F, c->sms) - 8; rows >= 8; rows -= 8) {
+      const int grid = (F + rows - 1) / rows;
+      if (grid > 2 * c->sms) break;
+      if (ffn_sub_layout(d, F, gated, grid, grid, SUB_MB).total <= SUB_HALF_SM) { m.sub_grid[1] = grid; break; }
+    }
   m.sub_C = C; m.sub_parts = parts;
   for (int v = 0; v < 2; ++v) { m.sub_self[v] = ps[v]; m.sub_cross[v] = pc[v]; }
   m.fused = true;
@@ -862,10 +873,11 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   a.mb = MB; a.err = &c->st->err;
   a.spin = c->spin_limit; a.skip_copies = c->debug_skip_copies ? 1 : 0;
   a.n_keys_dev = c->enc_len_dev;
-  // When the next kernel's blocks may start their requests.  Behind this kernel's token rows: its 64 KB a block otherwise queue in front
-  // of them (5-row pass 580 -> 552 us).  At once for a single row of more than 512 columns: the kernels are so short then that the
-  // requests would not be back in time (mT5-large 442 -> 416 us, T5-large 356 -> 354 us; 512 columns: 145 -> 135 us the other way).
-  a.early = MB == 1 && d > 512 ? 1 : 0;
+  // When the next kernel's blocks may start their requests.  Behind this kernel's token rows where those requests are large and would queue
+  // in front of them (T5-large, 5 rows: 580 -> 552 us; blocks of 9 to 16 rows: two chunks' kernels share the SMs), or where the kernels
+  // are shorter still than their prologue's gain (single rows of 512 columns: 145 -> 135 us); at once where a prologue would otherwise
+  // not be done in time (single rows of 1024 columns: mT5-large 442 -> 416 us; blocks of 512 columns: mT5-small 2 rows 215 -> 206 us).
+  a.early = MB == 1 ? d > 512 : d <= 512 && desc == m.desc;
   // S1-S3 / L1-L3 (layer 0: with S0 / L0, the rows come from the embedding table)
   if (l == 0 && c->fused_embed) {
     a.emb = (const __nv_bfloat16*)m.w.emb; a.tokens = m.desc->tokens + row0; a.vocab = mc.vocab;
@@ -895,10 +907,11 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   f.Wi0 = (const __nv_bfloat16*)w.wi0; f.Wi1 = (const __nv_bfloat16*)w.wi1;
   f.Wfo1 = m.wfo_one + (size_t)l * (Fd / 8) * d; f.Wfo8 = m.wfo_blk + (size_t)l * (Fd / 8) * pack_wfo_dpad(d);
   f.nparts = m.sub_parts;
-  f.L = ffn_sub_layout(d, Fd, gated, c->sms * m.sub_parts, c->sms, MB);
+  const int grid = m.sub_grid[MB == 1 ? 0 : 1];
+  f.L = ffn_sub_layout(d, Fd, gated, grid * m.sub_parts, grid, MB);
   for (int p = 0; p < m.sub_parts; ++p) {
     f.part = p; f.seed = p == 0 ? 1 : 0; f.x_zero = p == 0 ? xb : nullptr;
-    CUDA_TRY(c, launch_sub(c, MB == 1 ? ffn_sub_kernel<true> : ffn_sub_kernel<false>, c->sms, 1, (size_t)f.L.total, f));
+    CUDA_TRY(c, launch_sub(c, MB == 1 ? ffn_sub_kernel<true> : ffn_sub_kernel<false>, grid, 1, (size_t)f.L.total, f));
   }
   return BILD_OK;
 }
