@@ -264,6 +264,7 @@ __global__ void __cluster_dims__(CP_C, 1, 1) __launch_bounds__(CP_THREADS, 1) cl
   pdl_launch_dependents();
   const unsigned lim = (a.spin > SPIN_LIMIT ? a.spin : SPIN_LIMIT) * 4u;
   auto wait = [&](unsigned long long* bar, unsigned parity) {   // bounded; after a time-out nothing is waited for any more
+    __syncwarp();   // (a lane that polls must not keep a sibling from issuing a copy or a store)
     if (sub_try_cluster(smem_u32(bar), parity) || *(volatile int*)failed) return;
     for (unsigned it = 0; it < lim; ++it)
       if (sub_try_cluster(smem_u32(bar), parity)) return;

@@ -218,6 +218,7 @@ __global__ void __launch_bounds__(EF_THREADS, 1) enc_flash_kernel(const EncFlash
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       ea_group_sync(g);
       if ((tid & 127) == 0) mbar_arrive(smem_u32(&p_full[g]));
+      __syncwarp();   // (the arrival before its siblings poll)
       if (!mbar_wait(&o_full[g], par)) *a.err = BILD_ERR_TIMEOUT;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       ef_ld64(tl + 128 + g * 64, sr);

@@ -66,6 +66,7 @@ __host__ __device__ inline int sub_kv_stride(int dkv) { return ((dkv + 15) / 32)
 // Bounded wait for the weight copies: after `spin` unsuccessful polls the block records BILD_ERR_TIMEOUT for the host
 // and goes on (with whatever the shared memory holds), so that every block of the kernel still leaves.
 __device__ __forceinline__ void sub_wait(SubShared* sh, int* err, unsigned long long* bar, uint32_t parity, unsigned spin) {
+  __syncwarp();   // (a lane that polls must not keep a sibling from issuing a copy)
   const uint32_t b = smem_u32(bar);
   if (mbar_try(b, parity)) return;
   if (*(volatile int*)&sh->failed) return;
@@ -90,7 +91,9 @@ __device__ __forceinline__ bool sub_try_cluster(uint32_t bar, uint32_t parity) {
 }
 // Wait for the values the cluster's blocks store into this one (sub_push).  Every block sends its part after bounded waits of
 // its own, so the limit here is only a last bound, above theirs.
+// (The warp meets first: a lane that polls must not keep a sibling from sending what the others wait for.)
 __device__ __forceinline__ void sub_wait_exchange(SubShared* sh, int* err, unsigned long long* bar, unsigned spin) {
+  __syncwarp();
   const uint32_t b = smem_u32(bar);
   const unsigned lim = (spin > SPIN_LIMIT ? spin : SPIN_LIMIT) * 4u;
   for (unsigned it = 0; it < lim; ++it)
