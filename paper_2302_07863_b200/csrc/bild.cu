@@ -115,6 +115,7 @@ struct Model {
   // encoder GEMM: descriptors of the bf16 head / remainder matrices of the layer input, by row length (d, inner, d_ff)
   CUtensorMap tmAtt[6];       // encoder attention: queries, keys (heads, remainders each), transposed values
   bool enc_flash = false;     // encoder attention on tcgen05
+  CUtensorMap tmH64[2][3][2]; // the same in boxes of 64 rows
   CUtensorMap tmH[2][3][2];   // [buffer pair][row length d / inner / d_ff][head, remainder]
   bool enc_gemm = false;
   int index = 0;   // 0 small, 1 large
@@ -684,9 +685,15 @@ void setup_umma(bild_ctx* c, Model& m) {
   for (int pr = 0; pr < 2; ++pr)
     for (int i = 0; i < 3; ++i)
       if (!make_tmap(enc, c->eb[m.index].exh[pr], ecap128, Ks[i], &m.tmH[pr][i][0]) ||
-          !make_tmap(enc, c->eb[m.index].exl[pr], ecap128, Ks[i], &m.tmH[pr][i][1])) return;
-  if (cudaFuncSetAttribute(enc_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eg_smem_bytes<false>()) != cudaSuccess ||
-      cudaFuncSetAttribute(enc_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eg_smem_bytes<true>()) != cudaSuccess) {
+          !make_tmap(enc, c->eb[m.index].exl[pr], ecap128, Ks[i], &m.tmH[pr][i][1]) ||
+          !make_tmap(enc, c->eb[m.index].exh[pr], ecap128, Ks[i], &m.tmH64[pr][i][0], 64) ||
+          !make_tmap(enc, c->eb[m.index].exl[pr], ecap128, Ks[i], &m.tmH64[pr][i][1], 64)) return;
+  auto smem_ok = [](const void* k, size_t bytes) { return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess; };
+  if (!smem_ok((const void*)enc_gemm_kernel<false, false, 128>, eg_smem_bytes<false, false, 128>()) ||
+      !smem_ok((const void*)enc_gemm_kernel<true, false, 128>, eg_smem_bytes<true, false, 128>()) ||
+      !smem_ok((const void*)enc_gemm_kernel<false, false, 64>, eg_smem_bytes<false, false, 64>()) ||
+      !smem_ok((const void*)enc_gemm_kernel<false, true, 64>, std::max(eg_smem_bytes<false, true, 64>(2), eg_smem_bytes<false, true, 64>(4))) ||
+      !smem_ok((const void*)enc_gemm_kernel<true, true, 64>, std::max(eg_smem_bytes<true, true, 64>(2), eg_smem_bytes<true, true, 64>(4)))) {
     cudaGetLastError();
     return;
   }
@@ -1085,21 +1092,44 @@ cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, 
     if (e != cudaSuccess) return e;
   }
   const CUtensorMap* t = &m.tmaps[(size_t)layer * TM_PER_LAYER];
-  const bool gated = a.epi == EPI_GATED;
+  const CUtensorMap &t0 = t[which_map], &t1 = t[which_map == TM_EWI0 ? TM_EWI1 : which_map];
+  const bool gated = a.epi == EPI_GATED, resid = a.epi == EPI_RESID, small = E <= 64;
   __nv_bfloat16* oh = out_pair >= 0 ? c->eb[m.index].exh[out_pair] : nullptr;
   __nv_bfloat16* ol = out_pair >= 0 ? c->eb[m.index].exl[out_pair] : nullptr;
-  dim3 grid((a.N + UM_TILE_M - 1) / UM_TILE_M, tiles_tok);
-  if (a.epi == EPI_RESID && c->enc_split_k) {   // few tiles, long K: split K until the grid covers the SMs (at least 4 K blocks each)
-    const int tiles = (int)(grid.x * grid.y), nkb = a.K / UM_KB;
-    int z = 1;
+  const CUtensorMap* h = small ? m.tmH64[pair][ki] : m.tmH[pair][ki];
+  dim3 grid((a.N + UM_TILE_M - 1) / UM_TILE_M, small ? 1 : tiles_tok);
+  const int tiles = (int)(grid.x * grid.y), nkb = a.K / UM_KB;
+  int z = 1;
+  if (resid && c->enc_split_k) {   // few tiles, long K: split K until the grid covers the SMs (at least 4 K blocks each), sums by reductions at the L2
     while (z < 8 && tiles * (z * 2) <= c->sms && nkb / (z * 2) >= 4) z *= 2;
-    grid.z = z;
+  } else if (small && c->enc_split_k) {
+    // the other epilogues need the whole sum: a cluster of two or four blocks splits K.  64 ids, T5-large shapes, from kernel to kernel:
+    // q|k|v 10.9 -> 8.2 us, d_ff 9.4 -> 7.4 us, gated d_ff (mT5-large) 17.2 -> 11.6 us; encode 1337 -> 1248 us (mT5-large pair 1607 -> 1429).
+    // Not for longer inputs: their tile of 128 tokens takes twice the exchange, and encode of 200 ids went from 1551 to 1973 us.
+    while (z < 4 && tiles * (z * 2) <= c->sms && nkb / (z * 2) >= 2) z *= 2;
   }
-  if (gated)
-    return launch_k(c, enc_gemm_kernel<true>, grid, dim3(EG_THREADS), eg_smem_bytes<true>(), a, &c->st->err, oh, ol, qkv, t[which_map],
-                    t[which_map == TM_EWI0 ? TM_EWI1 : which_map], m.tmH[pair][ki][0], m.tmH[pair][ki][1]);
-  return launch_k(c, enc_gemm_kernel<false>, grid, dim3(EG_THREADS), eg_smem_bytes<false>(), a, &c->st->err, oh, ol, qkv, t[which_map],
-                  t[which_map], m.tmH[pair][ki][0], m.tmH[pair][ki][1]);
+  grid.z = z;
+  if (!resid && z > 1) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = dim3(EG_THREADS); cfg.stream = c->stream;
+    cfg.dynamicSmemBytes = gated ? eg_smem_bytes<true, true, 64>(z) : eg_smem_bytes<false, true, 64>(z);
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = z;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = c->use_pdl ? 2 : 1;
+    (*c->cnt)++;
+    auto kern = gated ? enc_gemm_kernel<true, true, 64> : enc_gemm_kernel<false, true, 64>;
+    return cudaLaunchKernelEx(&cfg, kern, a, &c->st->err, oh, ol, qkv, t0, t1, h[0], h[1]);
+  }
+  if (gated) {
+    grid.y = tiles_tok;
+    return launch_k(c, enc_gemm_kernel<true, false, 128>, grid, dim3(EG_THREADS), eg_smem_bytes<true, false, 128>(), a, &c->st->err, oh, ol, qkv, t0, t1,
+                    m.tmH[pair][ki][0], m.tmH[pair][ki][1]);
+  }
+  return launch_k(c, small ? enc_gemm_kernel<false, false, 64> : enc_gemm_kernel<false, false, 128>, grid, dim3(EG_THREADS),
+                  small ? eg_smem_bytes<false, false, 64>() : eg_smem_bytes<false, false, 128>(), a, &c->st->err, oh, ol, qkv, t0, t1, h[0], h[1]);
 }
 
 // Encoder attention on tcgen05; two blocks share a query tile's keys while the grid leaves half of the SMs idle (and there are two tiles).

@@ -26,6 +26,12 @@ namespace bild {
 constexpr int EG_THREADS = 512;   // thread 0 feeds the ring, thread 32 issues the MMAs, all 16 warps share the epilogue
 constexpr int EG_TOK = 128;   // tokens per tile
 
+__device__ __forceinline__ uint32_t sub_mapa_u32(uint32_t a, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+
 // Optional cycle stamps (build with -DBILD_STAMPS), summed over the blocks of the T5-large-shaped GEMMs of 512 tokens:
 // [class: QKV (24 row tiles), FFN-up (32), residual (8, K split)][slot]; slot 15 counts the blocks.  Slots 0-4: a thread
 // of warp 2 (start -> tensor memory allocated -> dependency wait returned -> all MMAs done -> epilogue done; 4: its loads
@@ -136,161 +142,40 @@ __global__ void __launch_bounds__(128) norm_split_kernel(const float* __restrict
   }
 }
 
-// bf16 x bf16 -> fp32, A and B K-major, M = 128, N = 256 (128 token rows of hi, then 128 of lo)
-constexpr uint32_t EG_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((256u >> 3) << 17) | ((128u >> 4) << 24);
+// bf16 x bf16 -> fp32, A and B K-major, M = 128, N = 2 TT (TT token rows of hi, then TT of lo)
+template <int TT>
+__host__ __device__ constexpr uint32_t eg_idesc() { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * TT >> 3) << 17) | ((128u >> 4) << 24); }
+template <int TT>
 __device__ __forceinline__ void eg_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(EG_IDESC), "r"(accumulate) : "memory");
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(eg_idesc<TT>()), "r"(accumulate) : "memory");
 }
 
-template <bool GATED>
-__host__ __device__ constexpr int eg_stages() { return GATED ? 3 : 4; }
-template <bool GATED>
-constexpr size_t eg_smem_bytes() { return 1024 + (size_t)eg_stages<GATED>() * (GATED ? 4 : 3) * 16384 + 256; }
+template <bool GATED, bool CL>
+__host__ __device__ constexpr int eg_stages() { return CL ? (GATED ? 2 : 3) : GATED ? 3 : 4; }
+template <bool GATED, int TT>
+__host__ __device__ constexpr int eg_stage_bytes() { return (GATED ? 2 : 1) * 16384 + 2 * TT * 128; }
+// room for the cluster's partial tiles: [matrix][rank][128 rows][token columns of a rank + 4]
+__host__ __device__ constexpr int eg_red_bytes(bool gated, int tt, int z) { return (gated ? 2 : 1) * z * 128 * (tt / z + 4) * 4; }
+template <bool GATED, bool CL, int TT>
+constexpr size_t eg_smem_bytes(int z = 1) {
+  return 1024 + (size_t)eg_stages<GATED, CL>() * eg_stage_bytes<GATED, TT>() + 256 + (CL ? eg_red_bytes(GATED, TT, z) : 0);
+}
 
 // Where the encoder's q | k | v projection leaves its result for enc_flash_kernel: bf16 heads and remainders, q and k [token][inner],
 // v transposed [inner][ldv] (whole tiles of tokens: what lies past the last one is zero, since its input rows are)
 struct EgQkv { __nv_bfloat16 *qh, *ql, *kh, *kl, *vh, *vl; int ldv; };
 
-template <bool GATED>
-__global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* err, __nv_bfloat16* oh, __nv_bfloat16* ol, const EgQkv qkv,
-                                                              const __grid_constant__ CUtensorMap tmW0,
-                                                              const __grid_constant__ CUtensorMap tmW1,
-                                                              const __grid_constant__ CUtensorMap tmHh,
-                                                              const __grid_constant__ CUtensorMap tmHl) {
-  constexpr int NST = eg_stages<GATED>();
-  constexpr int NMAT = GATED ? 2 : 1;
-  constexpr int STAGE = (NMAT + 2) * 16384;
-  constexpr int TCOLS = 256 * NMAT;
-  extern __shared__ unsigned char eg_raw[];
-  const int tid = threadIdx.x, warp = tid >> 5;
-#ifdef BILD_STAMPS
-  long long T0, T1 = 0, T2 = 0, T3 = 0, T4 = 0, TM1 = 0, TM2 = 0, TP1 = 0, TL = 0, TA = 0;
-#endif
-  EG_STAMP(T0);
-  const int n_base = blockIdx.x * UM_TILE_M, tok0 = blockIdx.y * EG_TOK;
-  // this block's share of the K blocks (gridDim.z splits, EPI_RESID only)
-  const int nkb_all = a.K / UM_KB, kb0 = (int)(((long long)blockIdx.z * nkb_all) / gridDim.z);
-  const int nkb = (int)(((long long)(blockIdx.z + 1) * nkb_all) / gridDim.z) - kb0;
-  unsigned char* base = (unsigned char*)(((uintptr_t)eg_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(base + (size_t)NST * STAGE);
-  uint64_t* empty = full + NST;
-  uint64_t* done = empty + NST;
-  uint32_t* tmem_slot = (uint32_t*)(done + 1);
-  if (tid == 0) {
-    for (int i = 0; i < NST; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
-    mbar_init(done, 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(TCOLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *tmem_slot;
-  EG_STAMP(T1);
-  // thread 0 feeds the ring; the weight tiles depend on nothing and are requested before the dependency wait
-  // for the first NST stages, the activation tiles of those stages follow after it (same barrier per stage)
-  auto load_weights = [&](int kb) {
-    unsigned char* st = base + (size_t)(kb % NST) * STAGE;
-    uint64_t* bar = &full[kb % NST];
-    mbar_expect_tx(bar, STAGE);
-    tma_load_2d(st, &tmW0, (kb0 + kb) * UM_KB, n_base, bar);
-    if (GATED) tma_load_2d(st + 16384, &tmW1, (kb0 + kb) * UM_KB, n_base, bar);
-  };
-  auto load_acts = [&](int kb) {
-    unsigned char* st = base + (size_t)(kb % NST) * STAGE;
-    uint64_t* bar = &full[kb % NST];
-    tma_load_2d(st + NMAT * 16384, &tmHh, (kb0 + kb) * UM_KB, tok0, bar);
-    tma_load_2d(st + (NMAT + 1) * 16384, &tmHl, (kb0 + kb) * UM_KB, tok0, bar);
-  };
-  if (tid == 0)
-    for (int kb = 0; kb < nkb && kb < NST; ++kb) load_weights(kb);
-  pdl_launch_dependents();
-  pdl_wait();   // the activation tiles were written by the kernel in front
-  EG_STAMP(T2);
-  if (tid == 0) {
-    asm volatile("fence.proxy.async;" ::: "memory");   // rows written with ordinary stores, read by the copy engine
-    for (int kb = 0; kb < nkb; ++kb) {
-      if (kb >= NST) {
-        if (!mbar_wait(&empty[kb % NST], ((kb / NST) - 1) & 1)) *err = BILD_ERR_TIMEOUT;
-        load_weights(kb);
-      }
-      load_acts(kb);
-    }
-    EG_STAMP(TP1);
-  } else if (tid == 32) {
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int st = kb % NST;
-      if (!mbar_wait(&full[st], (kb / NST) & 1)) *err = BILD_ERR_TIMEOUT;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-#ifdef BILD_STAMPS
-      if (kb == 0) TM1 = clock64();
-#endif
-      const uint32_t a0 = smem_u32(base + (size_t)st * STAGE);
-      const uint32_t bh = a0 + NMAT * 16384;   // hi tile, lo tile right behind it: one operand of 256 rows
-#pragma unroll
-      for (int kk = 0; kk < UM_KB / 16; ++kk) {
-        const uint64_t db = umma_desc_sw128(bh + kk * 32);
-        eg_mma(tmem, umma_desc_sw128(a0 + kk * 32), db, (kb | kk) ? 1u : 0u);
-        if (GATED) eg_mma(tmem + 256, umma_desc_sw128(a0 + 16384 + kk * 32), db, (kb | kk) ? 1u : 0u);
-      }
-      umma_commit(&empty[st]);   // the stage may be refilled once these MMAs have read it
-    }
-    umma_commit(done);
-    EG_STAMP(TM2);
-  }
-  __syncwarp();
-  if (!mbar_wait(done, 0)) *err = BILD_ERR_TIMEOUT;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  EG_STAMP(T3);
-
-  // ---- epilogue: a warp reads the 32 lanes (weight rows) of tensor memory that its number modulo 4 gives it access to; the
-  // four warps of a lane quarter share the 128 token columns, 32 each.  One warp per scheduler would be bound by the
-  // latency of its own instruction stream (measured: 5-10 us for the 128 columns), so all 16 warps of the block take part.
-  const int quarter = warp & 3, colgrp = warp >> 2;
-  const int n = n_base + quarter * 32 + (tid & 31);
-  const bool row_ok = n < a.N;
-  const uint32_t t0 = tmem + ((uint32_t)(quarter * 32) << 16);
-  int part = a.first_part, rr = n;
-  if (a.epi == EPI_HEADS) {
-    if (rr >= a.inner) { rr -= a.inner; ++part; }
-    if (rr >= a.inner) { rr -= a.inner; ++part; }
-  }
-  const int hh = a.epi == EPI_HEADS ? rr / a.dkv : 0, hc = a.epi == EPI_HEADS ? rr % a.dkv : 0;
-  constexpr int CH = GATED ? 16 : 32;   // token columns per turn (registers: four loads of CH columns in flight when gated)
-#pragma unroll 1
-  for (int c0 = colgrp * 32; c0 < colgrp * 32 + 32; c0 += CH) {
-    uint32_t rh[CH], rl[CH], gh[GATED ? CH : 1], gl[GATED ? CH : 1];
-    EG_STAMP(TA);
-    if constexpr (GATED) {
-      tmem_ld16_issue(t0 + c0, rh); tmem_ld16_issue(t0 + 128 + c0, rl);
-      tmem_ld16_issue(t0 + 256 + c0, gh); tmem_ld16_issue(t0 + 384 + c0, gl);
-    } else {
-      tmem_ld32_issue(t0 + c0, rh); tmem_ld32_issue(t0 + 128 + c0, rl);
-    }
-    tmem_ld_wait();
-    tmem_ld_pin(rh); tmem_ld_pin(rl);
-#ifdef BILD_STAMPS
-    TL += clock64() - TA;
-#endif
-    if constexpr (GATED) { tmem_ld_pin(gh); tmem_ld_pin(gl); }
-    float v0[CH];
-#pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      v0[j] = __uint_as_float(rh[j]) + __uint_as_float(rl[j]);
-      if constexpr (GATED) v0[j] = gelu_tanh(v0[j]) * (__uint_as_float(gh[j]) + __uint_as_float(gl[j]));
-    }
-    if (!row_ok) continue;
-    const int tokb = tok0 + c0;
-    int lim = a.M - tokb;   // token columns of this turn that exist
+// What becomes of CH token columns (tokb ..) of output row n: store / ReLU / residual add / scatter to q and the K/V layout.
+template <int CH>
+__device__ __forceinline__ void eg_emit(const LinArgs& a, __nv_bfloat16* oh, __nv_bfloat16* ol, const EgQkv& qkv, float (&v0)[CH], int n, int part,
+                                        int rr, int hh, int hc, int tokb, bool split) {
+    int lim = a.M - tokb;   // token columns that exist
     if (a.epi == EPI_RESID) {
       float* p = a.Y + (size_t)tokb * a.ldy + n;
-      if (gridDim.z > 1) {   // split over K: the partial tile is added to the stream where it lies
+      if (split) {   // split over K: the partial tile is added to the stream where it lies
 #pragma unroll
         for (int j = 0; j < CH; ++j)
           if (j < lim) atomicAdd(p + (size_t)j * a.ldy, v0[j]);
@@ -303,7 +188,7 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
           if (j < lim) p[(size_t)j * a.ldy] = old[j] + v0[j];
       }
     } else if (a.epi == EPI_HEADS && qkv.qh) {
-      if constexpr (!GATED) {
+      {
         if (part < 2) {
           __nv_bfloat16* ph = (part ? qkv.kh : qkv.qh) + (size_t)tokb * a.inner + rr;
           __nv_bfloat16* pl = (part ? qkv.kl : qkv.ql) + (size_t)tokb * a.inner + rr;
@@ -313,7 +198,18 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
             ph[(size_t)j * a.inner] = hv;
             pl[(size_t)j * a.inner] = __float2bfloat16_rn(v0[j] - __bfloat162float(hv));
           }
-        } else {   // 32 tokens of a channel: 64 bytes in a row
+        } else if constexpr (CH < 8) {
+          uint32_t hw[2], lw[2];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const __nv_bfloat162 hp = __floats2bfloat162_rn(v0[2 * i], v0[2 * i + 1]);
+            hw[i] = *reinterpret_cast<const uint32_t*>(&hp);
+            const __nv_bfloat162 lp = __floats2bfloat162_rn(v0[2 * i] - __uint_as_float(hw[i] << 16), v0[2 * i + 1] - __uint_as_float(hw[i] & 0xffff0000u));
+            lw[i] = *reinterpret_cast<const uint32_t*>(&lp);
+          }
+          *reinterpret_cast<uint2*>(qkv.vh + (size_t)rr * qkv.ldv + tokb) = make_uint2(hw[0], hw[1]);
+          *reinterpret_cast<uint2*>(qkv.vl + (size_t)rr * qkv.ldv + tokb) = make_uint2(lw[0], lw[1]);
+        } else {   // tokens of a channel: 16 bytes at a time
           uint4* ph = reinterpret_cast<uint4*>(qkv.vh + (size_t)rr * qkv.ldv + tokb);
           uint4* pl = reinterpret_cast<uint4*>(qkv.vl + (size_t)rr * qkv.ldv + tokb);
 #pragma unroll
@@ -368,6 +264,208 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
           if (j < lim) p[(size_t)j * a.ldy] = v0[j];
       }
     }
+}
+
+// CL: the gridDim.z blocks of a tile are a cluster that splits K (short inputs: a few tiles would leave most SMs idle, and one SM takes in about
+// 90 GB/s): their partial tiles meet in shared memory, every block the sum of its share of the token columns, and finishes them.
+// TT: tokens per tile (64: inputs of up to 64 tokens, half the activation bytes).
+template <bool GATED, bool CL, int TT>
+__global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* err, __nv_bfloat16* oh, __nv_bfloat16* ol, const EgQkv qkv,
+                                                              const __grid_constant__ CUtensorMap tmW0,
+                                                              const __grid_constant__ CUtensorMap tmW1,
+                                                              const __grid_constant__ CUtensorMap tmHh,
+                                                              const __grid_constant__ CUtensorMap tmHl) {
+  constexpr int NST = eg_stages<GATED, CL>();
+  constexpr int NMAT = GATED ? 2 : 1;
+  constexpr int STAGE = eg_stage_bytes<GATED, TT>();
+  constexpr int TCOLS = 256 * NMAT;
+  extern __shared__ unsigned char eg_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5;
+#ifdef BILD_STAMPS
+  long long T0, T1 = 0, T2 = 0, T3 = 0, T4 = 0, TM1 = 0, TM2 = 0, TP1 = 0, TL = 0, TA = 0;
+#endif
+  EG_STAMP(T0);
+  const int n_base = blockIdx.x * UM_TILE_M, tok0 = blockIdx.y * TT;
+  // this block's share of the K blocks (gridDim.z splits, EPI_RESID only)
+  const int nkb_all = a.K / UM_KB, kb0 = (int)(((long long)blockIdx.z * nkb_all) / gridDim.z);
+  const int nkb = (int)(((long long)(blockIdx.z + 1) * nkb_all) / gridDim.z) - kb0;
+  unsigned char* base = (unsigned char*)(((uintptr_t)eg_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(base + (size_t)NST * STAGE);
+  uint64_t* empty = full + NST;
+  uint64_t* done = empty + NST;
+  uint64_t* red = done + 1;   // CL: the partial tiles have arrived
+  uint32_t* tmem_slot = (uint32_t*)(red + 1);
+  if (tid == 0) {
+    for (int i = 0; i < NST; ++i) { mbar_init(&full[i], 1); mbar_init(&empty[i], 1); }
+    mbar_init(done, 1);
+    mbar_init(red, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(TCOLS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tmem_slot;
+  EG_STAMP(T1);
+  // thread 0 feeds the ring; the weight tiles depend on nothing and are requested before the dependency wait
+  // for the first NST stages, the activation tiles of those stages follow after it (same barrier per stage)
+  auto load_weights = [&](int kb) {
+    unsigned char* st = base + (size_t)(kb % NST) * STAGE;
+    uint64_t* bar = &full[kb % NST];
+    mbar_expect_tx(bar, STAGE);
+    tma_load_2d(st, &tmW0, (kb0 + kb) * UM_KB, n_base, bar);
+    if (GATED) tma_load_2d(st + 16384, &tmW1, (kb0 + kb) * UM_KB, n_base, bar);
+  };
+  auto load_acts = [&](int kb) {
+    unsigned char* st = base + (size_t)(kb % NST) * STAGE;
+    uint64_t* bar = &full[kb % NST];
+    tma_load_2d(st + NMAT * 16384, &tmHh, (kb0 + kb) * UM_KB, tok0, bar);
+    tma_load_2d(st + NMAT * 16384 + TT * 128, &tmHl, (kb0 + kb) * UM_KB, tok0, bar);
+  };
+  if (tid == 0)
+    for (int kb = 0; kb < nkb && kb < NST; ++kb) load_weights(kb);
+  if (CL) {
+    if (tid == 0) mbar_expect_tx(red, (uint32_t)(NMAT * 128 * TT * 4));
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (the barriers are set up: the cluster may write here)
+  }
+  pdl_launch_dependents();
+  pdl_wait();   // the activation tiles were written by the kernel in front
+  EG_STAMP(T2);
+  if (tid == 0) {
+    asm volatile("fence.proxy.async;" ::: "memory");   // rows written with ordinary stores, read by the copy engine
+    for (int kb = 0; kb < nkb; ++kb) {
+      if (kb >= NST) {
+        if (!mbar_wait(&empty[kb % NST], ((kb / NST) - 1) & 1)) *err = BILD_ERR_TIMEOUT;
+        load_weights(kb);
+      }
+      load_acts(kb);
+    }
+    EG_STAMP(TP1);
+  } else if (tid == 32) {
+    for (int kb = 0; kb < nkb; ++kb) {
+      const int st = kb % NST;
+      if (!mbar_wait(&full[st], (kb / NST) & 1)) *err = BILD_ERR_TIMEOUT;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#ifdef BILD_STAMPS
+      if (kb == 0) TM1 = clock64();
+#endif
+      const uint32_t a0 = smem_u32(base + (size_t)st * STAGE);
+      const uint32_t bh = a0 + NMAT * 16384;   // hi tile, lo tile right behind it: one operand of 256 rows
+#pragma unroll
+      for (int kk = 0; kk < UM_KB / 16; ++kk) {
+        const uint64_t db = umma_desc_sw128(bh + kk * 32);
+        eg_mma<TT>(tmem, umma_desc_sw128(a0 + kk * 32), db, (kb | kk) ? 1u : 0u);
+        if (GATED) eg_mma<TT>(tmem + 256, umma_desc_sw128(a0 + 16384 + kk * 32), db, (kb | kk) ? 1u : 0u);
+      }
+      umma_commit(&empty[st]);   // the stage may be refilled once these MMAs have read it
+    }
+    umma_commit(done);
+    EG_STAMP(TM2);
+  }
+  __syncwarp();
+  if (!mbar_wait(done, 0)) *err = BILD_ERR_TIMEOUT;
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  EG_STAMP(T3);
+
+  // ---- epilogue: a warp reads the 32 lanes (weight rows) of tensor memory that its number modulo 4 gives it access to; the
+  // four warps of a lane quarter share the 128 token columns, 32 each.  One warp per scheduler would be bound by the
+  // latency of its own instruction stream (measured: 5-10 us for the 128 columns), so all 16 warps of the block take part.
+  const int quarter = warp & 3, colgrp = warp >> 2;
+  const int n = n_base + quarter * 32 + (tid & 31);
+  const bool row_ok = n < a.N;
+  const uint32_t t0 = tmem + ((uint32_t)(quarter * 32) << 16);
+  int part = a.first_part, rr = n;
+  if (a.epi == EPI_HEADS) {
+    if (rr >= a.inner) { rr -= a.inner; ++part; }
+    if (rr >= a.inner) { rr -= a.inner; ++part; }
+  }
+  const int hh = a.epi == EPI_HEADS ? rr / a.dkv : 0, hc = a.epi == EPI_HEADS ? rr % a.dkv : 0;
+  if constexpr (CL) {
+    // this warp's quarter of the token columns, both halves added, to the rank that finishes them
+    constexpr int W4 = TT / 4;
+    static_assert(W4 == 16, "clusters take tiles of 64 tokens");
+    const int z = (int)gridDim.z, cpo = TT / z, rst = cpo + 4, rank = (int)cluster_rank(), c0 = colgrp * W4, owner = c0 / cpo;
+    float* red_buf = reinterpret_cast<float*>(base + (size_t)NST * STAGE + 256);
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const uint32_t bar = sub_mapa_u32(smem_u32(red), owner);
+#pragma unroll
+    for (int mat = 0; mat < NMAT; ++mat) {
+      uint32_t rh[W4], rl[W4];
+      tmem_ld16_issue(t0 + mat * 256 + c0, rh);
+      tmem_ld16_issue(t0 + mat * 256 + TT + c0, rl);
+      tmem_ld_wait();
+      tmem_ld_pin(rh); tmem_ld_pin(rl);
+      const uint32_t dst = sub_mapa_u32(smem_u32(red_buf + ((size_t)(mat * z + rank) * 128 + quarter * 32 + (tid & 31)) * rst + (c0 - owner * cpo)), owner);
+#pragma unroll
+      for (int j = 0; j < W4; j += 4) {
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = __uint_as_float(rh[j + e]) + __uint_as_float(rl[j + e]);
+        asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                     ::"r"(dst + j * 4), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])), "r"(bar)
+                     : "memory");
+      }
+    }
+    __syncwarp();
+    {   // (what the cluster's other blocks stored is visible behind it)
+      uint32_t ok = 0;
+      for (uint32_t it = 0; it < UM_SPIN_LIMIT && !ok; ++it)
+        asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+                     : "=r"(ok) : "r"(smem_u32(red)), "r"(0u) : "memory");
+      if (!ok) *err = BILD_ERR_TIMEOUT;
+    }
+    // the sums over the ranks, in rank order: this warp's quarter of the rank's columns, four at a time
+    const int cw = cpo / 4, row = quarter * 32 + (tid & 31);
+#pragma unroll 1
+    for (int c = colgrp * cw; c < (colgrp + 1) * cw; c += 4) {
+      float v[4] = {0.f, 0.f, 0.f, 0.f}, gt[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int rk = 0; rk < z; ++rk) {
+        const float4 p = *reinterpret_cast<const float4*>(red_buf + ((size_t)rk * 128 + row) * rst + c);
+        v[0] += p.x; v[1] += p.y; v[2] += p.z; v[3] += p.w;
+        if constexpr (GATED) {
+          const float4 q = *reinterpret_cast<const float4*>(red_buf + ((size_t)(z + rk) * 128 + row) * rst + c);
+          gt[0] += q.x; gt[1] += q.y; gt[2] += q.z; gt[3] += q.w;
+        }
+      }
+      if constexpr (GATED) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = gelu_tanh(v[e]) * gt[e];
+      }
+      if (row_ok) eg_emit<4>(a, oh, ol, qkv, v, n, part, rr, hh, hc, tok0 + rank * cpo + c, false);
+    }
+  } else {
+  constexpr int CW = TT / 4, CH = GATED ? 16 : CW;   // token columns per warp, and per turn (registers: four loads of CH columns in flight when gated)
+#pragma unroll 1
+  for (int c0 = colgrp * CW; c0 < colgrp * CW + CW; c0 += CH) {
+    uint32_t rh[CH], rl[CH], gh[GATED ? CH : 1], gl[GATED ? CH : 1];
+    EG_STAMP(TA);
+    if constexpr (GATED) {
+      tmem_ld16_issue(t0 + c0, rh); tmem_ld16_issue(t0 + TT + c0, rl);
+      tmem_ld16_issue(t0 + 256 + c0, gh); tmem_ld16_issue(t0 + 256 + TT + c0, gl);
+    } else if constexpr (CH == 16) {
+      tmem_ld16_issue(t0 + c0, rh); tmem_ld16_issue(t0 + TT + c0, rl);
+    } else {
+      tmem_ld32_issue(t0 + c0, rh); tmem_ld32_issue(t0 + TT + c0, rl);
+    }
+    tmem_ld_wait();
+    tmem_ld_pin(rh); tmem_ld_pin(rl);
+#ifdef BILD_STAMPS
+    TL += clock64() - TA;
+#endif
+    if constexpr (GATED) { tmem_ld_pin(gh); tmem_ld_pin(gl); }
+    float v0[CH];
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      v0[j] = __uint_as_float(rh[j]) + __uint_as_float(rl[j]);
+      if constexpr (GATED) v0[j] = gelu_tanh(v0[j]) * (__uint_as_float(gh[j]) + __uint_as_float(gl[j]));
+    }
+    if (!row_ok) continue;
+    eg_emit<CH>(a, oh, ol, qkv, v0, n, part, rr, hh, hc, tok0 + c0, gridDim.z > 1 && !CL);
+  }
   }
 #ifdef BILD_STAMPS
   T4 = clock64();

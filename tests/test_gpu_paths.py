@@ -83,3 +83,32 @@ def test_small_fp32_passes_match_oracle(torch_cuda, name, n_layers, d, H, dkv, F
         z = m.forward_one(st1, t)
         assert np.max(np.abs(buf[0].cpu().numpy() - z)) <= 1e-4 * max(1.0, np.max(np.abs(z)))
     ctx.close()
+
+
+@pytest.mark.parametrize("E", [1, 17, 63, 64, 65, 127, 128, 129, 200, 257, 300])
+@pytest.mark.parametrize("ffn,d,H,F", [("relu", 512, 8, 1024), ("gated_gelu", 512, 6, 1024)])
+def test_encoder_lengths_match_oracle(torch_cuda, E, ffn, d, H, F):
+    """Cross keys and values of every layer against the oracle around the tile sizes of the encoder's kernels (64 and 128 tokens a GEMM
+    tile, K split over a cluster or not, 64 keys and 128 queries an attention tile, one or two blocks per query tile)."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200.binding import BF16, Config, Context, model_cfg, upload_model
+    s = dataclasses.replace(MODEL_SHAPES["wide_s"], name="len_" + ffn, n_layers=2, d_model=d, n_heads=H, d_kv=64, d_ff=F, ffn=ffn, vocab=300)
+    key = (ffn, d)
+    if key not in _len_cache:
+        w = gen_model(s, 5, "bf16")
+        dev = upload_model(w, "cuda:0")
+        _len_cache.clear()
+        _len_cache[key] = (Context(Config(model_cfg(s, 3.0), model_cfg(s, 3.0), BF16, 320, 20, 8, 0, -1, 0), s, dev, s, dev), Model(s, w, 3.0))
+    ctx, m = _len_cache[key]
+    ids = np.random.default_rng(E).integers(2, 300, size=E).astype(np.int32)
+    ctx.encode(ids)
+    st = m.start(ids, 4)
+    for which in (0, 1):
+        for layer in range(2):
+            for what, ref in ((0, st.ck[layer]), (1, st.cv[layer])):
+                got = ctx.read_cache(which, what, layer, H, 320, 64)[:, :E]
+                want = ref.reshape(E, H, 64).transpose(1, 0, 2)
+                assert float(np.max(np.abs(got - want))) <= 2e-3 * max(1.0, float(np.max(np.abs(want)))), (which, layer, what)
+
+
+_len_cache = {}
