@@ -176,7 +176,8 @@ typedef struct {
   int32_t pdl;               /* 1: kernels of a pass are launched with programmatic dependent launch */
   int32_t fused;             /* fused sub-layer kernels: 0 off, 1 single-row passes, 2 also passes of 2 to 8 rows, 3 also
                               * blocks of 9 to 16 rows (as two chunks of up to 8 rows on two streams, layer l of the second
-                              * chunk waiting for the self-attention of layer l of the first) */
+                              * chunk waiting for the self-attention of layer l of the first) and the cluster kernel that runs
+                              * all layers of a pass of a small fp32 model */
   int32_t ffn_parts;         /* launches the fused feed-forward sub-layer is split into (0: fewest that fit) */
   int32_t block_simt;        /* 1: unfused block passes on the SIMT block GEMV */
   int32_t slice_mode;        /* unfused linear layers on the row-slice kernel: 0 off, 1 block passes, 2 also single rows */
@@ -187,7 +188,7 @@ typedef struct {
   int32_t unit_attn;         /* 1: unfused decoder attention on the chunked 256-thread kernel */
   int32_t umma;              /* 1: tcgen05 kernels (encoder linears; unfused block linears when slice_mode = 0) */
   int32_t enc_gemm;          /* 1: encoder linears as 128-token tcgen05 GEMM tiles */
-  int32_t enc_attn_mma;      /* 1: encoder self-attention on mma.sync tiles */
+  int32_t enc_attn_mma;      /* 1: encoder self-attention on tensor-core tiles (tcgen05 or mma.sync: enc_attn_groups) */
   int32_t enc_parallel;      /* 1: the two encoders run side by side on two streams, and the cross K/V projections of the
                               * decoder layers on three; 0: the whole set-up step on the context's stream */
   int32_t spin_limit;        /* polls before a bounded device-side wait gives up with BILD_ERR_TIMEOUT (0: 2^20) */
@@ -200,11 +201,13 @@ typedef struct {
                               * SWITCH kind (bodies: block pass, single-row pass, pass of 2 to 8 rows); 0: one IF node per
                               * kind of pass */
   int32_t enc_split_k;       /* 1: encoder GEMMs that add to the residual stream (output projection, second FFN matrix)
-                              * split K over more blocks, partial tiles added with reductions at the L2 */
+                              * split K over more blocks, partial tiles added with reductions at the L2; for up to 64 ids also
+                              * the others, over a cluster that adds its partial tiles in shared memory */
   int32_t head_stream;       /* single-row bf16 LM heads (rows of at most 1024 columns) on the streaming kernel: 0 off,
                               * 1 heads of slice_head_min_mb and more, 2 all */
-  int32_t enc_attn_groups;   /* encoder self-attention (enc_attn_mma): groups of four warps per block, each visiting every
-                              * n-th tile of 64 keys, partial results merged at the end; 1..3 */
+  int32_t enc_attn_groups;   /* encoder self-attention (enc_attn_mma): 3: tcgen05 kernel where it applies (enc_gemm, d_kv = 64);
+                              * 1, 2 (and 3 elsewhere): the mma.sync kernel with that many groups of four warps per block, each
+                              * visiting every n-th tile of 64 keys, partial results merged at the end */
 } bild_tuning;
 void bild_tuning_default(bild_tuning *t /*HOST out*/);
 /* bild_create with explicit switches; tuning == NULL means the defaults. */
