@@ -241,16 +241,15 @@ __device__ __forceinline__ float sub_inv(const SubShared* sh, int m, float inv_d
   return rsqrtf((((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]))) * inv_d + eps);
 }
 
-// the left operands of this warp's slice of the 16-row tile `mt` (chunks past the end of the rows: zero)
-__device__ __forceinline__ void sub_frags(const unsigned char* sW, int wst, int nrows, int d, int mt, int col0, int nch, int lane, uint4 (&f)[4][2]) {
+// the left operands of this warp's slice of half a 16-row tile (chunks past the end of the rows: zero; rows past the last one: the last one
+// again, their sums are not read)
+__device__ __forceinline__ void sub_frags8(const unsigned char* sW, int wst, int nrows, int d, int half, int col0, int nch, int lane, uint4 (&f)[4]) {
   const int g = lane >> 2, t = lane & 3;
-  const unsigned char* p0 = sW + (size_t)min(mt * 16 + g, nrows - 1) * wst + (col0 + 8 * t) * 2;
-  const unsigned char* p1 = sW + (size_t)min(mt * 16 + g + 8, nrows - 1) * wst + (col0 + 8 * t) * 2;
+  const unsigned char* p0 = sW + (size_t)min(half * 8 + g, nrows - 1) * wst + (col0 + 8 * t) * 2;
 #pragma unroll
   for (int ch = 0; ch < 4; ++ch) {
     const bool in = ch < nch && col0 + ch * 32 + 8 * t < d;
-    f[ch][0] = in ? *reinterpret_cast<const uint4*>(p0 + ch * 64) : make_uint4(0u, 0u, 0u, 0u);
-    f[ch][1] = in ? *reinterpret_cast<const uint4*>(p1 + ch * 64) : make_uint4(0u, 0u, 0u, 0u);
+    f[ch] = in ? *reinterpret_cast<const uint4*>(p0 + ch * 64) : make_uint4(0u, 0u, 0u, 0u);
   }
 }
 // the right operands: the warp's slice of the token rows
@@ -266,15 +265,15 @@ __device__ __forceinline__ void sub_bfrags(const uint32_t* Xs, int xst, int k, i
       if (!ONE) b.l[ONE ? 0 : ch] = *reinterpret_cast<const uint4*>(p + (size_t)SUB_MB * xst + ch * 16);
     }
 }
-// one 16-row tile; the warp's partial sums go to psum [warp][token][sub_pst(rows)]
+// one 16-row tile, its halves' operands f0 and f1 (`both`: the second one exists); the warp's partial sums go to psum [warp][token][sub_pst(rows)]
 template <bool ONE>
-__device__ __forceinline__ void sub_tile(const uint4 (&f)[4][2], const SubB<ONE>& b, int nch, int nrows, int mt, float* psum, int warp, int lane) {
+__device__ __forceinline__ void sub_tile(const uint4 (&f0)[4], const uint4 (&f1)[4], bool both, const SubB<ONE>& b, int nch, int nrows, int mt, float* psum, int warp, int lane) {
   const int g = lane >> 2, t = lane & 3, pst = sub_pst(nrows), row = mt * 16 + g;
   float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int ch = 0; ch < 4; ++ch)
     if (ch < nch) {
-      const uint4 a0 = f[ch][0], a1 = f[ch][1];
+      const uint4 a0 = f0[ch], a1 = both ? f1[ch] : make_uint4(0u, 0u, 0u, 0u);
       sub_mma(c, a0.x, a1.x, a0.y, a1.y, b.h[ch].x, b.h[ch].y);
       if (ONE) {
         sub_mma(e, a0.z, a1.z, a0.w, a1.w, b.h[ch].z, b.h[ch].w);
@@ -380,8 +379,8 @@ inline AttnSubPlan attn_sub_plan(int d, int dkv, int P, int C, int keys_cap, int
   const int need = std::min(64, sub_up16(per_rank)), want = std::min(128, sub_up16(std::max(per_rank, std::min(all_keys, keys_cap))));
   auto blen = [&](int kc) { return P == 3 ? (std::max(per_rank, kc) + MAXB + 8 + 3) / 4 * 4 : 4; };
   auto fits = [&](int kc, int lim) {
-    for (pl.late = 0; pl.late < (P == 3 && (P * dkv + C - 1) / C <= 32 ? 2 : 1); ++pl.late)   // (cross-attention: its keys are requested first
-      // thing, into an area of their own; more than 32 weight rows do not all wait in registers)
+    for (pl.late = 0; pl.late < (P == 3 && (P * dkv + C - 1) / C <= 24 ? 2 : 1); ++pl.late)   // (cross-attention: its keys are requested first
+      // thing, into an area of their own; more than 24 weight rows do not all wait in registers)
       if (attn_sub_layout(d, dkv, P, C, mb, kc, blen(kc), pl.late).total <= lim) return true;
     pl.late = 0;
     return false;
@@ -684,11 +683,13 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
   SUB_STAMP();            // 0: requests
   // the weight rows become operands (two 16-row tiles in registers), then the keys may take their place
   const int mt = (npr + 15) >> 4;
-  uint4 fr[2][4][2];
+  // (24 rows: 3 d_kv / 8 for d_kv = 64.  Half tiles, not whole ones: with 16 registers more the block variant spilled, and every pass of a
+  // block was slower for it: T5-large, 5 rows, 539 -> 517 us, 16 rows 824 -> 753; mT5-large, 4 to 5 rows, 637 -> 579)
+  uint4 hf[3][4];
   sub_wait(sh, a.err, &sh->wbar, 0, a.spin);
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-    if (i < mt) sub_frags(sWq, wst, npr, d, i, col0, nch, lane, fr[i]);
+  for (int i = 0; i < 3; ++i)
+    if (i * 8 < npr) sub_frags8(sWq, wst, npr, d, i, col0, nch, lane, hf[i]);
   if (a.L.kv_late) {
     __syncthreads();
     stage_cached(j0, min(min(j1, pos0), j0 + a.kc_keys));
@@ -711,12 +712,15 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
   {
     SubB<ONE> b;
     sub_bfrags<ONE>(Xs, xst, k, col0, nch, lane, b);
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (i < mt) sub_tile<ONE>(fr[i], b, nch, npr, i, psum, warp, lane);
-    if (mt > 2) {   // (heads over fewer than eight blocks; never with kv_late)
-      sub_frags(sWq, wst, npr, d, 2, col0, nch, lane, fr[0]);
-      sub_tile<ONE>(fr[0], b, nch, npr, 2, psum, warp, lane);
+    sub_tile<ONE>(hf[0], hf[1], npr > 8, b, nch, npr, 0, psum, warp, lane);
+    if (mt > 1) {   // (rows 24 and up: heads over fewer than eight blocks; never with kv_late)
+      if (npr > 24) sub_frags8(sWq, wst, npr, d, 3, col0, nch, lane, hf[0]);
+      sub_tile<ONE>(hf[2], hf[0], npr > 24, b, nch, npr, 1, psum, warp, lane);
+    }
+    if (mt > 2) {
+      sub_frags8(sWq, wst, npr, d, 4, col0, nch, lane, hf[0]);
+      if (npr > 40) sub_frags8(sWq, wst, npr, d, 5, col0, nch, lane, hf[1]);
+      sub_tile<ONE>(hf[0], hf[1], npr > 40, b, nch, npr, 2, psum, warp, lane);
     }
   }
   sub_cp_wait();          // (first chunk of keys / values)
@@ -1055,12 +1059,12 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) ffn_sub_kernel(const FfnSubArg
   // fraction of the memory's rate).  Both by bulk copies: 64 KB a block through the load units held up the shared-memory
   // accesses of the kernel in front on the same SM (5-row pass 594 -> 551 us without them).
   const int ust_fo = (ONE ? d : pack_wfo_dpad(d)) * 16 + 32;   // bytes from unit to unit: the lanes (row g, unit t) hit 32 banks
-  uint4 fr[2][4][2];
+  uint4 fr[4][4];
   if (nf > 0) {
     sub_wait(sh, a.err, &sh->wbar, 0, a.spin);
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (i * 16 < nrows) sub_frags(sWi, wst, nrows, d, i, col0, nch, lane, fr[i]);
+    for (int i = 0; i < 4; ++i)
+      if (i * 8 < nrows) sub_frags8(sWi, wst, nrows, d, i, col0, nch, lane, fr[i]);
     __syncthreads();
     const uint32_t ub = (uint32_t)(ust_fo - 32);
     if (tid == 0) mbar_expect(smem_u32(&sh->wbar), ub * (uint32_t)(nf >> 3));
@@ -1089,10 +1093,11 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) ffn_sub_kernel(const FfnSubArg
     sub_bfrags<ONE>(Xs, xst, k, col0, nch, lane, b);
 #pragma unroll
     for (int i = 0; i < 2; ++i)
-      if (i * 16 < nrows) sub_tile<ONE>(fr[i], b, nch, nrows, i, psum, warp, lane);
+      if (i * 16 < nrows) sub_tile<ONE>(fr[2 * i], fr[2 * i + 1], i * 16 + 8 < nrows, b, nch, nrows, i, psum, warp, lane);
     if (nrows > 32) {
-      sub_frags(sWi2, wst, nrows, d, 2, col0, nch, lane, fr[0]);
-      sub_tile<ONE>(fr[0], b, nch, nrows, 2, psum, warp, lane);
+      sub_frags8(sWi2, wst, nrows, d, 4, col0, nch, lane, fr[0]);
+      if (nrows > 40) sub_frags8(sWi2, wst, nrows, d, 5, col0, nch, lane, fr[1]);
+      sub_tile<ONE>(fr[0], fr[1], nrows > 40, b, nch, nrows, 2, psum, warp, lane);
     }
   }
   // W_fo into registers while the sums go round.  ONE: thread <-> the four output rows 4 tid .. 4 tid + 3, chunk q = columns 8 q .. 8 q + 7.
