@@ -984,6 +984,7 @@ struct FfnSubArgs {
   const uint4* Wfo8;         // ... and of the block variant
   int d, F, gated;
   int part, nparts;          // this launch covers the slices blockIdx.x * nparts + part of gridDim.x * nparts
+  int early;                 // 1: the next kernel may start at once, 0: once this kernel has its token rows
   int seed;                  // 1: the blocks add x_in for their share of the columns
   int mb;
   unsigned spin;             // polls of the weight barrier before the kernel gives up
@@ -1076,7 +1077,7 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) ffn_sub_kernel(const FfnSubArg
   }
   SUB_STAMP();            // 1: weights
   pdl_wait();
-  pdl_launch_dependents();   // (the next kernel's requests behind this kernel's own rows)
+  if (a.early) pdl_launch_dependents();
   SUB_STAMP();            // 2: dependency wait
   SubRows<ONE> rw;
   sub_rows_issue<ONE>(a.x_in, k, d, col, on, rw);
@@ -1087,6 +1088,7 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) ffn_sub_kernel(const FfnSubArg
       reinterpret_cast<float4*>(a.x_zero)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
   }
   sub_rows_split<ONE>(rw, k, col, stores, on, g4, Xs, xst, sh, sSeed, su0 * 4, su1 * 4, lane, warp);
+  if (!a.early) pdl_launch_dependents();
   SUB_STAMP();            // 3: token rows
   if (nf > 0) {   // hidden activations of the slice
     SubB<ONE> b;
