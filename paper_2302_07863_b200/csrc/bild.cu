@@ -914,9 +914,12 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   f.Wi0 = (const __nv_bfloat16*)w.wi0; f.Wi1 = (const __nv_bfloat16*)w.wi1;
   f.Wfo1 = m.wfo_one + (size_t)l * (Fd / 8) * d; f.Wfo8 = m.wfo_blk + (size_t)l * (Fd / 8) * pack_wfo_dpad(d);
   f.nparts = m.sub_parts;
-  // as a.early, except for the gated variant's blocks of up to 8 rows: their slices are the largest, what follows them would come late
-  // (mT5-large, 5 rows 579 us at once, 594 behind the rows; two chunks side by side, 16 rows: 903 at once, 842 behind; T5-large, 2 rows: 478, 468)
-  f.early = MB == 1 || d <= 512 || (gated && desc == m.desc);
+  // Single rows: ahead of the dependency wait, so that the next layer's first kernel, whose prologue is longer than this whole kernel, takes
+  // the SMs the kernel in front leaves (T5-large 351 -> 338 us, T5-small 81.4 -> 80.0, mT5-small 135 -> 133); not for gated slices of more
+  // than 512 columns, whose own weights would wait for it (mT5-large 408 us behind the wait, 429 ahead).  Blocks: as a.early, except for
+  // gated ones of up to 8 rows (mT5-large, 5 rows 579 us at once, 594 behind the rows; two chunks side by side, 16 rows: 903 at once, 842
+  // behind; T5-large, 2 rows: 478, 468).
+  f.early = MB == 1 ? (gated && d > 512 ? 1 : 2) : d <= 512 || (gated && desc == m.desc) ? 1 : 0;
   const int grid = m.sub_grid[MB == 1 ? 0 : 1];
   f.L = ffn_sub_layout(d, Fd, gated, grid * m.sub_parts, grid, MB);
   for (int p = 0; p < m.sub_parts; ++p) {

@@ -984,7 +984,7 @@ struct FfnSubArgs {
   const uint4* Wfo8;         // ... and of the block variant
   int d, F, gated;
   int part, nparts;          // this launch covers the slices blockIdx.x * nparts + part of gridDim.x * nparts
-  int early;                 // 1: the next kernel may start at once, 0: once this kernel has its token rows
+  int early;                 // when the next kernel may start: 2 ahead of this one's dependency wait, 1 behind it, 0 once this kernel has its token rows
   int seed;                  // 1: the blocks add x_in for their share of the columns
   int mb;
   unsigned spin;             // polls of the weight barrier before the kernel gives up
@@ -1076,8 +1076,9 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) ffn_sub_kernel(const FfnSubArg
     }
   }
   SUB_STAMP();            // 1: weights
+  if (a.early == 2) pdl_launch_dependents();
   pdl_wait();
-  if (a.early) pdl_launch_dependents();
+  if (a.early == 1) pdl_launch_dependents();
   SUB_STAMP();            // 2: dependency wait
   SubRows<ONE> rw;
   sub_rows_issue<ONE>(a.x_in, k, d, col, on, rw);
