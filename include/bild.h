@@ -405,6 +405,11 @@ int bild_op_lm_head_static(const void *W, int w_dtype, const float *X, const flo
  * max_enc_len (cross) or max_dec_len (self); count must be exactly that many floats. */
 int bild_debug_read_cache(bild_ctx *ctx, int which, int what, int layer, float *dst_host, size_t count);
 
+/* Test helper: how many of the kernels behind the set-up kernel of a single-step call (which: 0 small, 1 large; k tokens)
+ * may start before it is complete.  Must be 0: the kernels of a pass read what it writes without waiting for it.
+ * Nothing runs on the GPU (the launches are recorded in a graph that is dropped). */
+int bild_debug_setup_edges(bild_ctx *ctx, int which, int k, int *programmatic /*HOST out*/);
+
 /* Host-only: the relative-position bucket the library uses (T5's bucket function in
  * exact integer arithmetic).  which = 0: decoder, rel = query_pos - key_pos >= 0;
  * which = 1: encoder, rel = key_pos - query_pos.  Returns -1 on invalid arguments. */

@@ -27,7 +27,7 @@ EXPORTS = ["bild_query_workspace", "bild_create", "bild_create_tuned", "bild_tun
            "bild_fetch_result", "bild_time_pass", "bild_uses_tensor_cores", "bild_launch_count", "bild_last_error", "bild_op_linear",
            "bild_op_lm_head_scratch_bytes", "bild_op_lm_head", "bild_op_lm_head_static", "bild_debug_bucket",
            "bild_debug_read_cache", "bild_op_lm_head_sliced", "bild_op_lm_head_stream", "bild_op_sublayer_scratch_bytes", "bild_op_attn_sublayer",
-           "bild_op_ffn_sublayer", "bild_generate_sampled"]
+           "bild_op_ffn_sublayer", "bild_generate_sampled", "bild_debug_setup_edges"]
 
 
 class ModelCfg(C.Structure):
@@ -303,6 +303,13 @@ class Context:
         self.L.bild_debug_read_cache.argtypes = [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_void_p, C.c_size_t]
         self._check(self.L.bild_debug_read_cache(self.h, which, what, layer, out.ctypes.data, out.size))
         return out
+
+    def setup_edges(self, which: int, k: int) -> int:
+        """Kernels of a single-step call's pass that may start before its set-up kernel is complete (recorded, not run)."""
+        n = C.c_int()
+        self.L.bild_debug_setup_edges.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_int)]
+        self._check(self.L.bild_debug_setup_edges(self.h, which, k, C.byref(n)))
+        return n.value
 
     def uses_tensor_cores(self) -> bool:
         return bool(self.L.bild_uses_tensor_cores(self.h))

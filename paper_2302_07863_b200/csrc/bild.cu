@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <string>
 #include <vector>
@@ -363,8 +364,16 @@ void plan(bild_ctx* c, Bump& b) {
 }
 
 // ---- launches ------------------------------------------------------------------------
-// Every kernel of a pass is launched so that it may start while its predecessor drains
-// (programmatic dependent launch); each of them waits before touching dependent data.
+// Every kernel of a pass but the first is launched so that it may start while its predecessor drains
+// (programmatic dependent launch); each of them waits before touching what its predecessor writes.  The first is a
+// plain launch: the sub-layer kernels and the cluster pass read the call descriptor ahead of their wait, so the kernel
+// that wrote it (set_call_kernel, split_desc_kernel) has to be complete before any kernel of the pass starts.
+struct PlainLaunches {   // while one lives: launches without the programmatic attribute
+  bild_ctx* c;
+  bool was;
+  explicit PlainLaunches(bild_ctx* ctx) : c(ctx), was(ctx->use_pdl) { c->use_pdl = false; }
+  ~PlainLaunches() { c->use_pdl = was; }
+};
 template <typename... KArgs, typename... Args>
 cudaError_t launch_k(bild_ctx* c, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, Args... args) {
   cudaLaunchConfig_t cfg = {};
@@ -825,15 +834,13 @@ cudaError_t launch_cpass_rows(bild_ctx* c, Model& m, int mb, const CallDesc* des
   return launch_k(c, kern, dim3(CP_C), dim3(CP_THREADS), smem, a);
 }
 cudaError_t launch_cpass(bild_ctx* c, Model& m, int MBv) {
+  PlainLaunches plain(c);   // (first kernel of the pass)
   if (MBv <= SUB_MB) return launch_cpass_rows(c, m, MBv, m.desc, 0);
-  // 9 to 16 rows: two chunks, the second (plain launch: it stages keys of the first before any wait) behind the first
+  // 9 to 16 rows: two chunks, the second (a plain launch too: it stages keys of the first before any wait) behind the first
   split_desc_kernel<<<1, 1, 0, c->stream>>>(m.desc, m.desc_lo, m.desc_hi);
   (*c->cnt)++;
-  const bool pdl = c->use_pdl;
-  c->use_pdl = false;
   cudaError_t e = launch_cpass_rows(c, m, SUB_MB, m.desc_lo, 0);
   if (e == cudaSuccess) e = launch_cpass_rows(c, m, SUB_MB, m.desc_hi, SUB_CHUNK);
-  c->use_pdl = pdl;
   return e;
 }
 
@@ -860,8 +867,8 @@ cudaError_t launch_sub(bild_ctx* c, void (*kern)(Arg), int grid, int cluster, si
 
 // One layer of a decoder pass on the fused sub-layer kernels: the residual stream goes x -> xb -> xc -> x (self-attention,
 // cross-attention, feed-forward), each kernel clearing the buffer after its output.  desc / row0: the rows the kernels
-// work on (a whole pass, or one chunk of a block of 9 to 16 rows); first_plain: the layer's first kernel follows a
-// dependency on another stream and is launched without the programmatic-launch attribute; after_self: called once the
+// work on (a whole pass, or one chunk of a block of 9 to 16 rows); first_plain: the layer's first kernel is the first of its
+// pass or follows a dependency on another stream, and is launched without the programmatic-launch attribute; after_self: called once the
 // self-attention kernel is in the stream (its keys and values are what the next chunk's same layer waits for).
 template <typename F>
 int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int row0, bool first_plain, F after_self) {
@@ -931,7 +938,7 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
 
 int fused_layers(bild_ctx* c, Model& m, int MB) {
   for (int l = 0; l < m.c.n_layers; ++l) {
-    int rc = fused_layer(c, m, MB, l, m.desc, 0, false, [] { return (int)BILD_OK; });
+    int rc = fused_layer(c, m, MB, l, m.desc, 0, l == 0 && c->fused_embed, [] { return (int)BILD_OK; });
     if (rc) return rc;
   }
   return BILD_OK;
@@ -1198,8 +1205,10 @@ int decoder_pass(bild_ctx* c, int which, int MBv, float* logits_dbg, unsigned lo
   // (fused sub-layer kernels: the first one gathers the embedding rows itself; the buffer it adds into is clear, every
   // pass leaves it so and a generation starts with it cleared)
   if (small) CUDA_TRY(c, launch_cpass(c, m, MBv));
-  else if (!(fused && c->fused_embed))
+  else if (!(fused && c->fused_embed)) {
+    PlainLaunches plain(c);   // (first kernel of the pass)
     CUDA_TRY(c, launch_embed(c, m.w.emb, m.desc->tokens, &m.desc->k, 0, MB, d, mc.vocab, m.x, fused ? m.xb : nullptr));
+  }
   if (fused) {
     int rc = chunked ? fused_layers_two_chunks(c, m) : fused_layers(c, m, MBv);
     if (rc) return rc;
@@ -1415,9 +1424,10 @@ int add_cond(bild_ctx* c, cudaGraph_t g, const cudaGraphNode_t* deps, size_t nde
   return BILD_OK;
 }
 
-// Captures one decoder pass into `body`; returns the leaf nodes of the capture.
+// Captures one decoder pass into `body` (behind whatever `before` launches); returns the leaf nodes of the capture.
 int capture_pass(bild_ctx* c, cudaGraph_t body, int which, int MB, unsigned long long hw, unsigned long long hi,
-                 std::vector<cudaGraphNode_t>* leaves, int64_t* count, unsigned long long hi1 = 0, unsigned long long hi8 = 0) {
+                 std::vector<cudaGraphNode_t>* leaves, int64_t* count, unsigned long long hi1 = 0, unsigned long long hi8 = 0,
+                 const std::function<void()>& before = {}) {
   if (!c->cap_stream) CUDA_TRY(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
   CUDA_TRY(c, cudaStreamBeginCaptureToGraph(c->cap_stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   int64_t n = 0;
@@ -1425,6 +1435,7 @@ int capture_pass(bild_ctx* c, cudaGraph_t body, int which, int MB, unsigned long
   c->stream = c->cap_stream;
   c->cnt = &n;
   c->capturing = true;
+  if (before) before();
   int rc = decoder_pass(c, which, MB, nullptr, hw, hi, hi1, hi8);
   c->capturing = false;
   c->cnt = &c->launches;
@@ -1600,6 +1611,14 @@ int bild_reset_lengths(bild_ctx* c) {
 // One single-step call: k tokens through model `which`, results in pin_head.  One set-up kernel, the pass (a graph from the second call of
 // its kind on: 19 or 73 launches cost the host 45 or 170 us, and the capture more than one call gains) and one synchronisation; the cache
 // lengths are read back first only if a loop may have moved them.  T5-small step, host to host: 136 -> 105 us (the pass alone: 83).
+void launch_set_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha) {
+  TokList t{};
+  for (int i = 0; i < k; ++i) t.t[i] = tokens[i];
+  set_call_kernel<<<1, 1, 0, c->stream>>>(c->m[which].desc, c->st, which, k, alpha, t);
+  (*c->cnt)++;
+}
+int step_rows(int k) { return k == 1 ? 1 : k <= SUB_MB ? SUB_MB : MAXB; }   // rows the pass of a call over k tokens is built for
+
 int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha, float* logits_dbg) {
   if (!c->len_known) {
     int rc = read_state(c);
@@ -1608,12 +1627,9 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
   if ((which == 0 ? c->pin_state->S_len : c->pin_state->L_len) + k > c->cfg.max_dec_len)
     return fail(c, BILD_ERR_CAPACITY, which == 0 ? "small-model cache is full" : "large-model cache is full");
   c->len_known = false;
-  TokList t{};
-  for (int i = 0; i < k; ++i) t.t[i] = tokens[i];
-  set_call_kernel<<<1, 1, 0, c->stream>>>(c->m[which].desc, c->st, which, k, alpha, t);
-  (*c->cnt)++;
+  launch_set_call(c, which, tokens, k, alpha);
   CUDA_TRY(c, cudaGetLastError());
-  const int MBv = k == 1 ? 1 : k <= SUB_MB ? SUB_MB : MAXB;
+  const int MBv = step_rows(k);
   bild_ctx::StepGraph& s = c->step[which == 0 ? 0 : MBv == 1 ? 1 : MBv == SUB_MB ? 2 : 3];
   struct Publish { bild_ctx* c; ~Publish() { c->publish = false; } } publish{c};
   c->publish = true;
@@ -2310,6 +2326,31 @@ int bild_debug_read_cache(bild_ctx* c, int which, int what, int layer, float* ds
   const float* base = what == 0 ? m.crossK : what == 1 ? m.crossV : what == 2 ? m.selfK : m.selfV;
   CUDA_TRY(c, cudaMemcpyAsync(dst_host, base + (size_t)layer * n, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return BILD_OK;
+}
+
+// Test helper: records what a single-step call over k tokens enqueues on the plain-launch path (set-up kernel, then the pass) in a graph that
+// is never run, and counts the programmatic edges that leave the set-up kernel.
+int bild_debug_setup_edges(bild_ctx* c, int which, int k, int* programmatic) {
+  if (!c || !programmatic || (which != 0 && which != 1)) return fail(c, BILD_ERR_ARG, "null argument / which");
+  if (k < 1 || k > (which == 0 ? 1 : MAXB)) return fail(c, BILD_ERR_ARG, "k outside 1..16");
+  const int32_t tokens[MAXB] = {};
+  cudaGraph_t g = nullptr;
+  CUDA_TRY(c, cudaGraphCreate(&g, 0));
+  struct Drop { cudaGraph_t g; ~Drop() { cudaGraphDestroy(g); } } drop{g};
+  int64_t n = 0;
+  int rc = capture_pass(c, g, which, step_rows(k), 0, 0, nullptr, &n, 0, 0, [&] { launch_set_call(c, which, tokens, k, 0.f); });
+  if (rc) return rc;
+  cudaGraphNode_t root = nullptr;
+  size_t nr = 1, nd = 0;
+  CUDA_TRY(c, cudaGraphGetRootNodes(g, &root, &nr));
+  CUDA_TRY(c, cudaGraphNodeGetDependentNodes_v2(root, nullptr, nullptr, &nd));
+  std::vector<cudaGraphNode_t> dep(nd);
+  std::vector<cudaGraphEdgeData> edge(nd);
+  if (nd) CUDA_TRY(c, cudaGraphNodeGetDependentNodes_v2(root, dep.data(), edge.data(), &nd));
+  if (nr != 1 || nd < 1) return fail(c, BILD_ERR_STATE, "no kernel behind the set-up kernel");
+  *programmatic = 0;
+  for (size_t i = 0; i < nd; ++i) *programmatic += edge[i].type == cudaGraphDependencyTypeProgrammatic ? 1 : 0;
   return BILD_OK;
 }
 

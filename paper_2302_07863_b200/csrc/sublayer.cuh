@@ -656,8 +656,8 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
     }
   }
   // The call descriptor (row count, cache position) is written by kernels that have finished before the first kernel of a
-  // pass starts -- the head of the pass before, or a set-up kernel in front of the embedding -- never by the kernel in
-  // front of this one: it is read before the dependency wait, and with it the cached keys and values (rows below the
+  // pass starts (the head of the pass before, or a set-up kernel; that first kernel is a plain launch), never by a kernel
+  // of the pass that this one may overlap: it is read before the dependency wait, and with it the cached keys and values (rows below the
   // cache position, written by earlier passes; a second chunk of a block is launched only when the first chunk's rows
   // of this layer are complete) and the bias by distance.
   const int k = ONE ? 1 : min(a.desc->k, a.mb), pos0 = a.desc->pos0;

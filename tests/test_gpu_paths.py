@@ -112,3 +112,15 @@ def test_encoder_lengths_match_oracle(torch_cuda, E, ffn, d, H, F):
 
 
 _len_cache = {}
+
+
+@pytest.mark.parametrize("name,tuning", [("tiny", None), ("tiny", dict(fused=0)), ("odd_bf16", None), ("tiny_bf16", None), ("wide_bf16", None),
+                                         ("wide_bf16", dict(fused=1)), ("wide_bf16", dict(fused=2)), ("wide_bf16", dict(fused=0))])
+def test_pass_starts_behind_its_set_up_kernel(torch_cuda, name, tuning):
+    """No kernel of a single-step call's pass may start before the kernel that writes the call descriptor is complete, since the
+    kernels read the descriptor ahead of their dependency wait.  The launches are recorded, nothing runs."""
+    from paper_2302_07863_b200.synthetic import make_context
+    ctx, _, _ = make_context(name, 9.0, 9.0, tuning=tuning)
+    for which, k in ((0, 1), (1, 1), (1, 2), (1, 8), (1, 9), (1, 16)):
+        assert ctx.setup_edges(which, k) == 0, (which, k)
+    ctx.close()
