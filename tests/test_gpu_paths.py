@@ -124,3 +124,75 @@ def test_pass_starts_behind_its_set_up_kernel(torch_cuda, name, tuning):
     for which, k in ((0, 1), (1, 1), (1, 2), (1, 8), (1, 9), (1, 16)):
         assert ctx.setup_edges(which, k) == 0, (which, k)
     ctx.close()
+
+
+@pytest.mark.parametrize("name,scS,scL", [("tiny", 9.0, 9.0), ("odd_bf16", 9.0, 9.0), ("wide_bf16", 9.0, 11.0)])
+def test_single_step_calls_without_logits_match_oracle(torch_cuda, name, scS, scL):
+    """Calls without a logits buffer, as a host program makes them: the first two of a kind (small step; large pass of one row, of 2 to 8
+    and of 9 to 16) launch their kernels, the later ones replay a graph.  Results against the oracle for every call, on growing caches,
+    after rewinds, after an input of another length, after a reset and after generations (which move the caches on the device)."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200 import MODE_LARGE_ONLY, MODE_SMALL_ONLY
+    from paper_2302_07863_b200.synthetic import make_context
+    wl = WORKLOADS[name]
+    ctx, _, _ = make_context(name, scS, scL, max_enc_len=140, max_dec_len=130)
+    S, L = (Model(MODEL_SHAPES[m], gen_model(MODEL_SHAPES[m], wl.seed, wl.dtype), sc) for m, sc in ((wl.small, scS), (wl.large, scL)))
+    tol = 1e-4 if wl.dtype == "fp32" else 2e-3   # logit error e of the other tests; lse moves by at most e, gaps and distances by 2 e
+    rng = np.random.default_rng(3)
+    V, afb, arb = S.s.vocab, 0.4, 15.0
+
+    def check(o, Z, toks):
+        for i, z in enumerate(Z):
+            top, pmax, lse, gap = obild.max_prob(z)
+            if gap > 2 * tol:
+                assert (o.argmax[i] if len(toks) else o.argmax) == top
+            assert abs((o.lse[i] if len(toks) else o.lse) - lse) <= tol
+        if not len(toks):
+            assert abs(o.pmax - pmax) <= 2 * tol * pmax + 1e-6 and abs(o.max_logit - z[top]) <= tol
+            assert o.fallback == int(pmax < afb) or abs(pmax - afb) <= 2 * tol
+            return
+        d = [obild.max_prob(z)[2] - z[t] for z, t in zip(Z, toks[1:])]
+        assert all(abs(a - b) <= 2 * tol for a, b in zip(o.d, d))
+        if all(abs(x - arb) > 2 * tol for x in d):
+            assert o.first_violation == next((i for i, x in enumerate(d) if x > arb), -1)
+
+    def step(st):
+        t = int(rng.integers(2, V))
+        check(ctx.small_step(t, afb), [S.forward_one(st, t)], [])
+
+    def verify(st, k):
+        toks = [int(t) for t in rng.integers(2, V, size=k)]
+        check(ctx.large_verify(toks, arb), L.forward_block(st, toks), toks)
+
+    KINDS = (1, 5, 12, 8, 9, 2)
+    for E, again in ((23, 3), (131, 1)):
+        ids = rng.integers(2, V, size=E).astype(np.int32)
+        ctx.encode(ids)
+        stS, stL = S.start(ids, 130), L.start(ids, 130)
+        for _ in range(again):
+            for k in KINDS[:3]:
+                step(stS)
+                verify(stL, k)
+        for st, which in ((stS, 0), (stL, 1)):
+            st.rewind(2)
+            ctx.rewind(which, 2)
+        for k in KINDS:
+            step(stS)
+            verify(stL, k)
+        toks = ctx.generate(MODE_SMALL_ONLY, 0.0, 1.0, 7)["tokens"]
+        stS = S.start(ids, 130)
+        S.forward_block(stS, [0] + toks[:-1])
+        step(stS)
+        step(stS)
+        toks = ctx.generate(MODE_LARGE_ONLY, 0.0, 1.0, 7)["tokens"]
+        stL = L.start(ids, 130)
+        L.forward_block(stL, [0] + toks[:-1])
+        for k in KINDS:
+            verify(stL, k)
+        ctx.generate(MODE_SMALL_ONLY, 0.0, 1.0, 5)
+        ctx.reset()
+        stS, stL = S.start(ids, 130), L.start(ids, 130)
+        for k in KINDS:
+            step(stS)
+            verify(stL, k)
+    ctx.close()
