@@ -229,6 +229,11 @@ int bild_encode(bild_ctx *ctx, const int32_t *ids /*HOST*/, int n_ids);
 /* Reset the decode state only (keeps the encoder results of the last bild_encode). */
 int bild_reset(bild_ctx *ctx);
 
+/* The single-step calls below (bild_small_step, bild_large_verify) replay a CUDA graph of their pass from the third call of
+ * a kind on (small step; large pass of one row, of 2 to 8, of 9 to 16).  The first two calls of a kind on a context launch
+ * the kernels one by one and record and instantiate the graph while the GPU works; where a pass is shorter than that
+ * (models of a few layers) each of them takes up to about 100 us longer.  Calls with a logits_dbg buffer always launch. */
+
 /* One small-model step: feed `token` at the next position of the small model's
  * cache (cache length += 1) and return the arg-max / p_max / fallback test of the
  * next-token distribution (Section 3.3).  logits_dbg: DEVICE [vocab] fp32 or NULL;

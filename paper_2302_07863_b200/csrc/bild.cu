@@ -171,7 +171,7 @@ struct bild_ctx {
   HeadOut* pin_head = nullptr;
   bool len_known = false;         // pin_state holds the device's cache lengths and error flag (no call has moved them since)
   bool publish = false;           // the pass being enqueued writes its results to pin_head / pin_state
-  // single-step calls from the second of a kind on: the pass as a graph.  [0] small step, [1] large pass of one row, [2] of 2 to 8, [3] of more
+  // single-step calls from the third of a kind on: the pass as a graph.  [0] small step, [1] large pass of one row, [2] of 2 to 8, [3] of more
   struct StepGraph { cudaGraph_t g = nullptr; cudaGraphExec_t ex = nullptr; int64_t launches = 0; int calls = 0; } step[4];
   size_t ws_bytes = 0;
   // device-side loop: WHILE { small pass; IF (fallback) { large block pass } } and WHILE { large pass }
@@ -1608,9 +1608,6 @@ int bild_reset_lengths(bild_ctx* c) {
   return BILD_OK;
 }
 
-// One single-step call: k tokens through model `which`, results in pin_head.  One set-up kernel, the pass (a graph from the second call of
-// its kind on: 19 or 73 launches cost the host 45 or 170 us, and the capture more than one call gains) and one synchronisation; the cache
-// lengths are read back first only if a loop may have moved them.  T5-small step, host to host: 136 -> 105 us (the pass alone: 83).
 void launch_set_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha) {
   TokList t{};
   for (int i = 0; i < k; ++i) t.t[i] = tokens[i];
@@ -1619,6 +1616,27 @@ void launch_set_call(bild_ctx* c, int which, const int32_t* tokens, int k, float
 }
 int step_rows(int k) { return k == 1 ? 1 : k <= SUB_MB ? SUB_MB : MAXB; }   // rows the pass of a call over k tokens is built for
 
+// The graph of a kind of single-step call is built while the GPU is at the plain launches of its first calls: recorded behind the first,
+// instantiated behind the second.  The host would only wait meanwhile, so that no call pays for it whose pass is longer than the build
+// (T5 pair, us: recording 30, for 9 to 16 rows 65; instantiation 85 small step, 140, 9 to 16 rows 280).  Calls one to four, host to host:
+// small step 146, 138, 114, 98, pass of 5 rows 548, 562, 533, 535; with all of it in front of the second call's pass 115, 278, 98, 98 and
+// 546, 747, 536, 533.  A failure leaves the kind on plain launches.
+void step_graph_build(bild_ctx* c, bild_ctx::StepGraph& s, int which, int MBv) {
+  bool ok = true;
+  if (++s.calls == 1) {
+    ok = cudaGraphCreate(&s.g, 0) == cudaSuccess && capture_pass(c, s.g, which, MBv, 0, 0, nullptr, &s.launches) == BILD_OK;
+  } else if (s.calls == 2 && s.g) {
+    ok = cudaGraphInstantiate(&s.ex, s.g, 0) == cudaSuccess;
+    // the first launch of a graph uploads it (20 to 55 us): here, if the GPU is still busy
+    if (ok && cudaStreamQuery(c->stream) == cudaErrorNotReady) cudaGraphUpload(s.ex, c->stream);
+  }
+  if (!ok) drop_step_graph(s);
+  cudaGetLastError();
+}
+
+// One single-step call: k tokens through model `which`, results in pin_head.  One set-up kernel, the pass (a graph from the third call of
+// its kind on: 19 or 73 launches cost the host 45 or 170 us) and one synchronisation; the cache lengths are read back first only if a
+// loop may have moved them.  T5-small step, host to host: 143 us with launches and two read-backs, 115 with launches, 98 (the pass alone: 80).
 int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha, float* logits_dbg) {
   if (!c->len_known) {
     int rc = read_state(c);
@@ -1633,16 +1651,13 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
   bild_ctx::StepGraph& s = c->step[which == 0 ? 0 : MBv == 1 ? 1 : MBv == SUB_MB ? 2 : 3];
   struct Publish { bild_ctx* c; ~Publish() { c->publish = false; } } publish{c};
   c->publish = true;
-  if (!logits_dbg && !s.ex && ++s.calls == 2) {
-    int rc = cudaGraphCreate(&s.g, 0) == cudaSuccess ? capture_pass(c, s.g, which, MBv, 0, 0, nullptr, &s.launches) : (int)BILD_ERR_CUDA;
-    if (rc != BILD_OK || cudaGraphInstantiate(&s.ex, s.g, 0) != cudaSuccess) { cudaGetLastError(); drop_step_graph(s); }   // (plain launches then)
-  }
   if (!logits_dbg && s.ex) {
     CUDA_TRY(c, cudaGraphLaunch(s.ex, c->stream));
     c->launches += s.launches;
   } else {
     int rc = decoder_pass(c, which, MBv, logits_dbg);
     if (rc) return rc;
+    if (!logits_dbg) step_graph_build(c, s, which, MBv);
   }
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   if (c->pin_state->err) return fail(c, c->pin_state->err, "device-side error flag set");
