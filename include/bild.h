@@ -191,9 +191,11 @@ typedef struct {
   int32_t enc_attn_mma;      /* 1: encoder self-attention on tensor-core tiles (tcgen05 or mma.sync: enc_attn_groups) */
   int32_t enc_parallel;      /* 1: the two encoders run side by side on two streams, and the cross K/V projections of the
                               * decoder layers on three; 0: the whole set-up step on the context's stream */
-  int32_t spin_limit;        /* polls before a bounded device-side wait gives up with BILD_ERR_TIMEOUT (0: 2^20) */
-  int32_t debug_skip_copies; /* 1: the fused attention kernel announces its weight copies but does not issue them, so
-                              * that its bounded wait runs out (test of the time-out path; never set in production) */
+  int32_t spin_limit;        /* polls before a bounded wait of the fused sub-layer kernels or the cluster kernel gives up with
+                              * BILD_ERR_TIMEOUT (0: 2^20, which the other kernels' waits always use) */
+  int32_t debug_skip_copies; /* tests of the time-out path; never set in production.  1: the fused attention kernel announces its
+                              * weight copies but does not issue them, so that its bounded wait runs out.  2: a time-out is noted
+                              * in the encoder's place, as one of its kernels would */
   int32_t attn_all_keys;     /* fused attention: while a head has at most this many keys (and they fit one staged chunk)
                               * every block of the head's cluster attends over all of them, which saves the exchange
                               * and merge of per-block partial results; 0: keys always split over the cluster */
@@ -223,7 +225,8 @@ void bild_destroy(bild_ctx *ctx); /* frees the host-side context only */
  * encoder runs on a stream of the context's own, forked from and joined back into the
  * caller's stream with events, so work queued on the caller's stream after this call still
  * sees both encoders' results (bild_tuning.enc_parallel = 0 keeps everything on the caller's
- * stream). */
+ * stream).  A time-out of an encoder kernel is reported by the calls that decode from this input
+ * (all of them, whatever bild_reset or another generation does in between). */
 int bild_encode(bild_ctx *ctx, const int32_t *ids /*HOST*/, int n_ids);
 
 /* Reset the decode state only (keeps the encoder results of the last bild_encode). */

@@ -149,7 +149,7 @@ struct bild_ctx {
   bild_trace_rec* trace = nullptr;
   int trace_cap = 0;
   int* enc_ids = nullptr;
-  int* enc_len_dev = nullptr;
+  int* enc_len_dev = nullptr;              // [0] encoder ids of the present input, [1] error its encoder kernels reported
   int* bucket_tmp = nullptr;
   float* u_draw[2] = {nullptr, nullptr};   // uniform numbers by output position, small / large model (sampling variant)
   float top_p = 0.f;                       // > 0 while a sampled generation is set up or running
@@ -214,7 +214,7 @@ struct bild_ctx {
   int sub_parts_want = 0;            // 0: fewest launches of the feed-forward sub-layer that fit
   bool use_umma = true, use_enc_gemm = true;
   unsigned spin_limit = SPIN_LIMIT;
-  bool debug_skip_copies = false;
+  int debug_skip_copies = 0;
   bool capturing = false;            // launches are being recorded into a graph, not run
   int64_t graph_counted = 0;         // launches of the loop graphs already added to `launches`
 };
@@ -293,7 +293,7 @@ void plan(bild_ctx* c, Bump& b) {
   c->trace_cap = cap * (cfg.max_draft + 3);
   c->trace = b.take<bild_trace_rec>(c->trace_cap);
   c->enc_ids = b.take<int>(ecap);
-  c->enc_len_dev = b.take<int>(1);
+  c->enc_len_dev = b.take<int>(2);
   c->bucket_tmp = b.take<int>(std::max(cap, 2 * ecap));
   c->u_draw[0] = b.take<float>(cap + 1);
   c->u_draw[1] = b.take<float>(cap + 1);
@@ -794,7 +794,7 @@ int setup_cpass(bild_ctx* c, Model& m) {
   m.cpass = false;
   const bild_model_cfg& mc = m.c;
   const bool gated = mc.ffn_kind == BILD_FFN_GATED_GELU;
-  if (c->fused_on < 3 || c->debug_skip_copies || !cpass_size_ok(mc, c->cfg.dtype)) return BILD_OK;
+  if (c->fused_on < 3 || c->debug_skip_copies == 1 || !cpass_size_ok(mc, c->cfg.dtype)) return BILD_OK;
   int smem_max = 0, dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
     cudaGetLastError();
@@ -885,7 +885,7 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   AttnSubArgs a{};
   a.desc = desc; a.eps = mc.ln_eps; a.inv_d = 1.f / (float)d; a.d = d; a.I = I; a.H = H; a.dkv = dkv; a.dkv_shift = ilog2(dkv); a.C = C; a.c_shift = ilog2(C);
   a.mb = MB; a.err = &c->st->err;
-  a.spin = c->spin_limit; a.skip_copies = c->debug_skip_copies ? 1 : 0;
+  a.spin = c->spin_limit; a.skip_copies = c->debug_skip_copies == 1 ? 1 : 0;
   a.n_keys_dev = c->enc_len_dev;
   // When the next kernel's blocks may start their requests.  Behind this kernel's token rows where those requests are large and would queue
   // in front of them (T5-large, 5 rows: 580 -> 552 us; blocks of 9 to 16 rows: two chunks' kernels share the SMs), or where the kernels
@@ -1004,11 +1004,13 @@ bool umma_plan(int N, int K, bool gated, int* cs_out, int* nkb_out, bool many_ro
   return true;
 }
 
+int* encoder_err(bild_ctx* c) { return c->enc_len_dev + 1; }
+
 cudaError_t launch_umma(bild_ctx* c, const LinArgs& a, const CUtensorMap& t0, const CUtensorMap& t1, int cs, int nkb,
-                        int row_blocks = 1) {
+                        int* err, int row_blocks = 1) {
   const bool gated = a.epi == EPI_GATED;
   UmmaArgs u;
-  u.lin = a; u.cs = cs; u.nkb = nkb; u.err = &c->st->err;
+  u.lin = a; u.cs = cs; u.nkb = nkb; u.err = err;
   const int tiles = (a.N + UM_TILE_M - 1) / UM_TILE_M;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(tiles * cs, row_blocks); cfg.blockDim = dim3(UM_THREADS);
@@ -1086,7 +1088,7 @@ cudaError_t launch_dec_linear(bild_ctx* c, Model& m, int MB, const LinArgs& a, i
   }
   if (MB != 1 && m.umma && umma_plan(a.N, a.K, a.epi == EPI_GATED, &cs, &nkb)) {
     const CUtensorMap* t = &m.tmaps[(size_t)layer * TM_PER_LAYER];
-    return launch_umma(c, a, t[which_map], t[which_map == TM_WI0 ? TM_WI1 : which_map], cs, nkb);
+    return launch_umma(c, a, t[which_map], t[which_map == TM_WI0 ? TM_WI1 : which_map], cs, nkb, &c->st->err);
   }
   return launch_linear(c, c->cfg.dtype, MB, a);
 }
@@ -1134,15 +1136,15 @@ cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, 
     cfg.attrs = at; cfg.numAttrs = c->use_pdl ? 2 : 1;
     (*c->cnt)++;
     auto kern = gated ? enc_gemm_kernel<true, true, 64> : enc_gemm_kernel<false, true, 64>;
-    return cudaLaunchKernelEx(&cfg, kern, a, &c->st->err, oh, ol, qkv, t0, t1, h[0], h[1]);
+    return cudaLaunchKernelEx(&cfg, kern, a, encoder_err(c), oh, ol, qkv, t0, t1, h[0], h[1]);
   }
   if (gated) {
     grid.y = tiles_tok;
-    return launch_k(c, enc_gemm_kernel<true, false, 128>, grid, dim3(EG_THREADS), eg_smem_bytes<true, false, 128>(), a, &c->st->err, oh, ol, qkv, t0, t1,
+    return launch_k(c, enc_gemm_kernel<true, false, 128>, grid, dim3(EG_THREADS), eg_smem_bytes<true, false, 128>(), a, encoder_err(c), oh, ol, qkv, t0, t1,
                     m.tmH[pair][ki][0], m.tmH[pair][ki][1]);
   }
   return launch_k(c, small ? enc_gemm_kernel<false, false, 64> : enc_gemm_kernel<false, false, 128>, grid, dim3(EG_THREADS),
-                  small ? eg_smem_bytes<false, false, 64>() : eg_smem_bytes<false, false, 128>(), a, &c->st->err, oh, ol, qkv, t0, t1, h[0], h[1]);
+                  small ? eg_smem_bytes<false, false, 64>() : eg_smem_bytes<false, false, 128>(), a, encoder_err(c), oh, ol, qkv, t0, t1, h[0], h[1]);
 }
 
 // Encoder attention on tcgen05; two blocks share a query tile's keys while the grid leaves half of the SMs idle (and there are two tiles).
@@ -1175,7 +1177,7 @@ cudaError_t launch_enc_linear(bild_ctx* c, Model& m, const LinArgs& a, int rb, i
     return launch_enc_gemm(c, m, a, layer, which_map, split, pair, out_pair);
   if (m.umma && umma_plan(a.N, a.K, a.epi == EPI_GATED, &cs, &nkb, rb >= 4)) {
     const CUtensorMap* t = &m.tmaps[(size_t)layer * TM_PER_LAYER];
-    return launch_umma(c, a, t[which_map], t[which_map == TM_EWI0 ? TM_EWI1 : which_map], cs, nkb, rb);
+    return launch_umma(c, a, t[which_map], t[which_map == TM_EWI0 ? TM_EWI1 : which_map], cs, nkb, encoder_err(c), rb);
   }
   return launch_linear(c, c->cfg.dtype, MAXB, a, rb);
 }
@@ -1318,6 +1320,10 @@ int encoder_pass(bild_ctx* c, int which) {
   const int E = c->enc_len, ecap = c->cfg.max_enc_len, dt = c->cfg.dtype;
   const int rb = (E + MAXB - 1) / MAXB;
   CUDA_TRY(c, launch_embed(c, m.w.emb, c->enc_ids, nullptr, E, E, d, mc.vocab, B.ex));
+  if (c->debug_skip_copies == 2) {
+    fake_timeout_kernel<<<1, 1, 0, c->stream>>>(encoder_err(c));
+    (*c->cnt)++;
+  }
   for (int l = 0; l < mc.n_layers; ++l) {
     const bild_enc_layer& w = m.enc[l];
     LinArgs a{};
@@ -1331,14 +1337,14 @@ int encoder_pass(bild_ctx* c, int which) {
     if (m.enc_flash) {
       EncFlashArgs f{};
       f.bias = m.enc_bias; f.bias_ld = 2 * ecap - 1; f.bias_off = ecap - 1; f.n_keys_dev = c->enc_len_dev; f.M = E; f.H = H;
-      f.oh = B.exh[1]; f.ol = B.exl[1]; f.err = &c->st->err;
+      f.oh = B.exh[1]; f.ol = B.exl[1]; f.err = encoder_err(c);
       CUDA_TRY(c, launch_enc_flash(c, m, f));
     } else {
     BAttnArgs t{};
     t.q = B.eq; t.ldq = I; t.kc = B.ek; t.vc = B.ev; t.cap = ecap; t.out = B.eatt; t.ldo = I;
     t.bias = m.enc_bias; t.bias_ld = 2 * ecap - 1; t.bias_off = ecap - 1; t.mode = 2; t.dkv = dkv; t.H = H;
     t.n_keys_dev = c->enc_len_dev; t.M = E; t.part = m.att_part; t.counters = m.att_cnt; t.nsplit = 1;
-    t.err = &c->st->err;
+    t.err = encoder_err(c);
     CUDA_TRY(c, launch_battn(c, MAXB, t, rb, ecap, fuse ? B.exh[1] : nullptr, fuse ? B.exl[1] : nullptr));
     }
     LinArgs o{};
@@ -1666,7 +1672,7 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
 }
 
 int reset_state(bild_ctx* c, int mode, float afb, float arb, int max_len) {
-  reset_state_kernel<<<1, 1, 0, c->stream>>>(loop_ptrs(c), mode, afb, arb, max_len, c->cfg.max_draft,
+  reset_state_kernel<<<1, 1, 0, c->stream>>>(loop_ptrs(c), encoder_err(c), mode, afb, arb, max_len, c->cfg.max_draft,
                                              c->cfg.eos_id, c->cfg.start_id, c->trace_cap, c->top_p);
   c->len_known = false;
   (*c->cnt)++;
@@ -1747,7 +1753,7 @@ int bild_create_tuned(const bild_config* cfg, const bild_weights* small_w, const
     c->enc_parallel = t.enc_parallel != 0;
     c->enc_kv_streams = t.enc_parallel != 0;   // (one switch: everything of the set-up step on one stream, or not)
     c->spin_limit = t.spin_limit > 0 ? (unsigned)t.spin_limit : SPIN_LIMIT;
-    c->debug_skip_copies = t.debug_skip_copies != 0;
+    c->debug_skip_copies = std::min(2, std::max(0, t.debug_skip_copies));
     c->attn_all_keys = std::min(128, std::max(0, t.attn_all_keys));
     c->graph_switch = t.graph_switch != 0;
     c->enc_split_k = t.enc_split_k != 0;
@@ -1841,7 +1847,8 @@ int bild_encode(bild_ctx* c, const int32_t* ids, int n_ids) {
   c->encoded = false;
   c->enc_len = n_ids;
   CUDA_TRY(c, cudaMemcpyAsync(c->enc_ids, ids, n_ids * sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  CUDA_TRY(c, cudaMemcpyAsync(c->enc_len_dev, &c->enc_len, sizeof(int), cudaMemcpyHostToDevice, c->stream));
+  const int head[2] = {n_ids, 0};   // length; no error so far
+  CUDA_TRY(c, cudaMemcpyAsync(c->enc_len_dev, head, sizeof(head), cudaMemcpyHostToDevice, c->stream));
   // The two encoders are independent: the small model's runs on a side stream, forked from and joined
   // back into the caller's stream with events, while the large model's runs on the caller's stream.
   const bool early = c->cfg.early_exit_layers > 0;   // one encoder: the small model is a prefix of the large model's decoder

@@ -710,12 +710,16 @@ __global__ void rewind_kernel(DevState* st, int which, int new_len) {
   if (which == 0) st->S_len = new_len; else st->L_len = new_len;
 }
 
-__global__ void reset_state_kernel(LoopPtrs L, int mode, float alpha_fb, float alpha_rb, int max_len,
+// What an encoder kernel does whose bounded wait runs out (bild_tuning.debug_skip_copies = 2)
+__global__ void fake_timeout_kernel(int* err) { *err = BILD_ERR_TIMEOUT; }
+
+// enc_err: what the encoder of the present input reported (an error there stays with everything decoded from it)
+__global__ void reset_state_kernel(LoopPtrs L, const int* enc_err, int mode, float alpha_fb, float alpha_rb, int max_len,
                                    int max_draft, int eos_id, int start_id, int trace_cap, float top_p) {
   DevState* st = L.st;
   st->top_p = top_p;
   st->n = 0; st->S_len = 0; st->L_len = 0; st->drafts = 0;
-  st->fallback = 0; st->mode = mode; st->err = 0;
+  st->fallback = 0; st->mode = mode; st->err = *enc_err;
   st->max_len = max_len; st->max_draft = max_draft; st->eos_id = eos_id; st->start_id = start_id;
   st->alpha_fb = alpha_fb; st->alpha_rb = alpha_rb;
   st->n_trace = 0; st->trace_cap = trace_cap;

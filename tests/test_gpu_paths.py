@@ -196,3 +196,27 @@ def test_single_step_calls_without_logits_match_oracle(torch_cuda, name, scS, sc
             step(stS)
             verify(stL, k)
     ctx.close()
+
+
+@pytest.mark.parametrize("name,early_exit", [("tiny", 0), ("wide_bf16", 0), ("wide_bf16", 1)])
+def test_encoder_time_out_reaches_the_caller(torch_cuda, name, early_exit):
+    """A time-out noted while the encoder runs (bild_tuning.debug_skip_copies = 2 writes the code that an encoder kernel would): every call
+    that decodes from that input must report it, also behind a reset or a generation, which start from a fresh decode state."""
+    from paper_2302_07863_b200 import MODE_BILD, MODE_LARGE_ONLY, BildError
+    from paper_2302_07863_b200.synthetic import make_context
+    ctx, ids, wl = make_context(name, 9.0, 9.0, tuning=dict(debug_skip_copies=2), early_exit_layers=early_exit)
+
+    def times_out(f):
+        with pytest.raises(BildError) as e:
+            f()
+        assert e.value.code == -6
+    u = np.full(4, 0.5, np.float32)
+    for _ in range(2):
+        ctx.encode(ids)
+        times_out(lambda: ctx.small_step(0, 0.4))
+        ctx.reset()
+        times_out(lambda: ctx.large_verify([0, 5, 7], 10.0))
+        times_out(lambda: ctx.generate(MODE_BILD, 0.4, 10.0, 3))
+        times_out(lambda: ctx.generate(MODE_LARGE_ONLY, 0.4, 10.0, 2))
+        times_out(lambda: ctx.generate_sampled(MODE_BILD, 0.4, 10.0, 3, 0.8, u, u))
+    ctx.close()
