@@ -25,6 +25,10 @@ namespace bild {
 
 constexpr int EG_THREADS = 512;   // thread 0 feeds the ring, thread 32 issues the MMAs, all 16 warps share the epilogue
 constexpr int EG_TOK = 128;   // tokens per tile
+// Polls for the partial tiles of a cluster's other blocks: more than such a block may spend in front of its stores when every one of its
+// waits runs out (one per K block, 128 at most with K <= 16384 split in two, and one for their end), so that none of the blocks has left
+// when they arrive.
+constexpr uint32_t EG_PART_LIMIT = 160u * UM_SPIN_LIMIT;
 
 __device__ __forceinline__ uint32_t sub_mapa_u32(uint32_t a, int rank) {
   uint32_t r;
@@ -413,7 +417,7 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
     __syncwarp();
     {   // (what the cluster's other blocks stored is visible behind it)
       uint32_t ok = 0;
-      for (uint32_t it = 0; it < UM_SPIN_LIMIT && !ok; ++it)
+      for (uint32_t it = 0; it < EG_PART_LIMIT && !ok; ++it)
         asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
                      : "=r"(ok) : "r"(smem_u32(red)), "r"(0u) : "memory");
       if (!ok) *err = BILD_ERR_TIMEOUT;
