@@ -418,6 +418,9 @@ int bild_debug_read_cache(bild_ctx *ctx, int which, int what, int layer, float *
  * Nothing runs on the GPU (the launches are recorded in a graph that is dropped). */
 int bild_debug_setup_edges(bild_ctx *ctx, int which, int k, int *programmatic /*HOST out*/);
 
+/* Test helper: y[i] = 1 / x[i] as the attention kernels of the decoder passes form it.  x, y: DEVICE [n].  Asynchronous. */
+int bild_debug_reciprocal(const float *x /*DEVICE*/, float *y /*DEVICE*/, int n, void *cuda_stream);
+
 /* Host-only: the relative-position bucket the library uses (T5's bucket function in
  * exact integer arithmetic).  which = 0: decoder, rel = query_pos - key_pos >= 0;
  * which = 1: encoder, rel = key_pos - query_pos.  Returns -1 on invalid arguments. */

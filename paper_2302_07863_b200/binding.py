@@ -27,7 +27,8 @@ EXPORTS = ["bild_query_workspace", "bild_create", "bild_create_tuned", "bild_tun
            "bild_fetch_result", "bild_time_pass", "bild_uses_tensor_cores", "bild_launch_count", "bild_last_error", "bild_op_linear",
            "bild_op_lm_head_scratch_bytes", "bild_op_lm_head", "bild_op_lm_head_static", "bild_debug_bucket",
            "bild_debug_read_cache", "bild_op_lm_head_sliced", "bild_op_lm_head_stream", "bild_op_sublayer_scratch_bytes", "bild_op_attn_sublayer",
-           "bild_op_ffn_sublayer", "bild_generate_sampled", "bild_debug_setup_edges"]
+           "bild_op_ffn_sublayer", "bild_generate_sampled", "bild_debug_setup_edges",
+           "bild_debug_reciprocal"]
 
 
 class ModelCfg(C.Structure):

@@ -2351,6 +2351,13 @@ int bild_debug_read_cache(bild_ctx* c, int which, int what, int layer, float* ds
   return BILD_OK;
 }
 
+// Test helper: the reciprocal that the attention kernels normalise with.
+int bild_debug_reciprocal(const float* x, float* y, int n, void* cuda_stream) {
+  if (!x || !y || n < 1) return BILD_ERR_ARG;
+  sub_rcp_kernel<<<(n - 1) / 256 + 1, 256, 0, (cudaStream_t)cuda_stream>>>(x, y, n);
+  return cudaGetLastError() == cudaSuccess ? BILD_OK : BILD_ERR_CUDA;
+}
+
 // Test helper: records what a single-step call over k tokens enqueues on the plain-launch path (set-up kernel, then the pass) in a graph that
 // is never run, and counts the programmatic edges that leave the set-up kernel.
 int bild_debug_setup_edges(bild_ctx* c, int which, int k, int* programmatic) {

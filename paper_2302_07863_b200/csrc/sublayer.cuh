@@ -227,11 +227,16 @@ __device__ __forceinline__ void sub_rows_split(const SubRows<ONE>& rw, int k, in
   }
   __syncwarp();
 }
-// 1 / x to the last bit but one: the hardware's approximation and a Newton step (a full division is a chain several times as long)
+// 1 / x of a soft-max's sum (1 to the number of keys), relative error at most 2^-23: the hardware's approximation (its error, 2^-23, is
+// squared) and a Newton step of two roundings; a full division is a chain several times as long.  Not for 0 and infinity.
 __device__ __forceinline__ float sub_rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r * (2.f - x * r);
+  return r * fmaf(-x, r, 2.f);
+}
+__global__ void sub_rcp_kernel(const float* x, float* y, int n) {   // (for its test)
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) y[i] = sub_rcp(x[i]);
 }
 // 1 / rms of token row m from the warps' sums of squares (after the barrier behind the products)
 __device__ __forceinline__ float sub_inv(const SubShared* sh, int m, float inv_d, float eps) {

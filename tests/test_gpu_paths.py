@@ -220,3 +220,20 @@ def test_encoder_time_out_reaches_the_caller(torch_cuda, name, early_exit):
         times_out(lambda: ctx.generate(MODE_LARGE_ONLY, 0.4, 10.0, 2))
         times_out(lambda: ctx.generate_sampled(MODE_BILD, 0.4, 10.0, 3, 0.8, u, u))
     ctx.close()
+
+
+def test_reciprocal_of_softmax_sums(torch_cuda):
+    """The attention kernels' 1 / x against fp64 for every mantissa, at the exponents of a soft-max's sum (1 to 2048 keys and beyond).
+    Bound: an approximation of relative error 2^-23, squared by the Newton step, and the step's two roundings of 2^-24 each."""
+    from paper_2302_07863_b200 import binding
+    torch = torch_cuda
+    L = binding.lib()
+    L.bild_debug_reciprocal.argtypes = [binding.C.c_void_p, binding.C.c_void_p, binding.C.c_int, binding.C.c_void_p]
+    mant = torch.arange(1 << 23, device="cuda", dtype=torch.int32)
+    y = torch.empty(1 << 23, device="cuda")
+    for e in (-1, 0, 1, 5, 11, 12):
+        x = (mant | ((127 + e) << 23)).view(torch.float32)
+        assert L.bild_debug_reciprocal(x.data_ptr(), y.data_ptr(), x.numel(), torch.cuda.current_stream().cuda_stream) == 0
+        err = (y.double() * x.double() - 1.0).abs().max().item()
+        assert err <= 2.0 ** -23 + 2.0 ** -45, (e, err)
+    assert (y > 0).all()
