@@ -21,7 +21,7 @@
  * General rules
  *   - Every pointer is tagged HOST or DEVICE.  The library never allocates or
  *     frees device memory: weights, workspace and debug buffers are the caller's
- *     and must outlive the context.  bild_create allocates a small host-side
+ *     and must outlive the context (the weights unchanged: see bild_create).  bild_create allocates a small host-side
  *     context, freed by bild_destroy.
  *   - Every call returns a status (BILD_OK = 0 or a negative BILD_ERR_*), never
  *     throws, never aborts.  After an error the context is usable again after
@@ -161,9 +161,12 @@ int bild_query_workspace(const bild_config *cfg /*HOST*/, size_t *bytes /*HOST o
 /* Build a context.  `workspace` is DEVICE memory, 256-byte aligned, at least
  * bild_query_workspace bytes, caller-owned, used exclusively by this context until
  * bild_destroy.  `cuda_stream` is a cudaStream_t (NULL = default stream).  Device work done
- * here, on that stream, with a synchronisation before returning: the workspace is cleared
- * and the relative-position bias tables are expanded by distance.  The weights are read in
- * place by every kernel (no copies, no re-layout).  Errors: ARG, WORKSPACE, CUDA. */
+ * here, on that stream, with a synchronisation before returning: the workspace is cleared,
+ * the relative-position bias tables are expanded by distance, and what the decoder kernels
+ * read in an order of their own is copied into it (bf16: wfo of every decoder layer, twice;
+ * fp32 models of at most 2 MB a decoder layer: wo, wco and wfo).  All other weights are read
+ * in place.  So they must not change while the context exists: after an update of the weights
+ * create a new one.  Errors: ARG, WORKSPACE, CUDA. */
 int bild_create(const bild_config *cfg /*HOST*/, const bild_weights *small_w /*HOST*/,
                 const bild_weights *large_w /*HOST*/, void *workspace /*DEVICE*/,
                 size_t workspace_bytes, void *cuda_stream, bild_ctx **out /*HOST out*/);

@@ -237,3 +237,31 @@ def test_reciprocal_of_softmax_sums(torch_cuda):
         err = (y.double() * x.double() - 1.0).abs().max().item()
         assert err <= 2.0 ** -23 + 2.0 ** -45, (e, err)
     assert (y > 0).all()
+
+
+@pytest.mark.parametrize("name", ["tiny", "tiny_bf16"])
+def test_new_context_takes_updated_weights(torch_cuda, name):
+    """Some matrices are copied in another order when a context is created (W_fo; W_o and W_co of small fp32 models), so weights must not
+    change under a context; one created after an update in place uses the new values of all of them."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200.binding import BF16, FP32, Config, Context, model_cfg, upload_model
+    torch = torch_cuda
+    wl = WORKLOADS[name]
+    s = MODEL_SHAPES[wl.large]
+    dev = upload_model(gen_model(s, 1, wl.dtype), "cuda:0")
+    cfg = Config(model_cfg(s, 3.0), model_cfg(s, 3.0), BF16 if wl.dtype == "bf16" else FP32, 32, 20, 8, 0, -1, 0)
+    ids = np.arange(2, 30, dtype=np.int32)
+    old = Context(cfg, s, dev, s, dev)
+    w = gen_model(s, 2, wl.dtype)
+    for key, val in upload_model(w, "cuda:0").items():
+        dev[key].copy_(val)
+    new = Context(cfg, s, dev, s, dev)
+    m = Model(s, w, 3.0)
+    buf = torch.empty((16, s.vocab), dtype=torch.float32, device="cuda")
+    for k in (1, 5):
+        new.encode(ids)
+        new.large_verify([0, 5, 9, 4, 7][:k], 10.0, buf)
+        z = m.forward_block(m.start(ids, 20), [0, 5, 9, 4, 7][:k])
+        assert np.max(np.abs(buf[:k].cpu().numpy() - z)) <= (1e-4 if wl.dtype == "fp32" else 2e-3) * max(1.0, np.max(np.abs(z)))
+    old.close()
+    new.close()
