@@ -30,12 +30,6 @@ constexpr int EG_TOK = 128;   // tokens per tile
 // when they arrive.
 constexpr uint32_t EG_PART_LIMIT = 160u * UM_SPIN_LIMIT;
 
-__device__ __forceinline__ uint32_t sub_mapa_u32(uint32_t a, int rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
-}
-
 // Optional cycle stamps (build with -DBILD_STAMPS), summed over the blocks of the T5-large-shaped GEMMs of 512 tokens:
 // [class: QKV (24 row tiles), FFN-up (32), residual (8, K split)][slot]; slot 15 counts the blocks.  Slots 0-4: a thread
 // of warp 2 (start -> tensor memory allocated -> dependency wait returned -> all MMAs done -> epilogue done; 4: its loads
@@ -395,7 +389,7 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
     const int z = (int)gridDim.z, cpo = TT / z, rst = cpo + 4, rank = (int)cluster_rank(), c0 = colgrp * W4, owner = c0 / cpo;
     float* red_buf = reinterpret_cast<float*>(base + (size_t)NST * STAGE + 256);
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    const uint32_t bar = sub_mapa_u32(smem_u32(red), owner);
+    const uint32_t bar = cluster_map(smem_u32(red), owner);
 #pragma unroll
     for (int mat = 0; mat < NMAT; ++mat) {
       uint32_t rh[W4], rl[W4];
@@ -403,7 +397,7 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
       tmem_ld16_issue(t0 + mat * 256 + TT + c0, rl);
       tmem_ld_wait();
       tmem_ld_pin(rh); tmem_ld_pin(rl);
-      const uint32_t dst = sub_mapa_u32(smem_u32(red_buf + ((size_t)(mat * z + rank) * 128 + quarter * 32 + (tid & 31)) * rst + (c0 - owner * cpo)), owner);
+      const uint32_t dst = cluster_map(smem_u32(red_buf + ((size_t)(mat * z + rank) * 128 + quarter * 32 + (tid & 31)) * rst + (c0 - owner * cpo)), owner);
 #pragma unroll
       for (int j = 0; j < W4; j += 4) {
         float v[4];

@@ -45,11 +45,7 @@ struct NucleusShared {
   int token;
 };
 
-__device__ __forceinline__ unsigned ns_remote(const void* p, int rank) {
-  unsigned a;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  return a;
-}
+__device__ __forceinline__ unsigned ns_remote(const void* p, int rank) { return cluster_map(smem_u32(p), (uint32_t)rank); }
 __device__ __forceinline__ unsigned ns_ld(const unsigned* p, int rank) {
   unsigned v;
   asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(ns_remote(p, rank)) : "memory");

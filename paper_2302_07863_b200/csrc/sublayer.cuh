@@ -104,19 +104,14 @@ __device__ __forceinline__ void sub_wait_exchange(SubShared* sh, int* err, unsig
 // Stores into the shared memory of block `rank` of the cluster that count down the bytes its mbarrier `bar` expects: the
 // receiver waits for the bytes, nobody for a cluster-wide barrier with its release of everything written before (which cost
 // 883 cycles per exchange against 510 of these stores, eight blocks, 192 values each to everyone).
-__device__ __forceinline__ uint32_t sub_mapa(uint32_t a, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  return r;
-}
 __device__ __forceinline__ void sub_push(const float* dst, const unsigned long long* bar, uint32_t rank, float v) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-               ::"r"(sub_mapa(smem_u32(dst), rank)), "r"(__float_as_uint(v)), "r"(sub_mapa(smem_u32(bar), rank)) : "memory");
+               ::"r"(cluster_map(smem_u32(dst), rank)), "r"(__float_as_uint(v)), "r"(cluster_map(smem_u32(bar), rank)) : "memory");
 }
 __device__ __forceinline__ void sub_push4(const float* dst, const unsigned long long* bar, uint32_t rank, float4 v) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-               ::"r"(sub_mapa(smem_u32(dst), rank)), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
-               "r"(__float_as_uint(v.w)), "r"(sub_mapa(smem_u32(bar), rank)) : "memory");
+               ::"r"(cluster_map(smem_u32(dst), rank)), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)),
+               "r"(__float_as_uint(v.w)), "r"(cluster_map(smem_u32(bar), rank)) : "memory");
 }
 
 __device__ __forceinline__ void sub_mma(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
