@@ -891,6 +891,10 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   // in front of them (T5-large, 5 rows: 580 -> 552 us; blocks of 9 to 16 rows: two chunks' kernels share the SMs), or where the kernels
   // are shorter still than their prologue's gain (single rows of 512 columns: 145 -> 135 us); at once where a prologue would otherwise
   // not be done in time (single rows of 1024 columns: mT5-large 442 -> 416 us; blocks of 512 columns: mT5-small 2 rows 215 -> 206 us).
+  // The line at 512 columns lies between these models.  Widths in between (576 to 960, 12 layers, 256 encoder ids, all six choices of this and
+  // f.early below): blocks within 3 % of the best choice (640 columns, 2 rows: 204.5 us, 198.3 best), single rows within 1 % with ReLU and
+  // 6 % gated (576 columns: 155.4 us, 145.9 with f.early = 2).  No one line is best everywhere: at 512 columns such a model of 12 layers
+  // takes 149.8 us a single row, 136.3 with a.early = 1, where the T5-small shapes (6 layers, 512 ids) go from 80 to 82.
   a.early = MB == 1 ? d > 512 : d <= 512 && desc == m.desc;
   // S1-S3 / L1-L3 (layer 0: with S0 / L0, the rows come from the embedding table)
   if (l == 0 && c->fused_embed) {

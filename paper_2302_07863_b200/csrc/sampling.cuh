@@ -9,8 +9,9 @@
 // prefix whose probabilities add up to at least top_p; drawn token = first of the prefix at which the running sum
 // exceeds u times the prefix's total.  Both prefixes are found without sorting the row.
 //
-// One cluster of eight blocks owns the row, each an eighth of the vocabulary, every probability computed once and kept in
-// a register (up to 262144 tokens).  Probabilities below (1 - top_p) / V cannot belong to the nucleus (all of them
+// One cluster of eight blocks owns the row, each an eighth of the vocabulary, every probability computed once and kept by its
+// thread (up to 262144 tokens: 32 values; of the 64 registers a block of 1024 threads leaves each, 13 values are spilled).
+// Probabilities below (1 - top_p) / V cannot belong to the nucleus (all of them
 // together weigh less than what the nucleus leaves out), so:
 //   * up to 32 candidates are left (a peaked distribution, the usual one): one warp ranks them by comparing all pairs;
 //   * more: a radix search over the bit patterns of the probabilities, 11 + 10 + 9 bits, on histograms of counts and
@@ -28,7 +29,7 @@ namespace bild {
 
 constexpr int NS_THREADS = 1024;
 constexpr int NS_CLUSTER = 8;
-constexpr int NS_KEEP = 32;            // probabilities a thread keeps in registers
+constexpr int NS_KEEP = 32;            // probabilities a thread keeps
 constexpr int NS_CAND = 32;            // candidates one warp ranks
 constexpr int NS_BUCKETS = 2048;       // of the first radix level
 constexpr unsigned NS_NONE = 0xffffffffu;
