@@ -11,7 +11,7 @@
 // Such a layer is a few thousand multiply-adds per token row: a pass is bound by the latency of its instruction stream and of the
 // kernels in a row (eight a layer with one kernel per operation), not by bytes.  Eight blocks: the portable cluster size, and the
 // heads and slices of such models do not fill more.  Measured against one kernel per operation, 4 layers of 128 columns, 4 heads, d_ff
-// 512, passes with LM head: 1 row 71 -> 53 us, 2 rows 134 -> 72, 5 rows 155 -> 90, 8 rows 175 -> 99; 2 layers of 64 columns, 1 row 39 -> 31.
+// 512, passes with LM head: 1 row 72 -> 53 us, 2 rows 137 -> 72, 5 rows 158 -> 90, 8 rows 177 -> 98; 2 layers of 64 columns, 1 row 39 -> 29.
 // bf16 models of this size stay on the sub-layer kernels, whose tensor-core tiles are faster still (3 layers of 128 columns, 5 rows:
 // 55 us there, 82 us with this kernel on bf16 weights).
 // Sums run in a fixed order, so results do not depend on timing.

@@ -548,7 +548,7 @@ __device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk
 }
 
 // ONE: a single token row (the small model's step, the large model's single-row pass); else 2 to 8 rows.
-// Bound by the latency of its dependent chain (3-10 % of the memory's rate, 3-10 % of the tensor pipe): token rows from the L2,
+// Bound by the latency of its dependent chain (5 rows: 8 % of the memory's rate, 6-8 % of the tensor pipe while it runs): token rows from the L2,
 // products, exchange of q | k | v within the head's cluster, attention, [exchange of the ranks' records], output products, reductions
 // at the L2.  What is off the chain is done before the dependency wait: the weight rows wait as operands in registers, W_o's too,
 // the cached keys and values in shared memory.  Between barriers each warp works alone: three (four) block barriers and one
@@ -556,7 +556,7 @@ __device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk
 // Measured, T5-large shapes, pass of 24 layers, cache 32, 512 encoder keys, before -> after this form of the kernels (both
 // sub-layer kernels; before: token rows and norm for the whole block, then products from shared memory, cluster barriers, scores,
 // soft-max and values with a block barrier each): 1 row 473 -> 355 us, 5 rows 632 -> 550 us, 8 rows 691 -> 597 us, 16 rows
-// 1080 -> 831 us; T5-small 100 -> 83 us.
+// 1080 -> 831 us; T5-small 100 -> 83 us.  With the steps noted at their places since: 339, 506, 558, 748 and 80 us.
 template <bool ONE>
 __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubArgs a) {
   extern __shared__ __align__(1024) unsigned char sub_smem[];
