@@ -213,6 +213,10 @@ typedef struct {
   int32_t enc_attn_groups;   /* encoder self-attention (enc_attn_mma): 3: tcgen05 kernel where it applies (enc_gemm, d_kv = 64);
                               * 1, 2 (and 3 elsewhere): the mma.sync kernel with that many groups of four warps per block, each
                               * visiting every n-th tile of 64 keys, partial results merged at the end */
+  int32_t draft_ahead;       /* 1: in bild_generate* the small model goes on from its own candidate while the large model judges
+                              * the block in front, as long as large passes mostly end with that candidate; what it drafted
+                              * is dropped if one ends otherwise (tokens, trace and counts are those of the serial loop).
+                              * 0, and with early exit (shared caches), graph_switch = 0 or host_loop = 1: the serial loop */
 } bild_tuning;
 void bild_tuning_default(bild_tuning *t /*HOST out*/);
 /* bild_create with explicit switches; tuning == NULL means the defaults. */

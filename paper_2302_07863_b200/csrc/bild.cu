@@ -200,6 +200,8 @@ struct bild_ctx {
   bool graph_switch = true;          // the large pass of a loop iteration hangs off one SWITCH node (else: one IF node per kind of pass)
   unsigned long long sw_handle = 0;  // while the small pass of such a loop is captured: the SWITCH node's handle and body count
   int sw_bodies = 0;
+  bool draft_ahead = true;           // loop in rounds, the small model drafting on beside the large pass
+  unsigned long long side_handle = 0;   // while a pass of such a loop is captured: its model's WHILE node
   int attn_all_keys = 128;           // fused attention: caches up to this many keys are attended by every rank of a head
   bool unit_attn = true;             // decoder attention on the 256-thread chunked kernel
   bool uattn_smem_set = false;
@@ -1279,7 +1281,8 @@ int decoder_pass(bild_ctx* c, int which, int MBv, float* logits_dbg, unsigned lo
   h.scale = mc.logit_scale; h.V = mc.vocab; h.K = d; h.desc = m.desc; h.partials = m.head_part;
   h.counter = m.head_cnt; h.out = m.head_out; h.logits_dbg = logits_dbg; h.which = which; h.loop = loop_ptrs(c);
   h.cond_while = cond_while; h.cond_if = cond_if; h.cond_if1 = cond_if1; h.cond_if8 = cond_if8;
-  if (which == 0) { h.cond_switch = c->sw_handle; h.sw_bodies = c->sw_bodies; }
+  h.cond_side = c->side_handle;
+  if ((which == 1) == (c->side_handle != 0)) { h.cond_switch = c->sw_handle; h.sw_bodies = c->sw_bodies; }
   if (c->publish) { h.host_head = c->pin_head; h.host_state = c->pin_state; }
   h.pass_kind = which == 0 ? 0 : MBv == 1 ? 2 : MBv == SUB_MB ? 3 : 1;
   if (c->draw) {   // sampling: the head leaves its logits and the policy step to the kernel that draws the token
@@ -1423,7 +1426,7 @@ int build_bias_tables(bild_ctx* c) {
 
 // Adds a conditional node to `g` after `deps` and returns its body graph.
 int add_cond(bild_ctx* c, cudaGraph_t g, const cudaGraphNode_t* deps, size_t ndeps, cudaGraphConditionalHandle h,
-             cudaGraphConditionalNodeType type, cudaGraph_t* body) {
+             cudaGraphConditionalNodeType type, cudaGraph_t* body, cudaGraphNode_t* node_out = nullptr) {
   cudaGraphNodeParams p = {cudaGraphNodeTypeConditional};
   p.conditional.handle = h;
   p.conditional.type = type;
@@ -1431,6 +1434,7 @@ int add_cond(bild_ctx* c, cudaGraph_t g, const cudaGraphNode_t* deps, size_t nde
   cudaGraphNode_t node;
   CUDA_TRY(c, cudaGraphAddNode(&node, g, deps, ndeps, &p));
   *body = p.conditional.phGraph_out[0];
+  if (node_out) *node_out = node;
   return BILD_OK;
 }
 
@@ -1508,6 +1512,41 @@ int build_graphs(bild_ctx* c, int base) {
   return rc;
 }
 
+// The loop in rounds (round_step): WHILE { WHILE { SWITCH { large pass } } beside WHILE { small pass }; round_kernel }.
+int build_rounds(bild_ctx* c, cudaGraph_t g, int64_t* per_pass, int64_t* per_pass_large1, int64_t* per_pass_large8) {
+  const bool body8 = c->m[1].cpass || (c->m[1].fused && c->fused_on >= 2);   // passes of 2 to 8 rows have a body of their own
+  const int nb = body8 ? 3 : 2;
+  cudaGraphConditionalHandle hw, hl, hb, hs;
+  CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hw, g, 1, cudaGraphCondAssignDefault));
+  CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hl, g, 0, cudaGraphCondAssignDefault));
+  CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hb, g, (unsigned)nb, cudaGraphCondAssignDefault));
+  CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hs, g, 1, cudaGraphCondAssignDefault));
+  cudaGraph_t round = nullptr, large = nullptr, small = nullptr;
+  cudaGraphNode_t sides[2], node;
+  int rc = add_cond(c, g, nullptr, 0, hw, cudaGraphCondTypeWhile, &round);
+  if (rc == BILD_OK) rc = add_cond(c, round, nullptr, 0, hl, cudaGraphCondTypeWhile, &large, &sides[0]);
+  if (rc == BILD_OK) rc = add_cond(c, round, nullptr, 0, hs, cudaGraphCondTypeWhile, &small, &sides[1]);
+  if (rc) return rc;
+  cudaGraphNodeParams p = {cudaGraphNodeTypeConditional};
+  p.conditional.handle = hb; p.conditional.type = cudaGraphCondTypeSwitch; p.conditional.size = (unsigned)nb;
+  CUDA_TRY(c, cudaGraphAddNode(&node, large, nullptr, 0, &p));
+  struct Side { bild_ctx* c; ~Side() { c->side_handle = c->sw_handle = 0; c->sw_bodies = 0; } } side{c};
+  c->side_handle = hs;
+  rc = capture_pass(c, small, 0, 1, 0, 0, nullptr, &per_pass[0]);
+  c->side_handle = hl; c->sw_handle = hb; c->sw_bodies = nb;
+  if (rc == BILD_OK) rc = capture_pass(c, p.conditional.phGraph_out[0], 1, MAXB, 0, 0, nullptr, &per_pass[1]);
+  if (rc == BILD_OK) rc = capture_pass(c, p.conditional.phGraph_out[1], 1, 1, 0, 0, nullptr, per_pass_large1);
+  if (rc == BILD_OK && body8) rc = capture_pass(c, p.conditional.phGraph_out[2], 1, SUB_MB, 0, 0, nullptr, per_pass_large8);
+  if (rc) return rc;
+  LoopPtrs L = loop_ptrs(c);
+  int bodies = nb;
+  void* args[] = {&L, &bodies, &hw, &hl, &hb, &hs};
+  cudaKernelNodeParams k = {};
+  k.func = (void*)round_kernel; k.gridDim = dim3(1); k.blockDim = dim3(1); k.kernelParams = args;
+  CUDA_TRY(c, cudaGraphAddKernelNode(&node, round, sides, 2, &k));
+  return BILD_OK;
+}
+
 int build_graphs_once(bild_ctx* c, int base) {
   // launches per pass are recorded from the greedy graphs; the drawing kernels of the sampled ones are counted on the device
   int64_t dummy[2] = {0, 0}, dummy1 = 0, dummy8 = 0;
@@ -1516,7 +1555,12 @@ int build_graphs_once(bild_ctx* c, int base) {
   int64_t& per_pass_large8 = base == 0 ? c->per_pass_large8 : dummy8;
   cudaGraph_t* graph = c->graph + base;
   cudaGraphExec_t* exec = c->exec + base;
-  {  // BiLD (and small-only): WHILE { small pass ; IF { large block pass } ; IF { large single-row pass } }
+  if (c->graph_switch && c->draft_ahead && c->cfg.early_exit_layers == 0) {
+    CUDA_TRY(c, cudaGraphCreate(&graph[0], 0));
+    int rc = build_rounds(c, graph[0], per_pass, &per_pass_large1, &per_pass_large8);
+    if (rc) return rc;
+    CUDA_TRY(c, cudaGraphInstantiate(&exec[0], graph[0], 0));
+  } else {  // BiLD (and small-only): WHILE { small pass ; IF { large block pass } ; IF { large single-row pass } }
     CUDA_TRY(c, cudaGraphCreate(&graph[0], 0));
     cudaGraphConditionalHandle hw, hi, hi1, hi8 = 0;
     CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hw, graph[0], 1, cudaGraphCondAssignDefault));
@@ -1597,7 +1641,8 @@ int read_state(bild_ctx* c) {
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   {  // kernels launched by the loop graphs so far (the device counts the passes they ran)
     const long long* cp = c->pin_state->cum_passes;
-    const int64_t total = cp[0] * c->per_pass[0] + cp[1] * c->per_pass[1] + cp[2] * c->per_pass_large1 + cp[3] * c->per_pass_large8;
+    const int64_t total = cp[0] * c->per_pass[0] + cp[1] * c->per_pass[1] + cp[2] * c->per_pass_large1 + cp[3] * c->per_pass_large8 +
+                          c->pin_state->cum_rounds;
     c->launches += total - c->graph_counted;
     c->graph_counted = total;
     c->launches += c->pin_state->cum_draws - c->sampled_counted;
@@ -1714,6 +1759,7 @@ void bild_tuning_default(bild_tuning* t) {
   t->slice_min_kb = 3000; t->slice_mma_min = 3; t->slice_head = 2; t->slice_head_min_mb = 32; t->unit_attn = 1;
   t->umma = 1; t->enc_gemm = 1; t->enc_attn_mma = 1; t->enc_parallel = 1; t->spin_limit = 0; t->debug_skip_copies = 0;
   t->attn_all_keys = 128; t->graph_switch = 1; t->enc_split_k = 1; t->head_stream = 2; t->enc_attn_groups = EA_MAX_GROUPS;
+  t->draft_ahead = 1;
 }
 
 int bild_create(const bild_config* cfg, const bild_weights* small_w, const bild_weights* large_w, void* workspace,
@@ -1762,6 +1808,7 @@ int bild_create_tuned(const bild_config* cfg, const bild_weights* small_w, const
     c->graph_switch = t.graph_switch != 0;
     c->enc_split_k = t.enc_split_k != 0;
     c->head_stream = std::min(2, std::max(0, t.head_stream));
+    c->draft_ahead = t.draft_ahead != 0;
     c->enc_attn_groups = std::min(EA_MAX_GROUPS, std::max(1, t.enc_attn_groups));
   }
   {

@@ -37,6 +37,20 @@ struct HeadOut {
   int next_token;
 };
 
+// A block of drafts on its way to the large model, and what the small model's side looked like when it was handed over.
+struct DraftBlock {
+  int n;          // index of its last token
+  int proposed;   // the small model's candidate for n + 1
+  int last;       // 1: nothing is drafted behind it (end of sequence, max_len)
+  int slot;       // place of the large pass's record in the trace
+  int steps, fallbacks, forced, passes;   // counts to go back to if the drafts behind it do not stand
+};
+constexpr int BLOCK_RING = 8, TRUST_MAX = 3;   // (at most TRUST_MAX + 1 blocks are on their way)
+constexpr unsigned QUEUE_COUNT = 0xffffu;
+constexpr unsigned QUEUE_LARGE_IDLE = 1u << 16;   // no large pass is running or about to start
+constexpr unsigned QUEUE_SMALL_IDLE = 1u << 17;   // the small model has stopped
+constexpr unsigned QUEUE_DROP = 1u << 18;         // the last large pass ended otherwise than drafted: what is behind its block goes
+
 // Decode-loop state (Algorithm 1) kept on the device.
 struct DevState {
   int n;        // index of the last token of y
@@ -57,6 +71,13 @@ struct DevState {
   int pad1;
   long long cum_draws;       // token-drawing kernels run from the loop graphs since create
   long long cum_passes[4];   // passes run from the loop graphs since create: small, large block, large single row, large up to 8 rows
+  // Loop in rounds (round_step): the blocks of drafts handed to the large model, oldest first
+  DraftBlock block[BLOCK_RING];
+  unsigned block_head, block_tail;   // counted up by the large passes and by the small steps
+  unsigned queue;            // QUEUE_* flags, and the number of blocks handed over and not yet judged
+  int trust;                 // 0..TRUST_MAX, up when a large pass ends with the small model's candidate, down when it does not
+  int overrun;               // the loop was stopped by the guard on `passes`
+  long long cum_rounds;      // round_kernel launches since create
 };
 
 struct Partial {  // running soft-max statistics of a slice of the vocabulary

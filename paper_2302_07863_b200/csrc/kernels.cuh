@@ -346,14 +346,15 @@ struct LoopPtrs {
   CallDesc* descL;
 };
 
-__device__ inline void trace_add(const LoopPtrs& L, int kind, int pos, int token, int k, int m, float v) {
-  DevState* st = L.st;
-  const int i = st->n_trace++;
-  if (i < st->trace_cap) {
+__device__ inline void trace_put(const LoopPtrs& L, int i, int kind, int pos, int token, int k, int m, float v) {
+  if (i < L.st->trace_cap) {
     bild_trace_rec r;
     r.kind = kind; r.pos = pos; r.token = token; r.k = k; r.m = m; r.value = v;
     L.trace[i] = r;
   }
+}
+__device__ inline void trace_add(const LoopPtrs& L, int kind, int pos, int token, int k, int m, float v) {
+  trace_put(L, L.st->n_trace++, kind, pos, token, k, m, v);
 }
 
 __device__ inline void next_small(const LoopPtrs& L) {
@@ -365,15 +366,15 @@ __device__ inline void next_small(const LoopPtrs& L) {
   L.descS->targets[0] = -1;
 }
 
-__device__ inline void next_large(const LoopPtrs& L) {
+__device__ inline void next_large(const LoopPtrs& L, int n) {   // the tokens the large model has not seen, up to y[n]
   DevState* st = L.st;
-  const int k = st->n - st->L_len + 1;
+  const int k = n - st->L_len + 1;
   L.descL->k = k;
   L.descL->pos0 = st->L_len;
   L.descL->run_policy = 1;
   for (int i = 0; i < MAXB; ++i) {
-    L.descL->tokens[i] = i < k ? L.y[st->L_len + i] : 0;
-    L.descL->targets[i] = i < k - 1 ? L.y[st->L_len + i + 1] : -1;
+    L.descL->tokens[i] = i < k ? __ldcg(L.y + st->L_len + i) : 0;
+    L.descL->targets[i] = i < k - 1 ? __ldcg(L.y + st->L_len + i + 1) : -1;
   }
 }
 
@@ -396,15 +397,96 @@ __device__ inline void policy_tests(HeadOut* o, const CallDesc* desc, const DevS
   }
 }
 
-__device__ inline void policy_step(const LoopPtrs& L, const HeadOut* o, const CallDesc* desc, int which) {
+// ---- the loop in rounds ----
+// A round = [large passes | small steps] side by side, then round_kernel.  At a fallback the small model has a candidate for the position
+// too.  Most often the large pass ends with just that token and without a rollback, so the small model goes on from it while the pass is at
+// work: the block of drafts is handed over (block[], queue) and drafting continues.  A large pass that ends as proposed takes the next block,
+// if one is waiting; one that does not stops both sides, and round_step sets y, the caches, the trace and the counts back to
+// what the serial loop has after that pass.  Tokens, trace and counts are those of the serial loop in any case.
+// Neither side waits for the other inside a kernel: each leaves its WHILE node when it has nothing to do, which the flags in `queue`
+// tell the other, and the round ends when both have.
+// When it pays: T5 pair, five rows: a large pass takes 520 us, 650 with small steps beside it all the time, of which five are then done that
+// cost 82 us each by themselves; so a block that stands saves about 250 us, one that does not costs up to 130 and the wait for the
+// step at hand.  trust follows what the passes ended with, also while nothing is drafted ahead, and bounds the
+// number of blocks on their way: a pair that never agrees pays once a generation.
+
+// The small model's side at a fallback: hands its drafts over.
+__device__ inline void small_hands_over(const LoopPtrs& L, int candidate) {
+  DevState* st = L.st;
+  DraftBlock& b = st->block[st->block_tail++ % BLOCK_RING];
+  b.n = st->n; b.proposed = candidate;
+  b.last = st->n + 1 >= st->max_len || candidate == st->eos_id;
+  b.slot = st->n_trace++;
+  b.steps = st->stats.small_steps; b.fallbacks = st->stats.fallbacks; b.forced = st->stats.forced; b.passes = st->passes;
+  L.y[st->n + 1] = candidate;
+  __threadfence();
+  const unsigned q = atomicAdd(&st->queue, 1u);
+  const int waiting = (int)(q & QUEUE_COUNT) + 1;
+  // goes on unless a round is needed to start the large model, or enough blocks are on their way
+  if (!(q & (QUEUE_LARGE_IDLE | QUEUE_DROP)) && !b.last && waiting <= *(volatile int*)&st->trust) {
+    ++st->n;
+    st->drafts = 0;
+    next_small(L);
+  } else {
+    st->fallback = 1;
+    atomicOr(&st->queue, QUEUE_SMALL_IDLE);
+  }
+}
+
+// The end of a large pass in the loop in rounds (L_len, stats.large_calls, sum_k, rollbacks, discarded, trust: this side's only).
+// Returns whether the next block follows at once.
+__device__ inline bool large_settles(const LoopPtrs& L, const HeadOut* o, const CallDesc* desc) {
+  DevState* st = L.st;
+  const DraftBlock& b = st->block[st->block_head % BLOCK_RING];
+  const int proposed = __ldcg(&b.proposed), last = __ldcg(&b.last), slot = __ldcg(&b.slot);
+  const int k = desc->k, base = desc->pos0, mv = o->first_violation;
+  st->stats.large_calls++;
+  st->stats.sum_k += k;
+  const int j = base + (mv >= 0 ? mv + 1 : k), tok = o->argmax[mv >= 0 ? mv : k - 1];
+  if (mv >= 0) {            // rollback: drop y[j..], write the large model's token at j
+    st->stats.rollbacks++;
+    st->stats.discarded += base + k - j;
+    trace_put(L, slot, 4, j, tok, k, mv, o->d[mv]);
+  } else {
+    float dmax = 0.f;
+    for (int i = 0; i < k - 1; ++i) dmax = fmaxf(dmax, o->d[i]);
+    trace_put(L, slot, 3, j, tok, k, -1, dmax);
+  }
+  L.y[j] = tok;
+  st->L_len = j;
+  const bool stands = mv < 0 && tok == proposed;
+  st->trust = stands ? min(TRUST_MAX, st->trust + 1) : max(0, st->trust - 1);
+  if (!stands || last) {
+    __threadfence();
+    atomicOr(&st->queue, QUEUE_DROP | QUEUE_LARGE_IDLE);
+    return false;
+  }
+  st->block_head++;
+  // the next block at once while the small model is at work; else, or without one, this side stops and a new round begins
+  unsigned q = *(volatile unsigned*)&st->queue;
+  for (;;) {   // (at most as many turns as the small model changes the word meanwhile: one step's worth)
+    const bool more = (q & QUEUE_COUNT) > 1 && !(q & QUEUE_SMALL_IDLE);
+    const unsigned was = atomicCAS(&st->queue, q, more ? q - 1 : (q - 1) | QUEUE_LARGE_IDLE);
+    if (was == q) {
+      if (!more) return false;
+      __threadfence();
+      next_large(L, __ldcg(&st->block[st->block_head % BLOCK_RING].n));
+      return true;
+    }
+    q = was;
+  }
+}
+
+__device__ inline void policy_step(const LoopPtrs& L, const HeadOut* o, const CallDesc* desc, int which, bool rounds) {
   DevState* st = L.st;
   int* y = L.y;
   // Every pass adds a token or consumes a pending draft, so a run takes at most
   // (max_len + 1) * (max_draft + 2) passes; beyond that the loop is stopped with an error.
   if (++st->passes > (st->max_len + 1) * (st->max_draft + 2) + 8) {
     st->err = BILD_ERR_TIMEOUT;
-    st->done = 1;
+    st->done = st->overrun = 1;
     st->fallback = 0;
+    if (rounds) atomicOr(&st->queue, QUEUE_SMALL_IDLE);
     return;
   }
   if (which == 0) {
@@ -418,12 +500,17 @@ __device__ inline void policy_step(const LoopPtrs& L, const HeadOut* o, const Ca
       trace_add(L, 0, st->n, t, 0, -1, o->pmax);
       st->fallback = 0;
       st->done = (st->n >= st->max_len || t == st->eos_id) ? 1 : 0;
+      if (rounds && st->done) atomicOr(&st->queue, QUEUE_SMALL_IDLE);
       next_small(L);
     } else {
       if (confident) st->stats.forced++; else st->stats.fallbacks++;
       trace_add(L, confident ? 2 : 1, st->n + 1, t, 0, -1, o->pmax);
-      st->fallback = 1;
-      next_large(L);
+      if (rounds) {
+        small_hands_over(L, t);
+      } else {
+        st->fallback = 1;
+        next_large(L, st->n);
+      }
     }
   } else {
     const int k = desc->k, base = desc->pos0;
@@ -449,8 +536,58 @@ __device__ inline void policy_step(const LoopPtrs& L, const HeadOut* o, const Ca
     st->drafts = 0;
     st->fallback = 0;
     st->done = (st->n >= st->max_len || y[st->n] == st->eos_id) ? 1 : 0;
-    if (st->mode == BILD_MODE_LARGE_ONLY) next_large(L); else next_small(L);
+    if (st->mode == BILD_MODE_LARGE_ONLY) next_large(L, st->n); else next_small(L);
   }
+}
+
+// Between two rounds, both sides stopped, one thread.  rows: of the large pass to start (0: none); small: the small model goes on.
+__device__ inline void round_step(const LoopPtrs& L, int* rows, bool* small) {
+  DevState* st = L.st;
+  *rows = 0; *small = false;
+  st->cum_rounds++;
+  if (st->queue & QUEUE_DROP) {   // the serial loop's state behind the last large pass
+    const DraftBlock& b = st->block[st->block_head % BLOCK_RING];
+    st->n = st->S_len = st->L_len;
+    st->drafts = 0;
+    st->fallback = 0;
+    st->n_trace = b.slot + 1;
+    st->stats.small_steps = b.steps; st->stats.fallbacks = b.fallbacks; st->stats.forced = b.forced;
+    st->passes = b.passes;
+    st->done = (st->n >= st->max_len || L.y[st->n] == st->eos_id || st->overrun) ? 1 : 0;
+    st->block_head = st->block_tail;
+    st->queue = 0;
+    next_small(L);
+  }
+  const int waiting = (int)(st->queue & QUEUE_COUNT);
+  if (waiting > 0) {
+    next_large(L, st->block[st->block_head % BLOCK_RING].n);
+    *rows = L.descL->k;
+  }
+  if (!st->done) {
+    // at a fallback: on from the candidate if its block stands already, or ahead
+    if (!st->fallback) {
+      *small = true;
+    } else if (waiting == 0 || (waiting <= st->trust && !st->block[(st->block_tail - 1) % BLOCK_RING].last)) {
+      ++st->n;
+      st->drafts = 0;
+      st->fallback = 0;
+      next_small(L);
+      *small = true;
+    }
+  }
+  st->queue = (unsigned)waiting | (*rows ? 0u : QUEUE_LARGE_IDLE) | (*small ? 0u : QUEUE_SMALL_IDLE);
+}
+// nb bodies of the large passes' SWITCH node (their order: see HeadArgs); the value nb runs none
+__device__ inline unsigned large_body(int rows, int nb) { return rows == 1 ? 1u : nb == 3 && rows <= 8 ? 2u : 0u; }
+__global__ void round_kernel(LoopPtrs L, int nb, cudaGraphConditionalHandle go, cudaGraphConditionalHandle large, cudaGraphConditionalHandle body,
+                             cudaGraphConditionalHandle small) {
+  int rows;
+  bool steps;
+  round_step(L, &rows, &steps);
+  cudaGraphSetConditional(go, rows || steps ? 1u : 0u);
+  cudaGraphSetConditional(large, rows ? 1u : 0u);
+  cudaGraphSetConditional(body, large_body(rows, nb));
+  cudaGraphSetConditional(small, steps ? 1u : 0u);
 }
 
 // ---------------------------------------------------------------------------------
@@ -485,6 +622,8 @@ struct HeadArgs {
   // the pass over 2 to 8 rows; the value sw_bodies runs none
   unsigned long long cond_switch;
   int sw_bodies;
+  // loop in rounds (round_step): the WHILE node of this model's passes; cond_switch and sw_bodies are then set for the large model
+  unsigned long long cond_side;
   int pass_kind;                 // which pass counter the kernel bumps inside a loop graph: 0 small, 1 block, 2 single row, 3 up to 8 rows
   int defer_policy;              // sampling: the head leaves policy and loop control to the kernel that draws the token
   // single-step calls: pinned HOST memory the results are written to (five to fifty words over the bus, on their way while the
@@ -499,7 +638,22 @@ __device__ inline void policy_tail(const HeadArgs& a, HeadOut* o) {
   if (!a.loop.st) return;
   policy_tests(o, a.desc, a.loop.st, a.which);
   if (a.defer_policy) return;   // (the row the token is drawn from depends on the tests)
-  if (a.desc->run_policy) policy_step(a.loop, o, a.desc, a.which);
+  if (a.desc->run_policy) {
+    if (a.cond_side && a.which == 1) {
+      const bool more = large_settles(a.loop, o, a.desc);
+      a.loop.st->cum_passes[a.pass_kind]++;
+      cudaGraphSetConditional(a.cond_side, more ? 1u : 0u);
+      if (more) cudaGraphSetConditional(a.cond_switch, large_body(a.loop.descL->k, a.sw_bodies));
+      return;
+    }
+    policy_step(a.loop, o, a.desc, a.which, a.cond_side != 0);
+    if (a.cond_side) {
+      const DevState* st = a.loop.st;
+      a.loop.st->cum_passes[a.pass_kind]++;
+      cudaGraphSetConditional(a.cond_side, st->fallback || st->done || (*(const volatile unsigned*)&st->queue & QUEUE_DROP) ? 0u : 1u);
+      return;
+    }
+  }
   else if (a.which == 0) a.loop.st->S_len = a.desc->pos0 + 1;
   else a.loop.st->L_len = a.desc->pos0 + a.desc->k;
   if (a.host_head) {
@@ -725,9 +879,13 @@ __global__ void reset_state_kernel(LoopPtrs L, const int* enc_err, int mode, flo
   st->n_trace = 0; st->trace_cap = trace_cap;
   st->stats = bild_stats{0, 0, 0, 0, 0, 0, 0};
   st->passes = 0;
+  st->overrun = 0;
+  st->block_head = st->block_tail = 0;
+  st->queue = QUEUE_LARGE_IDLE;
+  st->trust = 1;
   L.y[0] = start_id;
   st->done = (max_len <= 0 || start_id == eos_id) ? 1 : 0;
-  if (mode == BILD_MODE_LARGE_ONLY) next_large(L); else next_small(L);
+  if (mode == BILD_MODE_LARGE_ONLY) next_large(L, st->n); else next_small(L);
 }
 
 }  // namespace bild

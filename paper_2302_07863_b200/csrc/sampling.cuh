@@ -300,7 +300,7 @@ nucleus_policy_kernel(HeadArgs a, const float* __restrict__ logits, const float*
   cluster_sync_all();   // the token is in rank 0; no block leaves while another may read its shared memory
   if (rank == 0 && tid == 0) {
     o->argmax[r] = sh.token;
-    if (a.cond_while) a.loop.st->cum_draws++;
+    if (a.cond_while || a.cond_side) atomicAdd((unsigned long long*)&a.loop.st->cum_draws, 1ull);   // (both models' at once)
     HeadArgs b = a;
     b.defer_policy = 0;
     policy_tail(b, o);

@@ -265,3 +265,57 @@ def test_new_context_takes_updated_weights(torch_cuda, name):
         assert np.max(np.abs(buf[:k].cpu().numpy() - z)) <= (1e-4 if wl.dtype == "fp32" else 2e-3) * max(1.0, np.max(np.abs(z)))
     old.close()
     new.close()
+
+
+@pytest.mark.parametrize("name,noise", [("tiny", 0.0), ("tiny", 0.03), ("tiny", None), ("tiny_bf16", 0.0), ("tiny_bf16", 0.03), ("wide_bf16", None)])
+@pytest.mark.parametrize("top_p", [0.0, 0.8])
+def test_drafting_ahead_is_the_serial_loop(torch_cuda, name, noise, top_p):
+    """The loop in rounds against the serial one (draft_ahead = 0): tokens, trace and counts.  The small model is the large one
+    (every large pass ends as proposed), the large one with `noise` on its weights (some do), or another model (hardly any does);
+    fallbacks from none to all, blocks from 1 row to the most, ends by length at the first places and by token anywhere."""
+    from paper_2302_07863_b200 import MODE_BILD, MODE_LARGE_ONLY, MODE_SMALL_ONLY
+    from paper_2302_07863_b200.binding import BF16, FP32, Config, Context, model_cfg, upload_model
+    wl = WORKLOADS[name]
+    sL = MODEL_SHAPES[wl.large]
+    wlarge = upload_model(gen_model(sL, wl.seed, wl.dtype), "cuda:0")
+    if noise is None:
+        sS = MODEL_SHAPES[wl.small]
+        wsmall = upload_model(gen_model(sS, wl.seed, wl.dtype), "cuda:0")
+    else:
+        import torch
+        torch.manual_seed(1)
+        sS, wsmall = sL, {k: (v.float() * (1 + noise * torch.randn_like(v.float()))).to(v.dtype) for k, v in wlarge.items()}
+    cap = 41
+    ids = np.random.default_rng(5).integers(2, sL.vocab, size=min(wl.enc_len, 32)).astype(np.int32)
+    u = np.random.default_rng(6).random((2, cap)).astype(np.float32)
+
+    def contexts(max_draft, eos):
+        cfg = Config(model_cfg(sS, 9.0), model_cfg(sL, 9.0), FP32 if wl.dtype == "fp32" else BF16, 32, cap, max_draft, 0, eos, 0)
+        out = [Context(cfg, sS, wsmall, sL, wlarge, tuning=t) for t in (None, dict(draft_ahead=0))]
+        for c in out:
+            c.encode(ids)
+        return out
+
+    def run(c, afb, arb, n, mode=MODE_BILD):
+        return c.generate_sampled(mode, afb, arb, n, top_p, u[0], u[1]) if top_p else c.generate(mode, afb, arb, n)
+
+    eos = -1
+    for max_draft in (10, 1, 4):
+        both = contexts(max_draft, eos)
+        r = run(both[1], 0.0, float("inf"), cap - 1)
+        p = sorted(t[5] for t in r["trace"] if t[0] != 3)
+        for q in (0.0, 0.2, 0.5, 1.1):   # share of the small model's steps that fall back (roughly: a run takes its own course)
+            i = int(q * len(p))
+            afb = 0.0 if i == 0 else 2.0 if i >= len(p) else (p[i - 1] + p[i]) / 2
+            for arb in (1.0, 6.0):
+                for n in (cap - 1,) if q != 0.5 else (1, 2, 3, 7, cap - 1):
+                    want, got = run(both[1], afb, arb, n), run(both[0], afb, arb, n)
+                    assert got["tokens"] == want["tokens"] and got["stats"] == want["stats"], (max_draft, q, arb, n)
+                    assert [t[:5] for t in got["trace"]] == [t[:5] for t in want["trace"]]
+                    # (fused sub-layers add partial sums in no fixed order: the last bits differ from run to run)
+                    assert np.allclose([t[5] for t in got["trace"]], [t[5] for t in want["trace"]], rtol=1e-4, atol=1e-5)
+        for mode in (MODE_SMALL_ONLY, MODE_LARGE_ONLY):
+            assert run(both[0], 0.4, 1.0, cap - 1, mode)["tokens"] == run(both[1], 0.4, 1.0, cap - 1, mode)["tokens"]
+        eos = want["tokens"][len(want["tokens"]) // 2] if max_draft == 10 else want["tokens"][-1]   # the next contexts end on it
+        for c in both:
+            c.close()
