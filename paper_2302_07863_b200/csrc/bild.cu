@@ -779,12 +779,26 @@ int setup_fused(bild_ctx* c, Model& m) {
   // attention kernel's in front and their weights arrive in its shadow (gated slices of 24 rows: 148 KB, of 16 rows: 112 KB; mT5-large,
   // 5 rows: a pass of two 642 -> 600 us, of five 642 -> 637, of sixteen 1033 -> 912)
   m.sub_grid[0] = m.sub_grid[1] = c->sms;
-  if (parts == 1 && ffn_sub_layout(d, F, gated, c->sms, c->sms, SUB_MB).total > SUB_HALF_SM)
-    for (int rows = ffn_sub_rows(F, c->sms) - 8; rows >= 8; rows -= 8) {
-      const int grid = (F + rows - 1) / rows;
-      if (grid > 2 * c->sms) break;
-      if (ffn_sub_layout(d, F, gated, grid, grid, SUB_MB).total <= SUB_HALF_SM) { m.sub_grid[1] = grid; break; }
-    }
+  if (parts == 1) {
+    const int units = F / 8, q0 = (units + c->sms - 1) / c->sms;   // slices are whole units of 8 rows
+    // no more blocks than the largest slice leaves work for: every block adds to all d outputs at the L2 and takes a place on an SM
+    // (T5-large, 512 units, 148 -> 128 blocks: 2 rows 479 -> 471 us, 5 rows 522 -> 507, 16 rows 760 -> 750)
+    m.sub_grid[1] = (units + q0 - 1) / q0;
+    if (ffn_sub_layout(d, F, gated, m.sub_grid[1], m.sub_grid[1], SUB_MB).total > SUB_HALF_SM)
+      for (int rows = 8 * q0 - 8; rows >= 8; rows -= 8) {
+        const int grid = (F + rows - 1) / rows;
+        if (grid > 2 * c->sms) break;
+        if (ffn_sub_layout(d, F, gated, grid, grid, SUB_MB).total <= SUB_HALF_SM) { m.sub_grid[1] = grid; break; }
+      }
+    // single rows: slices up to the 32 weight rows a block keeps in registers, down to 64 blocks (mT5-small, 128 units of a gated
+    // pair of matrices: 148 blocks 137 us a step, 128 137, 64 123, 43 126; T5-small, 256 units: 148 blocks 81.8, 128 80.1, 86 79.5, 64 79.8;
+    // and fewer blocks are in the way of a large pass beside them, round_step: T5 pair 655 -> 648 us a pass of 5 rows)
+    const int q = std::max(q0, std::min(4 / nmat, units / 64));
+    // (ungated slices that are that large anyway: one block per SM, 128 or 148 blocks of T5-large 338 and 341 us at 512 encoder ids, 402 and
+    // 391 at 1024)
+    m.sub_grid[0] = q == q0 && !gated ? c->sms : (units + q - 1) / q;
+    if (ffn_sub_layout(d, F, gated, m.sub_grid[0], m.sub_grid[0], 1).total > SUB_HALF_SM) m.sub_grid[0] = (units + q0 - 1) / q0;
+  }
   m.sub_C = C; m.sub_parts = parts;
   for (int v = 0; v < 2; ++v) { m.sub_self[v] = ps[v]; m.sub_cross[v] = pc[v]; }
   m.fused = true;
@@ -928,11 +942,10 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   f.Wfo1 = m.wfo_one + (size_t)l * (Fd / 8) * d; f.Wfo8 = m.wfo_blk + (size_t)l * (Fd / 8) * pack_wfo_dpad(d);
   f.nparts = m.sub_parts;
   // Single rows: ahead of the dependency wait, so that the next layer's first kernel, whose prologue is longer than this whole kernel, takes
-  // the SMs the kernel in front leaves (T5-large 351 -> 338 us, T5-small 81.4 -> 80.0, mT5-small 135 -> 133); not for gated slices of more
-  // than 512 columns, whose own weights would wait for it (mT5-large 408 us behind the wait, 429 ahead).  Blocks: as a.early, except for
+  // the SMs the kernel in front leaves (T5-large 351 -> 338 us, T5-small 81.4 -> 80.0, mT5-small 126 -> 123, mT5-large 417 -> 406).  Blocks: as a.early, except for
   // gated ones of up to 8 rows (mT5-large, 5 rows 579 us at once, 594 behind the rows; two chunks side by side, 16 rows: 903 at once, 842
   // behind; T5-large, 2 rows: 478, 468).
-  f.early = MB == 1 ? (gated && d > 512 ? 1 : 2) : d <= 512 || (gated && desc == m.desc) ? 1 : 0;
+  f.early = MB == 1 ? 2 : d <= 512 || (gated && desc == m.desc) ? 1 : 0;
   const int grid = m.sub_grid[MB == 1 ? 0 : 1];
   f.L = ffn_sub_layout(d, Fd, gated, grid * m.sub_parts, grid, MB);
   for (int p = 0; p < m.sub_parts; ++p) {
