@@ -586,8 +586,7 @@ constexpr int HEAD1_THREADS = 256;
 template <typename WT, int NCH, int RPW>   // NCH chunks of 256 columns per row, RPW rows per warp
 __global__ void __launch_bounds__(HEAD1_THREADS) head1_kernel(HeadArgs a) {
   constexpr int NW = HEAD1_THREADS / 32;
-  __shared__ Partial s_p[HEAD1_THREADS];
-  __shared__ int s_last;
+  __shared__ Partial s_p[NW];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int K = a.K, V = a.V;
   const int n0 = (blockIdx.x * NW + warp) * RPW;
@@ -651,54 +650,7 @@ __global__ void __launch_bounds__(HEAD1_THREADS) head1_kernel(HeadArgs a) {
     }
   }
   if (lane == 0) s_p[warp] = run;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Partial p = s_p[0];
-    for (int w2 = 1; w2 < NW; ++w2) p = combine(p, s_p[w2]);
-    a.partials[blockIdx.x] = p;
-    __threadfence();
-    const unsigned t = atomicAdd(a.counter, 1u);
-    s_last = (t == gridDim.x - 1);
-    if (s_last) *a.counter = 0;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  // merge: every thread requests its partials together, then combines them in index order
-  {
-    Partial q[8];
-    const int nb = (int)gridDim.x;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int b = threadIdx.x + j * HEAD1_THREADS;
-      q[j].m = -INFINITY; q[j].s = 0.f; q[j].idx = 0x7fffffff;
-      if (b < nb) { q[j].m = __ldcg(&a.partials[b].m); q[j].s = __ldcg(&a.partials[b].s); q[j].idx = __ldcg(&a.partials[b].idx); }
-    }
-    Partial p = q[0];
-#pragma unroll
-    for (int j = 1; j < 8; ++j) p = combine(p, q[j]);
-    for (int b = threadIdx.x + 8 * HEAD1_THREADS; b < nb; b += HEAD1_THREADS) {   // very large vocabularies
-      Partial t2;
-      t2.m = __ldcg(&a.partials[b].m); t2.s = __ldcg(&a.partials[b].s); t2.idx = __ldcg(&a.partials[b].idx);
-      p = combine(p, t2);
-    }
-    s_p[threadIdx.x] = p;
-  }
-  __syncthreads();
-  for (int stride = HEAD1_THREADS / 2; stride > 0; stride >>= 1) {
-    if (threadIdx.x < stride) s_p[threadIdx.x] = combine(s_p[threadIdx.x], s_p[threadIdx.x + stride]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const Partial p = s_p[0];
-    HeadOut* o = a.out;
-    o->argmax[0] = p.idx;
-    o->zmax[0] = p.m;
-    o->lse[0] = p.m + logf(p.s);
-    o->pmax = 1.f / p.s;
-    o->gather[0] = __ldcg(&o->gather[0]);
-    policy_tail(a, o);
-  }
+  head_row_end(a, s_p, NW);
 }
 
 // ---------------------------------------------------------------------------------
@@ -713,8 +665,7 @@ __global__ void __launch_bounds__(HEAD1_THREADS) head1_kernel(HeadArgs a) {
 template <int NCH, int R>   // NCH chunks of 256 columns per row, R rows per batch
 __global__ void __launch_bounds__(HEAD1_THREADS, 2) head_stream_kernel(HeadArgs a) {
   constexpr int NW = HEAD1_THREADS / 32, SH = R == 8 ? 2 : R == 4 ? 3 : 4;   // lane >> SH: the row of the batch this lane ends up with
-  __shared__ Partial s_p[HEAD1_THREADS];
-  __shared__ int s_last;
+  __shared__ Partial s_p[NW];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int K = a.K, V = a.V;
   const int tw = gridDim.x * NW, gw = blockIdx.x * NW + warp;
@@ -806,44 +757,7 @@ __global__ void __launch_bounds__(HEAD1_THREADS, 2) head_stream_kernel(HeadArgs 
     run = ((lane & o) == 0) ? combine(run, q) : combine(q, run);
   }
   if (lane == 0) s_p[warp] = run;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    Partial p = s_p[0];
-    for (int w2 = 1; w2 < NW; ++w2) p = combine(p, s_p[w2]);
-    a.partials[blockIdx.x] = p;
-    __threadfence();
-    const unsigned t = atomicAdd(a.counter, 1u);
-    s_last = (t == gridDim.x - 1);
-    if (s_last) *a.counter = 0;
-  }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  {   // merge: the grid has at most two blocks per SM, one partial each
-    Partial p;
-    p.m = -INFINITY; p.s = 0.f; p.idx = 0x7fffffff;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += HEAD1_THREADS) {
-      Partial t2;
-      t2.m = __ldcg(&a.partials[b].m); t2.s = __ldcg(&a.partials[b].s); t2.idx = __ldcg(&a.partials[b].idx);
-      p = combine(p, t2);
-    }
-    s_p[threadIdx.x] = p;
-  }
-  __syncthreads();
-  for (int stride = HEAD1_THREADS / 2; stride > 0; stride >>= 1) {
-    if (threadIdx.x < stride) s_p[threadIdx.x] = combine(s_p[threadIdx.x], s_p[threadIdx.x + stride]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    const Partial p = s_p[0];
-    HeadOut* o = a.out;
-    o->argmax[0] = p.idx;
-    o->zmax[0] = p.m;
-    o->lse[0] = p.m + logf(p.s);
-    o->pmax = 1.f / p.s;
-    o->gather[0] = __ldcg(&o->gather[0]);
-    policy_tail(a, o);
-  }
+  head_row_end(a, s_p, NW);
 }
 
 // ---------------------------------------------------------------------------------

@@ -346,55 +346,98 @@ struct LoopPtrs {
   CallDesc* descL;
 };
 
-__device__ inline void trace_put(const LoopPtrs& L, int i, int kind, int pos, int token, int k, int m, float v) {
-  if (i < L.st->trace_cap) {
+// What the policy of a pass reads of the state, in one go: the loads of one thread then share a trip to the L2 (read where they were used,
+// between its stores, they were a dozen trips: 2.6 us behind a small step of the T5 pair, 6 to 13 while the other model's kernels load the
+// memory system).  The head kernels issue them ahead of the merge of their partial results.
+struct PolicyIn {
+  float alpha_fb, alpha_rb;
+  int k, pos0, run_policy;
+  int n, drafts, mode, max_len, max_draft, eos_id, n_trace, trace_cap, passes, trust;
+  unsigned block_head, block_tail;
+  bild_stats stats;
+  long long cum_passes;
+};
+__device__ inline PolicyIn policy_in(const DevState* st, const CallDesc* desc, int pass_kind) {
+  PolicyIn p;
+  p.alpha_fb = st->alpha_fb; p.alpha_rb = st->alpha_rb;
+  p.k = desc->k; p.pos0 = desc->pos0; p.run_policy = desc->run_policy;
+  p.n = st->n; p.drafts = st->drafts; p.mode = st->mode; p.max_len = st->max_len; p.max_draft = st->max_draft;
+  p.eos_id = st->eos_id; p.n_trace = st->n_trace; p.trace_cap = st->trace_cap; p.passes = st->passes; p.trust = st->trust;
+  p.block_head = st->block_head; p.block_tail = st->block_tail;
+  p.stats = st->stats;
+  p.cum_passes = st->cum_passes[pass_kind];
+  return p;
+}
+// What a pass came to.
+struct PolicyOut {
+  int token;           // arg max of the row that counts (block pass: of the first violation, else of the last row)
+  float pmax;          // small model: its confidence
+  int fallback;
+  int mv;              // block pass: first violation of Eq. 3 or -1, its distance, the largest distance
+  float d_mv, d_max;
+  int after;           // what the policy decided: small model: 1 it goes on; block pass in rounds: rows of the pass that follows at once
+};
+
+__device__ inline void trace_put(const LoopPtrs& L, int cap, int i, int kind, int pos, int token, int k, int m, float v) {
+  if (i < cap) {
     bild_trace_rec r;
     r.kind = kind; r.pos = pos; r.token = token; r.k = k; r.m = m; r.value = v;
     L.trace[i] = r;
   }
 }
-__device__ inline void trace_add(const LoopPtrs& L, int kind, int pos, int token, int k, int m, float v) {
-  trace_put(L, L.st->n_trace++, kind, pos, token, k, m, v);
-}
 
-__device__ inline void next_small(const LoopPtrs& L) {
-  DevState* st = L.st;
+__device__ inline void next_small(const LoopPtrs& L, int pos, int token) {
   L.descS->k = 1;
-  L.descS->pos0 = st->S_len;
+  L.descS->pos0 = pos;
   L.descS->run_policy = 1;
-  L.descS->tokens[0] = L.y[st->n];
+  L.descS->tokens[0] = token;
   L.descS->targets[0] = -1;
 }
 
-__device__ inline void next_large(const LoopPtrs& L, int n) {   // the tokens the large model has not seen, up to y[n]
-  DevState* st = L.st;
-  const int k = n - st->L_len + 1;
+__device__ inline int next_large(const LoopPtrs& L, int len, int n) {   // the tokens the large model has not seen: y[len] to y[n]
+  const int k = n - len + 1;
+  int t[MAXB + 1];
+#pragma unroll
+  for (int i = 0; i <= MAXB; ++i) t[i] = i < k ? __ldcg(L.y + len + i) : -1;
   L.descL->k = k;
-  L.descL->pos0 = st->L_len;
+  L.descL->pos0 = len;
   L.descL->run_policy = 1;
+#pragma unroll
   for (int i = 0; i < MAXB; ++i) {
-    L.descL->tokens[i] = i < k ? __ldcg(L.y + st->L_len + i) : 0;
-    L.descL->targets[i] = i < k - 1 ? __ldcg(L.y + st->L_len + i + 1) : -1;
+    L.descL->tokens[i] = i < k ? t[i] : 0;
+    L.descL->targets[i] = t[i + 1];
   }
+  return k;
 }
 
-// Tests of Sections 3.3 / 3.4 on the head's per-row results (always run).
-__device__ inline void policy_tests(HeadOut* o, const CallDesc* desc, const DevState* st, int which) {
+// Tests of Sections 3.3 / 3.4 on the head's per-row results (always run).  token, pmax: of row 0 (what counts for the small model).
+__device__ inline PolicyOut policy_tests(HeadOut* o, const PolicyIn& p, int which, int token, float pmax) {
+  PolicyOut r;
+  r.mv = -1; r.d_mv = 0.f; r.d_max = 0.f; r.pmax = pmax; r.token = token; r.fallback = 0; r.after = 0;
   if (which == 0) {
-    o->fallback = (o->pmax < st->alpha_fb) ? 1 : 0;   // fallback iff p_max < alpha_FB
-    o->first_violation = -1;
-    o->next_token = o->argmax[0];
-  } else {
-    const int k = desc->k;
-    int mv = -1;
-    for (int i = 0; i < k - 1; ++i) {
-      o->d[i] = o->lse[i] - o->gather[i];             // -ln p_L(drafted token)
-      if (mv < 0 && o->d[i] > st->alpha_rb) mv = i;   // first violation of Eq. 3
+    r.fallback = pmax < p.alpha_fb ? 1 : 0;   // fallback iff p_max < alpha_FB
+  } else if (p.k > 1) {
+    const int k = p.k;
+    float d[MAXB];
+    int am[MAXB];
+#pragma unroll
+    for (int i = 0; i < MAXB; ++i)
+      if (i < k) { d[i] = o->lse[i] - o->gather[i]; am[i] = o->argmax[i]; }
+#pragma unroll
+    for (int i = 0; i < MAXB; ++i) {
+      if (i < k - 1) {
+        o->d[i] = d[i];                       // -ln p_L(drafted token)
+        r.d_max = fmaxf(r.d_max, d[i]);
+        if (r.mv < 0 && d[i] > p.alpha_rb) { r.mv = i; r.d_mv = d[i]; r.token = am[i]; }   // first violation of Eq. 3
+      } else if (i == k - 1 && r.mv < 0) {
+        r.token = am[i];
+      }
     }
-    o->first_violation = mv;
-    o->next_token = o->argmax[mv >= 0 ? mv : k - 1];
-    o->fallback = 0;
   }
+  o->fallback = r.fallback;
+  o->first_violation = r.mv;
+  o->next_token = r.token;
+  return r;
 }
 
 // ---- the loop in rounds ----
@@ -410,133 +453,145 @@ __device__ inline void policy_tests(HeadOut* o, const CallDesc* desc, const DevS
 // step at hand.  trust follows what the passes ended with, also while nothing is drafted ahead, and bounds the
 // number of blocks on their way: a pair that never agrees pays once a generation.
 
-// The small model's side at a fallback: hands its drafts over.
-__device__ inline void small_hands_over(const LoopPtrs& L, int candidate) {
+// The small model's side at a fallback: hands its drafts over.  Returns whether it goes on.
+__device__ inline bool small_hands_over(const LoopPtrs& L, const PolicyIn& p, int steps, int fallbacks, int forced, int candidate) {
   DevState* st = L.st;
-  DraftBlock& b = st->block[st->block_tail++ % BLOCK_RING];
-  b.n = st->n; b.proposed = candidate;
-  b.last = st->n + 1 >= st->max_len || candidate == st->eos_id;
-  b.slot = st->n_trace++;
-  b.steps = st->stats.small_steps; b.fallbacks = st->stats.fallbacks; b.forced = st->stats.forced; b.passes = st->passes;
-  L.y[st->n + 1] = candidate;
+  DraftBlock& b = st->block[p.block_tail % BLOCK_RING];
+  st->block_tail = p.block_tail + 1;
+  const bool last = p.n + 1 >= p.max_len || candidate == p.eos_id;
+  b.n = p.n; b.proposed = candidate; b.last = last;
+  b.slot = p.n_trace + 1;   // (behind the record of this fallback)
+  st->n_trace = p.n_trace + 2;
+  b.steps = steps; b.fallbacks = fallbacks; b.forced = forced; b.passes = p.passes + 1;
+  L.y[p.n + 1] = candidate;
   __threadfence();
   const unsigned q = atomicAdd(&st->queue, 1u);
   const int waiting = (int)(q & QUEUE_COUNT) + 1;
   // goes on unless a round is needed to start the large model, or enough blocks are on their way
-  if (!(q & (QUEUE_LARGE_IDLE | QUEUE_DROP)) && !b.last && waiting <= *(volatile int*)&st->trust) {
-    ++st->n;
+  if (!(q & (QUEUE_LARGE_IDLE | QUEUE_DROP)) && !last && waiting <= *(volatile int*)&st->trust) {
+    st->n = p.n + 1;
     st->drafts = 0;
-    next_small(L);
-  } else {
-    st->fallback = 1;
-    atomicOr(&st->queue, QUEUE_SMALL_IDLE);
+    next_small(L, p.pos0 + 1, candidate);
+    return true;
   }
+  st->fallback = 1;
+  atomicOr(&st->queue, QUEUE_SMALL_IDLE);
+  return false;
 }
 
-// The end of a large pass in the loop in rounds (L_len, stats.large_calls, sum_k, rollbacks, discarded, trust: this side's only).
-// Returns whether the next block follows at once.
-__device__ inline bool large_settles(const LoopPtrs& L, const HeadOut* o, const CallDesc* desc) {
+// The end of a large pass in the loop in rounds (L_len, block_head, trust and the counts of large calls, rows, rollbacks and dropped tokens
+// are this side's only).  Returns the rows of the block that follows at once, 0 if none does.
+__device__ inline int large_settles(const LoopPtrs& L, const PolicyIn& p, const PolicyOut& o) {
   DevState* st = L.st;
-  const DraftBlock& b = st->block[st->block_head % BLOCK_RING];
+  const DraftBlock& b = st->block[p.block_head % BLOCK_RING];
   const int proposed = __ldcg(&b.proposed), last = __ldcg(&b.last), slot = __ldcg(&b.slot);
-  const int k = desc->k, base = desc->pos0, mv = o->first_violation;
-  st->stats.large_calls++;
-  st->stats.sum_k += k;
-  const int j = base + (mv >= 0 ? mv + 1 : k), tok = o->argmax[mv >= 0 ? mv : k - 1];
-  if (mv >= 0) {            // rollback: drop y[j..], write the large model's token at j
-    st->stats.rollbacks++;
-    st->stats.discarded += base + k - j;
-    trace_put(L, slot, 4, j, tok, k, mv, o->d[mv]);
-  } else {
-    float dmax = 0.f;
-    for (int i = 0; i < k - 1; ++i) dmax = fmaxf(dmax, o->d[i]);
-    trace_put(L, slot, 3, j, tok, k, -1, dmax);
-  }
-  L.y[j] = tok;
-  st->L_len = j;
-  const bool stands = mv < 0 && tok == proposed;
-  st->trust = stands ? min(TRUST_MAX, st->trust + 1) : max(0, st->trust - 1);
-  if (!stands || last) {
-    __threadfence();
-    atomicOr(&st->queue, QUEUE_DROP | QUEUE_LARGE_IDLE);
-    return false;
-  }
-  st->block_head++;
-  // the next block at once while the small model is at work; else, or without one, this side stops and a new round begins
   unsigned q = *(volatile unsigned*)&st->queue;
-  for (;;) {   // (at most as many turns as the small model changes the word meanwhile: one step's worth)
+  const int j = p.pos0 + (o.mv >= 0 ? o.mv + 1 : p.k);
+  st->stats.large_calls = p.stats.large_calls + 1;
+  st->stats.sum_k = p.stats.sum_k + p.k;
+  if (o.mv >= 0) {          // rollback: drop y[j..], write the large model's token at j
+    st->stats.rollbacks = p.stats.rollbacks + 1;
+    st->stats.discarded = p.stats.discarded + p.pos0 + p.k - j;
+    trace_put(L, p.trace_cap, slot, 4, j, o.token, p.k, o.mv, o.d_mv);
+  } else {
+    trace_put(L, p.trace_cap, slot, 3, j, o.token, p.k, -1, o.d_max);
+  }
+  L.y[j] = o.token;
+  st->L_len = j;
+  const bool stands = o.mv < 0 && o.token == proposed;
+  st->trust = stands ? min(TRUST_MAX, p.trust + 1) : max(0, p.trust - 1);
+  if (!stands || last) {
+    atomicOr(&st->queue, QUEUE_DROP | QUEUE_LARGE_IDLE);
+    return 0;
+  }
+  st->block_head = p.block_head + 1;
+  // the next block at once while the small model is at work; else, or without one, this side stops and a new round begins
+  for (;;) {   // (a turn fails only because the small model has changed the word: it hands over at most TRUST_MAX blocks)
     const bool more = (q & QUEUE_COUNT) > 1 && !(q & QUEUE_SMALL_IDLE);
     const unsigned was = atomicCAS(&st->queue, q, more ? q - 1 : (q - 1) | QUEUE_LARGE_IDLE);
     if (was == q) {
-      if (!more) return false;
+      if (!more) return 0;
       __threadfence();
-      next_large(L, __ldcg(&st->block[st->block_head % BLOCK_RING].n));
-      return true;
+      return next_large(L, j, __ldcg(&st->block[(p.block_head + 1) % BLOCK_RING].n));
     }
     q = was;
   }
 }
 
-__device__ inline void policy_step(const LoopPtrs& L, const HeadOut* o, const CallDesc* desc, int which, bool rounds) {
+// Bookkeeping of a pass in the serial loop, and of a small step in rounds.
+__device__ inline void policy_step(const LoopPtrs& L, const PolicyIn& p, PolicyOut& o, int which, bool rounds) {
   DevState* st = L.st;
   int* y = L.y;
   // Every pass adds a token or consumes a pending draft, so a run takes at most
   // (max_len + 1) * (max_draft + 2) passes; beyond that the loop is stopped with an error.
-  if (++st->passes > (st->max_len + 1) * (st->max_draft + 2) + 8) {
+  st->passes = p.passes + 1;
+  if (p.passes + 1 > (p.max_len + 1) * (p.max_draft + 2) + 8) {
     st->err = BILD_ERR_TIMEOUT;
     st->done = st->overrun = 1;
-    st->fallback = 0;
+    st->fallback = o.fallback = o.after = 0;
     if (rounds) atomicOr(&st->queue, QUEUE_SMALL_IDLE);
     return;
   }
   if (which == 0) {
-    const int t = o->argmax[0];
-    st->stats.small_steps++;
-    st->S_len = desc->pos0 + 1;
-    const bool confident = !o->fallback;
-    if (st->mode == BILD_MODE_SMALL_ONLY || (confident && st->drafts < st->max_draft)) {
-      y[++st->n] = t;
-      st->drafts++;
-      trace_add(L, 0, st->n, t, 0, -1, o->pmax);
+    const int steps = p.stats.small_steps + 1;
+    st->stats.small_steps = steps;
+    st->S_len = p.pos0 + 1;
+    const bool confident = !o.fallback;
+    if (p.mode == BILD_MODE_SMALL_ONLY || (confident && p.drafts < p.max_draft)) {
+      const int n = p.n + 1;
+      y[n] = o.token;
+      st->n = n;
+      st->drafts = p.drafts + 1;
+      trace_put(L, p.trace_cap, p.n_trace, 0, n, o.token, 0, -1, o.pmax);
+      st->n_trace = p.n_trace + 1;
       st->fallback = 0;
-      st->done = (st->n >= st->max_len || t == st->eos_id) ? 1 : 0;
-      if (rounds && st->done) atomicOr(&st->queue, QUEUE_SMALL_IDLE);
-      next_small(L);
+      const bool done = n >= p.max_len || o.token == p.eos_id;
+      st->done = done;
+      if (rounds && done) atomicOr(&st->queue, QUEUE_SMALL_IDLE);
+      next_small(L, p.pos0 + 1, o.token);
+      o.after = !done;
+      o.fallback = 0;   // (of the loop: the small model alone takes every token)
     } else {
-      if (confident) st->stats.forced++; else st->stats.fallbacks++;
-      trace_add(L, confident ? 2 : 1, st->n + 1, t, 0, -1, o->pmax);
+      const int fallbacks = p.stats.fallbacks + (confident ? 0 : 1), forced = p.stats.forced + (confident ? 1 : 0);
+      st->stats.fallbacks = fallbacks; st->stats.forced = forced;
+      trace_put(L, p.trace_cap, p.n_trace, confident ? 2 : 1, p.n + 1, o.token, 0, -1, o.pmax);
       if (rounds) {
-        small_hands_over(L, t);
+        o.after = small_hands_over(L, p, steps, fallbacks, forced, o.token);
       } else {
+        st->n_trace = p.n_trace + 1;
         st->fallback = 1;
-        next_large(L, st->n);
+        o.fallback = 1;
+        o.after = next_large(L, st->L_len, p.n);
       }
     }
   } else {
-    const int k = desc->k, base = desc->pos0;
-    st->stats.large_calls++;
-    st->stats.sum_k += k;
-    const int mv = o->first_violation;
-    if (mv >= 0) {            // rollback: drop y[j..], write the large model's token at j
-      const int j = base + mv + 1;
-      st->stats.rollbacks++;
-      st->stats.discarded += st->n - j + 1;
-      y[j] = o->argmax[mv];
-      st->n = j;
+    st->stats.large_calls = p.stats.large_calls + 1;
+    st->stats.sum_k = p.stats.sum_k + p.k;
+    int j;
+    if (o.mv >= 0) {          // rollback: drop y[j..], write the large model's token at j
+      j = p.pos0 + o.mv + 1;
+      st->stats.rollbacks = p.stats.rollbacks + 1;
+      st->stats.discarded = p.stats.discarded + p.n - j + 1;
       st->S_len = j;
-      st->L_len = j;
-      trace_add(L, 4, j, y[j], k, mv, o->d[mv]);
+      trace_put(L, p.trace_cap, p.n_trace, 4, j, o.token, p.k, o.mv, o.d_mv);
     } else {
-      float dmax = 0.f;
-      for (int i = 0; i < k - 1; ++i) dmax = fmaxf(dmax, o->d[i]);
-      y[++st->n] = o->argmax[k - 1];
-      st->L_len = st->n;
-      trace_add(L, 3, st->n, y[st->n], k, -1, dmax);
+      j = p.n + 1;
+      trace_put(L, p.trace_cap, p.n_trace, 3, j, o.token, p.k, -1, o.d_max);
     }
+    y[j] = o.token;
+    st->n = st->L_len = j;
+    st->n_trace = p.n_trace + 1;
     st->drafts = 0;
     st->fallback = 0;
-    st->done = (st->n >= st->max_len || y[st->n] == st->eos_id) ? 1 : 0;
-    if (st->mode == BILD_MODE_LARGE_ONLY) next_large(L, st->n); else next_small(L);
+    const bool done = j >= p.max_len || o.token == p.eos_id;
+    st->done = done;
+    o.after = !done;
+    if (p.mode != BILD_MODE_LARGE_ONLY) {
+      next_small(L, j, o.token);
+    } else {   // (every pass of that loop has one row: the other places of the descriptor stay as reset_state_kernel left them)
+      L.descL->pos0 = j;
+      L.descL->tokens[0] = o.token;
+    }
   }
 }
 
@@ -556,12 +611,11 @@ __device__ inline void round_step(const LoopPtrs& L, int* rows, bool* small) {
     st->done = (st->n >= st->max_len || L.y[st->n] == st->eos_id || st->overrun) ? 1 : 0;
     st->block_head = st->block_tail;
     st->queue = 0;
-    next_small(L);
+    next_small(L, st->n, L.y[st->n]);
   }
   const int waiting = (int)(st->queue & QUEUE_COUNT);
   if (waiting > 0) {
-    next_large(L, st->block[st->block_head % BLOCK_RING].n);
-    *rows = L.descL->k;
+    *rows = next_large(L, st->L_len, st->block[st->block_head % BLOCK_RING].n);
   }
   if (!st->done) {
     // at a fallback: on from the candidate if its block stands already, or ahead
@@ -571,7 +625,7 @@ __device__ inline void round_step(const LoopPtrs& L, int* rows, bool* small) {
       ++st->n;
       st->drafts = 0;
       st->fallback = 0;
-      next_small(L);
+      next_small(L, st->n, L.y[st->n]);
       *small = true;
     }
   }
@@ -633,52 +687,123 @@ struct HeadArgs {
 };
 
 // What the last block of every LM-head kernel does once the per-row results are complete: the policy tests, the
-// bookkeeping of Algorithm 1, and (inside a loop graph) the choice of what runs next.
-__device__ inline void policy_tail(const HeadArgs& a, HeadOut* o) {
-  if (!a.loop.st) return;
-  policy_tests(o, a.desc, a.loop.st, a.which);
+// bookkeeping of Algorithm 1, and (inside a loop graph) the choice of what runs next.  p: policy_in; token, pmax: of row 0.
+__device__ inline void policy_tail(const HeadArgs& a, HeadOut* o, const PolicyIn& p, int token, float pmax) {
+  DevState* st = a.loop.st;
+  if (!st) return;
+  PolicyOut r = policy_tests(o, p, a.which, token, pmax);
   if (a.defer_policy) return;   // (the row the token is drawn from depends on the tests)
-  if (a.desc->run_policy) {
-    if (a.cond_side && a.which == 1) {
-      const bool more = large_settles(a.loop, o, a.desc);
-      a.loop.st->cum_passes[a.pass_kind]++;
-      cudaGraphSetConditional(a.cond_side, more ? 1u : 0u);
-      if (more) cudaGraphSetConditional(a.cond_switch, large_body(a.loop.descL->k, a.sw_bodies));
-      return;
+  if (a.cond_side) {            // loop in rounds
+    st->cum_passes[a.pass_kind] = p.cum_passes + 1;
+    if (a.which == 0) {
+      policy_step(a.loop, p, r, 0, true);
+      cudaGraphSetConditional(a.cond_side, r.after && !(*(const volatile unsigned*)&st->queue & QUEUE_DROP) ? 1u : 0u);
+    } else {
+      const int rows = large_settles(a.loop, p, r);
+      cudaGraphSetConditional(a.cond_side, rows ? 1u : 0u);
+      if (rows) cudaGraphSetConditional(a.cond_switch, large_body(rows, a.sw_bodies));
     }
-    policy_step(a.loop, o, a.desc, a.which, a.cond_side != 0);
-    if (a.cond_side) {
-      const DevState* st = a.loop.st;
-      a.loop.st->cum_passes[a.pass_kind]++;
-      cudaGraphSetConditional(a.cond_side, st->fallback || st->done || (*(const volatile unsigned*)&st->queue & QUEUE_DROP) ? 0u : 1u);
-      return;
-    }
+    return;
   }
-  else if (a.which == 0) a.loop.st->S_len = a.desc->pos0 + 1;
-  else a.loop.st->L_len = a.desc->pos0 + a.desc->k;
+  if (p.run_policy) policy_step(a.loop, p, r, a.which, false);
+  else if (a.which == 0) st->S_len = p.pos0 + 1;
+  else st->L_len = p.pos0 + p.k;
   if (a.host_head) {
     volatile HeadOut* w = a.host_head;
-    const int k = a.which == 0 ? 1 : a.desc->k;
+    const int k = a.which == 0 ? 1 : p.k;
     for (int i = 0; i < k; ++i) { w->argmax[i] = o->argmax[i]; w->lse[i] = o->lse[i]; w->d[i] = o->d[i]; }
     w->zmax[0] = o->zmax[0]; w->pmax = o->pmax; w->fallback = o->fallback;
     w->first_violation = o->first_violation; w->next_token = o->next_token;
     volatile DevState* v = a.host_state;
-    v->S_len = a.loop.st->S_len; v->L_len = a.loop.st->L_len; v->err = *(volatile int*)&a.loop.st->err;
+    v->S_len = st->S_len; v->L_len = st->L_len; v->err = *(volatile int*)&st->err;
   }
   if (a.cond_while) {
-    a.loop.st->cum_passes[a.pass_kind]++;
-    cudaGraphSetConditional(a.cond_while, a.loop.st->done ? 0u : 1u);
+    st->cum_passes[a.pass_kind] = p.cum_passes + 1;
+    cudaGraphSetConditional(a.cond_while, r.fallback || r.after ? 1u : 0u);
   }
-  // the large pass wanted next: the graph branch for its row count where that branch exists, else the block branch
-  const bool fb = a.loop.st->fallback != 0;
-  const int kn = a.loop.descL->k;
+  // behind a small step, the large pass wanted next: the graph branch for its row count where that branch exists, else the block branch
+  const bool fb = a.which == 0 && r.fallback != 0;
+  const int kn = r.after;
   const bool one_row = a.cond_if1 && fb && kn == 1;
   const bool upto8 = a.cond_if8 && fb && !one_row && kn <= 8;
   if (a.cond_if) cudaGraphSetConditional(a.cond_if, (fb && !one_row && !upto8) ? 1u : 0u);
   if (a.cond_if1) cudaGraphSetConditional(a.cond_if1, one_row ? 1u : 0u);
   if (a.cond_if8) cudaGraphSetConditional(a.cond_if8, upto8 ? 1u : 0u);
-  if (a.cond_switch)
-    cudaGraphSetConditional(a.cond_switch, !fb ? (unsigned)a.sw_bodies : kn == 1 ? 1u : (a.sw_bodies == 3 && kn <= 8) ? 2u : 0u);
+  if (a.cond_switch) cudaGraphSetConditional(a.cond_switch, fb ? large_body(kn, a.sw_bodies) : (unsigned)a.sw_bodies);
+}
+
+// s, a sum of exp(z - m), as one of exp(z - top)
+__device__ __forceinline__ float rebase_sum(float s, float m, float top) { return s == 0.f || m == top ? s : s * expf(m - top); }
+// The lanes' records as one, in every lane.
+__device__ __forceinline__ Partial warp_combine(Partial p) {
+  const float m = warp_max(p.m);
+  p.s = warp_sum(rebase_sum(p.s, p.m, m));
+  p.idx = (int)__reduce_min_sync(0xffffffffu, (unsigned)(p.m == m ? p.idx : 0x7fffffff));   // lowest index among equal maxima
+  p.m = m;
+  return p;
+}
+// The last block's merge: `nb` partial records, `stride` apart, by one warp.  All loads together, then one maximum, sum and index over the
+// lanes (a tree of pairs in shared memory, an exponential and a barrier a level, took 1.5 us more).  Every lane has the result.
+__device__ inline Partial warp_merge(const Partial* src, int nb, int stride, int lane) {
+  Partial p;
+  p.m = -INFINITY; p.s = 0.f; p.idx = 0x7fffffff;
+  for (int b0 = lane; b0 < nb; b0 += 10 * 32) {
+    Partial q[10];
+#pragma unroll
+    for (int j = 0; j < 10; ++j) {
+      const int b = b0 + 32 * j;
+      q[j].m = -INFINITY; q[j].s = 0.f; q[j].idx = 0x7fffffff;
+      if (b < nb) {
+        const Partial* r = src + (size_t)b * stride;
+        q[j].m = __ldcg(&r->m); q[j].s = __ldcg(&r->s); q[j].idx = __ldcg(&r->idx);
+      }
+    }
+    float m = p.m;
+#pragma unroll
+    for (int j = 0; j < 10; ++j) m = fmaxf(m, q[j].m);
+    float s = rebase_sum(p.s, p.m, m);
+    int idx = p.m == m ? p.idx : 0x7fffffff;
+#pragma unroll
+    for (int j = 0; j < 10; ++j) {
+      s += rebase_sum(q[j].s, q[j].m, m);
+      if (q[j].m == m) idx = min(idx, q[j].idx);
+    }
+    p.m = m; p.s = s; p.idx = idx;
+  }
+  return warp_combine(p);
+}
+
+// The end of a single-row head, every warp's record in s_p: the block's record, and in the block that arrives last the result.
+__device__ __forceinline__ void head_row_end(const HeadArgs& a, const Partial* s_p, int nw) {
+  __syncthreads();
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x;
+  Partial p;
+  p.m = -INFINITY; p.s = 0.f; p.idx = 0x7fffffff;
+  if (lane < nw) p = s_p[lane];
+  p = warp_combine(p);
+  unsigned t = 0u;
+  if (lane == 0) {
+    a.partials[blockIdx.x] = p;
+    __threadfence();
+    t = atomicAdd(a.counter, 1u);
+  }
+  if (__shfl_sync(0xffffffffu, t, 0) != gridDim.x - 1) return;
+  __threadfence();
+  PolicyIn in{};
+  if (lane == 0 && a.loop.st) in = policy_in(a.loop.st, a.desc, a.pass_kind);
+  p = warp_merge(a.partials, (int)gridDim.x, 1, lane);
+  if (lane == 0) {
+    *a.counter = 0;
+    HeadOut* o = a.out;
+    o->argmax[0] = p.idx;
+    o->zmax[0] = p.m;
+    o->lse[0] = p.m + logf(p.s);
+    const float pmax = 1.f / p.s;
+    o->pmax = pmax;
+    o->gather[0] = __ldcg(&o->gather[0]);
+    policy_tail(a, o, in, p.idx, pmax);
+  }
 }
 
 constexpr int HEAD_THREADS = 256;
@@ -821,7 +946,9 @@ __global__ void __launch_bounds__(HEAD_THREADS) lm_head_kernel(HeadArgs a) {
     HeadOut* o = a.out;
     // gather[] was written by other blocks before their tickets: read around L1
     for (int m = 0; m < mrows; ++m) o->gather[m] = __ldcg(&o->gather[m]);
-    policy_tail(a, o);
+    PolicyIn in{};
+    if (a.loop.st) in = policy_in(a.loop.st, a.desc, a.pass_kind);
+    policy_tail(a, o, in, o->argmax[0], o->pmax);
   }
 }
 
@@ -885,7 +1012,7 @@ __global__ void reset_state_kernel(LoopPtrs L, const int* enc_err, int mode, flo
   st->trust = 1;
   L.y[0] = start_id;
   st->done = (max_len <= 0 || start_id == eos_id) ? 1 : 0;
-  if (mode == BILD_MODE_LARGE_ONLY) next_large(L, st->n); else next_small(L);
+  if (mode == BILD_MODE_LARGE_ONLY) next_large(L, 0, 0); else next_small(L, 0, start_id);
 }
 
 }  // namespace bild

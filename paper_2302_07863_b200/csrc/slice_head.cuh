@@ -195,32 +195,10 @@ __global__ void __launch_bounds__(SH_THREADS) slice_head_kernel(HeadArgs a, int*
   csync256();
   if (!sh->last) return;
   __threadfence();
+  PolicyIn in{};
+  if (tid == 0 && a.loop.st) in = policy_in(a.loop.st, a.desc, a.pass_kind);
   for (int m = warp; m < M; m += SH_COMPUTE / 32) {
-    Partial p;
-    p.m = -INFINITY; p.s = 0.f; p.idx = 0x7fffffff;
-    // (the blocks' partial results of a lane are requested together, eight at a time, then combined in block order)
-    for (int b0 = lane; b0 < (int)gridDim.x; b0 += 8 * 32) {
-      Partial q[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int b = b0 + 32 * j;
-        q[j].m = -INFINITY; q[j].s = 0.f; q[j].idx = 0x7fffffff;
-        if (b < (int)gridDim.x) {
-          const Partial* src = &a.partials[(size_t)b * MAXB + m];
-          q[j].m = __ldcg(&src->m); q[j].s = __ldcg(&src->s); q[j].idx = __ldcg(&src->idx);
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 8; ++j) p = combine(p, q[j]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      Partial q;
-      q.m = __shfl_xor_sync(0xffffffffu, p.m, o);
-      q.s = __shfl_xor_sync(0xffffffffu, p.s, o);
-      q.idx = __shfl_xor_sync(0xffffffffu, p.idx, o);
-      p = ((lane & o) == 0) ? combine(p, q) : combine(q, p);
-    }
+    const Partial p = warp_merge(a.partials + m, (int)gridDim.x, MAXB, lane);
     if (lane == 0) {
       a.out->argmax[m] = p.idx;
       a.out->zmax[m] = p.m;
@@ -233,8 +211,14 @@ __global__ void __launch_bounds__(SH_THREADS) slice_head_kernel(HeadArgs a, int*
     __threadfence();
     HeadOut* o = a.out;
     // gather[] was written by other blocks before their tickets: read around L1
-    for (int m = 0; m < M; ++m) o->gather[m] = __ldcg(&o->gather[m]);
-    policy_tail(a, o);
+    float z[MAXB];
+#pragma unroll
+    for (int m = 0; m < MAXB; ++m)
+      if (m < M) z[m] = __ldcg(&o->gather[m]);
+#pragma unroll
+    for (int m = 0; m < MAXB; ++m)
+      if (m < M) o->gather[m] = z[m];
+    policy_tail(a, o, in, o->argmax[0], o->pmax);
   }
 }
 
