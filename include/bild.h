@@ -83,8 +83,9 @@ typedef struct {
    * decoder layers of the large model, with the large model's encoder, embedding, final norm and prediction
    * head.  small_cfg must then equal large_cfg except for n_layers (= n) and logit_scale; the small model's
    * weights argument is ignored (may be NULL); only the large model's encoder runs, and the two "models"
-   * share the cross-attention K/V and the self-attention cache of those n layers (a large pass rewrites the
-   * rows the small steps wrote, so the cache always holds the large model's own values).  0: two models. */
+   * share the cross-attention K/V of those n layers.  Each has self-attention rows of its own (those of the shared
+   * layers hold the same values up to the order of additions): the small model drafts on while a large pass
+   * writes its rows.  0: two models. */
   int32_t early_exit_layers;
 } bild_config;
 
@@ -216,7 +217,7 @@ typedef struct {
   int32_t draft_ahead;       /* 1: in bild_generate* the small model goes on from its own candidate while the large model judges
                               * the block in front, as long as large passes mostly end with that candidate; what it drafted
                               * is dropped if one ends otherwise (tokens, trace and counts are those of the serial loop).
-                              * 0, and with early exit (shared caches), graph_switch = 0 or host_loop = 1: the serial loop */
+                              * 0, and with graph_switch = 0 or host_loop = 1: the serial loop */
 } bild_tuning;
 void bild_tuning_default(bild_tuning *t /*HOST out*/);
 /* bild_create with explicit switches; tuning == NULL means the defaults. */

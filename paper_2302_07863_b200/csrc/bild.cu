@@ -145,6 +145,7 @@ struct bild_ctx {
   Model m[2];
   cudaStream_t stream = nullptr;
   DevState* st = nullptr;
+  DraftBlock* block = nullptr;
   int* y = nullptr;
   bild_trace_rec* trace = nullptr;
   int trace_cap = 0;
@@ -362,6 +363,7 @@ void plan(bild_ctx* c, Bump& b) {
       e.exl[pr] = b.take<__nv_bfloat16>(ecap128 * std::max(std::max(d, I), F));
     }
   }
+  c->block = b.take<DraftBlock>(BLOCK_RING);
   b.off = align_up(b.off, 256);
 }
 
@@ -1203,7 +1205,7 @@ cudaError_t launch_enc_linear(bild_ctx* c, Model& m, const LinArgs& a, int rb, i
 
 LoopPtrs loop_ptrs(bild_ctx* c) {
   LoopPtrs L;
-  L.st = c->st; L.y = c->y; L.trace = c->trace; L.descS = c->m[0].desc; L.descL = c->m[1].desc;
+  L.st = c->st; L.y = c->y; L.trace = c->trace; L.descS = c->m[0].desc; L.descL = c->m[1].desc; L.block = c->block;
   return L;
 }
 
@@ -1568,7 +1570,7 @@ int build_graphs_once(bild_ctx* c, int base) {
   int64_t& per_pass_large8 = base == 0 ? c->per_pass_large8 : dummy8;
   cudaGraph_t* graph = c->graph + base;
   cudaGraphExec_t* exec = c->exec + base;
-  if (c->graph_switch && c->draft_ahead && c->cfg.early_exit_layers == 0) {
+  if (c->graph_switch && c->draft_ahead) {
     CUDA_TRY(c, cudaGraphCreate(&graph[0], 0));
     int rc = build_rounds(c, graph[0], per_pass, &per_pass_large1, &per_pass_large8);
     if (rc) return rc;
@@ -1835,8 +1837,8 @@ int bild_create_tuned(const bild_config* cfg, const bild_weights* small_w, const
   plan(c, b);
   c->ws_bytes = b.off;
   if (workspace_bytes < b.off) { delete c; return BILD_ERR_WORKSPACE; }
-  if (early) {   // one cache for the shared layers: [layer][head][row][channel], the small model's layers come first
-    c->m[0].selfK = c->m[1].selfK; c->m[0].selfV = c->m[1].selfV;
+  if (early) {   // one encoder: its keys and values of the shared layers come first.  (The self-attention caches stay apart: the
+    // small model drafts on while a large pass writes rows of the same layers.)
     c->m[0].crossK = c->m[1].crossK; c->m[0].crossV = c->m[1].crossV;
   }
   const bild_weights* ws[2] = {early ? large_w : small_w, large_w};   // early exit: the small model is a prefix of the large one

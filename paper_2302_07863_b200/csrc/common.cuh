@@ -71,9 +71,8 @@ struct DevState {
   int pad1;
   long long cum_draws;       // token-drawing kernels run from the loop graphs since create
   long long cum_passes[4];   // passes run from the loop graphs since create: small, large block, large single row, large up to 8 rows
-  // Loop in rounds (round_step): the blocks of drafts handed to the large model, oldest first
-  DraftBlock block[BLOCK_RING];
-  unsigned block_head, block_tail;   // counted up by the large passes and by the small steps
+  // Loop in rounds (round_step)
+  unsigned block_head, block_tail;   // blocks of drafts the large model has judged and the small one handed over (places in LoopPtrs::block)
   unsigned queue;            // QUEUE_* flags, and the number of blocks handed over and not yet judged
   int trust;                 // 0..TRUST_MAX, up when a large pass ends with the small model's candidate, down when it does not
   int overrun;               // the loop was stopped by the guard on `passes`

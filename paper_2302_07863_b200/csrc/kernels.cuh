@@ -344,6 +344,7 @@ struct LoopPtrs {
   bild_trace_rec* trace;
   CallDesc* descS;
   CallDesc* descL;
+  DraftBlock* block;   // [BLOCK_RING] blocks of drafts on their way, oldest first
 };
 
 // What the policy of a pass reads of the state, in one go: the loads of one thread then share a trip to the L2 (read where they were used,
@@ -456,7 +457,7 @@ __device__ inline PolicyOut policy_tests(HeadOut* o, const PolicyIn& p, int whic
 // The small model's side at a fallback: hands its drafts over.  Returns whether it goes on.
 __device__ inline bool small_hands_over(const LoopPtrs& L, const PolicyIn& p, int steps, int fallbacks, int forced, int candidate) {
   DevState* st = L.st;
-  DraftBlock& b = st->block[p.block_tail % BLOCK_RING];
+  DraftBlock& b = L.block[p.block_tail % BLOCK_RING];
   st->block_tail = p.block_tail + 1;
   const bool last = p.n + 1 >= p.max_len || candidate == p.eos_id;
   b.n = p.n; b.proposed = candidate; b.last = last;
@@ -483,7 +484,7 @@ __device__ inline bool small_hands_over(const LoopPtrs& L, const PolicyIn& p, in
 // are this side's only).  Returns the rows of the block that follows at once, 0 if none does.
 __device__ inline int large_settles(const LoopPtrs& L, const PolicyIn& p, const PolicyOut& o) {
   DevState* st = L.st;
-  const DraftBlock& b = st->block[p.block_head % BLOCK_RING];
+  const DraftBlock& b = L.block[p.block_head % BLOCK_RING];
   const int proposed = __ldcg(&b.proposed), last = __ldcg(&b.last), slot = __ldcg(&b.slot);
   unsigned q = *(volatile unsigned*)&st->queue;
   const int j = p.pos0 + (o.mv >= 0 ? o.mv + 1 : p.k);
@@ -512,7 +513,7 @@ __device__ inline int large_settles(const LoopPtrs& L, const PolicyIn& p, const 
     if (was == q) {
       if (!more) return 0;
       __threadfence();
-      return next_large(L, j, __ldcg(&st->block[(p.block_head + 1) % BLOCK_RING].n));
+      return next_large(L, j, __ldcg(&L.block[(p.block_head + 1) % BLOCK_RING].n));
     }
     q = was;
   }
@@ -601,7 +602,7 @@ __device__ inline void round_step(const LoopPtrs& L, int* rows, bool* small) {
   *rows = 0; *small = false;
   st->cum_rounds++;
   if (st->queue & QUEUE_DROP) {   // the serial loop's state behind the last large pass
-    const DraftBlock& b = st->block[st->block_head % BLOCK_RING];
+    const DraftBlock& b = L.block[st->block_head % BLOCK_RING];
     st->n = st->S_len = st->L_len;
     st->drafts = 0;
     st->fallback = 0;
@@ -615,13 +616,13 @@ __device__ inline void round_step(const LoopPtrs& L, int* rows, bool* small) {
   }
   const int waiting = (int)(st->queue & QUEUE_COUNT);
   if (waiting > 0) {
-    *rows = next_large(L, st->L_len, st->block[st->block_head % BLOCK_RING].n);
+    *rows = next_large(L, st->L_len, L.block[st->block_head % BLOCK_RING].n);
   }
   if (!st->done) {
     // at a fallback: on from the candidate if its block stands already, or ahead
     if (!st->fallback) {
       *small = true;
-    } else if (waiting == 0 || (waiting <= st->trust && !st->block[(st->block_tail - 1) % BLOCK_RING].last)) {
+    } else if (waiting == 0 || (waiting <= st->trust && !L.block[(st->block_tail - 1) % BLOCK_RING].last)) {
       ++st->n;
       st->drafts = 0;
       st->fallback = 0;

@@ -267,18 +267,21 @@ def test_new_context_takes_updated_weights(torch_cuda, name):
     new.close()
 
 
-@pytest.mark.parametrize("name,noise", [("tiny", 0.0), ("tiny", 0.03), ("tiny", None), ("tiny_bf16", 0.0), ("tiny_bf16", 0.03), ("wide_bf16", None)])
+@pytest.mark.parametrize("name,noise", [("tiny", 0.0), ("tiny", 0.03), ("tiny", None), ("tiny_bf16", 0.0), ("tiny_bf16", 0.03), ("wide_bf16", None), ("wide_bf16", "exit")])
 @pytest.mark.parametrize("top_p", [0.0, 0.8])
 def test_drafting_ahead_is_the_serial_loop(torch_cuda, name, noise, top_p):
     """The loop in rounds against the serial one (draft_ahead = 0): tokens, trace and counts.  The small model is the large one
-    (every large pass ends as proposed), the large one with `noise` on its weights (some do), or another model (hardly any does);
+    (every large pass ends as proposed), the large one with `noise` on its weights (some do), another model (hardly any does) or the
+    large one's first layer;
     fallbacks from none to all, blocks from 1 row to the most, ends by length at the first places and by token anywhere."""
     from paper_2302_07863_b200 import MODE_BILD, MODE_LARGE_ONLY, MODE_SMALL_ONLY
     from paper_2302_07863_b200.binding import BF16, FP32, Config, Context, model_cfg, upload_model
     wl = WORKLOADS[name]
     sL = MODEL_SHAPES[wl.large]
     wlarge = upload_model(gen_model(sL, wl.seed, wl.dtype), "cuda:0")
-    if noise is None:
+    if noise == "exit":
+        sS, wsmall = dataclasses.replace(sL, n_layers=1), wlarge
+    elif noise is None:
         sS = MODEL_SHAPES[wl.small]
         wsmall = upload_model(gen_model(sS, wl.seed, wl.dtype), "cuda:0")
     else:
@@ -290,7 +293,8 @@ def test_drafting_ahead_is_the_serial_loop(torch_cuda, name, noise, top_p):
     u = np.random.default_rng(6).random((2, cap)).astype(np.float32)
 
     def contexts(max_draft, eos):
-        cfg = Config(model_cfg(sS, 9.0), model_cfg(sL, 9.0), FP32 if wl.dtype == "fp32" else BF16, 32, cap, max_draft, 0, eos, 0)
+        cfg = Config(model_cfg(sS, 9.0), model_cfg(sL, 9.0), FP32 if wl.dtype == "fp32" else BF16, 32, cap, max_draft, 0, eos,
+                     1 if noise == "exit" else 0)
         out = [Context(cfg, sS, wsmall, sL, wlarge, tuning=t) for t in (None, dict(draft_ahead=0))]
         for c in out:
             c.encode(ids)
