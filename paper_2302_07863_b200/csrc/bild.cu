@@ -1500,7 +1500,7 @@ int capture_pass(bild_ctx* c, cudaGraph_t body, int which, int MB, unsigned long
 
 // Builds the two device-side loops (CUDA graphs with conditional nodes).  The head
 // kernel's last block sets the WHILE handle to "not done" and the IF handle to "fallback".
-int build_graphs_once(bild_ctx* c, int base);
+int build_graph_once(bild_ctx* c, int base, bool alone);
 
 void drop_graphs(bild_ctx* c) {
   for (int i = 0; i < 4; ++i) {
@@ -1517,24 +1517,25 @@ void drop_step_graph(bild_ctx::StepGraph& s) {
   s.g = nullptr;
 }
 
-// base 0: the greedy loops; base 2: the loops of the sampling variant (a token-drawing kernel after every LM head)
-int build_graphs(bild_ctx* c, int base) {
-  if (c->exec[base] && c->exec[base + 1]) return BILD_OK;
-  // if a loop body refuses programmatic edges, the graphs are built again with plain launches
+// base 0: a greedy loop; base 2: one of the sampling variant (a token-drawing kernel after every LM head).  alone: the loop of the large
+// model alone, else the other one; each is built when it is first asked for.
+int build_graph(bild_ctx* c, int base, bool alone) {
+  if (c->exec[base + alone]) return BILD_OK;
+  // if a loop body refuses programmatic edges, the graph is built again with plain launches
   const bool want_pdl = c->use_pdl;
   c->draw = base == 2;
-  int rc = build_graphs_once(c, base);
-  if (rc != BILD_OK && c->graph_switch) {   // no SWITCH nodes here: one IF node per kind of pass
+  int rc = build_graph_once(c, base, alone);
+  if (rc != BILD_OK && !alone && c->graph_switch) {   // no SWITCH nodes here: one IF node per kind of pass
     drop_graphs(c);
     cudaGetLastError();
     c->graph_switch = false;
-    rc = build_graphs_once(c, base);
+    rc = build_graph_once(c, base, alone);
   }
   if (rc != BILD_OK && want_pdl) {
     drop_graphs(c);
     cudaGetLastError();
     c->use_pdl = false;
-    rc = build_graphs_once(c, base);
+    rc = build_graph_once(c, base, alone);
   }
   c->draw = false;
   if (rc != BILD_OK) { drop_graphs(c); cudaGetLastError(); }
@@ -1576,7 +1577,7 @@ int build_rounds(bild_ctx* c, cudaGraph_t g, int64_t* per_pass, int64_t* per_pas
   return BILD_OK;
 }
 
-int build_graphs_once(bild_ctx* c, int base) {
+int build_graph_once(bild_ctx* c, int base, bool alone) {
   // launches per pass are recorded from the greedy graphs; the drawing kernels of the sampled ones are counted on the device
   int64_t dummy[2] = {0, 0}, dummy1 = 0, dummy8 = 0;
   int64_t* per_pass = base == 0 ? c->per_pass : dummy;
@@ -1584,12 +1585,12 @@ int build_graphs_once(bild_ctx* c, int base) {
   int64_t& per_pass_large8 = base == 0 ? c->per_pass_large8 : dummy8;
   cudaGraph_t* graph = c->graph + base;
   cudaGraphExec_t* exec = c->exec + base;
-  if (c->graph_switch && c->draft_ahead) {
+  if (!alone && c->graph_switch && c->draft_ahead) {
     CUDA_TRY(c, cudaGraphCreate(&graph[0], 0));
     int rc = build_rounds(c, graph[0], per_pass, &per_pass_large1, &per_pass_large8);
     if (rc) return rc;
     CUDA_TRY(c, cudaGraphInstantiate(&exec[0], graph[0], 0));
-  } else {  // BiLD (and small-only): WHILE { small pass ; IF { large block pass } ; IF { large single-row pass } }
+  } else if (!alone) {  // BiLD (and small-only): WHILE { small pass ; IF { large block pass } ; IF { large single-row pass } }
     CUDA_TRY(c, cudaGraphCreate(&graph[0], 0));
     cudaGraphConditionalHandle hw, hi, hi1, hi8 = 0;
     CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hw, graph[0], 1, cudaGraphCondAssignDefault));
@@ -1650,7 +1651,7 @@ int build_graphs_once(bild_ctx* c, int base) {
     CUDA_TRY(c, cudaGraphInstantiate(&exec[0], graph[0], 0));
     }
   }
-  {  // large-only greedy: WHILE { large pass with k = 1 }
+  if (alone) {  // large-only greedy: WHILE { large pass with k = 1 }
     CUDA_TRY(c, cudaGraphCreate(&graph[1], 0));
     cudaGraphConditionalHandle hw;
     CUDA_TRY(c, cudaGraphConditionalHandleCreate(&hw, graph[1], 1, cudaGraphCondAssignDefault));
@@ -2052,13 +2053,14 @@ int generate_async(bild_ctx* c, int mode, float alpha_fb, float alpha_rb, int ma
   if (!c->host_loop) {
     // device-side loop: no host involvement between the first and the last token
     const int base = sampled ? 2 : 0;
-    int rc = build_graphs(c, base);
+    const bool alone = mode == BILD_MODE_LARGE_ONLY;
+    int rc = build_graph(c, base, alone);
     if (rc) return rc;
     rc = reset_state(c, mode, alpha_fb, alpha_rb, max_len);
     if (rc) return rc;
     if (max_len == 0 || c->cfg.start_id == c->cfg.eos_id) return BILD_OK;
     // passes the loop may run: bounded by the guard of the device-side policy
-    CUDA_TRY(c, cudaGraphLaunch(c->exec[base + (mode == BILD_MODE_LARGE_ONLY ? 1 : 0)], c->stream));
+    CUDA_TRY(c, cudaGraphLaunch(c->exec[base + alone], c->stream));
     return BILD_OK;
   }
   int rc = reset_state(c, mode, alpha_fb, alpha_rb, max_len);
