@@ -706,7 +706,9 @@ void setup_umma(bild_ctx* c, Model& m) {
       !smem_ok((const void*)enc_gemm_kernel<true, false, 128>, eg_smem_bytes<true, false, 128>()) ||
       !smem_ok((const void*)enc_gemm_kernel<false, false, 64>, eg_smem_bytes<false, false, 64>()) ||
       !smem_ok((const void*)enc_gemm_kernel<false, true, 64>, std::max(eg_smem_bytes<false, true, 64>(2), eg_smem_bytes<false, true, 64>(4))) ||
-      !smem_ok((const void*)enc_gemm_kernel<true, true, 64>, std::max(eg_smem_bytes<true, true, 64>(2), eg_smem_bytes<true, true, 64>(4)))) {
+      !smem_ok((const void*)enc_gemm_kernel<true, true, 64>, std::max(eg_smem_bytes<true, true, 64>(2), eg_smem_bytes<true, true, 64>(4))) ||
+      !smem_ok((const void*)enc_gemm_kernel<false, true, 64, true>, std::max(eg_nrm_smem<false>(2), eg_nrm_smem<false>(4))) ||
+      !smem_ok((const void*)enc_gemm_kernel<true, true, 64, true>, std::max(eg_nrm_smem<true>(2), eg_nrm_smem<true>(4)))) {
     cudaGetLastError();
     return;
   }
@@ -1122,11 +1124,6 @@ cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, 
   const EgQkv qkv = which_map == TM_EQKV && m.enc_flash ? c->eb[m.index].qkv : EgQkv{};
   const int E = a.M, tiles_tok = (E + EG_TOK - 1) / EG_TOK;
   const int ki = a.K == m.c.d_model ? 0 : a.K == m.inner ? 1 : 2;
-  if (split) {
-    cudaError_t e = launch_k(c, norm_split_kernel, dim3(tiles_tok * EG_TOK / 4), dim3(128), 0, a.X, a.ldx, a.gain, a.eps, E, a.K,
-                             c->eb[m.index].exh[pair], c->eb[m.index].exl[pair]);
-    if (e != cudaSuccess) return e;
-  }
   const CUtensorMap* t = &m.tmaps[(size_t)layer * TM_PER_LAYER];
   const CUtensorMap &t0 = t[which_map], &t1 = t[which_map == TM_EWI0 ? TM_EWI1 : which_map];
   const bool gated = a.epi == EPI_GATED, resid = a.epi == EPI_RESID, small = E <= 64;
@@ -1145,10 +1142,17 @@ cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, 
     while (z < 4 && tiles * (z * 2) <= c->sms && nkb / (z * 2) >= 2) z *= 2;
   }
   grid.z = z;
+  // up to 64 ids the kernel normalises the residual stream itself, where only this layer needs the result
+  const bool nrm = split && a.gain && !resid && z > 1 && (which_map == TM_EQKV || which_map == TM_EWI0) && (nkb + z - 1) / z <= EG_NRM_KB;
+  if (split && !nrm) {
+    cudaError_t e = launch_k(c, norm_split_kernel, dim3(tiles_tok * EG_TOK / 4), dim3(128), 0, a.X, a.ldx, a.gain, a.eps, E, a.K,
+                             c->eb[m.index].exh[pair], c->eb[m.index].exl[pair]);
+    if (e != cudaSuccess) return e;
+  }
   if (!resid && z > 1) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid; cfg.blockDim = dim3(EG_THREADS); cfg.stream = c->stream;
-    cfg.dynamicSmemBytes = gated ? eg_smem_bytes<true, true, 64>(z) : eg_smem_bytes<false, true, 64>(z);
+    cfg.dynamicSmemBytes = nrm ? (gated ? eg_nrm_smem<true>(z) : eg_nrm_smem<false>(z)) : gated ? eg_smem_bytes<true, true, 64>(z) : eg_smem_bytes<false, true, 64>(z);
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 1; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = z;
@@ -1156,7 +1160,8 @@ cudaError_t launch_enc_gemm(bild_ctx* c, Model& m, const LinArgs& a, int layer, 
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = c->use_pdl ? 2 : 1;
     (*c->cnt)++;
-    auto kern = gated ? enc_gemm_kernel<true, true, 64> : enc_gemm_kernel<false, true, 64>;
+    auto kern = nrm ? (gated ? enc_gemm_kernel<true, true, 64, true> : enc_gemm_kernel<false, true, 64, true>)
+                    : gated ? enc_gemm_kernel<true, true, 64> : enc_gemm_kernel<false, true, 64>;
     return cudaLaunchKernelEx(&cfg, kern, a, encoder_err(c), oh, ol, qkv, t0, t1, h[0], h[1]);
   }
   if (gated) {
