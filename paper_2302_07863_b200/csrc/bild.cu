@@ -768,6 +768,7 @@ int setup_fused(bild_ctx* c, Model& m) {
   if (parts > 8) return BILD_OK;
   if (cudaFuncSetAttribute(attn_sub_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess ||
       cudaFuncSetAttribute(attn_sub_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess ||
+      cudaFuncSetAttribute(attn_sub_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess ||
       cudaFuncSetAttribute(ffn_sub_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess ||
       cudaFuncSetAttribute(ffn_sub_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) {
     cudaGetLastError();
@@ -924,8 +925,8 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   a.Wp = (const __nv_bfloat16*)w.wqkv; a.Wo = (const __nv_bfloat16*)w.wo;
   a.kc = m.selfK + kvoff * cap; a.vc = m.selfV + kvoff * cap; a.cap = cap; a.bias = m.dec_bias; a.bias_ld = cap; a.self = 1;
   const AttnSubPlan& pls = m.sub_self[MB == 1 ? 0 : 1];
-  a.kc_keys = pls.kc; a.bias_len = pls.bias_len; a.red_keys = pls.red_keys;
-  a.L = attn_sub_layout(d, dkv, 3, C, MB, a.kc_keys, a.bias_len, pls.late);
+  a.kc_keys = pls.kc; a.kc_main = pls.kc_main; a.bias_len = pls.bias_len; a.red_keys = pls.red_keys;
+  a.L = attn_sub_layout(d, dkv, 3, C, MB, a.kc_keys, a.bias_len, pls.late, pls.kc_main, pls.kvst);
   CUDA_TRY(c, launch_sub(c, MB == 1 ? attn_sub_kernel<true> : attn_sub_kernel<false>, H * C, C, (size_t)a.L.total, a, !first_plain));
   int rc = after_self();
   if (rc) return rc;
@@ -935,9 +936,9 @@ int fused_layer(bild_ctx* c, Model& m, int MB, int l, const CallDesc* desc, int 
   a.Wp = (const __nv_bfloat16*)w.wcq; a.Wo = (const __nv_bfloat16*)w.wco;
   a.kc = m.crossK + kvoff * ecap; a.vc = m.crossV + kvoff * ecap; a.cap = ecap; a.bias = nullptr; a.bias_ld = 0; a.self = 0;
   const AttnSubPlan& plc = m.sub_cross[MB == 1 ? 0 : 1];
-  a.kc_keys = plc.kc; a.bias_len = plc.bias_len; a.red_keys = plc.red_keys;
-  a.L = attn_sub_layout(d, dkv, 1, C, MB, a.kc_keys, a.bias_len, plc.late);
-  CUDA_TRY(c, launch_sub(c, MB == 1 ? attn_sub_kernel<true> : attn_sub_kernel<false>, H * C, C, (size_t)a.L.total, a));
+  a.kc_keys = plc.kc; a.kc_main = plc.kc_main; a.bias_len = plc.bias_len; a.red_keys = plc.red_keys;
+  a.L = attn_sub_layout(d, dkv, 1, C, MB, a.kc_keys, a.bias_len, plc.late, plc.kc_main, plc.kvst);
+  CUDA_TRY(c, launch_sub(c, MB == 1 ? attn_sub_kernel<true> : plc.wide() ? attn_sub_kernel<false, true> : attn_sub_kernel<false>, H * C, C, (size_t)a.L.total, a));
   // S7-S8 / L7-L8
   FfnSubArgs f{};
   f.desc = desc; f.eps = mc.ln_eps; f.inv_d = 1.f / (float)d; f.d = d; f.F = Fd; f.gated = gated ? 1 : 0; f.mb = MB; f.spin = c->spin_limit;
@@ -2287,7 +2288,7 @@ int bild_op_attn_sublayer(int self, const void* Wp, const void* Wo, const float*
   if (cudaMemsetAsync(o.err, 0, 4, s) != cudaSuccess) return BILD_ERR_CUDA;
   if (cudaMemcpyAsync(o.nkeys, &n_before, sizeof(int), cudaMemcpyHostToDevice, s) != cudaSuccess) return BILD_ERR_CUDA;
   if (cudaMemsetAsync(x_out, 0, (size_t)M * d * sizeof(float), s) != cudaSuccess) return BILD_ERR_CUDA;   // the kernel accumulates into it
-  auto kern = MB == 1 ? attn_sub_kernel<true> : attn_sub_kernel<false>;
+  auto kern = MB == 1 ? attn_sub_kernel<true> : pl.wide() ? attn_sub_kernel<false, true> : attn_sub_kernel<false>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess) return BILD_ERR_CUDA;
   AttnSubArgs a{};
   a.desc = o.desc; a.eps = eps; a.inv_d = 1.f / (float)d; a.d = d; a.I = I; a.H = H; a.dkv = dkv; a.dkv_shift = ilog2(dkv); a.C = C; a.c_shift = ilog2(C);
@@ -2295,7 +2296,8 @@ int bild_op_attn_sublayer(int self, const void* Wp, const void* Wo, const float*
   a.n_keys_dev = o.nkeys; a.x_in = x_in; a.x_out = x_out; a.x_zero = o.zero; a.gain = gain;
   a.Wp = (const __nv_bfloat16*)Wp; a.Wo = (const __nv_bfloat16*)Wo; a.kc = kc; a.vc = vc; a.cap = cap;
   a.bias = bias_by_dist; a.bias_ld = cap; a.self = self ? 1 : 0;
-  a.L = attn_sub_layout(d, dkv, P, C, MB, kc_keys, bias_len, pl.late);
+  a.kc_main = pl.kc_main;
+  a.L = attn_sub_layout(d, dkv, P, C, MB, kc_keys, bias_len, pl.late, pl.kc_main, pl.kvst);
   if (launch_sub(&tmp, kern, H * C, C, (size_t)a.L.total, a) != cudaSuccess) return BILD_ERR_CUDA;
   return op_finish(s, o);
 }

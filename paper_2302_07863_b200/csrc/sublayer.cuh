@@ -152,9 +152,11 @@ __device__ __forceinline__ void sub_split3(float x, float y, uint32_t& h, uint32
 __host__ __device__ inline int sub_chunks(int d) { return ((d + 31) / 32 + 7) / 8; }                 // 32-column chunks per warp: 1..4
 __host__ __device__ inline int sub_wst(int d) { return (d * 2 + 127) / 128 * 128 + 64; }            // bytes from weight row to weight row: 64 mod 128
 __host__ __device__ inline int sub_xst(int d) { return (d / 2 + 31) / 32 * 32 + 16; }               // words from token row to token row: 16 mod 32
-__host__ __device__ inline int sub_pst(int rows) { return (rows + 15) / 16 * 16 + 4; }              // floats of partial sums per token: 2 p = 8 mod 32
+__host__ __device__ inline int sub_pst(int rows, bool half = false) {   // floats of partial sums per token: 2 p = 8 (half a tile: 24) mod 32
+  return half ? 12 : (rows + 15) / 16 * 16 + 4;
+}
 __host__ __device__ inline int sub_xs_bytes(int d, int mb) { return (mb == 1 ? 3 : 2 * SUB_MB) * sub_xst(d) * 4; }
-__host__ __device__ inline int sub_psum_bytes(int rows, int mb) { return 8 * (mb == 1 ? 1 : SUB_MB) * sub_pst(rows) * 4; }
+__host__ __device__ inline int sub_psum_bytes(int rows, int mb, bool half = false) { return 8 * (mb == 1 ? 1 : SUB_MB) * sub_pst(rows, half) * 4; }
 
 template <bool ONE>
 struct SubRows { float4 v[ONE ? 1 : SUB_MB]; };
@@ -266,9 +268,10 @@ __device__ __forceinline__ void sub_bfrags(const uint32_t* Xs, int xst, int k, i
     }
 }
 // one 16-row tile, its halves' operands f0 and f1 (`both`: the second one exists); the warp's partial sums go to psum [warp][token][sub_pst(rows)]
-template <bool ONE>
+// HALF: of a block variant with up to 8 weight rows
+template <bool ONE, bool HALF = false>
 __device__ __forceinline__ void sub_tile(const uint4 (&f0)[4], const uint4 (&f1)[4], bool both, const SubB<ONE>& b, int nch, int nrows, int mt, float* psum, int warp, int lane) {
-  const int g = lane >> 2, t = lane & 3, pst = sub_pst(nrows), row = mt * 16 + g;
+  const int g = lane >> 2, t = lane & 3, pst = sub_pst(nrows, HALF), row = mt * 16 + g;
   float c[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int ch = 0; ch < 4; ++ch)
@@ -293,7 +296,8 @@ __device__ __forceinline__ void sub_tile(const uint4 (&f0)[4], const uint4 (&f1)
     }
   } else {
     float* p = psum + (size_t)(warp * SUB_MB + 2 * t) * pst + row;
-    p[0] = c[0]; p[pst] = c[1]; p[8] = c[2]; p[pst + 8] = c[3];
+    p[0] = c[0]; p[pst] = c[1];
+    if (!HALF) { p[8] = c[2]; p[pst + 8] = c[3]; }
   }
 }
 // dot product (weight row, token row) over all warps, in a fixed order
@@ -309,7 +313,7 @@ __device__ __forceinline__ float sub_total(const float* psum, int row, int m, in
 // ------------------------------------------------------------------------------------------------
 // Attention sub-layer
 // ------------------------------------------------------------------------------------------------
-struct AttnSubLayout { int wq, kv, kv_late, xs, rec, rrec, qkv, psum, sa, out, bias, seed, sh, total; };
+struct AttnSubLayout { int wq, kv, kv2_k, kv2_v, kv_late, xs, rec, rrec, qkv, psum, sa, out, bias, seed, sh, total; };
 
 struct AttnSubArgs {
   const CallDesc* desc;
@@ -332,6 +336,7 @@ struct AttnSubArgs {
   int self;
   int d, I, H, dkv, dkv_shift, C, c_shift;
   int kc_keys;               // keys per staged chunk
+  int kc_main;               // WIDE: of them in the main area (the rest where the weight rows were)
   int red_keys;              // up to this many keys every rank attends over ALL keys of the head (no second exchange)
   int bias_len;              // floats reserved for the staged bias
   int mb;                    // token rows the shared memory is sized for
@@ -346,21 +351,26 @@ struct AttnSubArgs {
 // this kernel's and run their prologue and weight fetch in its shadow (and so that 16 clusters of 8 are resident at
 // once: above that size an SM takes one block, and a B200 then holds only 15 such clusters).
 // late: the keys / values are staged where the projection's weight rows were, once those wait in registers.
-inline AttnSubLayout attn_sub_layout(int d, int dkv, int P, int C, int mb, int kc, int bias_len, int late) {
+// kc_main < kc: the keys from there on are.  kvst: floats from key to key.
+inline AttnSubLayout attn_sub_layout(int d, int dkv, int P, int C, int mb, int kc, int bias_len, int late, int kc_main, int kvst) {
   AttnSubLayout L;
   const int npr = (P * dkv + C - 1) / C, no = (d + C - 1) / C, rec = dkv + SUB_RECPAD;
-  const int wq_b = sub_up16(npr * sub_wst(d)), kv_b = sub_up16(kc * (sub_kv_stride(dkv) + dkv + 4) * 4);
+  const int wq_b = sub_up16(std::max(npr * sub_wst(d), (kc - kc_main) * (kvst + dkv + 4) * 4)), kv_b = sub_up16(kc_main * (kvst + dkv + 4) * 4);
   int off = 0;
   L.kv_late = late;
   L.wq = off; off += late ? std::max(wq_b, kv_b) : wq_b;
   L.kv = late ? L.wq : off; off += late ? 0 : kv_b;
+  // floats from where a key / value past kc_main would follow the others to where it is: behind L.wq, keys first
+  L.kv2_k = (L.wq - L.kv) / 4 - kc_main * kvst;
+  L.kv2_v = (L.wq - L.kv) / 4 + (kc - kc_main) * kvst - kc_main * (dkv + 4) - kc_main * kvst;
   // token rows; afterwards the warps' records and the ranks' records
   L.xs = off; L.rec = off; L.rrec = off + sub_up16(8 * mb * rec * 4);
   off += std::max(sub_up16(sub_xs_bytes(d, mb)), sub_up16(8 * mb * rec * 4) + sub_up16(C * mb * rec * 4));
   L.qkv = off; off += sub_up16(mb * (P * dkv + 16) * 4);
-  // partial sums of the products; afterwards the merged head output and the output tile (block variant)
-  L.psum = off; L.sa = off; L.out = off + sub_up16(mb * (dkv + 4) * 4);
-  off += std::max(sub_up16(sub_psum_bytes(npr, mb)), mb == 1 ? 0 : sub_up16(mb * (dkv + 4) * 4) + sub_up16(SUB_MB * (no + 4) * 4));
+  // partial sums of the products; afterwards the merged head output (block variant)
+  L.psum = off; L.sa = off; L.out = L.rec;   // (the output tile: the records are merged by then)
+  static_assert(SUB_MB * (SUB_THREADS / 2 + 4) * 4 <= 8 * SUB_MB * (16 + SUB_RECPAD) * 4, "at most 128 outputs a block, records of 16 channels and more");
+  off += std::max(sub_up16(sub_psum_bytes(npr, mb, kc_main < kc)), mb == 1 ? 0 : sub_up16(mb * (dkv + 4) * 4));
   L.bias = off; off += sub_up16(bias_len * 4);
   L.seed = off; off += sub_up16(mb * no * 4);
   L.sh = off; off += sub_up16((int)sizeof(SubShared));
@@ -372,7 +382,12 @@ inline AttnSubLayout attn_sub_layout(int d, int dkv, int P, int C, int mb, int k
 // `all_keys` > 0 asks for a chunk that holds up to that many keys so that short caches need no second exchange; the
 // chunk shrinks until the layout for passes of `mb` rows (1: the single-row kernel, SUB_MB: the block kernel; each has a plan
 // of its own) stays under `prefer` bytes (half an SM), else under `limit`.
-struct AttnSubPlan { int kc, bias_len, red_keys, late; bool ok; };
+struct AttnSubPlan {
+  int kc, bias_len, red_keys, late;
+  bool ok;
+  int kc_main, kvst;   // keys of a chunk in the main area, floats from key to key
+  bool wide() const { return kc_main < kc; }
+};
 inline AttnSubPlan attn_sub_plan(int d, int dkv, int P, int C, int keys_cap, int all_keys, int prefer, int limit, int mb) {
   AttnSubPlan pl;
   const int per_rank = (keys_cap + C - 1) / C;
@@ -381,7 +396,7 @@ inline AttnSubPlan attn_sub_plan(int d, int dkv, int P, int C, int keys_cap, int
   auto fits = [&](int kc, int lim) {
     for (pl.late = 0; pl.late < (P == 3 && (P * dkv + C - 1) / C <= 24 ? 2 : 1); ++pl.late)   // (cross-attention: its keys are requested first
       // thing, into an area of their own; more than 24 weight rows do not all wait in registers)
-      if (attn_sub_layout(d, dkv, P, C, mb, kc, blen(kc), pl.late).total <= lim) return true;
+      if (attn_sub_layout(d, dkv, P, C, mb, kc, blen(kc), pl.late, kc, sub_kv_stride(dkv)).total <= lim) return true;
     pl.late = 0;
     return false;
   };
@@ -391,6 +406,16 @@ inline AttnSubPlan attn_sub_plan(int d, int dkv, int P, int C, int keys_cap, int
   pl.kc = kc; pl.bias_len = blen(kc); pl.ok = fits(kc, limit);
   if (fits(kc, prefer)) pl.ok = true;
   else fits(kc, limit);
+  pl.kc_main = kc; pl.kvst = sub_kv_stride(dkv);
+  // Cross-attention of many keys: closer rows (two-way bank conflicts on the keys) and the room of the weight rows for the last keys hold a
+  // rank's whole share of up to 1024 encoder keys in one chunk (a second one is staged and waited for inside the chain:
+  // T5-large, 1024 ids, 200 cached rows, 2 / 5 / 8 rows 537 / 574 / 650 -> 509 / 544 / 620 us a pass, 800 ids 515 / 552 / 620 -> 492 / 527 / 593).
+  if (P == 1 && mb > 1 && per_rank > kc && all_keys > 0 && (dkv + C - 1) / C <= 8) {
+    const int st = dkv + 4, row_b = (st + dkv + 4) * 4, rest = sub_up16(((dkv + C - 1) / C) * sub_wst(d)) / row_b, wide = std::min(128, per_rank), main = wide - rest;
+    if (wide > kc && main >= 16 && rest > 0 && attn_sub_layout(d, dkv, P, C, mb, wide, blen(wide), 0, main, st).total <= prefer) {
+      kc = pl.kc = wide; pl.kc_main = main; pl.kvst = st; pl.late = 0; pl.bias_len = blen(wide); pl.ok = true;
+    }
+  }
   pl.red_keys = all_keys > 0 ? kc : 0;
   return pl;
 }
@@ -557,7 +582,9 @@ __device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk
 // sub-layer kernels; before: token rows and norm for the whole block, then products from shared memory, cluster barriers, scores,
 // soft-max and values with a block barrier each): 1 row 473 -> 355 us, 5 rows 632 -> 550 us, 8 rows 691 -> 597 us, 16 rows
 // 1080 -> 831 us; T5-small 100 -> 83 us.  With the steps noted at their places since: 339, 506, 558, 748 and 80 us.
-template <bool ONE>
+// WIDE: cross-attention of a block whose last keys of a chunk lie where the weight rows were (attn_sub_plan); a kernel of its own, since the
+// others would spill registers for it.
+template <bool ONE, bool WIDE = false>
 __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubArgs a) {
   extern __shared__ __align__(1024) unsigned char sub_smem[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -565,14 +592,14 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
   const int h = blockIdx.x >> a.c_shift, r = (int)cluster_rank();
   const int pr0 = (r * R) >> a.c_shift, npr = (((r + 1) * R) >> a.c_shift) - pr0;   // rows of the head's q|k|v projection
   const int no = d >> a.c_shift, o0 = r * no;                                         // output rows of W_o
-  const int wst = sub_wst(d), xst = sub_xst(d), kvst = sub_kv_stride(dkv), qst = R + 16, recst = dkv + SUB_RECPAD;
+  const int wst = sub_wst(d), xst = sub_xst(d), kvst = WIDE ? dkv + 4 : sub_kv_stride(dkv), qst = R + 16, recst = dkv + SUB_RECPAD;
   const int vst = dkv + 4;   // row stride of the staged values: the rows 2 t and channels 4 g of a tile hit 32 banks
   unsigned char* sWq = sub_smem + a.L.wq;
   uint32_t* Xs = reinterpret_cast<uint32_t*>(sub_smem + a.L.xs);
   float* sRec = reinterpret_cast<float*>(sub_smem + a.L.rec);     // [8 warps][mb][recst]
   float* sRrec = reinterpret_cast<float*>(sub_smem + a.L.rrec);   // [C ranks][mb][recst]
   float* sK = reinterpret_cast<float*>(sub_smem + a.L.kv);
-  float* sV = sK + (size_t)a.kc_keys * kvst;
+  float* sV = sK + (size_t)(WIDE ? a.kc_main : a.kc_keys) * kvst;
   float* sQKV = reinterpret_cast<float*>(sub_smem + a.L.qkv);     // [mb][qst]
   float* psum = reinterpret_cast<float*>(sub_smem + a.L.psum);
   float* sBias = reinterpret_cast<float*>(sub_smem + a.L.bias);
@@ -627,14 +654,17 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
   if (on) g4 = __ldg(reinterpret_cast<const float4*>(a.gain + col));
   const float* Kh = a.kc + (size_t)h * a.cap * dkv;
   const float* Vh = a.vc + (size_t)h * a.cap * dkv;
-  // stages keys / values [c0, c1) of the cache into sK / sV rows 0.. (asynchronous 16-byte copies)
-  auto stage_cached = [&](int c0, int c1) {
+  // places of a chunk's key jj
+  auto k_at = [&](int jj) { return sK + ((size_t)jj * kvst + (WIDE && jj >= a.kc_main ? a.L.kv2_k : 0)); };
+  auto v_at = [&](int jj) { return sV + ((size_t)jj * vst + (WIDE && jj >= a.kc_main ? a.L.kv2_v : 0)); };
+  // stages keys / values [c0 + r0, c1) of the cache into the places r0.. (asynchronous 16-byte copies)
+  auto stage_cached = [&](int c0, int c1, int r0 = 0) {
     const int up_sh = a.dkv_shift - 2, units = (c1 - c0) << up_sh;
 #pragma unroll 1
-    for (int i = tid; i < units; i += SUB_THREADS) {
+    for (int i = tid + (r0 << up_sh); i < units; i += SUB_THREADS) {
       const int jj = i >> up_sh, u = (i & ((1 << up_sh) - 1)) * 4;
-      sub_cp16(sK + (size_t)jj * kvst + u, Kh + (size_t)(c0 + jj) * dkv + u);
-      sub_cp16(sV + (size_t)jj * vst + u, Vh + (size_t)(c0 + jj) * dkv + u);
+      sub_cp16(k_at(jj) + u, Kh + (size_t)(c0 + jj) * dkv + u);
+      sub_cp16(v_at(jj) + u, Vh + (size_t)(c0 + jj) * dkv + u);
     }
   };
   // Few keys: every rank attends over all of them (the keys of the cache come from the L2, those of this pass from the
@@ -645,7 +675,7 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
     n_keys = min(*a.n_keys_dev, a.cap);
     red = n_keys <= a.red_keys;
     j0 = red ? 0 : (r * n_keys) >> a.c_shift; j1 = red ? n_keys : ((r + 1) * n_keys) >> a.c_shift;
-    stage_cached(j0, min(j1, j0 + a.kc_keys));
+    stage_cached(j0, min(j1, j0 + (WIDE ? a.kc_main : a.kc_keys)));
     // a share of more than one chunk: the later chunks are asked into the L2 now (they are staged when the first is used up)
     const int later = (j1 - j0 - a.kc_keys) * dkv / 32;   // 128-byte lines of keys (as many again of values)
 #pragma unroll 1
@@ -694,6 +724,10 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
     __syncthreads();
     stage_cached(j0, min(min(j1, pos0), j0 + a.kc_keys));
   }
+  if (WIDE && j1 - j0 > a.kc_main) {   // the last keys of the first chunk
+    __syncthreads();
+    stage_cached(j0, min(j1, j0 + a.kc_keys), a.kc_main);
+  }
   SUB_STAMP();            // 1: weights in registers
   pdl_wait();
   SUB_STAMP();            // 2: dependency wait
@@ -707,17 +741,17 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
   sub_rows_split<ONE>(rw, k, col, stores, on, g4, Xs, xst, sh, sSeed, h == 0 ? o0 : 0, h == 0 ? o0 + no : 0, lane, warp);
   if (!a.early) pdl_launch_dependents();
   SUB_STAMP();            // 3: token rows
-  const int pst = sub_pst(npr);
+  const int pst = sub_pst(npr, WIDE);
   // ---- phase A: this rank's q|k|v rows for all token rows -----------------------------------
   {
     SubB<ONE> b;
     sub_bfrags<ONE>(Xs, xst, k, col0, nch, lane, b);
-    sub_tile<ONE>(hf[0], hf[1], npr > 8, b, nch, npr, 0, psum, warp, lane);
-    if (mt > 1) {   // (rows 24 and up: heads over fewer than eight blocks; never with kv_late)
+    sub_tile<ONE, WIDE>(hf[0], hf[1], !WIDE && npr > 8, b, nch, npr, 0, psum, warp, lane);
+    if (!WIDE && mt > 1) {   // (rows 24 and up: heads over fewer than eight blocks; never with kv_late)
       if (npr > 24) sub_frags8(sWq, wst, npr, d, 3, col0, nch, lane, hf[0]);
       sub_tile<ONE>(hf[2], hf[0], npr > 24, b, nch, npr, 1, psum, warp, lane);
     }
-    if (mt > 2) {
+    if (!WIDE && mt > 2) {
       sub_frags8(sWq, wst, npr, d, 4, col0, nch, lane, hf[0]);
       if (npr > 40) sub_frags8(sWq, wst, npr, d, 5, col0, nch, lane, hf[1]);
       sub_tile<ONE>(hf[0], hf[1], npr > 40, b, nch, npr, 2, psum, warp, lane);
@@ -797,8 +831,8 @@ __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubA
     }
     // keys of this pass come from the exchange buffer
     const int own0 = a.self ? pos0 - c0 : nk;
-    auto kp = [&](int j) { return j >= own0 ? sQKV + (size_t)(j - own0) * qst + dkv : sK + (size_t)j * kvst; };
-    auto vp = [&](int j) { return j >= own0 ? sQKV + (size_t)(j - own0) * qst + 2 * dkv : sV + (size_t)j * vst; };
+    auto kp = [&](int j) { return j >= own0 ? sQKV + (size_t)(j - own0) * qst + dkv : k_at(j); };
+    auto vp = [&](int j) { return j >= own0 ? sQKV + (size_t)(j - own0) * qst + 2 * dkv : v_at(j); };
     if (ONE) sub_attend_one(q1, dkv >> 4, dkv, nk, kp, vp, sBias, pos0 - c0 - dist_lo, a.self != 0, s1, warp, lane);
     else sub_attend_block(q8, dkv, nk, kp, vp, sBias, pos0 + og - c0 - dist_lo, a.self != 0, a.self ? min(nk - 1, pos0 + og_k - c0) : nk - 1, s8, warp, lane);
   }

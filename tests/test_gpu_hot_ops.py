@@ -98,6 +98,16 @@ def test_attention_sublayer_matches_numpy(M, self_attn, d, H, dkv, cap, n_before
         assert np.array_equal(Kg[:, :n_before], K[:, :n_before]) and np.array_equal(Kg[:, n_before + M:], K[:, n_before + M:])
 
 
+@pytest.mark.parametrize("M", [2, 8])
+@pytest.mark.parametrize("d,H,cap,n", [(1024, 16, 704, 700), (1024, 16, 1024, 1024), (1024, 16, 1024, 1023), (1024, 16, 1024, 777), (1024, 16, 1024, 776),
+                                       (1024, 16, 1024, 129), (1024, 16, 1024, 128), (1024, 16, 1024, 97), (1024, 16, 1024, 98), (1024, 16, 1024, 3),
+                                       (1024, 16, 2048, 2048), (512, 8, 900, 897), (512, 6, 1024, 1009)])
+def test_cross_attention_of_blocks_over_many_keys(M, d, H, cap, n):
+    """Capacities whose chunk of keys goes on where the weight rows were: shares below, at and past the main area's end, several
+    chunks, and few keys that every block of a head attends over (bounds as in the test above)."""
+    test_attention_sublayer_matches_numpy(M, False, d, H, 64, cap, n)
+
+
 @pytest.mark.parametrize("M,V,K", [(1, 32128, 1024), (5, 32128, 1024), (16, 32128, 1024), (1, 250112, 512), (1, 250112, 1024),
                                    (5, 250112, 1024), (16, 250112, 1024), (3, 773, 64)])
 def test_sliced_head_matches_numpy_over_the_whole_vocabulary(M, V, K):
