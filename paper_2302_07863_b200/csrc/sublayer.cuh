@@ -581,7 +581,7 @@ __device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk
 // Measured, T5-large shapes, pass of 24 layers, cache 32, 512 encoder keys, before -> after this form of the kernels (both
 // sub-layer kernels; before: token rows and norm for the whole block, then products from shared memory, cluster barriers, scores,
 // soft-max and values with a block barrier each): 1 row 473 -> 355 us, 5 rows 632 -> 550 us, 8 rows 691 -> 597 us, 16 rows
-// 1080 -> 831 us; T5-small 100 -> 83 us.  With the steps noted at their places since: 339, 506, 558, 748 and 80 us.
+// 1080 -> 831 us; T5-small 100 -> 83 us.  With the steps noted at their places since: 340, 505, 557, 740 and 78 us.
 // WIDE: cross-attention of a block whose last keys of a chunk lie where the weight rows were (attn_sub_plan); a kernel of its own, since the
 // others would spill registers for it.
 template <bool ONE, bool WIDE = false>
