@@ -111,15 +111,14 @@ __global__ void __launch_bounds__(EF_THREADS, 1) enc_flash_kernel(const EncFlash
   unsigned char* sKV = sQ + 2 * 16384;
   float* sBias = reinterpret_cast<float*>(sKV + EF_STAGES * EF_STAGE);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, h = blockIdx.x / CS, r0 = blockIdx.y * EF_ROWS, rank = CS > 1 ? (int)cluster_rank() : 0;
-  __shared__ uint64_t k_full[EF_STAGES], k_free[EF_STAGES], v_full[EF_STAGES], v_free[EF_STAGES], q_full, q_there, s_full[4], p_full[4], o_full[2], o_done;
+  __shared__ uint64_t k_full[EF_STAGES], k_free[EF_STAGES], v_full[EF_STAGES], v_free[EF_STAGES], q_full, q_there, s_full[4], p_full[4], o_full[4], o_done;
   __shared__ uint32_t tmem_slot;
   if (tid == 0) {
     for (int i = 0; i < EF_STAGES; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_free[i], 1); mbar_init(&v_full[i], 1); mbar_init(&v_free[i], 1); }
     mbar_init(&q_full, 1);
     mbar_init(&q_there, 4);
     mbar_init(&o_done, 1);
-    for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 1); }   // (by tile: a group may be two ahead of the products)
-    for (int i = 0; i < 2; ++i) mbar_init(&o_full[i], 1);
+    for (int i = 0; i < 4; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 1); mbar_init(&o_full[i], 1); }   // by tile: a group may be two ahead of the products
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 9) {
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(EF_THREADS, 1) enc_flash_kernel(const EncFlash
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t v = smem_u32(sKV + st * EF_STAGE) + 16384;
       ef_product(tmem + 256 + g * 64, tmem + (t & 3) * 64, v, v + 8192, t >= 2);   // (the probabilities lie where the scores were)
-      umma_commit(&o_full[g]);
+      umma_commit(&o_full[t & 3]);
       umma_commit(&v_free[st]);
       if (t + 4 < tiles) scores(t + 4);   // (behind the products that read the probabilities there: MMAs run in order)
     }
@@ -240,8 +239,8 @@ __global__ void __launch_bounds__(EF_THREADS, 1) enc_flash_kernel(const EncFlash
         // only beyond are the sums brought to the new one.
         const bool far = !((mx - m) * LOG2E <= 8.f);
         if (__any_sync(0xffffffffu, far)) {
-          // (the products of this group's tile before: the latest that can be complete, and those before it are, behind these scores)
-          if (!mbar_wait(&o_full[g], ((t - 2) >> 1) & 1)) *a.err = BILD_ERR_TIMEOUT;
+          // (the products of this group's tile before; those of tile t - 6, the barrier's phase before, are long behind these scores)
+          if (!mbar_wait(&o_full[(t - 2) & 3], ((t - 2) >> 2) & 1)) *a.err = BILD_ERR_TIMEOUT;
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const float nw = far ? fmaxf(m, mx) : m, sc = m == nw ? 1.f : ef_exp2((m - nw) * LOG2E);
           m = nw;
