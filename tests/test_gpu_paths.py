@@ -111,6 +111,28 @@ def test_encoder_lengths_match_oracle(torch_cuda, E, ffn, d, H, F):
                 assert float(np.max(np.abs(got - want))) <= 2e-3 * max(1.0, float(np.max(np.abs(want)))), (which, layer, what)
 
 
+
+@pytest.mark.parametrize("E", [300, 700])
+def test_encoder_attention_with_maxima_far_apart(torch_cuda, E):
+    """Relative-position biases of N(0, 20): the maximum of a row's scores grows by far more than 2^8 from one tile of keys to a later one, so that
+    the sums kept so far are rescaled (the bias is added in fp32: bounds as above)."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200.binding import BF16, Config, Context, model_cfg, upload_model
+    s = dataclasses.replace(MODEL_SHAPES["wide_s"], name="far", n_layers=1, d_model=512, n_heads=8, d_kv=64, d_ff=512, ffn="relu", vocab=300)
+    w = gen_model(s, 5, "bf16")
+    w["enc.rel_bias"] = w["enc.rel_bias"] * np.float32(20)
+    dev = upload_model(w, "cuda:0")
+    ctx, m = Context(Config(model_cfg(s, 3.0), model_cfg(s, 3.0), BF16, 704, 20, 8, 0, -1, 0), s, dev, s, dev), Model(s, w, 3.0)
+    ids = np.random.default_rng(E).integers(2, 300, size=E).astype(np.int32)
+    ctx.encode(ids)
+    st = m.start(ids, 4)
+    for what, ref in ((0, st.ck[0]), (1, st.cv[0])):
+        got = ctx.read_cache(1, what, 0, 8, 704, 64)[:, :E]
+        want = ref.reshape(E, 8, 64).transpose(1, 0, 2)
+        assert float(np.max(np.abs(got - want))) <= 2e-3 * max(1.0, float(np.max(np.abs(want)))), what
+    ctx.close()
+
+
 _len_cache = {}
 
 
