@@ -516,10 +516,13 @@ __global__ void __launch_bounds__(EG_THREADS) enc_gemm_kernel(LinArgs a, int* er
           const float4 p = *reinterpret_cast<const float4*>(sSq + rk * TT + rank * cpo + c);
           t.x += p.x; t.y += p.y; t.z += p.z; t.w += p.w;
         }
-        const float inv[4] = {rsqrtf(t.x / (float)a.K + a.eps), rsqrtf(t.y / (float)a.K + a.eps), rsqrtf(t.z / (float)a.K + a.eps),
-                              rsqrtf(t.w / (float)a.K + a.eps)};
+        const float ss[4] = {t.x, t.y, t.z, t.w};
+        const int lim = a.M - (tok0 + rank * cpo + c);   // past the last token: zero, also where eps = 0 leaves nothing to divide by
 #pragma unroll
-        for (int e = 0; e < 4; ++e) { v[e] *= inv[e]; gt[e] *= inv[e]; }
+        for (int e = 0; e < 4; ++e) {
+          const float inv = e < lim ? rsqrtf(ss[e] / (float)a.K + a.eps) : 0.f;
+          v[e] *= inv; gt[e] *= inv;
+        }
       }
       if constexpr (GATED) {
 #pragma unroll

@@ -133,6 +133,37 @@ def test_encoder_attention_with_maxima_far_apart(torch_cuda, E):
     ctx.close()
 
 
+@pytest.mark.parametrize("E", [17, 63, 64])
+@pytest.mark.parametrize("ffn,H", [("relu", 8), ("gated_gelu", 6)])
+def test_norms_without_epsilon(torch_cuda, E, ffn, H):
+    """ln_eps = 0: rows that do not exist (the encoder's tiles past the last id, the places of a block pass past its last row) have no
+    squares to divide by, and nothing of them may reach a row that does exist.  Cross keys and values, logits of 1, 5 and 9 rows."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200.binding import BF16, Config, Context, model_cfg, upload_model
+    torch = torch_cuda
+    s = dataclasses.replace(MODEL_SHAPES["wide_s"], name="eps_" + ffn, n_layers=2, d_model=512, n_heads=H, d_kv=64, d_ff=1024, ffn=ffn, vocab=300, eps=0.0)
+    w = gen_model(s, 5, "bf16")
+    dev = upload_model(w, "cuda:0")
+    ctx, m = Context(Config(model_cfg(s, 3.0), model_cfg(s, 3.0), BF16, 96, 20, 8, 0, -1, 0), s, dev, s, dev), Model(s, w, 3.0)
+    ids = np.random.default_rng(E).integers(2, 300, size=E).astype(np.int32)
+    ctx.encode(ids)
+    st = m.start(ids, 20)
+    for layer in range(2):
+        for what, ref in ((0, st.ck[layer]), (1, st.cv[layer])):
+            got = ctx.read_cache(1, what, layer, H, 96, 64)[:, :E]
+            want = ref.reshape(E, H, 64).transpose(1, 0, 2)
+            assert float(np.max(np.abs(got - want))) <= 2e-3 * max(1.0, float(np.max(np.abs(want)))), (layer, what)
+    buf = torch.empty((16, 300), dtype=torch.float32, device="cuda")
+    toks = [int(t) for t in np.random.default_rng(1).integers(2, 300, size=15)]
+    at = 0
+    for k in (1, 5, 9):
+        ctx.large_verify(toks[at:at + k], 10.0, buf)
+        z = m.forward_block(st, toks[at:at + k])
+        assert np.max(np.abs(buf[:k].cpu().numpy() - z)) <= 2e-3 * max(1.0, np.max(np.abs(z))), k
+        at += k
+    ctx.close()
+
+
 _len_cache = {}
 
 
