@@ -217,7 +217,8 @@ typedef struct {
   int32_t draft_ahead;       /* 1: in bild_generate* the small model goes on from its own candidate while the large model judges
                               * the block in front, as long as large passes mostly end with that candidate; what it drafted
                               * is dropped if one ends otherwise (tokens, trace and counts are those of the serial loop).
-                              * 0, and with graph_switch = 0 or host_loop = 1: the serial loop */
+                              * 0, and with graph_switch = 0 or host_loop = 1: the serial loop, 1 to 2 % faster for two models
+                              * that never agree (unrelated random ones), a fifth slower for a pair that mostly does */
 } bild_tuning;
 void bild_tuning_default(bild_tuning *t /*HOST out*/);
 /* bild_create with explicit switches; tuning == NULL means the defaults. */
@@ -270,6 +271,10 @@ int bild_rewind(bild_ctx *ctx, int which, int new_len);
  * tokens_out: HOST [max_len]; *n_tokens: number written.  trace_out: HOST
  * [trace_cap] or NULL; *n_trace = records produced (records beyond trace_cap are
  * counted but dropped).  mode: BILD_MODE_*.  Synchronises.
+ * The loop is a CUDA graph, recorded and instantiated inside the first call that asks for it.  There are four on a
+ * context: BiLD and the small model alone share one, the large model alone has its own, and bild_generate_sampled has another
+ * two; a program that uses several warms up each (T5-large pair: 1.6 ms BiLD, 3 on the process's first context, 0.4 to 0.8 ms
+ * the large model alone, as much again for sampling).
  * Errors: STATE (no encode), CAPACITY (max_len + 1 > max_dec_len), ARG, CUDA. */
 int bild_generate(bild_ctx *ctx, int mode, float alpha_fb, float alpha_rb, int max_len,
                   int32_t *tokens_out /*HOST*/, int *n_tokens /*HOST out*/,

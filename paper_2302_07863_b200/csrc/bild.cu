@@ -175,8 +175,8 @@ struct bild_ctx {
   // single-step calls from the third of a kind on: the pass as a graph.  [0] small step, [1] large pass of one row, [2] of 2 to 8, [3] of more
   struct StepGraph { cudaGraph_t g = nullptr; cudaGraphExec_t ex = nullptr; int64_t launches = 0; int calls = 0; } step[4];
   size_t ws_bytes = 0;
-  // device-side loop: WHILE { small pass; IF (fallback) { large block pass } } and WHILE { large pass }
-  // [0], [1]: greedy; [2], [3]: the same two loops with the token-drawing kernel after every LM head
+  // device-side loops, each built when it is first asked for (build_graph): [0] BiLD or the small model alone, in rounds (build_rounds) or
+  // serial; [1] the large model alone; [2], [3]: the same two with the token-drawing kernel after every LM head
   cudaGraph_t graph[4] = {nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t exec[4] = {nullptr, nullptr, nullptr, nullptr};
   int64_t sampled_counted = 0;
@@ -1504,8 +1504,9 @@ int capture_pass(bild_ctx* c, cudaGraph_t body, int which, int MB, unsigned long
   return BILD_OK;
 }
 
-// Builds the two device-side loops (CUDA graphs with conditional nodes).  The head
-// kernel's last block sets the WHILE handle to "not done" and the IF handle to "fallback".
+// Builds one device-side loop (a CUDA graph with conditional nodes), recorded by build_rounds, or in place: the serial loop and the
+// large model's own, whose WHILE handle the last block of every LM-head kernel sets to "not done", and the handles of the large
+// pass's SWITCH or IF nodes to what the small step asks for.
 int build_graph_once(bild_ctx* c, int base, bool alone);
 
 void drop_graphs(bild_ctx* c) {
@@ -2065,7 +2066,7 @@ int generate_async(bild_ctx* c, int mode, float alpha_fb, float alpha_rb, int ma
     rc = reset_state(c, mode, alpha_fb, alpha_rb, max_len);
     if (rc) return rc;
     if (max_len == 0 || c->cfg.start_id == c->cfg.eos_id) return BILD_OK;
-    // passes the loop may run: bounded by the guard of the device-side policy
+    // (how many passes it may run is bounded by the guard in policy_step)
     CUDA_TRY(c, cudaGraphLaunch(c->exec[base + alone], c->stream));
     return BILD_OK;
   }

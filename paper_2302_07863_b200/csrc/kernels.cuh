@@ -449,10 +449,15 @@ __device__ inline PolicyOut policy_tests(HeadOut* o, const PolicyIn& p, int whic
 // what the serial loop has after that pass.  Tokens, trace and counts are those of the serial loop in any case.
 // Neither side waits for the other inside a kernel: each leaves its WHILE node when it has nothing to do, which the flags in `queue`
 // tell the other, and the round ends when both have.
-// When it pays: T5 pair, five rows: a large pass takes 520 us, 650 with small steps beside it all the time, of which five are then done that
-// cost 82 us each by themselves; so a block that stands saves about 250 us, one that does not costs up to 130 and the wait for the
+// When it pays: T5 pair, five rows: a large pass takes 505 us, 650 with small steps beside it all the time, of which five are then done that
+// cost 78 us each by themselves; so a block that stands saves about 250 us, one that does not costs up to 150 and the wait for the
 // step at hand.  trust follows what the passes ended with, also while nothing is drafted ahead, and bounds the
-// number of blocks on their way: a pair that never agrees pays once a generation.
+// number of blocks on their way.
+// What that costs a pair that never agrees (two random models), against the serial loop, 64 tokens: T5 pair 13.22 -> 13.41 ms, mT5 pair 16.93 ->
+// 17.23 (256 tokens, 1024 ids, T5 pair: 66.5 -> 67.3): the one block a generation begins with, and up to 8 us a large pass for the two
+// turns of a round.  Starting at trust 0, with no block ahead before a pass has ended as proposed, leaves 13.29 -> 13.37 and 16.94 -> 16.95 of it, and
+// costs the pairs that do agree 1 to 2.5 % (10.81 -> 11.06 ms, T5 pair, 64 tokens; mT5 pair 17.08 -> 17.23): those are what the method is
+// for, so it starts at 1.
 
 // The small model's side at a fallback: hands its drafts over.  Returns whether it goes on.
 __device__ inline bool small_hands_over(const LoopPtrs& L, const PolicyIn& p, int steps, int fallbacks, int forced, int candidate) {
@@ -524,7 +529,10 @@ __device__ inline void policy_step(const LoopPtrs& L, const PolicyIn& p, PolicyO
   DevState* st = L.st;
   int* y = L.y;
   // Every pass adds a token or consumes a pending draft, so a run takes at most
-  // (max_len + 1) * (max_draft + 2) passes; beyond that the loop is stopped with an error.
+  // (max_len + 1) * (max_draft + 2) passes; beyond that the loop is stopped with an error.  In rounds the small steps alone are counted, those
+  // ahead among them (what is dropped goes out of the count: DraftBlock::passes).  Of a run's L large passes, each of which needs a block that a
+  // small step handed over and leaves at least one more token settled, the steps in front are at most L (max_draft + 1); a step ahead of
+  // the last of them adds a token, so there are at most max_len - L of those, and the same bound holds.
   st->passes = p.passes + 1;
   if (p.passes + 1 > (p.max_len + 1) * (p.max_draft + 2) + 8) {
     st->err = BILD_ERR_TIMEOUT;
