@@ -216,7 +216,9 @@ typedef struct {
                               * visiting every n-th tile of 64 keys, partial results merged at the end */
   int32_t draft_ahead;       /* 1: in bild_generate* the small model goes on from its own candidate while the large model judges
                               * the block in front, as long as large passes mostly end with that candidate; what it drafted
-                              * is dropped if one ends otherwise (tokens, trace and counts are those of the serial loop).
+                              * is dropped if one ends otherwise (tokens, trace and counts are those of the serial loop).  Blocks of
+                              * two and more rows that wait together are judged in one pass of up to 16 rows, at the precision each
+                              * has alone, where the kernels add in no fixed order anyway (fused = 3, bf16).
                               * 0, and with graph_switch = 0 or host_loop = 1: the serial loop, 1 to 2 % faster for two models
                               * that never agree (unrelated random ones), a fifth slower for a pair that mostly does */
 } bild_tuning;
@@ -432,6 +434,11 @@ int bild_debug_read_cache(bild_ctx *ctx, int which, int what, int layer, float *
  * may start before it is complete.  Must be 0: the kernels of a pass read what it writes without waiting for it.
  * Nothing runs on the GPU (the launches are recorded in a graph that is dropped). */
 int bild_debug_setup_edges(bild_ctx *ctx, int which, int k, int *programmatic /*HOST out*/);
+
+/* Test helper: what the loops on the device (host_loop = 0) have run since the context was created: [0] small steps, [1] large passes of
+ * one row, [2] of 2 to 8 rows, [3] of other numbers (of 2 to 16, where the kernels make no difference), [4] rollbacks in a block of drafts that was not
+ * the first of its large pass.  A block of drafts counts once in bild_stats.large_calls, however many share a pass.  Synchronises. */
+int bild_debug_loop_counts(bild_ctx *ctx, int64_t counts[5] /*HOST out*/);
 
 /* Test helper: y[i] = 1 / x[i] as the attention kernels of the decoder passes form it.  x, y: DEVICE [n].  Asynchronous. */
 int bild_debug_reciprocal(const float *x /*DEVICE*/, float *y /*DEVICE*/, int n, void *cuda_stream);

@@ -28,7 +28,7 @@ EXPORTS = ["bild_query_workspace", "bild_create", "bild_create_tuned", "bild_tun
            "bild_op_lm_head_scratch_bytes", "bild_op_lm_head", "bild_op_lm_head_static", "bild_debug_bucket",
            "bild_debug_read_cache", "bild_op_lm_head_sliced", "bild_op_lm_head_stream", "bild_op_sublayer_scratch_bytes", "bild_op_attn_sublayer",
            "bild_op_ffn_sublayer", "bild_generate_sampled", "bild_debug_setup_edges",
-           "bild_debug_reciprocal"]
+           "bild_debug_reciprocal", "bild_debug_loop_counts"]
 
 
 class ModelCfg(C.Structure):
@@ -311,6 +311,13 @@ class Context:
         self.L.bild_debug_setup_edges.argtypes = [C.c_void_p, C.c_int, C.c_int, C.POINTER(C.c_int)]
         self._check(self.L.bild_debug_setup_edges(self.h, which, k, C.byref(n)))
         return n.value
+
+    def loop_counts(self) -> dict:
+        """Passes run by the loops on the device since the context was created, by kind, and rollbacks in a block behind another of its pass."""
+        n = (C.c_int64 * 5)()
+        self.L.bild_debug_loop_counts.argtypes = [C.c_void_p, C.POINTER(C.c_int64)]
+        self._check(self.L.bild_debug_loop_counts(self.h, n))
+        return dict(zip(("small", "large1", "large8", "large_more", "later_rollbacks"), n))
 
     def uses_tensor_cores(self) -> bool:
         return bool(self.L.bild_uses_tensor_cores(self.h))

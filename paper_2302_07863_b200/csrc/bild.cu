@@ -1300,6 +1300,7 @@ cudaError_t launch_enc_linear(bild_ctx* c, Model& m, const LinArgs& a, int rb, i
 LoopPtrs loop_ptrs(bild_ctx* c) {
   LoopPtrs L;
   L.st = c->st; L.y = c->y; L.trace = c->trace; L.descS = c->m[0].desc; L.descL = c->m[1].desc; L.block = c->block;
+  L.share = c->m[1].fused && !c->m[1].cpass && c->fused_on >= 3;   // (where decoder_pass takes 2 to 16 rows to the sub-layer kernels)
   return L;
 }
 
@@ -2534,6 +2535,17 @@ int bild_debug_read_cache(bild_ctx* c, int which, int what, int layer, float* ds
   const float* base = what == 0 ? m.crossK : what == 1 ? m.crossV : what == 2 ? m.selfK : m.selfV;
   CUDA_TRY(c, cudaMemcpyAsync(dst_host, base + (size_t)layer * n, n * sizeof(float), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return BILD_OK;
+}
+
+// Test helper: what the loop graphs have run since the context was created.
+int bild_debug_loop_counts(bild_ctx* c, int64_t* counts) {
+  if (!c || !counts) return fail(c, BILD_ERR_ARG, "null argument");
+  int rc = read_state(c);
+  if (rc) return rc;
+  const DevState& s = *c->pin_state;
+  const long long v[5] = {s.cum_passes[0], s.cum_passes[2], s.cum_passes[3], s.cum_passes[1], s.cum_later};
+  for (int i = 0; i < 5; ++i) counts[i] = v[i];
   return BILD_OK;
 }
 

@@ -89,6 +89,7 @@ struct DevState {
   unsigned ends;             // the running large pass: bit i: row i is the last one of a block
   unsigned call;             // (of the host's mirror) the last single-step call whose results are complete
   long long cum_rounds;      // round_kernel launches since create
+  long long cum_later;       // rollbacks since create in a block behind another one of the same large pass
 };
 
 struct Partial {  // running soft-max statistics of a slice of the vocabulary

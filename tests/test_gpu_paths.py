@@ -471,6 +471,53 @@ def test_several_blocks_of_drafts_in_a_large_pass(torch_cuda, dtype, later, top_
             c.close()
 
 
+@pytest.mark.parametrize("dtype,tuning", [("bf16", {}), ("bf16", dict(fused=0, enc_split_k=0)), ("fp32", {}), ("small_fp32", {})])
+@pytest.mark.parametrize("all_alone", [True, False])
+def test_blocks_that_share_a_pass_are_computed_as_alone(torch_cuda, dtype, tuning, all_alone):
+    """Drafts pile up in front of a slow large model (as below).  Blocks of one row (all of them, or some) keep the kernels of a single row, with 24
+    mantissa bits of the activations: values of the trace and the large model's cached keys and values against the serial loop's, where every block has a pass
+    of its own.  One kernel per operation and fp32: the same to the last bit, whatever the timing."""
+    from paper_2302_07863_b200 import MODE_BILD
+    from paper_2302_07863_b200.binding import BF16, FP32, Config, Context, model_cfg, upload_model
+    sL = dataclasses.replace(MODEL_SHAPES["tiny_l" if dtype == "small_fp32" else "wide_l"], n_layers=12)
+    sS = dataclasses.replace(sL, n_layers=1)
+    w = upload_model(gen_model(sL, 4, "bf16" if dtype == "bf16" else "fp32"), "cuda:0")
+    for name in w:
+        if name.startswith("dec.") and not name.startswith("dec.0.") and name.split(".")[-1] in ("wo", "wco", "wfo"):
+            w[name] *= 0.05   # (small enough that the small model's tokens stand, and what later layers compute still shows)
+    cap, n = 61, 60
+    cfg = Config(model_cfg(sS, 9.0), model_cfg(sL, 9.0), BF16 if dtype == "bf16" else FP32, 32, cap, 4, 0, -1, 1)
+    both = [Context(cfg, sS, w, sL, w, tuning=dict(tuning, **t)) for t in ({}, dict(draft_ahead=0))]
+    for c in both:
+        c.encode(np.random.default_rng(5).integers(2, sL.vocab, size=24).astype(np.int32))
+    afb = 2.0
+    if not all_alone:
+        p = sorted(t[5] for t in both[1].generate(MODE_BILD, 0.0, float("inf"), n)["trace"] if t[0] != 3)
+        i = int(0.7 * len(p))
+        afb = (p[i - 1] + p[i]) / 2
+    want = both[1].generate(MODE_BILD, afb, float("inf"), n)
+    keys = [both[1].read_cache(1, what, layer, sL.n_heads, cap, sL.d_kv)[:, :n - 8] for layer in range(12) for what in (2, 3)]
+    exact = dtype != "bf16" or "fused" in tuning
+    for _ in range(4):
+        before = both[0].loop_counts()
+        got = both[0].generate(MODE_BILD, afb, float("inf"), n)
+        ran = {k: v - before[k] for k, v in both[0].loop_counts().items()}
+        assert got["tokens"] == want["tokens"] and got["stats"] == want["stats"]
+        alone = sum(1 for t in want["trace"] if t[0] == 3 and t[3] == 1)
+        passes = ran["large1"] + ran["large8"] + ran["large_more"]
+        assert ran["large1"] >= alone and (not all_alone or passes == ran["large1"])
+        assert not exact or passes == want["stats"]["large_calls"]
+        a, b = [t[5] for t in got["trace"]], [t[5] for t in want["trace"]]
+        # (fused sub-layers add partial sums in no fixed order, 1e-7 each, through 12 layers: 6e-7 of the cached keys seen with single rows, 3e-6 with one
+        # row in a block of 16 mantissa bits; two more rows a block: those 16 bits fall otherwise where the sums do)
+        assert a == b if exact else np.allclose(a, b, rtol=1e-4, atol=1e-5)
+        for i, k in enumerate(keys):
+            g = both[0].read_cache(1, 2 + i % 2, i // 2, sL.n_heads, cap, sL.d_kv)[:, :n - 8]
+            assert np.array_equal(g, k) if exact else np.max(np.abs(g - k)) <= (1.5e-6 if all_alone else 2e-5) * np.max(np.abs(k)), i
+    for c in both:
+        c.close()
+
+
 @pytest.mark.parametrize("n_layers,d,H,E", [(3, 128, 2, 5), (1, 64, 1, 64), (2, 128, 3, 65), (3, 192, 4, 130), (50, 64, 1, 40), (50, 64, 5, 200)])
 def test_cross_kv_of_all_layers_in_one_launch(torch_cuda, n_layers, d, H, E):
     """Cross-attention keys and values of every decoder layer against the oracle: row tiles that do not fill a pair of blocks, more layers than a
