@@ -249,6 +249,7 @@ namespace {
 
 int fail(bild_ctx* c, int code, const std::string& msg) {
   if (c) c->err = msg;
+  if (code == BILD_ERR_CUDA) cudaGetLastError();   // (reported here: not by the next call's checks of its launches too)
   return code;
 }
 #define CUDA_TRY(ctx, expr)                                                               \

@@ -629,3 +629,38 @@ def test_rewinds_reach_the_device_by_every_way(torch_cuda, name):
     with pytest.raises(Exception):
         ctx.rewind(0, 3)   # the cache holds 2 rows
     ctx.close()
+
+
+def _captured(ctx, call):
+    """`call` while the context's stream is being captured into a graph that is dropped: nothing of it runs, and the wait at its end is an error."""
+    from cuda.bindings import runtime as cudart
+    from paper_2302_07863_b200 import BildError
+    assert cudart.cudaStreamBeginCapture(ctx.stream.cuda_stream, cudart.cudaStreamCaptureMode.cudaStreamCaptureModeRelaxed)[0] == 0
+    with pytest.raises(BildError):
+        call()
+    cudart.cudaStreamEndCapture(ctx.stream.cuda_stream)   # (reports that the capture was cut short)
+
+
+def _context_on_a_stream(torch):
+    from paper_2302_07863_b200.binding import BF16, Config, Context, model_cfg, upload_model
+    s = MODEL_SHAPES["wide_s"]
+    dev = upload_model(gen_model(s, 5, "bf16"), "cuda:0")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()   # (the weights were written on another stream)
+    ctx = Context(Config(model_cfg(s, 3.0), model_cfg(s, 3.0), BF16, 32, 20, 8, 0, -1, 0), s, dev, s, dev, stream=stream)
+    ctx.encode(np.arange(2, 20, dtype=np.int32))
+    return ctx
+
+
+@pytest.mark.parametrize("call", ["step", "verify", "generate", "read"])
+def test_an_error_is_reported_once(torch_cuda, call):
+    """The call behind one that failed on the host checks its own launches, not that one's."""
+    from paper_2302_07863_b200 import MODE_BILD
+    ctx = _context_on_a_stream(torch_cuda)
+    want = ctx.small_step(7, 0.4).lse
+    ctx.reset()
+    _captured(ctx, {"step": lambda: ctx.small_step(7, 0.4), "verify": lambda: ctx.large_verify([7], 10.0), "read": lambda: ctx.fetch_result(4),
+                    "generate": lambda: ctx.generate(MODE_BILD, 0.4, 10.0, 3)}[call])
+    ctx.reset()
+    assert abs(ctx.small_step(7, 0.4).lse - want) <= 1e-5
+    ctx.close()
