@@ -1743,13 +1743,13 @@ int build_graph_once(bild_ctx* c, int base, bool alone) {
   return BILD_OK;
 }
 
-// The lengths bild_rewind has set, for what reads them on the device other than a single-step call.
+// The lengths bild_rewind has set, for what reads them on the device other than a single-step call.  (len_ahead stays until the device is known to
+// have them: what is enqueued here or by a step may fail, or be recorded into the caller's graph.)
 int flush_lengths(bild_ctx* c) {
   if (!c->len_ahead) return BILD_OK;
   set_lengths_kernel<<<1, 1, 0, c->stream>>>(c->st, c->pin_state->S_len, c->pin_state->L_len);
   (*c->cnt)++;
   CUDA_TRY(c, cudaGetLastError());
-  c->len_ahead = false;
   return BILD_OK;
 }
 
@@ -1759,6 +1759,7 @@ int read_state(bild_ctx* c) {
   c->len_known = false;
   CUDA_TRY(c, cudaMemcpyAsync(c->pin_state, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
   CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  c->len_ahead = false;
   {  // kernels launched by the loop graphs so far (the device counts the passes they ran)
     const long long* cp = c->pin_state->cum_passes;
     const int64_t total = cp[0] * c->per_pass[0] + cp[1] * c->per_pass[1] + cp[2] * c->per_pass_large1 + cp[3] * c->per_pass_large8 +
@@ -1779,6 +1780,7 @@ int bild_reset_lengths(bild_ctx* c) {
   int rc = reset_state(c, BILD_MODE_BILD, 0.f, INFINITY, c->cfg.max_dec_len - 1);
   if (rc) return rc;
   c->pin_state->S_len = c->pin_state->L_len = 0;
+  c->len_ahead = false;
   c->len_known = true;
   return BILD_OK;
 }
@@ -1823,7 +1825,6 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
   CallArgs& a = *c->pin_call;   // (the call before has ended: its first kernel has read it)
   a.k = k; a.alpha = alpha; a.S_len = c->pin_state->S_len; a.L_len = c->pin_state->L_len; a.call = ++c->calls ? c->calls : ++c->calls;
   for (int i = 0; i < MAXB; ++i) a.tokens[i] = i < k ? tokens[i] : 0;
-  c->len_ahead = false;
   const int MBv = step_rows(k);
   bild_ctx::StepGraph& s = c->step[which == 0 ? 0 : MBv == 1 ? 1 : MBv == SUB_MB ? 2 : 3];
   struct Publish { bild_ctx* c; ~Publish() { c->publish = false; } } publish{c};
@@ -1849,6 +1850,7 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
     std::atomic_thread_fence(std::memory_order_acquire);
   }
   if (!seen) CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  c->len_ahead = false;
   if (c->pin_state->err) return fail(c, c->pin_state->err, "device-side error flag set");
   c->len_known = true;
   return BILD_OK;
@@ -1857,7 +1859,7 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
 int reset_state(bild_ctx* c, int mode, float afb, float arb, int max_len) {
   reset_state_kernel<<<1, 1, 0, c->stream>>>(loop_ptrs(c), encoder_err(c), mode, afb, arb, max_len, c->cfg.max_draft,
                                              c->cfg.eos_id, c->cfg.start_id, c->trace_cap, c->top_p);
-  c->len_known = c->len_ahead = false;
+  c->len_known = false;
   (*c->cnt)++;
   CUDA_TRY(c, cudaGetLastError());
   // the buffer the first fused sub-layer kernel of a pass adds into: every pass leaves it clear; cleared here as well, so
@@ -2156,13 +2158,14 @@ int generate_async(bild_ctx* c, int mode, float alpha_fb, float alpha_rb, int ma
     if (rc) return rc;
     rc = reset_state(c, mode, alpha_fb, alpha_rb, max_len);
     if (rc) return rc;
-    if (max_len == 0 || c->cfg.start_id == c->cfg.eos_id) return BILD_OK;
     // (how many passes it may run is bounded by the guard in policy_step)
-    CUDA_TRY(c, cudaGraphLaunch(c->exec[base + alone], c->stream));
+    if (max_len > 0 && c->cfg.start_id != c->cfg.eos_id) CUDA_TRY(c, cudaGraphLaunch(c->exec[base + alone], c->stream));
+    c->len_ahead = false;   // the lengths are the loop's now
     return BILD_OK;
   }
   int rc = reset_state(c, mode, alpha_fb, alpha_rb, max_len);
   if (rc) return rc;
+  c->len_ahead = false;
   struct DrawGuard { bild_ctx* c; ~DrawGuard() { c->draw = false; } } guard_draw{c};
   c->draw = sampled;
   // Debug loop driver: the policy still runs on the device; the host reads two flags per step.
