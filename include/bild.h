@@ -253,7 +253,8 @@ int bild_reset(bild_ctx *ctx);
  * next-token distribution (Section 3.3).  logits_dbg: DEVICE [vocab] fp32 or NULL;
  * when given, the scaled logits are also written there (debug; the normal path
  * never stores them).  Returns once the results are complete (everything queued on the stream
- * before the call has run by then; with logits_dbg the stream is synchronised). */
+ * before the call has run by then; with logits_dbg the stream is synchronised).  The calling thread polls for them, for up
+ * to 20 ms, then it waits as a synchronisation does; under cudaDeviceScheduleBlockingSync or ...Yield it only does the latter. */
 int bild_small_step(bild_ctx *ctx, int32_t token, float alpha_fb, bild_step_out *out /*HOST*/,
                     float *logits_dbg /*DEVICE or NULL*/);
 

@@ -1809,6 +1809,14 @@ void step_graph_build(bild_ctx* c, bild_ctx::StepGraph& s, int which, int MBv) {
   cudaGetLastError();
 }
 
+// Whether a wait may poll: not where the process asked for waits that leave the CPU to others (cudaDeviceScheduleBlockingSync, ...Yield).
+bool may_poll() {
+  unsigned flags = 0;
+  if (cudaGetDeviceFlags(&flags) != cudaSuccess) { cudaGetLastError(); return false; }
+  flags &= cudaDeviceScheduleMask;
+  return flags == cudaDeviceScheduleAuto || flags == cudaDeviceScheduleSpin;
+}
+
 // One single-step call: k tokens through model `which`, results in pin_head.  The call's tokens, threshold and cache lengths (those of a
 // rewind in front among them) lie in pinned memory, which the pass's first kernel reads: one graph launch from the third call of a kind on (19 or
 // 73 launches cost the host 45 or 170 us), whose last kernel writes the results back.  The state is read back first only if a loop may have
@@ -1840,9 +1848,10 @@ int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha,
     if (!logits_dbg) step_graph_build(c, s, which, MBv);
   }
   // The head's last write ends the call, a few us ahead of what a synchronisation takes to notice the end of the graph; what is left of the pass
-  // then writes nothing.  A pass that does not get there, in time or at all, is left to the synchronisation.
+  // then writes nothing.  A pass that does not get there, in time or at all, is left to the synchronisation, and so are all where the device's
+  // scheduling flags forbid to poll.
   bool seen = false;
-  if (!logits_dbg) {
+  if (!logits_dbg && may_poll()) {
     const volatile unsigned* call = &c->pin_state->call;
     const auto t0 = std::chrono::steady_clock::now();
     for (int it = 1; !(seen = *call == a.call); ++it)

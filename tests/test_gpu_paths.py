@@ -697,3 +697,37 @@ def test_rewinds_outlive_a_call_that_does_not_run(torch_cuda, call, graphs):
     # (fused sub-layers add partial sums in no fixed order; at another place of the caches the results are off by 1e-3)
     assert np.allclose(results(ctx), want, rtol=1e-5, atol=1e-5)
     ctx.close()
+
+
+def test_steps_wait_as_the_device_flags_say(torch_cuda):
+    """cudaDeviceScheduleBlockingSync: a step behind 15 ms of other work on its stream leaves the CPU alone while it waits.  (In a process of
+    its own: the flags belong to the device's context.)"""
+    import os
+    import subprocess
+    import sys
+    code = """
+import time
+from cuda.bindings import runtime as r
+assert r.cudaSetDeviceFlags(r.cudaDeviceScheduleBlockingSync)[0] == 0
+import torch
+from paper_2302_07863_b200.synthetic import make_context
+ctx, ids, _ = make_context("wide_bf16", 9.0, 9.0)
+ctx.encode(ids)
+for t in range(4):
+    ctx.small_step(t, 0.4)
+share = []
+for t in range(5):
+    torch.cuda._sleep(30_000_000)   # clocks
+    a, b = time.perf_counter(), time.thread_time()
+    ctx.small_step(t, 0.4)
+    a, b = time.perf_counter() - a, time.thread_time() - b
+    assert a > 5e-3, a
+    share.append(b / a)
+ctx.close()
+print("share", sorted(share)[2])
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0, out.stderr
+    # a blocked thread uses some tens of microseconds of 15 ms, a polling one all of them
+    assert float(out.stdout.split("share")[1]) < 0.3, out.stdout
