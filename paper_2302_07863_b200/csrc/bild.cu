@@ -2246,6 +2246,7 @@ int bild_op_linear(const void* W, int w_dtype, const float* X, const float* gain
   if (w_dtype != BILD_FP32 && w_dtype != BILD_BF16) return BILD_ERR_ARG;
   bild_ctx tmp;
   tmp.stream = (cudaStream_t)cuda_stream;
+  tmp.use_pdl = false;   // (the kernels read weights ahead of their dependency wait, and here the kernel in front may have written them)
   LinArgs a{};
   a.W0 = W; a.X = X; a.ldx = K; a.gain = gain; a.eps = eps; a.Y = Y; a.ldy = N; a.N = N; a.K = K; a.M = M;
   a.epi = EPI_STORE;

@@ -731,3 +731,19 @@ print("share", sorted(share)[2])
     assert out.returncode == 0, out.stderr
     # a blocked thread uses some tens of microseconds of 15 ms, a polling one all of them
     assert float(out.stdout.split("share")[1]) < 0.3, out.stdout
+
+
+@pytest.mark.parametrize("M", [1, 5, 16])
+def test_linear_on_weights_the_kernel_in_front_wrote(torch_cuda, M):
+    """bild_op_linear whose matrix is the result of the call before, which lets the kernel behind it start early: the product of the two, with other
+    numbers in the same memory each time."""
+    from paper_2302_07863_b200 import op_linear
+    torch = torch_cuda
+    g = torch.Generator("cuda").manual_seed(1)
+    for i in range(8):
+        A, B, X = (torch.randn(size, device="cuda", generator=g) for size in ((1024, 2048), (16, 2048), (M, 1024)))
+        W = op_linear(A, B, None, 0.0, 16, 1024, 2048)             # [16][1024] = B A^T
+        Y = op_linear(W, X, None, 0.0, M, 16, 1024)                # [M][16] = X W^T
+        want = X.double() @ (B.double() @ A.double().T).T
+        # fp32 sums of 2048 and then 1024 terms in other orders: a few 1e-7 of the sums' magnitude
+        assert (Y.double() - want).abs().max().item() <= 1e-5 * want.abs().max().item(), i
