@@ -183,6 +183,32 @@ def test_encoder_attention_with_maxima_far_apart(torch_cuda, E):
     ctx.close()
 
 
+@pytest.mark.parametrize("spread", [1, 20])
+def test_encoder_attention_of_one_block_over_several_tiles(torch_cuda, spread):
+    """More (head, query tile) pairs than half of the SMs, so that one block takes all key tiles of a query tile: its two groups exchange their
+    results where queries and keys were; biases of N(0, 1) and, so that sums are rescaled on the way, of N(0, 20).  Tiles of 128 keys and their halves."""
+    from oracle.t5 import Model
+    from paper_2302_07863_b200.binding import BF16, Config, Context, model_cfg, upload_model
+    H, cap = 16, 1008
+    sms = torch_cuda.cuda.get_device_properties(0).multi_processor_count
+    s = dataclasses.replace(MODEL_SHAPES["wide_s"], name="one", n_layers=1, d_model=256, n_heads=H, d_kv=64, d_ff=512, ffn="relu", vocab=300)
+    w = gen_model(s, 5, "bf16")
+    w["enc.rel_bias"] = w["enc.rel_bias"] * np.float32(spread)
+    dev = upload_model(w, "cuda:0")
+    ctx, m = Context(Config(model_cfg(s, 3.0), model_cfg(s, 3.0), BF16, cap, 20, 8, 0, -1, 0), s, dev, s, dev), Model(s, w, 3.0)
+    for E in (513, 576, 577, 640, 641, 1000):
+        assert 2 * H * ((E + 127) // 128) > sms
+        ids = np.random.default_rng(E).integers(2, 300, size=E).astype(np.int32)
+        ctx.encode(ids)
+        st = m.start(ids, 4)
+        for what, ref in ((0, st.ck[0]), (1, st.cv[0])):
+            got = ctx.read_cache(1, what, 0, H, cap, 64)[:, :E]
+            want = ref.reshape(E, H, 64).transpose(1, 0, 2)
+            # (bound: 16 mantissa bits of the activations, as above)
+            assert float(np.max(np.abs(got - want))) <= 2e-3 * max(1.0, float(np.max(np.abs(want)))), (E, what)
+    ctx.close()
+
+
 @pytest.mark.parametrize("E", [17, 63, 64])
 @pytest.mark.parametrize("ffn,H", [("relu", 8), ("gated_gelu", 6)])
 def test_norms_without_epsilon(torch_cuda, E, ffn, H):
