@@ -544,6 +544,50 @@ def test_blocks_that_share_a_pass_are_computed_as_alone(torch_cuda, dtype, tunin
         c.close()
 
 
+@pytest.mark.parametrize("top_p", [0.0, 0.05, 0.2])
+def test_large_passes_do_take_several_blocks(torch_cuda, top_p):
+    """What the test above is about happens: over a sweep, fewer large passes than blocks, passes of more than 8 rows, rollbacks in a block behind
+    another one of its pass, drawn tokens that stand behind others (top_p = 0.05: mostly of a nucleus of one); tokens, trace and counts against the serial loop."""
+    from paper_2302_07863_b200 import MODE_BILD
+    from paper_2302_07863_b200.binding import BF16, Config, Context, model_cfg, upload_model
+    sL = dataclasses.replace(MODEL_SHAPES["wide_l"], n_layers=12)
+    sS = dataclasses.replace(sL, n_layers=1)
+    w = upload_model(gen_model(sL, 4, "bf16"), "cuda:0")
+    for name in w:
+        if name.startswith("dec.") and not name.startswith("dec.0.") and name.split(".")[-1] in ("wo", "wco", "wfo"):
+            w[name] *= 0.0
+    cap = 120
+    u = np.random.default_rng(6).random((2, cap)).astype(np.float32)
+    ran, blocks = {}, 0
+    for max_draft in (3, 4):
+        cfg = Config(model_cfg(sS, 9.0), model_cfg(sL, 9.0), BF16, 32, cap, max_draft, 0, -1, 1)
+        both = [Context(cfg, sS, w, sL, w, tuning=t) for t in (None, dict(draft_ahead=0))]
+
+        def run(c, afb, arb):
+            return c.generate_sampled(MODE_BILD, afb, arb, cap - 1, top_p, u[0], u[1]) if top_p else c.generate(MODE_BILD, afb, arb, cap - 1)
+
+        for c in both:
+            c.encode(np.random.default_rng(5).integers(2, sL.vocab, size=24).astype(np.int32))
+        p = sorted(t[5] for t in run(both[1], 0.0, float("inf"))["trace"] if t[0] != 3)
+        for q in (0.0, 0.15, 0.3, 0.5):
+            i = int(q * len(p))
+            for arb in (1.0, 2.0, 4.0):
+                afb = (p[i - 1] + p[i]) / 2 if i else 0.0
+                want, got = run(both[1], afb, arb), run(both[0], afb, arb)
+                assert got["tokens"] == want["tokens"] and got["stats"] == want["stats"], (max_draft, q, arb)
+                assert [t[:5] for t in got["trace"]] == [t[:5] for t in want["trace"]]
+                # (fused sub-layers add partial sums in no fixed order; every row is computed with the bits it has alone)
+                assert np.allclose([t[5] for t in got["trace"]], [t[5] for t in want["trace"]], rtol=1e-4, atol=1e-5)
+                blocks += want["stats"]["large_calls"]
+        for k, n in both[0].loop_counts().items():
+            ran[k] = ran.get(k, 0) + n
+        for c in both:
+            c.close()
+    assert ran["large1"] + ran["large8"] + ran["large_more"] <= blocks - 40, (ran, blocks)
+    assert ran["large_more"] >= 5, ran
+    assert ran["later_rollbacks"] >= 1 or top_p == 0.2, ran
+
+
 @pytest.mark.parametrize("n_layers,d,H,E", [(3, 128, 2, 5), (1, 64, 1, 64), (2, 128, 3, 65), (3, 192, 4, 130), (50, 64, 1, 40), (50, 64, 5, 200)])
 def test_cross_kv_of_all_layers_in_one_launch(torch_cuda, n_layers, d, H, E):
     """Cross-attention keys and values of every decoder layer against the oracle: row tiles that do not fill a pair of blocks, more layers than a
