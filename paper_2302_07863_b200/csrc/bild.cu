@@ -530,8 +530,7 @@ template <typename WT, int MB, int RW>
 cudaError_t launch_linear_t(bild_ctx* c, const LinArgs& a, int rows_y) {
   const int nwarps = LIN_THREADS / 32;
   dim3 grid((a.N + nwarps * RW - 1) / (nwarps * RW), rows_y);
-  const int kc = (MB == 1) ? a.K : std::min(a.K, LIN_KC);
-  const size_t smem = (size_t)MB * kc * sizeof(float);
+  const size_t smem = (size_t)MB * std::min(a.K, LIN_KC) * sizeof(float);
   const bool gated = a.epi == EPI_GATED;
   auto kern = gated ? linear_kernel<WT, MB, RW, true> : linear_kernel<WT, MB, RW, false>;
   if (smem > 47 * 1024) {   // (beside it the kernel's own scale factors: rows of 768 columns are just over the default)
@@ -918,7 +917,8 @@ cudaError_t launch_sub(bild_ctx* c, void (*kern)(Arg), int grid, int cluster, si
   return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-// Single-row passes: whether the LM head is the streaming one.  (Smaller heads than slice_head_min_bytes stay on the GEMV head.)
+// Single-row passes: whether the LM head is the streaming one (head_stream = 2: of any size; 1: from slice_head_min_bytes on, smaller heads then
+// stay on the GEMV head).
 bool uses_head_stream(bild_ctx* c, const Model& m) {
   const bool big_head = (size_t)m.c.vocab * m.c.d_model * 2 >= c->slice_head_min_bytes;
   return c->head_stream >= (big_head ? 1 : 2) && c->sms > 0 && (size_t)2 * c->sms <= head_partial_count(m.c.vocab) && c->cfg.dtype == BILD_BF16 &&
@@ -1408,7 +1408,7 @@ int decoder_pass(bild_ctx* c, int which, int MBv, float* logits_dbg, unsigned lo
   };
   const int head_tr = (MB == 1 && d <= 512) ? 32 : 16;   // rows per tile of the tensor-core head
   const size_t sh_smem = slice_head_smem_bytes(d, head_tr);
-  // single-row passes: only heads of 32 MB and more (smaller ones stay on the GEMV head)
+  // the others, in single-row passes: the tensor-core head from slice_head_min_bytes on (slice_head = 2), the GEMV head below
   const bool big_head = (size_t)mc.vocab * d * 2 >= c->slice_head_min_bytes;
   if (MB == 1 && uses_head_stream(c, m)) {
     CUDA_TRY(c, launch_head_stream(c, h, c->sms));   // single row: the vocabulary streamed through registers
