@@ -27,7 +27,8 @@
  *     throws, never aborts.  After an error the context is usable again after
  *     bild_encode.  bild_last_error gives a message for the last failing call.
  *   - All work is enqueued on the CUDA stream given to bild_create.  Calls that
- *     return results in host memory synchronise that stream before returning.
+ *     return results in host memory synchronise that stream before returning, or, the
+ *     single-step calls, wait until their results are complete.
  *   - A context is not thread-safe; use one context per host thread.
  */
 #ifndef BILD_H
@@ -219,8 +220,8 @@ typedef struct {
                               * is dropped if one ends otherwise (tokens, trace and counts are those of the serial loop).  Blocks of
                               * two and more rows that wait together are judged in one pass of up to 16 rows, at the precision each
                               * has alone, where the kernels add in no fixed order anyway (fused = 3, bf16).
-                              * 0, and with graph_switch = 0 or host_loop = 1: the serial loop, 1 to 2 % faster for two models
-                              * that never agree (unrelated random ones), a fifth slower for a pair that mostly does */
+                              * 0, and with graph_switch = 0 or host_loop = 1: the serial loop, 0 to 2 % faster for two models
+                              * that never agree (unrelated random ones), 30 to 40 % slower for a pair that mostly does */
 } bild_tuning;
 void bild_tuning_default(bild_tuning *t /*HOST out*/);
 /* bild_create with explicit switches; tuning == NULL means the defaults. */

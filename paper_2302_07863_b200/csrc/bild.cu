@@ -1794,8 +1794,8 @@ int step_rows(int k) { return k == 1 ? 1 : k <= SUB_MB ? SUB_MB : MAXB; }   // r
 // The graph of a kind of single-step call is built while the GPU is at the plain launches of its first calls: recorded behind the first,
 // instantiated behind the second.  The host would only wait meanwhile, so that no call pays for it whose pass is longer than the build
 // (T5 pair, us: recording 30, for 9 to 16 rows 65; instantiation 85 small step, 140, 9 to 16 rows 280).  Calls one to four, host to host:
-// small step 146, 138, 114, 98, pass of 5 rows 548, 562, 533, 535; with all of it in front of the second call's pass 115, 278, 98, 98 and
-// 546, 747, 536, 533.  A failure leaves the kind on plain launches.
+// small step 134, 128, 98, 80, pass of 5 rows 539, 533, 506, 506 (with earlier kernels 146, 138, 114, 98 and 548, 562, 533, 535, where all of it in front of
+// the second call's pass was 115, 278, 98, 98 and 546, 747, 536, 533).  A failure leaves the kind on plain launches.
 void step_graph_build(bild_ctx* c, bild_ctx::StepGraph& s, int which, int MBv) {
   bool ok = true;
   if (++s.calls == 1) {
@@ -1821,7 +1821,7 @@ bool may_poll() {
 // rewind in front among them) lie in pinned memory, which the pass's first kernel reads: one graph launch from the third call of a kind on (19 or
 // 73 launches cost the host 45 or 170 us), whose last kernel writes the results back.  The state is read back first only if a loop may have
 // moved it.  T5-small step behind a rewind, host to host: with launches and two read-backs 143 us, launches alone 115, a kernel each for the
-// rewind and the call's arguments in front of the graph and a synchronisation behind it 101, now 92 (the pass alone: 78).
+// rewind and the call's arguments in front of the graph and a synchronisation behind it 101, this 92 (the pass alone: 78); with the present kernels 82 (72).
 int step_call(bild_ctx* c, int which, const int32_t* tokens, int k, float alpha, float* logits_dbg) {
   if (!c->len_known) {
     int rc = read_state(c);

@@ -593,7 +593,7 @@ __device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk
 // Measured, T5-large shapes, pass of 24 layers, cache 32, 512 encoder keys, before -> after this form of the kernels (both
 // sub-layer kernels; before: token rows and norm for the whole block, then products from shared memory, cluster barriers, scores,
 // soft-max and values with a block barrier each): 1 row 473 -> 355 us, 5 rows 632 -> 550 us, 8 rows 691 -> 597 us, 16 rows
-// 1080 -> 831 us; T5-small 100 -> 83 us.  With the steps noted at their places since: 340, 505, 557, 740 and 78 us.
+// 1080 -> 831 us; T5-small 100 -> 83 us.  With the steps noted at their places since: 311, 500, 552, 740 and 72 us.
 // WIDE: cross-attention of a block whose last keys of a chunk lie where the weight rows were (attn_sub_plan); a kernel of its own, since the
 // others would spill registers for it.
 // AHEAD (single rows): asks for some of the LM head's weights on the way (head_share); instances of their own, since the few instructions cost
@@ -603,7 +603,8 @@ __device__ __forceinline__ void sub_attend_block(const SubQ8& q, int dkv, int nk
 // trip count is a constant; the widths of 512, 768 and 1024, others go by DQ = 0.  These kernels are a chain of a few instructions at a time, so the index
 // arithmetic and the branches that go are time.  General kernels -> FIX -> with DQ: a step of the T5-small shapes 78.1 -> 74.0 -> 71.9 us, mT5-small
 // 117.9 -> 113.4 -> 109.2, single-row pass of T5-large 336.6 -> 327.2 -> 311.3, mT5-large 397.0 -> 392.8 -> 373.7.  The block kernels, at the limit of their
-// registers, spill some with FIX (5 rows 502 -> 522 us) and take every shape.
+// registers, spill some with FIX, head width and cluster size
+// together (5 rows 502 -> 522 us; DQ or KIND by itself was not tried there but for WIDE), and take every shape.
 constexpr int SUB_CROSS = 0, SUB_SELF = 1, SUB_EITHER = 2;
 template <bool ONE, bool WIDE = false, bool AHEAD = false, bool FIX = false, int KIND = SUB_EITHER, int DQ = 0>
 __global__ void __launch_bounds__(SUB_THREADS, 2) attn_sub_kernel(const AttnSubArgs a) {
